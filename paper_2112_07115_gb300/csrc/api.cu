@@ -244,18 +244,25 @@ struct dcem_scene {
   WedgeF* wedgesf = nullptr;   // ... the same in FP32
   WedgeTopo* wtopo = nullptr;  // ... and topology
   int nw = 0;
-  int* wperm = nullptr;        // wedge clusters: the wedges in spatial order, 32 per cluster,
-  float* wcbox = nullptr;      // and the clusters' boxes (per frame)
+  int* wperm = nullptr;        // the wedges in spatial order (mask words of 32),
+  float* wgbox = nullptr;      // and the boxes of the groups of 8 (per frame)
   int nwc = 0;
   bool diffraction = false;
   unsigned long long* dsurv = nullptr;  // diffraction: pre-test survivor list
   RPlane* rplanes = nullptr;   // diffraction combined with a reflection: reflector planes
   int* rmembers = nullptr;     // ... their triangle ids and sort keys
   float* rkeys = nullptr;
+  float4* quads = nullptr;     // ... and per triangle the wall quad it is part of (wall_quads)
+  unsigned* vis = nullptr;     // ... what each end point may see (k_refl_visible), and its words
+  size_t vis_cap = 0;
   int nrp = 0;
   int diff_refl = 0;               // reflections with diffraction (0..3, see the header)
   unsigned* rmask = nullptr;   // two reflections: the pre-test's wedge masks, and their words
   size_t rmask_cap = 0;
+  unsigned* wobs = nullptr;    // ... per wedge the receivers' sides: count, start, next slot (3 nw)
+  DiffObs* dobs = nullptr;     // ... and their list
+  unsigned dobs_cap = 0;
+  unsigned long long* dexact = nullptr;  // survivors past the occlusion test (dsurv_cap slots)
   unsigned dsurv_cap = 0;
   int diff_order = 1;          // diffraction: most wedges on one path (1-3)
   int4* dseq2 = nullptr;       // ... the frame's wedge pairs and triples, the pair relation
@@ -397,8 +404,8 @@ void scene_free(dcem_scene* s) {
   dfree(s->tri_mat_d); dfree(s->v9d); dfree(s->nodes); dfree(s->qnodes); dfree(s->qframe);
   dfree(s->q4_kid); dfree(s->q4_src); dfree(s->q4_count); dfree(s->q4_roots); dfree(s->q4_scr); dfree(s->leaf_parent); dfree(s->arrive);
   dfree(s->dsched); dfree(s->dlvl); dfree(s->tri_obj_d); dfree(s->wedges); dfree(s->wedgesf); dfree(s->wtopo);
-  dfree(s->wperm); dfree(s->wcbox); dfree(s->dsurv);
-  dfree(s->rplanes); dfree(s->rmembers); dfree(s->rkeys); dfree(s->rmask);
+  dfree(s->wperm); dfree(s->wgbox); dfree(s->dsurv); dfree(s->dexact); dfree(s->wobs); dfree(s->dobs);
+  dfree(s->rplanes); dfree(s->rmembers); dfree(s->rkeys); dfree(s->rmask); dfree(s->quads); dfree(s->vis);
   dfree(s->dseq2); dfree(s->dseq3); dfree(s->drel);
   dfree(s->g_items); dfree(s->g_param); dfree(s->g_out); dfree(s->g_err); dfree(s->g_paths);
   dfree(s->g_rx); dfree(s->g_theta);
@@ -635,12 +642,30 @@ int ensure_rx(dcem_scene* s, int nrx, int nlinks, int bucket_cap) {
   return DCEM_OK;
 }
 
-// The wedge masks of the two-reflection pre-test (k_refl2_masks): one word
-// per (end point: ntx transmitters and nrx receivers, reflector plane or
-// none, wedge cluster).
+// The wedge masks of the two-reflection pre-test (k_refl_single): one word
+// per (end point: ntx transmitters and nrx receivers, reflector plane, wedge
+// cluster); and the list of the receivers' sides by wedge (grown on demand).
+// Words before the end points' rows: the any-words of both sides and the
+// lists of their groups.
+static size_t vis_head(const dcem_scene* s) {
+  return 2 * (size_t)s->nwc + 2 * (size_t)((s->nw + kWedgeGroup - 1) / kWedgeGroup + 1);
+}
 static int ensure_rmask(dcem_scene* s, int ntx, int nrx) {
-  if (!(s->diffraction && s->nw > 0 && s->diff_refl >= 2 && s->nrp > 0)) return DCEM_OK;
-  const size_t need = (size_t)(ntx + nrx) * (size_t)(s->nrp + 1) * (size_t)s->nwc;
+  if (!(s->diffraction && s->nw > 0 && s->diff_refl >= 1 && s->nrp > 0)) return DCEM_OK;
+  const size_t words = (size_t)(ntx + nrx) * (size_t)((s->nrp + 31) / 32 + s->nwc) + vis_head(s);
+  if (words > s->vis_cap) {
+    dfree(s->vis);
+    s->vis_cap = 0;
+    CK(dalloc(&s->vis, words));
+    s->vis_cap = words;
+  }
+  if (s->diff_refl < 2) return DCEM_OK;
+  const size_t need = (size_t)(ntx + nrx) * (size_t)s->nrp * (size_t)s->nwc;
+  if (!s->wobs) CK(dalloc(&s->wobs, 3 * (size_t)s->nw));
+  if (!s->dobs) {
+    CK(dalloc(&s->dobs, (size_t)16384));
+    s->dobs_cap = 16384;
+  }
   if (s->rmask && need <= s->rmask_cap) return DCEM_OK;
   if (need > ((size_t)1 << 31)) return DCEM_ERR_CAPACITY;
   dfree(s->rmask);
@@ -853,6 +878,98 @@ void group_planes(const std::vector<float>& tris, const std::vector<int>& tri_ob
     planes.push_back(p);
     i = j;
   }
+  // in spatial order (the Morton code of the boxes' middles, 10 bits per
+  // axis), so that neighbouring lanes take neighbouring planes
+  double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
+  auto mid = [](const RPlane& p, int k) { return 0.5 * ((double)p.box[k] + p.box[k + 3]); };
+  for (const RPlane& p : planes)
+    for (int k = 0; k < 3; ++k) {
+      lo[k] = std::min(lo[k], mid(p, k));
+      hi[k] = std::max(hi[k], mid(p, k));
+    }
+  auto code = [&](const RPlane& p) {
+    uint64_t m = 0;
+    for (int k = 0; k < 3; ++k) {
+      const double u = hi[k] > lo[k] ? (mid(p, k) - lo[k]) / (hi[k] - lo[k]) : 0.0;
+      const uint64_t q = (uint64_t)std::min(1023.0, std::max(0.0, std::floor(u * 1024.0)));
+      for (int b = 0; b < 10; ++b) m |= ((q >> b) & 1ull) << (3 * b + k);
+    }
+    return m;
+  };
+  std::stable_sort(planes.begin(), planes.end(), [&](const RPlane& x, const RPlane& y) { return code(x) < code(y); });
+}
+
+// Per triangle the convex quad it forms with a coplanar neighbour (both
+// static, of one plane group, sharing an edge with identical vertices): the
+// neighbour that gives the largest one; corners in order, .w of the first 1.
+// A triangle without such a neighbour is its own quad (last corner doubled);
+// moving triangles have none (.w 0).
+std::vector<float4> wall_quads(const std::vector<float>& tris, const std::vector<int>& tri_obj,
+                               const std::vector<RPlane>& planes, const std::vector<int>& members) {
+  const int ntri = (int)tri_obj.size();
+  std::vector<float4> out(4 * (size_t)std::max(ntri, 1), make_float4(0.f, 0.f, 0.f, 0.f));
+  typedef std::array<float, 3> V;
+  struct Edge {
+    int plane;
+    V a, b;
+    int tri, k;  // edge from vertex k to k + 1
+  };
+  std::vector<Edge> e;
+  auto vert = [&](int t, int k) {
+    const float* p = &tris[9 * (size_t)t + 3 * (k % 3)];
+    return V{p[0], p[1], p[2]};
+  };
+  auto put = [&](int t, const V* c) {
+    for (int k = 0; k < 4; ++k) out[4 * (size_t)t + k] = make_float4(c[k][0], c[k][1], c[k][2], k == 0 ? 1.0f : 0.0f);
+  };
+  for (int i = 0; i < ntri; ++i) {
+    if (tri_obj[i] >= 0) continue;
+    const V c[4] = {vert(i, 0), vert(i, 1), vert(i, 2), vert(i, 2)};
+    put(i, c);
+  }
+  for (size_t p = 0; p < planes.size(); ++p)
+    for (int m = planes[p].first; m < planes[p].first + planes[p].count; ++m)
+      for (int k = 0; k < 3; ++k) {
+        V a = vert(members[m], k), b = vert(members[m], k + 1);
+        if (b < a) std::swap(a, b);
+        e.push_back(Edge{(int)p, a, b, members[m], k});
+      }
+  std::sort(e.begin(), e.end(), [](const Edge& x, const Edge& y) {
+    if (x.plane != y.plane) return x.plane < y.plane;
+    if (x.a != y.a) return x.a < y.a;
+    if (x.b != y.b) return x.b < y.b;
+    return x.tri < y.tri;
+  });
+  std::vector<double> best(ntri, 0.0);
+  for (size_t i = 0; i + 1 < e.size(); ++i) {
+    const Edge &x = e[i], &y = e[i + 1];
+    if (x.plane != y.plane || x.a != y.a || x.b != y.b || x.tri == y.tri) continue;
+    // corners around the union: x's edge start, y's far vertex, x's edge end, x's far vertex
+    const V c[4] = {vert(x.tri, x.k), vert(y.tri, y.k + 2), vert(x.tri, x.k + 1), vert(x.tri, x.k + 2)};
+    const double* n = planes[x.plane].n;
+    int pos = 0, neg = 0;
+    double area = 0.0;
+    for (int k = 0; k < 4; ++k) {
+      const V &a = c[k], &b = c[(k + 1) & 3], &d = c[(k + 2) & 3];
+      const double u[3] = {(double)b[0] - a[0], (double)b[1] - a[1], (double)b[2] - a[2]};
+      const double v[3] = {(double)d[0] - b[0], (double)d[1] - b[1], (double)d[2] - b[2]};
+      const double w = n[0] * (u[1] * v[2] - u[2] * v[1]) + n[1] * (u[2] * v[0] - u[0] * v[2]) +
+                       n[2] * (u[0] * v[1] - u[1] * v[0]);
+      const double lu = std::sqrt(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+      const double lv = std::sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+      if (w > 1e-6 * lu * lv) ++pos;
+      else if (w < -1e-6 * lu * lv) ++neg;
+      area += w;
+    }
+    if (pos != 4 && neg != 4) continue;  // not convex
+    area = std::fabs(area);
+    for (int t : {x.tri, y.tri})
+      if (area > best[t]) {
+        best[t] = area;
+        put(t, c);
+      }
+  }
+  return out;
 }
 
 bool same_traversal(const dcem_params& a, const dcem_params& b) {
@@ -1312,13 +1429,14 @@ int dcem_scene_set_diffraction(dcem_scene* s, int32_t on, int32_t* n_wedges) {
       CK(dalloc(&s->wedges, s->nw));
       CK(dalloc(&s->wedgesf, s->nw));
       CK(dalloc(&s->wperm, s->nw));
-      CK(dalloc(&s->wcbox, 6 * (size_t)s->nwc));
+      CK(dalloc(&s->wgbox, 6 * (size_t)((s->nw + kWedgeGroup - 1) / kWedgeGroup)));
       CK(cudaMemcpy(s->wtopo, w.data(), sizeof(WedgeTopo) * w.size(), cudaMemcpyHostToDevice));
       CK(cudaMemcpy(s->wperm, perm.data(), sizeof(int) * perm.size(), cudaMemcpyHostToDevice));
     }
   }
   if (on && s->nw && !s->dsurv) {  // grown (and the frame traced again) when a frame needs more
     CK(dalloc(&s->dsurv, (size_t)1024));
+    CK(dalloc(&s->dexact, (size_t)1024));
     s->dsurv_cap = 1024;
   }
   s->diffraction = on != 0;
@@ -1342,6 +1460,9 @@ int dcem_scene_set_diffraction_reflections(dcem_scene* s, int32_t on, int32_t* n
       CK(cudaMemcpy(s->rplanes, planes.data(), sizeof(RPlane) * planes.size(), cudaMemcpyHostToDevice));
       CK(cudaMemcpy(s->rmembers, members.data(), sizeof(int) * members.size(), cudaMemcpyHostToDevice));
       CK(cudaMemcpy(s->rkeys, keys.data(), sizeof(float) * keys.size(), cudaMemcpyHostToDevice));
+      const std::vector<float4> quads = wall_quads(s->tris_h, s->tri_obj_h, planes, members);
+      CK(dalloc(&s->quads, quads.size()));
+      CK(cudaMemcpy(s->quads, quads.data(), sizeof(float4) * quads.size(), cudaMemcpyHostToDevice));
     }
   }
   s->diff_refl = on;
@@ -1605,9 +1726,10 @@ static void make_plan(dcem_scene* s, int nrx, const dcem_params* p, bool coheren
   q.wtopo = s->wtopo;
   q.nw = s->nw;
   q.wperm = s->wperm;
-  q.wcbox = s->wcbox;
+  q.wgbox = s->wgbox;
   q.nwc = s->nwc;
   q.dsurv = s->dsurv;
+  q.dexact = s->dexact;
   q.dsurv_cap = s->dsurv_cap;
   const bool dr = q.wedges && s->diff_refl && s->nrp > 0;
   q.rplanes = dr ? s->rplanes : nullptr;
@@ -1621,8 +1743,17 @@ static void make_plan(dcem_scene* s, int nrx, const dcem_params* p, bool coheren
   q.rmembers = dr ? s->rmembers : nullptr;
   q.rkeys = dr ? s->rkeys : nullptr;
   q.nrp = dr ? s->nrp : 0;
+  q.quads = dr ? s->quads : nullptr;
+  q.vis_any = dr ? s->vis : nullptr;
+  q.vis_grp = dr ? reinterpret_cast<int*>(s->vis + 2 * (size_t)s->nwc) : nullptr;
+  q.vis = dr ? s->vis + vis_head(s) : nullptr;
   q.drefl2 = dr && s->diff_refl >= 2 ? 1 : 0;
   q.rmask = q.drefl2 ? s->rmask : nullptr;
+  q.wobs_cnt = q.drefl2 ? s->wobs : nullptr;
+  q.wobs_off = q.drefl2 ? s->wobs + s->nw : nullptr;
+  q.wobs_pos = q.drefl2 ? s->wobs + 2 * (size_t)s->nw : nullptr;
+  q.dobs = q.drefl2 ? s->dobs : nullptr;
+  q.dobs_cap = q.drefl2 ? s->dobs_cap : 0;
   q.dmid = dr && s->diff_refl >= 3 && dord >= 2 ? 1 : 0;
   // sticky mode: the previous frame's kept paths (when the cache is valid),
   // and this frame's
@@ -1804,10 +1935,10 @@ static int capture_frame(dcem_scene* s, const FramePlan& P, FrameGraph& G) {
 static int diffraction_launches(const FramePlan& P) {
   const PathArgs& q = P.q;
   if (!q.wedges) return 0;
-  int n = 1 + (q.drefl2 && q.rplanes ? 1 : 0);  // wedge geometry, cluster boxes
+  int n = 1 + (q.rplanes ? 1 : 0);  // wedge geometry, cluster boxes
   if (P.nlinks > 0) {
-    n += 2;  // first-order pre-test, exact stage
-    if (q.rplanes) n += 1 + (q.drefl2 ? 2 : 0);  // one reflection; wedge masks, two reflections
+    n += 3;  // first-order pre-test, occlusion, exact stage
+    if (q.rplanes) n += 3 + (q.drefl2 ? 4 : 0);  // visibility, one reflection; two: room, lists, join, double
     if (q.diff_order >= 2 && q.nw > 1)  // relation, pairs, [pairs around a plane], [triples], chains
       n += q.diff_order + 1 + (q.dmid ? 1 : 0);
   }
@@ -1968,7 +2099,13 @@ static int frame_finish(dcem_scene* s, const float* tx, int32_t ntx, const float
         cap = (unsigned)want;
         return DCEM_OK;
       };
+      unsigned had = s->dsurv_cap;
       if ((rc = grow(c[0].n_dsurv, s->dsurv_cap, s->dsurv)) != DCEM_OK) return rc;
+      if (s->dsurv_cap != had) {
+        dfree(s->dexact);
+        CK(dalloc(&s->dexact, (size_t)s->dsurv_cap));
+      }
+      if (s->dobs && (rc = grow(c[0].n_dobs, s->dobs_cap, s->dobs)) != DCEM_OK) return rc;
       if (s->dseq2 && (rc = grow(c[0].n_dpair, s->dseq2_cap, s->dseq2)) != DCEM_OK) return rc;
       if (s->dseq3 && (rc = grow(c[0].n_dtrip, s->dseq3_cap, s->dseq3)) != DCEM_OK) return rc;
     }
@@ -2009,7 +2146,7 @@ static int frame_finish(dcem_scene* s, const float* tx, int32_t ntx, const float
     S.child_rays = (int32_t)std::min<unsigned long long>(sp, 0x7fffffffull);
   }
   S.keys_reused = (int32_t)c[0].n_val_reused;
-  S.diff_candidates = (int32_t)std::min(c[0].n_dsurv, 0x7fffffffu);
+  S.diff_candidates = (int32_t)std::min(c[0].n_dexact, 0x7fffffffu);
   S.diff_pairs = (int32_t)std::min(c[0].n_dpair, 0x7fffffffu);
   S.diff_triples = (int32_t)std::min(c[0].n_dtrip, 0x7fffffffu);
   S.tri_tests = (int64_t)c[0].tri_tests;

@@ -54,7 +54,14 @@ struct WedgeF {
   float3 p0, e, t0, y0;
   float len, npi;
 };
-constexpr int kWedgeCluster = 32;  // wedges per cluster (a warp's lanes)
+// A receiver's image in plane p about a wedge: along the edge, off its line,
+// from its start, angle and the angle's tolerance (negative: not certain).
+struct DiffObs {
+  int rx, p;
+  float z, r, l, phi, tol, pad;
+};
+constexpr int kWedgeCluster = 32;  // wedges per mask word
+constexpr int kWedgeGroup = 8;     // wedges per box
 
 // Wedge topology (fixed for a rigid object): faces ta < tb, the local
 // indices of the edge's vertices in ta and of the faces' third vertices.
@@ -148,6 +155,8 @@ struct DevCounters {
   unsigned int n_val_reused;       // coherent frames: distinct keys whose validation was reused
   unsigned int n_dpair;            // diffraction of order >= 2: wedge pairs past the pre-test
   unsigned int n_dtrip;            // ... triples
+  unsigned int n_dobs;             // two reflections: the receivers' one-reflection sides of all wedges
+  unsigned int n_dexact;           // diffraction: candidates past the FP32 occlusion test
 };
 
 // Sticky mode: a valid path kept for the next frame (link, depth, sequence).

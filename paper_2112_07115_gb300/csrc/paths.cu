@@ -1015,13 +1015,15 @@ __global__ void k_wedge_geom(const float4* __restrict__ tris, const int* __restr
   }
 }
 
-// Each cluster's box (one warp per cluster of kWedgeCluster wedges in the
-// order perm): the min and max over its edges' two ends in FP32.
-__global__ void k_wedge_boxes(const WedgeF* __restrict__ wf, const int* __restrict__ perm, int nw, int nwc,
+// Each wedge group's box (kWedgeGroup wedges in the order perm, one lane
+// each): the min and max over its edges' two ends in FP32.
+__global__ void k_wedge_boxes(const WedgeF* __restrict__ wf, const int* __restrict__ perm, int nw,
                               float* __restrict__ box) {
-  const int lane = threadIdx.x & 31;
-  for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nwc; c += (gridDim.x * blockDim.x) >> 5) {
-    const int i = c * kWedgeCluster + lane;
+  const int lane = threadIdx.x & (kWedgeGroup - 1), ng = (nw + kWedgeGroup - 1) / kWedgeGroup;
+  // whole warps walk the groups (kWedgeGroup divides 32), so the shuffles below are complete
+  const int nwarp = (gridDim.x * blockDim.x) >> 5, per = 32 / kWedgeGroup;
+  for (int w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w0 * per < ng; w0 += nwarp) {
+    const int g = w0 * per + (threadIdx.x & 31) / kWedgeGroup, i = g * kWedgeGroup + lane;
     float lo[3] = {3e38f, 3e38f, 3e38f}, hi[3] = {-3e38f, -3e38f, -3e38f};
     if (i < nw) {
       const WedgeF f = wf[perm[i]];
@@ -1032,12 +1034,12 @@ __global__ void k_wedge_boxes(const WedgeF* __restrict__ wf, const int* __restri
         hi[k] = fmaxf(p[k], q[k]);
       }
     }
-    for (int o = 16; o > 0; o >>= 1)
+    for (int o = kWedgeGroup / 2; o > 0; o >>= 1)
       for (int k = 0; k < 3; ++k) {
         lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], o));
         hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
       }
-    if (lane < 6) box[6 * (size_t)c + lane] = lane < 3 ? lo[lane] : hi[lane - 3];
+    if (g < ng && lane < 6) box[6 * (size_t)g + lane] = lane < 3 ? lo[lane] : hi[lane - 3];
   }
 }
 
@@ -1212,33 +1214,6 @@ __device__ __forceinline__ bool diffract_refl_candidate(const WedgeF& W, const R
       X.y > P.box[4] + mb || X.z > P.box[5] + mb)
     return false;
   return true;
-}
-
-__global__ void __launch_bounds__(256) k_diffract_refl_pre(PathArgs a, int nlinks) {
-  const long total = (long)nlinks * a.nw * a.nrp * 2;
-  const int lane = threadIdx.x & 31;
-  const long stride = (long)gridDim.x * blockDim.x;
-  for (long base = (long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < total; base += stride) {
-    long idx = base + lane;
-    bool keep = false;
-    if (idx < total) {
-      long r = idx >> 1;
-      int p = (int)(r % a.nrp);
-      r /= a.nrp;
-      int w = (int)(r % a.nw), link = (int)(r / a.nw);
-      keep = diffract_refl_candidate(a.wf[w], a.rplanes[p], a.txs[link / a.nrx], a.rx[link % a.nrx],
-                                     (idx & 1) != 0);
-    }
-    unsigned m = __ballot_sync(0xffffffffu, keep);
-    if (!m) continue;
-    unsigned at = 0;
-    if (lane == 0) at = atomicAdd(&a.ctr->n_dsurv, (unsigned)__popc(m));
-    at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
-    if (keep) {
-      if (at < a.dsurv_cap) a.dsurv[at] = kReflTag | (unsigned long long)idx;
-      else atomicOr(&a.ctr->err, ERR_DIFF_OVERFLOW);
-    }
-  }
 }
 
 // Image, Keller point and reflection point for plane (n, c): false when the
@@ -1741,13 +1716,18 @@ __device__ __forceinline__ float3 chain_observer32(const PathArgs& a, int rho) {
 // inside its box? The legs fill the triangle S, A, B; its section by the
 // plane lies within the box of the crossings of its three sides, so the
 // answer is "no" when S, A and B lie on one side of the plane (by more than
-// the margin m), or when that box, widened by m, misses the plane's box.
-__device__ __forceinline__ bool plane_reachable(const RPlane& Pl, float3 S, float3 A, float3 B, float m) {
+// the margin m), or when that box, widened by m, misses the plane's box;
+// else [lo, hi] is the part of it (widened by m) that holds the crossings.
+__device__ __forceinline__ bool leg_window(const RPlane& Pl, float3 S, float3 A, float3 B, float m, float* lo,
+                                           float* hi) {
   const float3 n = f3(Pl.nf[0], Pl.nf[1], Pl.nf[2]);
   const float c = Pl.cf;
   const float ds = fdot3(n, S) - c, da = fdot3(n, A) - c, db = fdot3(n, B) - c;
   if ((ds > m && da > m && db > m) || (ds < -m && da < -m && db < -m)) return false;
-  float lo[3] = {3e38f, 3e38f, 3e38f}, hi[3] = {-3e38f, -3e38f, -3e38f};
+  for (int k = 0; k < 3; ++k) {
+    lo[k] = 3e38f;
+    hi[k] = -3e38f;
+  }
   bool any = false;
   const float3 P0[3] = {S, S, A}, P1[3] = {A, B, B};
   const float d0[3] = {ds, ds, da}, d1[3] = {da, db, db};
@@ -1772,9 +1752,17 @@ __device__ __forceinline__ bool plane_reachable(const RPlane& Pl, float3 S, floa
     any = true;
   }
   if (!any) return false;
-  for (int k = 0; k < 3; ++k)
-    if (hi[k] < Pl.box[k] - m || lo[k] > Pl.box[3 + k] + m) return false;
-  return true;
+  bool meet = true;
+  for (int k = 0; k < 3; ++k) {
+    lo[k] = fmaxf(lo[k], Pl.box[k]) - m;
+    hi[k] = fminf(hi[k], Pl.box[3 + k]) + m;
+    meet = meet && lo[k] <= hi[k];
+  }
+  return meet;
+}
+__device__ __forceinline__ bool plane_reachable(const RPlane& Pl, float3 S, float3 A, float3 B, float m) {
+  float lo[3], hi[3];
+  return leg_window(Pl, S, A, B, m, lo, hi);
 }
 
 // The relation of consecutive wedges in a chain, once per frame (moving
@@ -2984,37 +2972,48 @@ __device__ __noinline__ void diffract_multi(const PathArgs& a, unsigned long lon
 constexpr unsigned long long kRefl2Tag = kReflTag | (1ull << 61);
 constexpr unsigned long long kRefl2Mask = (1ull << 61) - 1ull;
 
-// Can a leg from S to some point of `box` cross plane P1 inside P1's box?
-// With every corner of the box across the plane from S, the legs' crossings
-// lie within the box of the corner legs' crossings; "no" when every corner
-// lies on S's side (no leg crosses the plane) or when the crossings' box,
-// widened by m, misses P1's box.
-__device__ __forceinline__ bool box_reachable(const RPlane& P1, float3 S, const float* box, float m) {
-  const float3 n = f3(P1.nf[0], P1.nf[1], P1.nf[2]);
-  const float c = P1.cf;
-  const float ds = fdot3(n, S) - c;
-  if (fabsf(ds) <= m) return true;
-  float lo[3] = {3e38f, 3e38f, 3e38f}, hi[3] = {-3e38f, -3e38f, -3e38f};
-  int same = 0;
-  for (int q = 0; q < 8; ++q) {
-    const float3 X = f3((q & 1) ? box[3] + m : box[0] - m, (q & 2) ? box[4] + m : box[1] - m,
-                        (q & 4) ? box[5] + m : box[2] - m);
-    const float dx = fdot3(n, X) - c;
-    if (fabsf(dx) <= m) return true;
-    if ((dx > 0.0f) == (ds > 0.0f)) {
-      ++same;
-      continue;
+// Where the legs from S to the points of `box` (lo, hi) cross plane P inside
+// P's box: false when none can, else [lo, hi] becomes a box that holds every
+// such crossing. Legs to the corners across the plane from S bound the
+// crossings of the box's part there; where the plane cuts the box (a corner
+// on S's side, or within m of the plane), the cut is itself a set of
+// crossings, bounded by the box. No conclusion for S within m of the plane.
+__device__ __forceinline__ bool box_window(const RPlane& P, float3 S, float m, float* lo, float* hi) {
+  const float3 n = f3(P.nf[0], P.nf[1], P.nf[2]);
+  const float ds = fdot3(n, S) - P.cf;
+  if (fabsf(ds) <= m) {
+    for (int k = 0; k < 3; ++k) {
+      lo[k] = P.box[k];
+      hi[k] = P.box[3 + k];
     }
-    const float t = ds / (ds - dx);
-    const float x = S.x + t * (X.x - S.x), y = S.y + t * (X.y - S.y), z = S.z + t * (X.z - S.z);
-    lo[0] = fminf(lo[0], x); lo[1] = fminf(lo[1], y); lo[2] = fminf(lo[2], z);
-    hi[0] = fmaxf(hi[0], x); hi[1] = fmaxf(hi[1], y); hi[2] = fmaxf(hi[2], z);
+    return true;
   }
-  if (same == 8) return false;
-  if (same > 0) return true;
-  for (int k = 0; k < 3; ++k)
-    if (hi[k] < P1.box[k] - m || lo[k] > P1.box[3 + k] + m) return false;
-  return true;
+  float wl[3] = {3e38f, 3e38f, 3e38f}, wh[3] = {-3e38f, -3e38f, -3e38f};
+  bool any = false, cut = false;
+#pragma unroll 2  // (the kernels that inline this are bound by instruction fetch)
+  for (int q = 0; q < 8; ++q) {
+    const float3 X = f3((q & 1) ? hi[0] + m : lo[0] - m, (q & 2) ? hi[1] + m : lo[1] - m, (q & 4) ? hi[2] + m : lo[2] - m);
+    const float dx = fdot3(n, X) - P.cf, sd = ds > 0.0f ? dx : -dx;  // sd > 0: on S's side
+    if (sd >= -m) cut = true;
+    if (sd > m) continue;
+    any = true;
+    const float t = fminf(fmaxf(ds / (ds - dx), 0.0f), 1.0f);
+    const float x = S.x + t * (X.x - S.x), y = S.y + t * (X.y - S.y), z = S.z + t * (X.z - S.z);
+    wl[0] = fminf(wl[0], x); wl[1] = fminf(wl[1], y); wl[2] = fminf(wl[2], z);
+    wh[0] = fmaxf(wh[0], x); wh[1] = fmaxf(wh[1], y); wh[2] = fmaxf(wh[2], z);
+  }
+  if (!any) return false;
+  bool meet = true;
+  for (int k = 0; k < 3; ++k) {
+    if (cut) {
+      wl[k] = fminf(wl[k], lo[k] - m);
+      wh[k] = fmaxf(wh[k], hi[k] + m);
+    }
+    lo[k] = fmaxf(wl[k], P.box[k]) - m;
+    hi[k] = fminf(wh[k], P.box[3 + k]) + m;
+    meet = meet && lo[k] <= hi[k];
+  }
+  return meet;
 }
 
 // The crossing X of the unfolded leg a0 -> a1 with plane P, within margins
@@ -3072,60 +3071,17 @@ __device__ __forceinline__ bool refl2_candidate(const WedgeF& W, const RPlane& P
   return diffract_candidate(W, make_float4(S.x, S.y, S.z, 0.0f), make_float4(O.x, O.y, O.z, 0.0f));
 }
 
-static_assert(kWedgeCluster == 32, "a wedge cluster is one warp's lanes and one mask word");
-
-// Wedge masks of the two-reflection pre-test, per frame. For every end point
-// X (the transmitters, then the receivers) and plane p, bit i of word
-// (X, p, c) is set when the i-th wedge of cluster c could take part in a
-// path with a reflection on p next to X: X's image in p outside the wedge,
-// and some leg from the image to the edge crossing p inside its box
-// (plane_reachable). Plane index nrp stands for no reflection: X itself
-// outside the wedge. A path with one reflection on each side of the wedge
-// needs its wedge in the transmitter's mask for p1 and the receiver's for
-// p2; one with both reflections on one side, in the other end point's mask
-// for no reflection.
-__global__ void __launch_bounds__(256) k_refl2_masks(PathArgs a, int ntx) {
-  const int np1 = a.nrp + 1;
-  const long nitem = (long)(ntx + a.nrx) * np1 * a.nwc;
-  const int lane = threadIdx.x & 31;
-  const long nwarp = (long)gridDim.x * (blockDim.x >> 5);
-  for (long it = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < nitem; it += nwarp) {
-    const int c = (int)(it % a.nwc);
-    const long r = it / a.nwc;
-    const int p = (int)(r % np1), x = (int)(r / np1);
-    const float4 xv = x < ntx ? a.txs[x] : a.rx[x - ntx];
-    float3 X = f3(xv.x, xv.y, xv.z);
-    const int i = c * kWedgeCluster + lane;
-    bool bit = false;
-    if (i < a.nw) {
-      const WedgeF W = a.wf[a.wperm[i]];
-      if (p == a.nrp) {
-        bit = !surely_inside(W, X);
-      } else {
-        const RPlane& Pl = a.rplanes[p];
-        X = mirror32(X, f3(Pl.nf[0], Pl.nf[1], Pl.nf[2]), Pl.cf);
-        float3 A, B;
-        edge_ends(W, A, B);
-        const float mg = 0.1f + 1e-4f * (fabsf(X.x) + fabsf(X.y) + fabsf(X.z) + W.len);
-        bit = plane_reachable(Pl, X, A, B, mg) && !surely_inside(W, X);
-      }
-    }
-    const unsigned mk = __ballot_sync(0xffffffffu, bit);
-    if (lane == 0) a.rmask[it] = mk;
-  }
-}
+static_assert(kWedgeCluster == 32 && kWedgeGroup == 8, "a mask word holds four groups, a warp four octets");
 
 // The images of block (kind, link, p1, p2): S, O the diffraction's source
 // and observer, S1 the transmitter's image in P1 (kind 0), O1 the
-// receiver's image in P2 (kind 2); m the block's margin.
+// receiver's image in P2 (kind 2).
 __device__ __forceinline__ void refl2_images(const PathArgs& a, int kind, int link, const RPlane& P1,
-                                             const RPlane& P2, float3& S, float3& S1, float3& O, float3& O1,
-                                             float& m) {
+                                             const RPlane& P2, float3& S, float3& S1, float3& O, float3& O1) {
   const float4 tv = a.txs[link / a.nrx], rv = a.rx[link % a.nrx];
   const float3 T = f3(tv.x, tv.y, tv.z), R = f3(rv.x, rv.y, rv.z);
   const float3 n1 = f3(P1.nf[0], P1.nf[1], P1.nf[2]);
   const float3 n2 = f3(P2.nf[0], P2.nf[1], P2.nf[2]);
-  m = 0.1f + 1e-4f * (fabsf(T.x) + fabsf(T.y) + fabsf(T.z) + fabsf(R.x) + fabsf(R.y) + fabsf(R.z));
   S = S1 = T;
   O = O1 = R;
   if (kind == 0) {
@@ -3140,131 +3096,716 @@ __device__ __forceinline__ void refl2_images(const PathArgs& a, int kind, int li
   }
 }
 
-// Block b's parts: kind, link and the two planes (32-bit division when b fits).
-__device__ __forceinline__ void refl2_block(const PathArgs& a, int nlinks, long b, int& kind, int& link, int& p1,
-                                            int& p2) {
-  if (b < 0x7fffffffL) {
-    unsigned r = (unsigned)b;
-    p2 = (int)(r % (unsigned)a.nrp);
-    r /= (unsigned)a.nrp;
-    p1 = (int)(r % (unsigned)a.nrp);
-    r /= (unsigned)a.nrp;
-    link = (int)(r % (unsigned)nlinks);
-    kind = (int)(r / (unsigned)nlinks);
+// Survivor codes of one and two reflections around a first-order diffraction.
+__device__ __forceinline__ unsigned long long refl1_code(const PathArgs& a, int link, int w, int p, bool first) {
+  return kReflTag | ((((unsigned long long)link * a.nw + w) * a.nrp + p) * 2 + (first ? 1 : 0));
+}
+__device__ __forceinline__ unsigned long long refl2_code(const PathArgs& a, int nlinks, int kind, int link, int p1,
+                                                         int p2, int w) {
+  const unsigned long long b = (((unsigned long long)kind * nlinks + link) * a.nrp + p1) * a.nrp + p2;
+  return kRefl2Tag | (b * a.nw + w);
+}
+struct ReflCand {
+  int kind, link, w, p1, p2;  // kind 0-2 as above; 3: one reflection (p1) before the wedge, 4: after it
+};
+__device__ __forceinline__ ReflCand refl_decode(const PathArgs& a, int nlinks, unsigned long long code) {
+  ReflCand c;
+  if ((code >> 61) & 1ull) {
+    unsigned long long v = code & kRefl2Mask;
+    c.w = (int)(v % (unsigned)a.nw);
+    v /= (unsigned)a.nw;
+    c.p2 = (int)(v % (unsigned)a.nrp);
+    v /= (unsigned)a.nrp;
+    c.p1 = (int)(v % (unsigned)a.nrp);
+    v /= (unsigned)a.nrp;
+    c.link = (int)(v % (unsigned)nlinks);
+    c.kind = (int)(v / (unsigned)nlinks);
   } else {
-    long r = b;
-    p2 = (int)(r % a.nrp);
-    r /= a.nrp;
-    p1 = (int)(r % a.nrp);
-    r /= a.nrp;
-    link = (int)(r % nlinks);
-    kind = (int)(r / nlinks);
+    unsigned long long v = code & ~kReflTag;
+    c.kind = (v & 1ull) ? 3 : 4;
+    v >>= 1;
+    c.p1 = c.p2 = (int)(v % (unsigned)a.nrp);
+    v /= (unsigned)a.nrp;
+    c.w = (int)(v % (unsigned)a.nw);
+    c.link = (int)(v / (unsigned)a.nw);
+  }
+  return c;
+}
+
+// ---- candidates by end point ----
+// The candidates (link, wedge, planes) are a product of two sides that are
+// nearly independent: the transmitter's image after 0, 1 or 2 reflections
+// against a wedge, and the receiver's. Forming each side once and joining
+// the two at the wedge costs a few percent of testing every (kind, link,
+// plane pair) block on its own (8 x 8 city blocks, 64 receivers, 321 planes:
+// 19.8M blocks, 24.5 ms; this form 1.2 ms in all):
+//   k_refl_visible the planes and wedges each end point may see at all
+//   k_refl_single  every (end point, plane): the wedges that the image sees
+//                  through the plane's box. Such a side with no reflection
+//                  on the other end gives the one-reflection candidates;
+//                  with two reflections on, the sets are also kept as mask
+//                  words and the receivers' sides counted per wedge
+//   k_refl_lists   the receivers' one-reflection sides listed by wedge
+//   k_refl_join    every transmitter side with one reflection against its
+//                  wedge's list: one reflection on each side of the wedge
+//   k_refl_double  every (end point, plane, plane): the wedges that the
+//                  double image sees, against the other ends: both
+//                  reflections on one side
+// The joins apply the closed-form Keller point and the angle rules
+// (side_pair, the rules of diffract_candidate on precomputed sides); what
+// passes goes through the full FP32 test (refl_candidates_take).
+
+// A point about a wedge: along the edge, off the edge line, from the edge's
+// start, and its angle (sure: tol >= 0).
+struct WedgeSide {
+  float z, r, l, phi, tol;
+};
+__device__ __forceinline__ void side_zr(const WedgeF& W, float3 X, WedgeSide& s, float3& p) {
+  const float3 d = f3(X.x - W.p0.x, X.y - W.p0.y, X.z - W.p0.z);
+  s.z = fdot3(d, W.e);
+  p = f3(d.x - W.e.x * s.z, d.y - W.e.y * s.z, d.z - W.e.z * s.z);
+  s.r = sqrtf(fdot3(p, p));
+  s.l = sqrtf(fdot3(d, d));
+}
+__device__ __forceinline__ void side_angle(const WedgeF& W, float3 p, WedgeSide& s) {
+  bool sure;
+  s.phi = wedge_angle32(p, W.t0, W.y0, s.r, s.l, sure, s.tol);
+  if (!sure) s.tol = -1.0f;
+}
+__device__ __forceinline__ WedgeSide wedge_side(const WedgeF& W, float3 X) {
+  WedgeSide s;
+  float3 p;
+  side_zr(W, X, s, p);
+  side_angle(W, p, s);
+  return s;
+}
+// The Keller point of two sides within the edge (margins of diffract_candidate)?
+__device__ __forceinline__ bool side_keller(float len, const WedgeSide& s, const WedgeSide& o) {
+  if (!(s.r > 1e-3f && o.r > 1e-3f)) return true;
+  const float zq = s.z + (o.z - s.z) * s.r / (s.r + o.r);
+  const float mz = 0.05f + 1e-5f * (s.l + o.l);
+  return !(zq < -mz || zq > len + mz);
+}
+// ... and the angle rules (the angles of both sides known)?
+__device__ __forceinline__ bool side_rules(float npi, const WedgeSide& s, const WedgeSide& o) {
+  if (!(s.r > 1e-3f && o.r > 1e-3f)) return true;
+  const bool ss = s.tol >= 0.0f, so = o.tol >= 0.0f;
+  if ((ss && s.phi > npi + s.tol) || (so && o.phi > npi + o.tol)) return false;
+  return !(ss && so && fabsf(o.phi - s.phi) < 3.14159265f - (s.tol + o.tol));
+}
+
+// Does an image X (of an end point, in plane Pl last) see wedge W: the
+// wedge not facing away, and some leg to its edge crossing Pl in its box?
+// For a double image, the legs must also have crossed the first plane Pf on
+// their way from the single image Xf to the crossings with Pl.
+__device__ __forceinline__ bool image_sees(const RPlane& Pl, const WedgeF& W, float3 X, const RPlane* Pf, float3 Xf) {
+  float3 A, B;
+  edge_ends(W, A, B);
+  const float mg = 0.1f + 1e-4f * (fabsf(X.x) + fabsf(X.y) + fabsf(X.z) + W.len);
+  float lo[3], hi[3];
+  return leg_window(Pl, X, A, B, mg, lo, hi) && (!Pf || box_window(*Pf, Xf, mg, lo, hi)) && !surely_inside(W, X);
+}
+// ... and a group of wedges, by its box.
+__device__ __forceinline__ bool image_sees_group(const PathArgs& a, const RPlane& Pl, int g, float3 X, float m,
+                                                 const RPlane* Pf, float3 Xf) {
+  const float* gb = a.wgbox + 6 * (size_t)g;
+  float lo[3] = {gb[0], gb[1], gb[2]}, hi[3] = {gb[3], gb[4], gb[5]};
+  return box_window(Pl, X, m, lo, hi) && (!Pf || box_window(*Pf, Xf, m, lo, hi));
+}
+// The next four of the lanes in mask `gm`, whose groups are g, to the warp's
+// four octets: this lane's place in the wedge order, -1 for none.
+__device__ __forceinline__ int octet_wedge(const PathArgs& a, int g, unsigned& gm) {
+  const int lane = threadIdx.x & 31;
+  int src = -1;
+  for (int k = 0; k < 4 && gm; ++k, gm &= gm - 1u)
+    if (lane >> 3 == k) src = __ffs(gm) - 1;
+  const int i = __shfl_sync(0xffffffffu, g, max(src, 0)) * kWedgeGroup + (lane & 7);
+  return src >= 0 && i < a.nw ? i : -1;
+}
+__device__ __forceinline__ float3 plane_image(const RPlane& P, float3 X) {
+  return mirror32(X, f3(P.nf[0], P.nf[1], P.nf[2]), P.cf);
+}
+__device__ __forceinline__ float3 end_point(const PathArgs& a, int ntx, int x) {
+  const float4 v = x < ntx ? a.txs[x] : a.rx[x - ntx];
+  return f3(v.x, v.y, v.z);
+}
+__device__ __forceinline__ float image_margin(float3 X, float3 Y) {
+  return 0.1f + 1e-4f * (fabsf(X.x) + fabsf(X.y) + fabsf(X.z) + fabsf(Y.x) + fabsf(Y.y) + fabsf(Y.z));
+}
+
+// ---- what an end point can see ----
+// In built-up scenes most reflector planes and wedges are hidden from a given
+// end point behind one wall, and every real leg from an end point must be
+// free: so the planes and wedges that are certainly hidden from it as a
+// whole take no part as its first reflection or as the wedge it sees
+// directly. (8 x 8 city blocks: the side lists shrink four to eight times a
+// side.) A target is hidden when one convex wall quad -- two static coplanar
+// triangles that share an edge -- is crossed strictly inside, by the margins
+// of leg_surely_blocked, by the legs to every corner of the target: the
+// crossings of the legs to the points between the corners lie between
+// theirs. The quads tried are those the leg to the target's middle crosses.
+
+// Does quad q (q[0].w != 0) cut off point X from E with margin?
+__device__ __forceinline__ bool quad_between(const float4* __restrict__ q, float3 E, float3 X, float eps_occ) {
+  const float4 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3];
+  if (q0.w == 0.0f) return false;
+  const float3 c[4] = {f3(q0.x, q0.y, q0.z), f3(q1.x, q1.y, q1.z), f3(q2.x, q2.y, q2.z), f3(q3.x, q3.y, q3.z)};
+  const float3 dv = f3(X.x - E.x, X.y - E.y, X.z - E.z);
+  const float dl = sqrtf(fdot3(dv, dv));
+  const float3 nv = cross3(f3(c[1].x - c[0].x, c[1].y - c[0].y, c[1].z - c[0].z),
+                           f3(c[2].x - c[0].x, c[2].y - c[0].y, c[2].z - c[0].z));
+  const float nn = sqrtf(fdot3(nv, nv)), dn = fdot3(dv, nv);
+  if (!(dl > 0.0f && fabsf(dn) > 1e-3f * dl * nn)) return false;
+  const float u = fdot3(f3(c[0].x - E.x, c[0].y - E.y, c[0].z - E.z), nv) / dn;
+  const float slack = 2e-3f + 1e-6f * (fabsf(E.x) + fabsf(E.y) + fabsf(E.z) + dl);
+  const float mu = 0.01f * (1.0f + dl * nn / fabsf(dn)) + slack, nu = mu / dl;
+  if (!(u > eps_occ + nu && u < 1.0f - eps_occ - nu)) return false;
+  const float3 H = f3(E.x + dv.x * u, E.y + dv.y * u, E.z + dv.z * u);
+  for (int k = 0; k < 4; ++k) {
+    const float3 a = c[k], b = c[(k + 1) & 3];
+    const float3 e = f3(b.x - a.x, b.y - a.y, b.z - a.z);
+    const float el = sqrtf(fdot3(e, e));
+    if (el > 0.0f && !(fdot3(cross3(e, f3(H.x - a.x, H.y - a.y, H.z - a.z)), nv) > mu * el * nn)) return false;
+  }
+  return true;
+}
+
+// Are all points of the box lo..hi, or (seg) of the segment lo-hi, certainly
+// hidden from E behind one quad?
+__device__ __noinline__ bool surely_hidden(const PathArgs& a, float3 E, float3 lo, float3 hi, bool seg, TStack& st) {
+  const float3 mid = f3(0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z));
+  const RayPre rp = ray_pre(E, f3(mid.x - E.x, mid.y - E.y, mid.z - E.z));
+  st.reset();
+  int cur = a.bvh.root0;  // static triangles only
+  for (int visits = 0; visits <= a.bvh.max_visits; ++visits) {
+    if (cur == kEmpty) {
+      if (st.empty()) break;
+      cur = st.pop();
+      continue;
+    }
+    if (cur >= 0) {
+      const float4* n = a.bvh.nodes + 4 * (size_t)DCEM_IDX(cur, a.bvh.nnodes);
+      float4 n0 = __ldg(n), n1 = __ldg(n + 1), n2 = __ldg(n + 2), n3 = __ldg(n + 3);
+      float tn0, tn1;
+      const bool h0 = slab(rp, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, 1.0f, tn0);
+      const bool h1 = slab(rp, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, 1.0f, tn1);
+      const int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
+      if (h0 && h1) {
+        if (!st.push(c1)) return false;
+        cur = c0;
+      } else {
+        cur = h0 ? c0 : h1 ? c1 : kEmpty;
+      }
+      continue;
+    }
+    const int id = __float_as_int(__ldg(&a.bvh.tris[3 * (size_t)DCEM_IDX(~cur, a.bvh.ntris)]).w);
+    cur = kEmpty;
+    const float4* q = a.quads + 4 * (size_t)DCEM_IDX(id, a.bvh.ntris);
+    bool all = quad_between(q, E, mid, a.eps_occ);
+    for (int k = 0; all && k < (seg ? 2 : 8); ++k) {
+      const float3 X = seg ? (k ? hi : lo) : f3((k & 1) ? hi.x : lo.x, (k & 2) ? hi.y : lo.y, (k & 4) ? hi.z : lo.z);
+      all = quad_between(q, E, X, a.eps_occ);
+    }
+    if (all) return true;
+  }
+  return false;
+}
+
+// Per end point the planes, then the wedges (in the order wperm) it may see,
+// one warp per word. A wedge the end point is inside of is not seen. Both
+// orders are spatial, so that a warp's legs run close together.
+__global__ void __launch_bounds__(64) k_refl_visible(PathArgs a, int ntx) {
+  extern __shared__ int sstk[];
+  TStack st;
+  bind_stack(st, sstk, kStackTrace);
+  const int npw = (a.nrp + 31) / 32, row = npw + a.nwc, lane = threadIdx.x & 31;
+  const long nitem = (long)(ntx + a.nrx) * row, nwarp = (long)gridDim.x * (blockDim.x >> 5);
+  for (long it = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < nitem; it += nwarp) {
+    const int x = (int)(it / row), c = (int)(it - (long)x * row);
+    const float3 E = end_point(a, ntx, x);
+    bool see = false;
+    if (c < npw) {
+      const int p = c * 32 + lane;
+      if (p < a.nrp) {
+        const float* b = a.rplanes[p].box;
+        see = !surely_hidden(a, E, f3(b[0], b[1], b[2]), f3(b[3], b[4], b[5]), false, st);
+      }
+    } else {
+      const int i = (c - npw) * kWedgeCluster + lane;
+      if (i < a.nw) {
+        const WedgeF W = a.wf[a.wperm[i]];
+        float3 A, B;
+        edge_ends(W, A, B);
+        see = !surely_inside(W, E) && !surely_hidden(a, E, A, B, true, st);
+      }
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, see);
+    if (lane == 0) a.vis[it] = m;
+  }
+}
+// The wedges some transmitter (words 0 .. nwc - 1) or some receiver sees, and
+// lists of the groups that hold any (per side a count, then the groups).
+__global__ void __launch_bounds__(256) k_refl_visible_any(PathArgs a, int ntx) {
+  __shared__ unsigned cnt;
+  const int npw = (a.nrp + 31) / 32, row = npw + a.nwc, side = blockIdx.x;
+  const int ng = (a.nw + kWedgeGroup - 1) / kWedgeGroup;
+  int* list = a.vis_grp + (size_t)side * (ng + 1);
+  if (threadIdx.x == 0) cnt = 0u;
+  __syncthreads();
+  for (int c0 = 0; c0 < a.nwc; c0 += 32) {  // lanes: words, warps: end points
+    __shared__ unsigned part[32];
+    const int c = c0 + (threadIdx.x & 31);
+    if (threadIdx.x < 32) part[threadIdx.x] = 0u;
+    __syncthreads();
+    if (c < a.nwc) {
+      unsigned m = 0;
+      const int x1 = side ? ntx + a.nrx : ntx;
+      for (int x = (side ? ntx : 0) + (threadIdx.x >> 5); x < x1; x += 8) m |= a.vis[(long)x * row + npw + c];
+      atomicOr(&part[threadIdx.x & 31], m);
+    }
+    __syncthreads();
+    if (threadIdx.x < 32 && c < a.nwc) {
+      const unsigned m = part[threadIdx.x];
+      a.vis_any[side * a.nwc + c] = m;
+      for (int k = 0; k < 4; ++k)
+        if ((m >> (8 * k)) & 0xffu) list[1 + atomicAdd(&cnt, 1u)] = 4 * c + k;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) list[0] = (int)cnt;
+}
+__device__ __forceinline__ bool sees_plane(const PathArgs& a, int x, int p) {
+  const int npw = (a.nrp + 31) / 32;
+  return (a.vis[(long)x * (npw + a.nwc) + p / 32] >> (p & 31)) & 1u;
+}
+// (i: the wedge's place in the order wperm)
+__device__ __forceinline__ bool sees_wedge(const PathArgs& a, int x, int i) {
+  const int npw = (a.nrp + 31) / 32;
+  return (a.vis[(long)x * (npw + a.nwc) + npw + i / kWedgeCluster] >> (i % kWedgeCluster)) & 1u;
+}
+
+// Two FIFO queues per warp in shared memory, so that each stage runs on full
+// warps: sides (end point, planes, wedge) waiting to be joined with the
+// other ends, and candidates waiting for the full test. At most 31 entries
+// wait when up to 32 join, so rings of 64 hold them.
+constexpr int kReflWarps = 8, kReflRing = 64;
+struct ReflQueues {
+  int4 side[kReflWarps][kReflRing];  // item, first plane from it, second or -1, wedge (place in wperm)
+  unsigned long long cand[kReflWarps][kReflRing];
+};
+struct ReflRing {  // warp-uniform
+  int sh = 0, st = 0, ch = 0, ct = 0;
+};
+
+// The oldest `nn` candidates of the warp through the full FP32 test; those
+// that pass join the survivor list.
+__device__ __noinline__ void refl_candidates_take(const PathArgs& a, int nlinks, const unsigned long long* q, int head,
+                                                  int nn) {
+  const int lane = threadIdx.x & 31;
+  bool keep = false;
+  unsigned long long code = 0;
+  if (lane < nn) {
+    code = q[(head + lane) & (kReflRing - 1)];
+    const ReflCand c = refl_decode(a, nlinks, code);
+    const WedgeF W = a.wf[c.w];
+    if (c.kind >= 3) {
+      keep = diffract_refl_candidate(W, a.rplanes[c.p1], a.txs[c.link / a.nrx], a.rx[c.link % a.nrx], c.kind == 3);
+    } else {
+      float3 S, S1, O, O1;
+      refl2_images(a, c.kind, c.link, a.rplanes[c.p1], a.rplanes[c.p2], S, S1, O, O1);
+      keep = refl2_candidate(W, a.rplanes[c.p1], a.rplanes[c.p2], c.kind, S, S1, O, O1);
+    }
+  }
+  const unsigned mk = __ballot_sync(0xffffffffu, keep);
+  if (!mk) return;
+  unsigned at = 0;
+  if (lane == 0) at = atomicAdd(&a.ctr->n_dsurv, (unsigned)__popc(mk));
+  at = __shfl_sync(0xffffffffu, at, 0) + __popc(mk & ((1u << lane) - 1u));
+  if (keep) {
+    if (at < a.dsurv_cap) a.dsurv[at] = code;
+    else atomicOr(&a.ctr->err, ERR_DIFF_OVERFLOW);
   }
 }
 
-// A block's record in a warp's ring: its images, planes, kind and index.
-struct Refl2Blk {
-  float3 S, S1, O, O1;
-  int p1, p2, kind;
-  long b;
-};
-constexpr int kRefl2Queue = 64;  // queue entries and block records per warp
+// Lanes with `add` push their candidate; 32 waiting go through the test.
+__device__ __forceinline__ void refl_push(const PathArgs& a, int nlinks, unsigned long long* q, ReflRing& r, bool add,
+                                          unsigned long long code) {
+  const unsigned m = __ballot_sync(0xffffffffu, add);
+  if (!m) return;
+  const int lane = threadIdx.x & 31;
+  if (add) q[(r.ct + __popc(m & ((1u << lane) - 1u))) & (kReflRing - 1)] = code;
+  r.ct += __popc(m);
+  __syncwarp();
+  if (r.ct - r.ch >= 32) {
+    refl_candidates_take(a, nlinks, q, r.ch, 32);
+    r.ch += 32;
+    __syncwarp();
+  }
+}
 
-// One warp per block (kind, link, p1, p2). Its wedges: with one reflection
-// on each side, those in both end points' masks (k_refl2_masks); with both
-// on one side, the wedges of the clusters that the unfolded legs can reach
-// through the planes' boxes (lane c tests cluster c), less those the other,
-// real end point lies inside. The candidates wait in a per-warp FIFO queue
-// in shared memory and go through refl2_candidate 32 at a time, so that the
-// test runs on full warps; each entry names its wedge and its block's record
-// in a ring of 64. At most 63 entries wait, each block with an entry adds
-// one, so a record is overwritten only after its entries left the queue.
-__global__ void __launch_bounds__(256, 3) k_diffract_refl2_pre(PathArgs a, int nlinks) {
-  __shared__ Refl2Blk rec[8][kRefl2Queue];
-  __shared__ int qw[8][kRefl2Queue];
-  __shared__ unsigned char qs[8][kRefl2Queue];
-  const long nblk = 3L * nlinks * a.nrp * a.nrp;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const long nwarp = (long)gridDim.x * (blockDim.x >> 5);
-  const int np1 = a.nrp + 1, ntx = nlinks / a.nrx;
-  // warp-uniform: queue head and tail (entries head .. tail - 1), next record
-  int head = 0, tail = 0, nrec = 0;
-  // the oldest min(tail - head, 32) entries through the test
-  auto drain = [&]() {
-    const int nn = min(tail - head, 32);
-    bool keep = false;
-    int w = 0;
-    long b = 0;
-    if (lane < nn) {
-      const int e = (head + lane) & (kRefl2Queue - 1);
-      w = qw[wid][e];
-      const Refl2Blk& R = rec[wid][qs[wid][e]];
-      b = R.b;
-      keep = refl2_candidate(a.wf[w], a.rplanes[R.p1], a.rplanes[R.p2], R.kind, R.S, R.S1, R.O, R.O1);
+// Work items by end point: the transmitters, each split into a.rsub runs of
+// receivers (few transmitters against many receivers would otherwise leave
+// their pairs to a few warps), then the receivers.
+__device__ __forceinline__ int item_end(const PathArgs& a, int ntx, int v) {
+  return v < ntx * a.rsub ? v / a.rsub : v - ntx * a.rsub + ntx;
+}
+
+// The oldest `nn` sides of the warp against the other ends without a
+// reflection: a transmitter's side against the item's run of receivers, a
+// receiver's against every transmitter. (Entries name the item, not the end point.)
+__device__ __noinline__ void refl_sides_take(const PathArgs& a, int ntx, int nlinks, const int4* sq,
+                                             unsigned long long* cq, ReflRing& r, int nn) {
+  const int lane = threadIdx.x & 31;
+  int4 s = make_int4(0, 0, -1, 0);
+  WedgeSide me{};
+  WedgeF W{};
+  int y0 = 0, y1 = 0, at = 0;
+  if (lane < nn) {
+    s = sq[(r.sh + lane) & (kReflRing - 1)];
+    at = s.w;
+    s.w = a.wperm[at];
+    const int v = s.x;
+    s.x = item_end(a, ntx, v);
+    W = a.wf[s.w];
+    float3 X = plane_image(a.rplanes[s.y], end_point(a, ntx, s.x));
+    if (s.z >= 0) X = plane_image(a.rplanes[s.z], X);
+    me = wedge_side(W, X);
+    if (s.x < ntx) {
+      const int run = (a.nrx + a.rsub - 1) / a.rsub;
+      y0 = (v % a.rsub) * run;
+      y1 = min(a.nrx, y0 + run);
+    } else {
+      y1 = ntx;
     }
-    head += nn;
-    const unsigned mk = __ballot_sync(0xffffffffu, keep);
-    if (!mk) return;
-    unsigned at = 0;
-    if (lane == 0) at = atomicAdd(&a.ctr->n_dsurv, (unsigned)__popc(mk));
-    at = __shfl_sync(0xffffffffu, at, 0) + __popc(mk & ((1u << lane) - 1u));
-    if (keep) {
-      if (at < a.dsurv_cap) a.dsurv[at] = kRefl2Tag | ((unsigned long long)b * a.nw + w);
-      else atomicOr(&a.ctr->err, ERR_DIFF_OVERFLOW);
-    }
-  };
-  for (long b = (long)blockIdx.x * (blockDim.x >> 5) + wid; b < nblk; b += nwarp) {
-    int kind, link, p1, p2;
-    refl2_block(a, nlinks, b, kind, link, p1, p2);
-    if (kind != 1 && p1 == p2) continue;  // two reflections in a row on one plane
-    const RPlane &P1 = a.rplanes[p1], &P2 = a.rplanes[p2];
-    float3 S, S1, O, O1;
-    float m;
-    refl2_images(a, kind, link, P1, P2, S, S1, O, O1, m);
-    if (kind == 0 && !box_reachable(P1, S1, P2.box, m)) continue;
-    if (kind == 2 && !box_reachable(P2, O1, P1.box, m)) continue;
-    const int t = link / a.nrx, rr = link % a.nrx;
-    const unsigned* mt = a.rmask + ((long)t * np1 + (kind == 1 ? p1 : a.nrp)) * a.nwc;
-    const unsigned* mr = a.rmask + ((long)(ntx + rr) * np1 + (kind == 1 ? p2 : a.nrp)) * a.nwc;
-    int slot = -1;  // this block's record (written with its first entry)
-    for (int c0 = 0; c0 < a.nwc; c0 += 32) {
-      const int c = c0 + lane;
-      unsigned word = 0;
-      if (c < a.nwc) {
-        if (kind == 1) {
-          word = mt[c] & mr[c];
-        } else {
-          word = kind == 0 ? mr[c] : mt[c];
-          const float* cb = a.wcbox + 6 * (size_t)c;
-          if (word && !(kind == 0 ? box_reachable(P2, S, cb, m) : box_reachable(P1, O, cb, m))) word = 0;
-        }
+  }
+  const int most = __reduce_max_sync(0xffffffffu, max(y1 - y0, 0));
+  for (int k = 0; k < most; ++k) {
+    const int y = y0 + k, yx = s.x < ntx ? ntx + y : y;
+    bool ok = y < y1 && sees_wedge(a, yx, at);
+    if (ok) {
+      const float3 Y = end_point(a, ntx, yx);
+      WedgeSide o;
+      float3 p;
+      side_zr(W, Y, o, p);
+      ok = side_keller(W.len, me, o);
+      if (ok) {
+        side_angle(W, p, o);
+        ok = side_rules(W.npi, me, o);
       }
-      for (unsigned cm = __ballot_sync(0xffffffffu, word != 0); cm; cm &= cm - 1u) {
-        const int src = __ffs(cm) - 1;
-        const unsigned wd = __shfl_sync(0xffffffffu, word, src);
-        if (slot < 0) {
-          slot = nrec++ & (kRefl2Queue - 1);
-          if (lane == 0) {
-            Refl2Blk& R = rec[wid][slot];
-            R.S = S; R.S1 = S1; R.O = O; R.O1 = O1;
-            R.p1 = p1; R.p2 = p2; R.kind = kind; R.b = b;
-          }
+    }
+    unsigned long long code = 0;
+    if (ok) {
+      const bool tx = s.x < ntx;
+      const int link = tx ? s.x * a.nrx + y : y * a.nrx + (s.x - ntx);
+      code = s.z < 0 ? refl1_code(a, link, s.w, s.y, tx)
+                     : refl2_code(a, nlinks, tx ? 0 : 2, link, tx ? s.y : s.z, tx ? s.z : s.y, s.w);
+    }
+    refl_push(a, nlinks, cq, r, ok, code);
+  }
+}
+
+// The wedges of cluster c that lanes with `bit` hold join the side queue.
+__device__ __forceinline__ void side_push(const PathArgs& a, int ntx, int nlinks, int4* sq, unsigned long long* cq,
+                                          ReflRing& r, bool bit, int4 s) {
+  const unsigned m = __ballot_sync(0xffffffffu, bit);
+  if (!m) return;
+  const int lane = threadIdx.x & 31;
+  if (bit) sq[(r.st + __popc(m & ((1u << lane) - 1u))) & (kReflRing - 1)] = s;
+  r.st += __popc(m);
+  __syncwarp();
+  if (r.st - r.sh >= 32) {
+    refl_sides_take(a, ntx, nlinks, sq, cq, r, 32);
+    r.sh += 32;
+    __syncwarp();
+  }
+}
+__device__ __forceinline__ void refl_flush(const PathArgs& a, int ntx, int nlinks, int4* sq, unsigned long long* cq,
+                                           ReflRing& r) {
+  if (r.st > r.sh) refl_sides_take(a, ntx, nlinks, sq, cq, r, r.st - r.sh);
+  __syncwarp();
+  if (r.ct > r.ch) refl_candidates_take(a, nlinks, cq, r.ch, r.ct - r.ch);
+}
+
+// One warp per (end point, plane): lanes test the wedge groups' boxes first
+// (most are out of the image's window), then the wedges, four groups at once.
+__global__ void __launch_bounds__(256) k_refl_single(PathArgs a, int ntx, int nlinks) {
+  __shared__ ReflQueues Q;
+  const long nitem = ((long)ntx * a.rsub + a.nrx) * a.nrp;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const long nwarp = (long)gridDim.x * kReflWarps;
+  const int ng = (a.nw + kWedgeGroup - 1) / kWedgeGroup;
+  ReflRing r;
+  for (long it = (long)blockIdx.x * kReflWarps + wid; it < nitem; it += nwarp) {
+    const int p = (int)(it % a.nrp), v = (int)(it / a.nrp), x = item_end(a, ntx, v);
+    if (!sees_plane(a, x, p)) continue;
+    const RPlane& Pl = a.rplanes[p];
+    const float3 E = end_point(a, ntx, x), X = plane_image(Pl, E);
+    const float m = image_margin(E, X);
+    for (int g0 = 0; g0 < ng; g0 += 32) {
+      const bool near = g0 + lane < ng && image_sees_group(a, Pl, g0 + lane, X, m, nullptr, X);
+      for (unsigned gm = __ballot_sync(0xffffffffu, near); gm;) {
+        const int i = octet_wedge(a, g0 + lane, gm);
+        int w = 0;
+        bool bit = false;
+        if (i >= 0) {
+          w = a.wperm[i];
+          bit = image_sees(Pl, a.wf[w], X, nullptr, X);
         }
-        const bool bit = (wd >> lane) & 1u;
-        const unsigned bm = __ballot_sync(0xffffffffu, bit);
-        if (bit) {
-          const int e = (tail + __popc(bm & ((1u << lane) - 1u))) & (kRefl2Queue - 1);
-          qw[wid][e] = a.wperm[(c0 + src) * kWedgeCluster + lane];
-          qs[wid][e] = (unsigned char)slot;
+        if (bit && a.drefl2) {
+          atomicOr(&a.rmask[((long)x * a.nrp + p) * a.nwc + i / kWedgeCluster], 1u << (i % kWedgeCluster));
+          if (x >= ntx) atomicAdd(&a.wobs_cnt[w], 1u);
         }
-        tail += __popc(bm);
-        __syncwarp();
-        if (tail - head >= 32) drain();
-        __syncwarp();
+        side_push(a, ntx, nlinks, Q.side[wid], Q.cand[wid], r, bit, make_int4(v, p, -1, i));
       }
     }
   }
-  while (tail > head) drain();
+  refl_flush(a, ntx, nlinks, Q.side[wid], Q.cand[wid], r);
+}
+
+// Room in the observer list for every wedge's receiver sides.
+__global__ void k_refl_room(PathArgs a) {
+  for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < a.nw; w += gridDim.x * blockDim.x) {
+    const unsigned n = a.wobs_cnt[w];
+    const unsigned at = n ? atomicAdd(&a.ctr->n_dobs, n) : 0u;
+    a.wobs_off[w] = a.wobs_pos[w] = at;
+    if (n && (unsigned long long)at + n > a.dobs_cap) atomicOr(&a.ctr->err, ERR_DIFF_OVERFLOW);
+  }
+}
+
+// The receivers' one-reflection sides into their wedges' lists, from the
+// mask words: one warp per (receiver, plane).
+__global__ void __launch_bounds__(256) k_refl_lists(PathArgs a, int ntx) {
+  const long nitem = (long)a.nrx * a.nrp;
+  const int lane = threadIdx.x & 31;
+  const long nwarp = (long)gridDim.x * (blockDim.x >> 5);
+  for (long it = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < nitem; it += nwarp) {
+    const int p = (int)(it % a.nrp), rx = (int)(it / a.nrp);
+    const float3 X = plane_image(a.rplanes[p], end_point(a, ntx, ntx + rx));
+    const unsigned* row = a.rmask + ((long)(ntx + rx) * a.nrp + p) * a.nwc;
+    for (int c0 = 0; c0 < a.nwc; c0 += 32) {
+      const unsigned word = c0 + lane < a.nwc ? row[c0 + lane] : 0u;
+      for (unsigned cm = __ballot_sync(0xffffffffu, word != 0); cm; cm &= cm - 1u) {
+        const int src = __ffs(cm) - 1;
+        const unsigned wd = __shfl_sync(0xffffffffu, word, src);
+        if (!((wd >> lane) & 1u)) continue;
+        const int w = a.wperm[(c0 + src) * kWedgeCluster + lane];
+        const WedgeSide s = wedge_side(a.wf[w], X);
+        const unsigned at = atomicAdd(&a.wobs_pos[w], 1u);
+        if (at < a.dobs_cap) a.dobs[at] = DiffObs{rx, p, s.z, s.r, s.l, s.phi, s.tol, 0.0f};
+      }
+      __syncwarp();
+    }
+  }
+}
+
+// One reflection on each side of the wedge: one warp per (transmitter,
+// plane, cluster) mask word and eighth of the lists, its lanes over that
+// part of the list of each wedge in the word.
+constexpr int kJoinParts = 8;
+__global__ void __launch_bounds__(256) k_refl_join(PathArgs a, int ntx, int nlinks) {
+  __shared__ unsigned long long cq[kReflWarps][kReflRing];
+  const long nitem = (long)ntx * a.nrp * a.nwc * kJoinParts;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const long nwarp = (long)gridDim.x * kReflWarps;
+  ReflRing r;
+  for (long part = (long)blockIdx.x * kReflWarps + wid; part < nitem; part += nwarp) {
+    const long it = part / kJoinParts;
+    unsigned word = a.rmask[it];
+    if (!word) continue;
+    const int c = (int)(it % a.nwc);
+    const long tp = it / a.nwc;
+    const int p1 = (int)(tp % a.nrp), t = (int)(tp / a.nrp);
+    const float3 S = plane_image(a.rplanes[p1], end_point(a, ntx, t));
+    for (; word; word &= word - 1u) {
+      const int w = a.wperm[c * kWedgeCluster + __ffs(word) - 1];
+      const WedgeF W = a.wf[w];
+      const WedgeSide me = wedge_side(W, S);
+      const unsigned n = a.wobs_cnt[w], off = a.wobs_off[w];
+      if ((unsigned long long)off + n > a.dobs_cap) continue;  // the list overflowed: the frame is traced again
+      for (unsigned i0 = 32 * (unsigned)(part % kJoinParts); i0 < n; i0 += 32 * kJoinParts) {
+        bool ok = i0 + lane < n;
+        unsigned long long code = 0;
+        if (ok) {
+          const DiffObs o = a.dobs[off + i0 + lane];
+          const WedgeSide os{o.z, o.r, o.l, o.phi, o.tol};
+          ok = side_keller(W.len, me, os) && side_rules(W.npi, me, os);
+          if (ok) code = refl2_code(a, nlinks, 1, t * a.nrx + o.rx, p1, o.p, w);
+        }
+        refl_push(a, nlinks, cq[wid], r, ok, code);
+      }
+    }
+  }
+  if (r.ct > r.ch) refl_candidates_take(a, nlinks, cq[wid], r.ch, r.ct - r.ch);
+}
+
+// Both reflections on one side of the wedge: lanes take (end point, first
+// plane from it, second plane) and keep those whose second plane's box the
+// image can reach through the first's; for each of them the warp tests the
+// groups' boxes against the double image, then the groups' wedges.
+__global__ void __launch_bounds__(256) k_refl_double(PathArgs a, int ntx, int nlinks) {
+  __shared__ ReflQueues Q;
+  const long nitem = ((long)ntx * a.rsub + a.nrx) * a.nrp * a.nrp;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const long stride = (long)gridDim.x * blockDim.x;
+  const int ng = (a.nw + kWedgeGroup - 1) / kWedgeGroup;
+  ReflRing r;
+  for (long base = (long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < nitem; base += stride) {
+    const long it = base + lane;
+    int v = 0, pa = 0, pb = 0;
+    float m = 0.0f;
+    bool pass = false;
+    if (it < nitem) {
+      pb = (int)(it % a.nrp);
+      const long q = it / a.nrp;
+      pa = (int)(q % a.nrp);
+      v = (int)(q / a.nrp);
+      const int x = item_end(a, ntx, v);
+      if (pa != pb && sees_plane(a, x, pa)) {  // two reflections in a row are on different planes
+        const float3 E = end_point(a, ntx, x), X1 = plane_image(a.rplanes[pa], E);
+        const RPlane& Pb = a.rplanes[pb];
+        m = image_margin(E, plane_image(Pb, X1));
+        float lo[3] = {Pb.box[0], Pb.box[1], Pb.box[2]}, hi[3] = {Pb.box[3], Pb.box[4], Pb.box[5]};
+        pass = box_window(a.rplanes[pa], X1, m, lo, hi);
+      }
+    }
+    for (unsigned pm = __ballot_sync(0xffffffffu, pass); pm; pm &= pm - 1u) {
+      const int who = __ffs(pm) - 1;
+      const int uv = __shfl_sync(0xffffffffu, v, who), ux = item_end(a, ntx, uv), ua = __shfl_sync(0xffffffffu, pa, who),
+                ub = __shfl_sync(0xffffffffu, pb, who);
+      const float um = __shfl_sync(0xffffffffu, m, who);
+      const RPlane &Pa = a.rplanes[ua], &Pb = a.rplanes[ub];
+      const float3 U1 = plane_image(Pa, end_point(a, ntx, ux)), U = plane_image(Pb, U1);
+      // the wedges the other ends see
+      const unsigned* opp = a.vis_any + (ux < ntx ? a.nwc : 0);
+      const int* grp = a.vis_grp + (ux < ntx ? ng + 1 : 0);
+      const int n = grp[0];
+      for (int k0 = 0; k0 < n; k0 += 32) {
+        const int g = k0 + lane < n ? grp[1 + k0 + lane] : -1;
+        const bool near = g >= 0 && image_sees_group(a, Pb, g, U, um, &Pa, U1);
+        for (unsigned gm = __ballot_sync(0xffffffffu, near); gm;) {
+          const int i = octet_wedge(a, g, gm);
+          bool bit = false;
+          if (i >= 0 && ((opp[i / kWedgeCluster] >> (i % kWedgeCluster)) & 1u))
+            bit = image_sees(Pb, a.wf[a.wperm[i]], U, &Pa, U1);
+          side_push(a, ntx, nlinks, Q.side[wid], Q.cand[wid], r, bit, make_int4(uv, ua, ub, i));
+        }
+      }
+    }
+  }
+  refl_flush(a, ntx, nlinks, Q.side[wid], Q.cand[wid], r);
+}
+
+// ---- occlusion before the exact stage ----
+// Nearly every candidate of the tests above has its Keller point and
+// reflection points in place and a building in between (8 x 8 city blocks:
+// 183k candidates, 313 paths), and the exact stage's FP64 work per
+// candidate is two orders of magnitude dearer than an FP32 traversal. So the
+// candidates whose legs are certainly blocked (leg_surely_blocked around the
+// FP32 estimate of the points) are dropped here. The estimate is trusted to
+// the margins of the candidate tests where it is well conditioned: both ends
+// half a metre off the edge line, legs more than 3 degrees off the planes
+// they cross; elsewhere the candidate is kept. Chains were tested by
+// k_diff_multi_pre; with transmission on, a first-order leg may cross walls.
+
+// The crossing of the unfolded leg a0 -> a1 with plane P; false when the leg
+// is within 3 degrees of the plane. delta: the larger of its value and the
+// crossing's margin.
+__device__ __forceinline__ bool plane_cross32(const RPlane& P, float3 a0, float3 a1, float3& X, float& delta) {
+  const float3 n = f3(P.nf[0], P.nf[1], P.nf[2]);
+  const float3 dv = f3(a1.x - a0.x, a1.y - a0.y, a1.z - a0.z);
+  const float den = fdot3(n, dv), len = sqrtf(fdot3(dv, dv));
+  if (!(fabsf(den) > 0.05f * len)) return false;
+  const float t = (P.cf - fdot3(n, a0)) / den;
+  X = f3(a0.x + t * dv.x, a0.y + t * dv.y, a0.z + t * dv.z);
+  delta = fmaxf(delta, 0.1f + 2e-4f * (len + sqrtf(fdot3(X, X))));
+  return true;
+}
+
+__device__ __forceinline__ bool diff_blocked(const PathArgs& a, int nlinks, unsigned long long code, TStack& st) {
+  ReflCand c;
+  const unsigned kind = (unsigned)(code >> kKindShift);
+  if (kind == 2u) {
+    c = refl_decode(a, nlinks, code);
+  } else if (kind == 0u && a.max_trans == 0) {
+    c.kind = 5;
+    c.link = (int)(code / (unsigned)a.nw);
+    c.w = (int)(code % (unsigned)a.nw);
+    c.p1 = c.p2 = 0;
+  } else {
+    return false;
+  }
+  const WedgeF W = a.wf[c.w];
+  const float4 tv = a.txs[c.link / a.nrx], rv = a.rx[c.link % a.nrx];
+  const float3 T = f3(tv.x, tv.y, tv.z), R = f3(rv.x, rv.y, rv.z);
+  float3 S = T, S1 = T, O = R, O1 = R;
+  if (c.kind <= 2) refl2_images(a, c.kind, c.link, a.rplanes[c.p1], a.rplanes[c.p2], S, S1, O, O1);
+  else if (c.kind == 3) S = plane_image(a.rplanes[c.p1], T);
+  else if (c.kind == 4) O = plane_image(a.rplanes[c.p1], R);
+  WedgeSide s, o;
+  float3 p;
+  side_zr(W, S, s, p);
+  side_zr(W, O, o, p);
+  if (!(s.r > 0.5f && o.r > 0.5f)) return false;
+  const float zq = s.z + (o.z - s.z) * s.r / (s.r + o.r);
+  const float3 Qp = edge_point(W, zq);
+  float delta = 0.05f + 1e-5f * (s.l + o.l);
+  // the path's points between T and R, and the wedge's place among them
+  float3 P[5];
+  int np = 0, at = 0;
+  P[np++] = T;
+  float3 X, Y;
+  if (c.kind == 0) {
+    if (!plane_cross32(a.rplanes[c.p2], S, Qp, Y, delta) || !plane_cross32(a.rplanes[c.p1], S1, Y, X, delta))
+      return false;
+    P[np++] = X;
+    P[np++] = Y;
+  } else if (c.kind == 1 || c.kind == 3) {
+    if (!plane_cross32(a.rplanes[c.p1], S, Qp, X, delta)) return false;
+    P[np++] = X;
+  }
+  at = np;
+  P[np++] = Qp;
+  if (c.kind == 2) {
+    if (!plane_cross32(a.rplanes[c.p1], Qp, O, X, delta) || !plane_cross32(a.rplanes[c.p2], X, O1, Y, delta))
+      return false;
+    P[np++] = X;
+    P[np++] = Y;
+  } else if (c.kind == 1 || c.kind == 4) {
+    if (!plane_cross32(a.rplanes[c.kind == 1 ? c.p2 : c.p1], Qp, O, X, delta)) return false;
+    P[np++] = X;
+  }
+  P[np++] = R;
+  const int ta = a.wtopo[c.w].ta, tb = a.wtopo[c.w].tb;
+  for (int q = 0; q + 1 < np; ++q) {
+    const bool ends = q == at || q + 1 == at;  // the wedge's faces do not block the legs at Q
+    const float3 dv = f3(P[q + 1].x - P[q].x, P[q + 1].y - P[q].y, P[q + 1].z - P[q].z);
+    if (leg_surely_blocked(a.bvh, P[q], dv, delta, a.eps_occ, ends ? ta : -1, ends ? tb : -1, -1, -1, st)) return true;
+  }
+  return false;
+}
+
+__global__ void __launch_bounds__(64) k_diff_unblocked(PathArgs a, int nlinks) {
+  extern __shared__ int sstk[];
+  TStack st;
+  bind_stack(st, sstk, kStackTrace);
+  const unsigned n = min(a.ctr->n_dsurv, a.dsurv_cap);
+  const int lane = threadIdx.x & 31;
+  // few candidates: a few lanes of every warp, so that all SMs share the
+  // traversals' latency; many: full warps of consecutive candidates (which
+  // come from one warp above, so their legs run close together)
+  const unsigned nwarp = gridDim.x * (blockDim.x >> 5), per = min(32u, max(1u, (n + nwarp - 1) / nwarp));
+  for (unsigned i0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per; i0 < n; i0 += nwarp * per) {
+    const unsigned i = i0 + lane;
+    const bool mine = lane < (int)per && i < n;
+    const unsigned long long code = mine ? a.dsurv[i] : 0ull;
+    const bool keep = mine && !diff_blocked(a, nlinks, code, st);
+    const unsigned mk = __ballot_sync(0xffffffffu, keep);
+    if (!mk) continue;
+    unsigned at = 0;
+    if (lane == 0) at = atomicAdd(&a.ctr->n_dexact, (unsigned)__popc(mk));
+    at = __shfl_sync(0xffffffffu, at, 0) + __popc(mk & ((1u << lane) - 1u));
+    if (keep) a.dexact[at] = code;
+  }
 }
 
 __device__ __forceinline__ d3w mirror_d(d3w x, d3w n, double c) { return x - n * (2.0 * (dotw(n, x) - c)); }
@@ -3464,20 +4005,22 @@ __global__ void __launch_bounds__(256) k_diffract_pre(PathArgs a, int nlinks) {
 
 // Pass 2 over the survivors: the exact FP64 test, the occlusion legs and the
 // UTD field. The SM's FP64 pipe is narrow and a warp instruction costs it the
-// same whatever the number of active lanes, so survivor i goes to block
-// i mod grid, slot i / grid: every SM gets an equal share, packed into its
-// first warp while there are few survivors and into more warps as they grow
-// (orders 2 and 3 can leave many), instead of a few SMs taking whole batches.
+// same whatever the number of active lanes, but with the few survivors left
+// after the occlusion test the pipe is mostly idle (12% busy on the city) and
+// the time is the longest lane's chain of dependent operations plus the
+// other lanes' divergent branches: so survivor i goes to block i mod grid,
+// slot i / grid, and the slots fill the warps one lane at a time.
 constexpr int kDiffThreads = 256;
 __global__ void __launch_bounds__(kDiffThreads) k_diffract(PathArgs a) {
   extern __shared__ int sstk[];
   TStack st;
   bind_stack(st, sstk, kStackTrace);
-  const unsigned n = min(a.ctr->n_dsurv, a.dsurv_cap);
+  const unsigned n = min(a.ctr->n_dexact, a.dsurv_cap);
   const double k = 2.0 * M_PI * a.freq / 299792458.0, lam = 299792458.0 / a.freq;
   unsigned ovf = 0;
-  for (unsigned i = blockIdx.x + gridDim.x * threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const unsigned long long c = a.dsurv[i];
+  const unsigned slot = (threadIdx.x & 31) * (kDiffThreads / 32) + (threadIdx.x >> 5);
+  for (unsigned i = blockIdx.x + gridDim.x * slot; i < n; i += gridDim.x * blockDim.x) {
+    const unsigned long long c = a.dexact[i];
     const unsigned kind = (unsigned)(c >> kKindShift);
     if (kind == 2u && ((c >> 61) & 1ull)) diffract_refl2(a, c & kRefl2Mask, k, lam, ovf, st);
     else if (kind == 2u) diffract_refl_pair(a, c & ~kReflTag, k, lam, ovf, st);
@@ -3628,26 +4171,34 @@ cudaError_t launch_dedupe(const PathArgs& a, int grid, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_diffract(const PathArgs& a, int nlinks, int sms, cudaStream_t st) {
+cudaError_t launch_diffract(const PathArgs& args, int nlinks, int sms, cudaStream_t st) {
+  PathArgs a = args;
   if (!a.wedges || a.nw <= 0) return cudaSuccess;
-  k_wedge_geom<<<(a.nw + 255) / 256, 256, 0, st>>>(a.tris, a.slot_of_id, a.wtopo, a.nw, a.wedges, a.wf);
-  if (a.drefl2 && a.rplanes && a.nrp > 0)
-    k_wedge_boxes<<<(a.nwc * 32 + 255) / 256, 256, 0, st>>>(a.wf, a.wperm, a.nw, a.nwc, a.wcbox);
+  k_wedge_geom<<<(a.nw + 31) / 32, 32, 0, st>>>(a.tris, a.slot_of_id, a.wtopo, a.nw, a.wedges, a.wf);
+  if (a.rplanes && a.nrp > 0)
+    k_wedge_boxes<<<(a.nw + 255) / 256, 256, 0, st>>>(a.wf, a.wperm, a.nw, a.wgbox);
   if (nlinks > 0) {
     long total = (long)nlinks * a.nw;
     long g = std::min<long>((total + 255) / 256, 8L * sms);
     k_diffract_pre<<<(int)std::max<long>(g, 1), 256, 0, st>>>(a, nlinks);
     if (a.rplanes && a.nrp > 0) {
-      long tr = (long)nlinks * a.nw * a.nrp * 2;
-      long gr = std::min<long>((tr + 255) / 256, 8L * sms);
-      k_diffract_refl_pre<<<(int)std::max<long>(gr, 1), 256, 0, st>>>(a, nlinks);
+      const int ntx = nlinks / a.nrx;
+      a.rsub = std::max(1, std::min((a.nrx + 7) / 8, a.nrx / ntx));
+      auto warps = [&](long n) { return (int)std::max<long>(std::min<long>((n + 7) / 8, 8L * sms), 1); };
       if (a.drefl2) {
-        const int ntx = nlinks / a.nrx;
-        long nm = (long)(ntx + a.nrx) * (a.nrp + 1) * a.nwc;
-        k_refl2_masks<<<(int)std::max<long>(std::min<long>((nm + 7) / 8, 8L * sms), 1), 256, 0, st>>>(a, ntx);
-        long nblk = 3L * nlinks * a.nrp * a.nrp;
-        long g2 = std::min<long>((nblk + 7) / 8, 8L * sms);
-        k_diffract_refl2_pre<<<(int)std::max<long>(g2, 1), 256, 0, st>>>(a, nlinks);
+        cudaMemsetAsync(a.wobs_cnt, 0, sizeof(unsigned) * (size_t)a.nw, st);
+        cudaMemsetAsync(a.rmask, 0, sizeof(unsigned) * (size_t)(ntx + a.nrx) * a.nrp * a.nwc, st);
+      }
+      const long nvis = (long)(ntx + a.nrx) * ((a.nrp + 31) / 32 + a.nwc);
+      k_refl_visible<<<(int)std::min<long>((nvis + 1) / 2, 16L * sms), 64, 64 * kStackTrace * sizeof(int), st>>>(a, ntx);
+      k_refl_visible_any<<<2, 256, 0, st>>>(a, ntx);
+      k_refl_single<<<warps(((long)ntx * a.rsub + a.nrx) * a.nrp), 256, 0, st>>>(a, ntx, nlinks);
+      if (a.drefl2) {
+        k_refl_room<<<(a.nw + 255) / 256, 256, 0, st>>>(a);
+        k_refl_lists<<<warps((long)a.nrx * a.nrp), 256, 0, st>>>(a, ntx);
+        k_refl_join<<<warps((long)ntx * a.nrp * a.nwc * kJoinParts), 256, 0, st>>>(a, ntx, nlinks);
+        a.rsub = std::max(1, a.rsub / 4);
+        k_refl_double<<<warps((((long)ntx * a.rsub + a.nrx) * a.nrp * a.nrp + 31) / 32), 256, 0, st>>>(a, ntx, nlinks);
       }
     }
     PathArgs b = a;  // chains: transmitters, and the reflector planes applied to them
@@ -3666,6 +4217,7 @@ cudaError_t launch_diffract(const PathArgs& a, int nlinks, int sms, cudaStream_t
       if (a.diff_order >= 3) k_diff_triples<<<8 * sms, 256, 0, st>>>(b);
       k_diff_multi_pre<<<8 * sms, 256, 256 * kStackTrace * sizeof(int), st>>>(b);
     }
+    k_diff_unblocked<<<8 * sms, 64, 64 * kStackTrace * sizeof(int), st>>>(b, nlinks);
     k_diffract<<<sms, kDiffThreads, kDiffThreads * kStackTrace * sizeof(int), st>>>(b);
   }
   return cudaGetLastError();

@@ -53,12 +53,14 @@ struct PathArgs {
   WedgeF* wf;                     // the same in FP32 (pre-tests)
   const WedgeTopo* wtopo;
   int nw;
-  // wedge clusters: the wedges in a fixed spatial order (wperm), 32 per
-  // cluster, and each cluster's box of its edges (6 floats, every frame)
+  // the wedges in a fixed spatial order (wperm): nwc mask words of
+  // kWedgeCluster, and the boxes of the groups of kWedgeGroup (6 floats
+  // each, every frame)
   const int* wperm;
-  float* wcbox;
+  float* wgbox;
   int nwc;
-  unsigned long long* dsurv;      // (link, wedge) pair indices past the FP32 pre-test
+  unsigned long long* dsurv;      // candidates past the FP32 pre-tests
+  unsigned long long* dexact;     // ... and past the FP32 occlusion test (same capacity)
   unsigned dsurv_cap;
   // one reflection before or after a diffraction (null: off): reflector
   // planes and their member triangle ids
@@ -66,9 +68,20 @@ struct PathArgs {
   const int* rmembers;             // per plane its members, sorted by their lowest coordinate
   const float* rkeys;              // along the plane's axis, and that coordinate
   int nrp;
+  const float4* quads;            // per triangle id: the convex wall quad it is part of (corners; .w of
+                                  // the first 0: none)
+  int rsub;                       // runs of receivers per transmitter item (set by launch_diffract)
+  unsigned* vis;                  // per end point: bits of the planes, then of the wedges it may see
+  unsigned* vis_any;              // the wedges some transmitter, then some receiver may see
+  int* vis_grp;                   // ... and the groups that hold any: per side a count and the list
   int drefl2;                     // 1: also two reflections around a first-order diffraction
-  unsigned* rmask;                // with drefl2: the wedge masks of k_refl2_masks, one word per
-                                  // (end point: transmitters then receivers, plane or none, cluster)
+  unsigned* rmask;                // with drefl2: the wedge masks of k_refl_single, one word per
+                                  // (end point: transmitters then receivers, plane, cluster)
+  unsigned* wobs_cnt;             // with drefl2, per wedge: the receivers' one-reflection sides,
+  unsigned* wobs_off;             // where they start in dobs, and the next free slot there
+  unsigned* wobs_pos;
+  DiffObs* dobs;
+  unsigned dobs_cap;
   int dmid;                       // 1: also a reflection between the two wedges of an order-2 chain
   // diffraction of order 2 and 3 (diff_order <= 1: off): the wedge pairs
   // (v, w1, w2, -1), the pairs with a reflection on plane p between them
