@@ -245,6 +245,7 @@ struct dcem_scene {
   WedgeTopo* wtopo = nullptr;  // ... and topology
   int nw = 0;
   int* wperm = nullptr;        // the wedges in spatial order (mask words of 32),
+  int* wplace = nullptr;       // their places in that order,
   float* wgbox = nullptr;      // and the boxes of the groups of 8 (per frame)
   int nwc = 0;
   bool diffraction = false;
@@ -269,6 +270,8 @@ struct dcem_scene {
   int4* dseq3 = nullptr;
   unsigned dseq2_cap = 0, dseq3_cap = 0;
   unsigned* drel = nullptr;
+  unsigned* dobs1 = nullptr;   // ... order 3: stage-1 rows of the related pairs, after the bits of
+  size_t dobs1_cap = 0;        // the pairs' second wedges (ensure_obs1)
   double2* g_items = nullptr;  // field derivatives: per-item results, their parameter,
   int* g_param = nullptr;      // staged outputs and the error flag (dcem_path_gradients)
   double* g_out = nullptr;
@@ -404,9 +407,9 @@ void scene_free(dcem_scene* s) {
   dfree(s->tri_mat_d); dfree(s->v9d); dfree(s->nodes); dfree(s->qnodes); dfree(s->qframe);
   dfree(s->q4_kid); dfree(s->q4_src); dfree(s->q4_count); dfree(s->q4_roots); dfree(s->q4_scr); dfree(s->leaf_parent); dfree(s->arrive);
   dfree(s->dsched); dfree(s->dlvl); dfree(s->tri_obj_d); dfree(s->wedges); dfree(s->wedgesf); dfree(s->wtopo);
-  dfree(s->wperm); dfree(s->wgbox); dfree(s->dsurv); dfree(s->dexact); dfree(s->wobs); dfree(s->dobs);
+  dfree(s->wperm); dfree(s->wplace); dfree(s->wgbox); dfree(s->dsurv); dfree(s->dexact); dfree(s->wobs); dfree(s->dobs);
   dfree(s->rplanes); dfree(s->rmembers); dfree(s->rkeys); dfree(s->rmask); dfree(s->quads); dfree(s->vis);
-  dfree(s->dseq2); dfree(s->dseq3); dfree(s->drel);
+  dfree(s->dseq2); dfree(s->dseq3); dfree(s->drel); dfree(s->dobs1);
   dfree(s->g_items); dfree(s->g_param); dfree(s->g_out); dfree(s->g_err); dfree(s->g_paths);
   dfree(s->g_rx); dfree(s->g_theta);
   dfree(s->roots); dfree(s->root_box); dfree(s->perm); dfree(s->prim); dfree(s->mats);
@@ -650,16 +653,21 @@ int ensure_rx(dcem_scene* s, int nrx, int nlinks, int bucket_cap) {
 static size_t vis_head(const dcem_scene* s) {
   return 2 * (size_t)s->nwc + 2 * (size_t)((s->nw + kWedgeGroup - 1) / kWedgeGroup + 1);
 }
+// Are the end points' visibility rows used: with reflector planes or chains.
+static bool uses_vis(const dcem_scene* s) {
+  return s->diffraction && s->nw > 0 && s->quads && ((s->diff_refl && s->nrp > 0) || (s->diff_order >= 2 && s->nw > 1));
+}
 static int ensure_rmask(dcem_scene* s, int ntx, int nrx) {
-  if (!(s->diffraction && s->nw > 0 && s->diff_refl >= 1 && s->nrp > 0)) return DCEM_OK;
-  const size_t words = (size_t)(ntx + nrx) * (size_t)((s->nrp + 31) / 32 + s->nwc) + vis_head(s);
+  if (!uses_vis(s)) return DCEM_OK;
+  const int nrp = s->diff_refl ? s->nrp : 0;
+  const size_t words = (size_t)(ntx + nrx) * (size_t)((nrp + 31) / 32 + s->nwc) + vis_head(s);
   if (words > s->vis_cap) {
     dfree(s->vis);
     s->vis_cap = 0;
     CK(dalloc(&s->vis, words));
     s->vis_cap = words;
   }
-  if (s->diff_refl < 2) return DCEM_OK;
+  if (s->diff_refl < 2 || s->nrp == 0) return DCEM_OK;
   const size_t need = (size_t)(ntx + nrx) * (size_t)s->nrp * (size_t)s->nwc;
   if (!s->wobs) CK(dalloc(&s->wobs, 3 * (size_t)s->nw));
   if (!s->dobs) {
@@ -671,6 +679,24 @@ static int ensure_rmask(dcem_scene* s, int ntx, int nrx) {
   dfree(s->rmask);
   CK(dalloc(&s->rmask, std::max<size_t>(need, 1)));
   s->rmask_cap = std::max<size_t>(need, 1);
+  return DCEM_OK;
+}
+
+// Order 3: the stage-1 rows (k_diff_stage1), one bit per (wedge pair,
+// receiver), kept while they take at most 256 MB (above, the rows' traffic
+// and room outweigh the repeated tests).
+static size_t obs1_words(const dcem_scene* s, int nrx) {
+  if (!(s->diffraction && s->diff_order >= 3 && s->nw > 2)) return 0;
+  const size_t n = (size_t)s->nw * s->nw * (size_t)((nrx + 31) / 32) + (size_t)((s->nw + 31) / 32);
+  return n <= ((size_t)64 << 20) ? n : 0;
+}
+static int ensure_obs1(dcem_scene* s, int nrx) {
+  const size_t n = obs1_words(s, nrx);
+  if (n <= s->dobs1_cap) return DCEM_OK;
+  dfree(s->dobs1);
+  s->dobs1_cap = 0;
+  CK(dalloc(&s->dobs1, n));
+  s->dobs1_cap = n;
   return DCEM_OK;
 }
 
@@ -1429,6 +1455,10 @@ int dcem_scene_set_diffraction(dcem_scene* s, int32_t on, int32_t* n_wedges) {
       CK(dalloc(&s->wedges, s->nw));
       CK(dalloc(&s->wedgesf, s->nw));
       CK(dalloc(&s->wperm, s->nw));
+      std::vector<int> place(perm.size());
+      for (size_t i = 0; i < perm.size(); ++i) place[perm[i]] = (int)i;
+      CK(dalloc(&s->wplace, s->nw));
+      CK(cudaMemcpy(s->wplace, place.data(), sizeof(int) * place.size(), cudaMemcpyHostToDevice));
       CK(dalloc(&s->wgbox, 6 * (size_t)((s->nw + kWedgeGroup - 1) / kWedgeGroup)));
       CK(cudaMemcpy(s->wtopo, w.data(), sizeof(WedgeTopo) * w.size(), cudaMemcpyHostToDevice));
       CK(cudaMemcpy(s->wperm, perm.data(), sizeof(int) * perm.size(), cudaMemcpyHostToDevice));
@@ -1442,6 +1472,15 @@ int dcem_scene_set_diffraction(dcem_scene* s, int32_t on, int32_t* n_wedges) {
   s->diffraction = on != 0;
   if (n_wedges) *n_wedges = s->nw;
   return DCEM_OK;
+}
+
+static cudaError_t upload_quads(dcem_scene* s, const std::vector<float4>& quads) {
+  if (s->quads) return cudaSuccess;
+  cudaError_t e = dalloc(&s->quads, quads.size());
+  if (e == cudaSuccess)
+    e = cudaMemcpy(s->quads, quads.data(), sizeof(float4) * quads.size(), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) dfree(s->quads);
+  return e;
 }
 
 int dcem_scene_set_diffraction_reflections(dcem_scene* s, int32_t on, int32_t* n_planes) {
@@ -1460,9 +1499,7 @@ int dcem_scene_set_diffraction_reflections(dcem_scene* s, int32_t on, int32_t* n
       CK(cudaMemcpy(s->rplanes, planes.data(), sizeof(RPlane) * planes.size(), cudaMemcpyHostToDevice));
       CK(cudaMemcpy(s->rmembers, members.data(), sizeof(int) * members.size(), cudaMemcpyHostToDevice));
       CK(cudaMemcpy(s->rkeys, keys.data(), sizeof(float) * keys.size(), cudaMemcpyHostToDevice));
-      const std::vector<float4> quads = wall_quads(s->tris_h, s->tri_obj_h, planes, members);
-      CK(dalloc(&s->quads, quads.size()));
-      CK(cudaMemcpy(s->quads, quads.data(), sizeof(float4) * quads.size(), cudaMemcpyHostToDevice));
+      CK(upload_quads(s, wall_quads(s->tris_h, s->tri_obj_h, planes, members)));
     }
   }
   s->diff_refl = on;
@@ -1477,6 +1514,13 @@ int dcem_scene_set_diffraction_order(dcem_scene* s, int32_t max_order) {
     CK(dalloc(&s->dseq2, (size_t)4096));
     s->dseq2_cap = 4096;
     CK(dalloc(&s->drel, ((size_t)s->nw * s->nw + 31) / 32));
+    if (!s->quads) {
+      std::vector<RPlane> planes;
+      std::vector<int> members;
+      std::vector<float> keys;
+      group_planes(s->tris_h, s->tri_obj_h, planes, members, keys);
+      CK(upload_quads(s, wall_quads(s->tris_h, s->tri_obj_h, planes, members)));
+    }
   }
   if (max_order >= 3 && !s->dseq3 && s->nw > 2) {
     CK(dalloc(&s->dseq3, (size_t)4096));
@@ -1726,6 +1770,7 @@ static void make_plan(dcem_scene* s, int nrx, const dcem_params* p, bool coheren
   q.wtopo = s->wtopo;
   q.nw = s->nw;
   q.wperm = s->wperm;
+  q.wplace = s->wplace;
   q.wgbox = s->wgbox;
   q.nwc = s->nwc;
   q.dsurv = s->dsurv;
@@ -1740,13 +1785,18 @@ static void make_plan(dcem_scene* s, int nrx, const dcem_params* p, bool coheren
   q.dseq3 = dord >= 3 ? s->dseq3 : nullptr;
   q.dseq3_cap = dord >= 3 ? s->dseq3_cap : 0;
   q.drel = dord >= 2 ? s->drel : nullptr;
+  const bool rows = dord >= 3 && obs1_words(s, nrx) > 0;
+  q.dsecond = rows ? s->dobs1 : nullptr;
+  q.dobs1 = rows ? s->dobs1 + (s->nw + 31) / 32 : nullptr;
+  q.dobs1_row = (nrx + 31) / 32;
   q.rmembers = dr ? s->rmembers : nullptr;
   q.rkeys = dr ? s->rkeys : nullptr;
   q.nrp = dr ? s->nrp : 0;
-  q.quads = dr ? s->quads : nullptr;
-  q.vis_any = dr ? s->vis : nullptr;
-  q.vis_grp = dr ? reinterpret_cast<int*>(s->vis + 2 * (size_t)s->nwc) : nullptr;
-  q.vis = dr ? s->vis + vis_head(s) : nullptr;
+  const bool uv = uses_vis(s);
+  q.quads = uv ? s->quads : nullptr;
+  q.vis_any = uv ? s->vis : nullptr;
+  q.vis_grp = uv ? reinterpret_cast<int*>(s->vis + 2 * (size_t)s->nwc) : nullptr;
+  q.vis = uv ? s->vis + vis_head(s) : nullptr;
   q.drefl2 = dr && s->diff_refl >= 2 ? 1 : 0;
   q.rmask = q.drefl2 ? s->rmask : nullptr;
   q.wobs_cnt = q.drefl2 ? s->wobs : nullptr;
@@ -1937,10 +1987,10 @@ static int diffraction_launches(const FramePlan& P) {
   if (!q.wedges) return 0;
   int n = 1 + (q.rplanes ? 1 : 0);  // wedge geometry, cluster boxes
   if (P.nlinks > 0) {
-    n += 3;  // first-order pre-test, occlusion, exact stage
-    if (q.rplanes) n += 3 + (q.drefl2 ? 4 : 0);  // visibility, one reflection; two: room, lists, join, double
+    n += 3 + (q.vis ? 1 : 0);  // first-order pre-test, occlusion, exact stage, visibility
+    if (q.rplanes) n += 2 + (q.drefl2 ? 4 : 0);  // visibility, one reflection; two: room, lists, join, double
     if (q.diff_order >= 2 && q.nw > 1)  // relation, pairs, [pairs around a plane], [triples], chains
-      n += q.diff_order + 1 + (q.dmid ? 1 : 0);
+      n += q.diff_order + 1 + (q.dmid ? 1 : 0) + (q.dobs1 ? 1 : 0);
   }
   return n;
 }
@@ -2038,6 +2088,7 @@ static int frame_begin(dcem_scene* s, const float* tx, int32_t ntx, const float*
   const int nlinks = ntx * nrx;
   if ((rc = ensure_rx(s, nrx, nlinks, s->bucket_cap)) != DCEM_OK) return rc;
   if ((rc = ensure_rmask(s, ntx, nrx)) != DCEM_OK) return rc;
+  if ((rc = ensure_obs1(s, nrx)) != DCEM_OK) return rc;
   cudaStream_t st = s->st;
   for (int t = 0; t < ntx; ++t)
     s->txs_h[t] = make_float4(tx[3 * t], tx[3 * t + 1], tx[3 * t + 2], alpha_eff_of(s->set_rays_h[t], p));

@@ -146,7 +146,10 @@ __device__ __forceinline__ d3 mk3(double x, double y, double z) { return d3{x, y
 __device__ __forceinline__ d3 operator+(d3 a, d3 b) { return mk3(a.x + b.x, a.y + b.y, a.z + b.z); }
 __device__ __forceinline__ d3 operator-(d3 a, d3 b) { return mk3(a.x - b.x, a.y - b.y, a.z - b.z); }
 __device__ __forceinline__ d3 operator*(d3 a, double s) { return mk3(a.x * s, a.y * s, a.z * s); }
-__device__ __forceinline__ double dd(d3 a, d3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
+// Dot products and complex products use explicit fused operations (half the
+// FP64 instructions); cross products do not, so that those of parallel
+// vectors with equal rounded products stay exactly zero.
+__device__ __forceinline__ double dd(d3 a, d3 b) { return fma(a.z, b.z, fma(a.y, b.y, a.x * b.x)); }
 __device__ __forceinline__ d3 dx(d3 a, d3 b) {
   return mk3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
 }
@@ -235,7 +238,9 @@ struct zd {
 __device__ __forceinline__ zd Z(double r, double i = 0.0) { return zd{r, i}; }
 __device__ __forceinline__ zd operator+(zd a, zd b) { return Z(a.re + b.re, a.im + b.im); }
 __device__ __forceinline__ zd operator-(zd a, zd b) { return Z(a.re - b.re, a.im - b.im); }
-__device__ __forceinline__ zd operator*(zd a, zd b) { return Z(a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re); }
+__device__ __forceinline__ zd operator*(zd a, zd b) {
+  return Z(fma(a.re, b.re, -(a.im * b.im)), fma(a.re, b.im, a.im * b.re));
+}
 __device__ __forceinline__ zd operator*(zd a, double s) { return Z(a.re * s, a.im * s); }
 __device__ __forceinline__ zd zdiv(zd a, zd b) {
   double d = b.re * b.re + b.im * b.im;
@@ -259,7 +264,9 @@ __device__ __forceinline__ float fdot3(float3 a, float3 b) { return a.x * b.x + 
 struct z3 {
   zd x, y, z;
 };
-__device__ __forceinline__ zd zdot(z3 e, d3 v) { return e.x * v.x + e.y * v.y + e.z * v.z; }
+__device__ __forceinline__ zd zdot(z3 e, d3 v) {
+  return Z(fma(e.z.re, v.z, fma(e.y.re, v.y, e.x.re * v.x)), fma(e.z.im, v.z, fma(e.y.im, v.y, e.x.im * v.x)));
+}
 __device__ __forceinline__ d3 dir_of(d3 a, d3 b) { return du(b - a); }  // unit vector a -> b
 // Polarisation of an isotropic antenna along unit d: u - (u.d) d, normalised
 // (a fixed axis instead when u is along d; the path is then flagged).
@@ -689,6 +696,19 @@ __global__ void __launch_bounds__(kFieldThreads) k_val_field(PathArgs a) {
 // ---------------------------------------------------------------------------
 // first-order edge diffraction (Sec. III step 5) with the UTD
 // ---------------------------------------------------------------------------
+// -1/n and 1/(2n + 1) for the erf series below (a division costs about ten
+// dependent FP64 operations, the rest of a term six).
+struct ErfTab {
+  double a[200], b[200];
+  constexpr ErfTab() : a(), b() {
+    for (int n = 1; n < 200; ++n) {
+      a[n] = -1.0 / n;
+      b[n] = 1.0 / (2 * n + 1);
+    }
+  }
+};
+__constant__ ErfTab kErfTab = ErfTab();
+
 // erfc(z) for Re z > 0: the Maclaurin series of erf (Abramowitz & Stegun
 // 7.1.5) for |z| < 3, else the continued fraction of A&S 7.1.14, truncated
 // after 40, 30 or 20 terms for |z| from 3, 3.5 or 4.5 on (relative error
@@ -700,8 +720,8 @@ __device__ zd erfc_z(zd z) {
   if (az < 3.0) {
     zd z2 = z * z, term = z, sum = z;
     for (int n = 1; n < 200; ++n) {
-      term = term * z2 * (-1.0 / n);
-      zd t = term * (1.0 / (2 * n + 1));
+      term = term * z2 * kErfTab.a[n];
+      zd t = term * kErfTab.b[n];
       sum = sum + t;
       if (fabs(t.re) + fabs(t.im) < 1e-17 * (fabs(sum.re) + fabs(sum.im))) break;
     }
@@ -714,7 +734,9 @@ __device__ zd erfc_z(zd z) {
   zd A0 = Z(1.0), A1 = z, B0 = Z(0.0), B1 = Z(1.0);
   const int nt = az < 3.5 ? 40 : az < 4.5 ? 30 : 20;
   for (int k = 1; k <= nt; ++k) {
-    zd A2 = z * A1 + A0 * (0.5 * k), B2 = z * B1 + B0 * (0.5 * k);
+    const double h = 0.5 * k;
+    const zd za = z * A1, zb = z * B1;
+    zd A2 = Z(fma(A0.re, h, za.re), fma(A0.im, h, za.im)), B2 = Z(fma(B0.re, h, zb.re), fma(B0.im, h, zb.im));
     A0 = A1;
     A1 = A2;
     B0 = B1;
@@ -767,6 +789,18 @@ __device__ zd utd_term(double n, double beta, double s, double kL, unsigned& fl)
 // with face reflection factors r0, rn. The prefactor and the four terms do
 // not depend on r0 and rn, so the soft and hard coefficients share them
 // (utd_parts once, utd_coeff per polarisation).
+// The exact stage takes a survivor with a group of kDiffLanes lanes that run
+// the same code on the same values and split what is independent: the four
+// terms here, the two faces' Fresnel factors, the legs' occlusion.
+constexpr int kDiffLanes = 4;
+__device__ __forceinline__ int diff_lane() { return threadIdx.x & (kDiffLanes - 1); }
+__device__ __forceinline__ unsigned diff_mask() {
+  return ((1u << kDiffLanes) - 1u) << ((threadIdx.x & 31) & ~(kDiffLanes - 1));
+}
+__device__ __forceinline__ zd diff_from(zd v, int lane) {  // the value of a lane of the group
+  const unsigned m = diff_mask();
+  return Z(__shfl_sync(m, v.re, lane, kDiffLanes), __shfl_sync(m, v.im, lane, kDiffLanes));
+}
 struct UtdParts {
   zd pre, t[4];
 };
@@ -774,11 +808,10 @@ __device__ UtdParts utd_parts(double n, double phi, double phip, double beta0, d
   const double h = 0.70710678118654752440;
   UtdParts u;
   u.pre = Z(-h, h) * (1.0 / (2.0 * n * sqrt(2.0 * M_PI * k) * sin(beta0)));  // -e^{-j pi/4} / (...)
-  double bm = phi - phip, bp = phi + phip, kL = k * L;
-  u.t[0] = utd_term(n, bm, 1.0, kL, fl);
-  u.t[1] = utd_term(n, bm, -1.0, kL, fl);
-  u.t[2] = utd_term(n, bp, -1.0, kL, fl);
-  u.t[3] = utd_term(n, bp, 1.0, kL, fl);
+  // terms: (phi - phi', +), (phi - phi', -), (phi + phi', -), (phi + phi', +)
+  const int q = diff_lane();
+  const zd t = utd_term(n, q < 2 ? phi - phip : phi + phip, q == 0 || q == 3 ? 1.0 : -1.0, k * L, fl);
+  for (int j = 0; j < 4; ++j) u.t[j] = diff_from(t, j);
   return u;
 }
 __device__ zd utd_coeff(const UtdParts& u, zd r0, zd rn) {
@@ -798,6 +831,18 @@ __device__ void fresnel_d(float4 mt, double freq, double ct, zd& te, zd& tm) {
   tm = zdiv(ec * ct - root, ec * ct + root);
 }
 
+// ... of a wedge's two faces at once (te, tm of face 0, then of face n).
+__device__ __forceinline__ void fresnel_faces(float4 ma, double cta, float4 mb, double ctb, double freq, zd& r0s,
+                                              zd& r0h, zd& rns, zd& rnh) {
+  const bool second = diff_lane() & 1;
+  zd te, tm;
+  fresnel_d(second ? mb : ma, freq, second ? ctb : cta, te, tm);
+  r0s = diff_from(te, 0);
+  r0h = diff_from(tm, 0);
+  rns = diff_from(te, 1);
+  rnh = diff_from(tm, 1);
+}
+
 struct d3w {
   double x, y, z;
 };
@@ -805,7 +850,7 @@ __device__ __forceinline__ d3w D3(double x, double y, double z) { return d3w{x, 
 __device__ __forceinline__ d3w operator-(d3w a, d3w b) { return D3(a.x - b.x, a.y - b.y, a.z - b.z); }
 __device__ __forceinline__ d3w operator+(d3w a, d3w b) { return D3(a.x + b.x, a.y + b.y, a.z + b.z); }
 __device__ __forceinline__ d3w operator*(d3w a, double s) { return D3(a.x * s, a.y * s, a.z * s); }
-__device__ __forceinline__ double dotw(d3w a, d3w b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
+__device__ __forceinline__ double dotw(d3w a, d3w b) { return fma(a.z, b.z, fma(a.y, b.y, a.x * b.x)); }
 __device__ __forceinline__ d3w crossw(d3w a, d3w b) {
   return D3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
 }
@@ -947,13 +992,18 @@ __device__ __noinline__ int leg_crossings(const PathArgs& a, d3w p, d3w q, int e
   return n;
 }
 
-// FP32 any-hit of the open segment a -> b, the wedge faces (and a reflecting
-// triangle) excluded.
-__device__ __noinline__ bool leg_occluded(const PathArgs& a, d3w p, d3w q, int ex0, int ex1, unsigned& ovf,
-                                             TStack& st, int ex2 = -1) {
-  d3w dv = q - p;
-  RayPre rp = ray_pre(f3((float)p.x, (float)p.y, (float)p.z), f3((float)dv.x, (float)dv.y, (float)dv.z));
-  return any_hit(a.bvh, rp, a.eps_occ, 1.0f - a.eps_occ, ex0, ex1, ovf, st, ex2);
+// FP32 any-hit of the legs between the n points P of a path, two triangles
+// excluded at each point; the legs are shared out over the group's lanes.
+__device__ __noinline__ bool legs_occluded(const PathArgs& a, const d3w* P, const int (*ex)[2], int n, unsigned& ovf,
+                                           TStack& st) {
+  bool hit = false;
+  for (int q = diff_lane(); q + 1 < n && !hit; q += kDiffLanes) {
+    const d3w dv = P[q + 1] - P[q];
+    const RayPre rp = ray_pre(f3((float)P[q].x, (float)P[q].y, (float)P[q].z),
+                              f3((float)dv.x, (float)dv.y, (float)dv.z));
+    hit = any_hit(a.bvh, rp, a.eps_occ, 1.0f - a.eps_occ, ex[q][0], ex[q][1], ovf, st, ex[q + 1][0], ex[q + 1][1]);
+  }
+  return __any_sync(diff_mask(), hit);
 }
 
 // Wedge geometry from the current world triangles (moving objects' wedges
@@ -1077,8 +1127,10 @@ __device__ __forceinline__ void diffract_pair(const PathArgs& a, long idx, doubl
     if (n1 < 0) return;
     n2 = leg_crossings(a, Q, R, W.ta, W.tb, W.tb, W.tb, c2, mt - n1, ovf, st);
     if (n2 < 0) return;
-  } else if (leg_occluded(a, T, Q, W.ta, W.tb, ovf, st) || leg_occluded(a, Q, R, W.ta, W.tb, ovf, st)) {
-    return;
+  } else {
+    const d3w P[3] = {T, Q, R};
+    const int ex[3][2] = {{-1, -1}, {W.ta, W.tb}, {-1, -1}};
+    if (legs_occluded(a, P, ex, 3, ovf, st)) return;
   }
   unsigned fl = 0;
   d3w qt = Q - T, rq = R - Q;
@@ -1095,8 +1147,7 @@ __device__ __forceinline__ void diffract_pair(const PathArgs& a, long idx, doubl
   const float4 mb =
       a.mats[__float_as_int(a.tris[3 * (size_t)DCEM_IDX(a.slot_of_id[DCEM_IDX(W.tb, a.bvh.ntris)], a.bvh.ntris) + 1].w)];
   zd r0s, r0h, rns, rnh;
-  fresnel_d(ma, a.freq, fabs(sin(phip)), r0s, r0h);
-  fresnel_d(mb, a.freq, fabs(sin(n * M_PI - phi)), rns, rnh);
+  fresnel_faces(ma, fabs(sin(phip)), mb, fabs(sin(n * M_PI - phi)), a.freq, r0s, r0h, rns, rnh);
   const UtdParts up = utd_parts(n, phi, phip, beta0, L, k, fl);
   zd Ds = utd_coeff(up, r0s, rns);
   zd Dh = utd_coeff(up, r0h, rnh);
@@ -1118,6 +1169,7 @@ __device__ __forceinline__ void diffract_pair(const PathArgs& a, long idx, doubl
     g *= pow(10.0, -(double)mt.w / 20.0);
   }
   zd amp = proj * A * (lam / (4.0 * M_PI) * g);
+  if (diff_lane() != 0) return;  // one lane of the group writes the record
   unsigned uu = atomicAdd(&a.ctr->n_unique, 1u);
   if (uu >= a.ucap) {
     atomicOr(&a.ctr->err, ERR_UNIQUE_OVERFLOW);
@@ -1316,7 +1368,9 @@ __device__ int member_at(const PathArgs& a, const RPlane& G, d3w x, const int* e
 struct zv3 {
   zd x, y, z;
 };
-__device__ __forceinline__ zd zvdot(zv3 E, d3w v) { return E.x * v.x + E.y * v.y + E.z * v.z; }
+__device__ __forceinline__ zd zvdot(zv3 e, d3w v) {
+  return Z(fma(e.z.re, v.z, fma(e.y.re, v.y, e.x.re * v.x)), fma(e.z.im, v.z, fma(e.y.im, v.y, e.x.im * v.x)));
+}
 
 // One survivor: exact geometry on the plane, the member triangle holding the
 // reflection point, the geometry again on that triangle's own plane, the
@@ -1345,15 +1399,10 @@ __device__ __forceinline__ void diffract_refl_pair(const PathArgs& a, unsigned l
   if (!refl_geometry(W, nj, dotw(nj, v0), T, R, first, g)) return;
   if (!inside_tri64(v0, v1, v2, g.P)) return;
   const d3w Q = g.Q, Pp = g.P;
-  if (first) {
-    if (leg_occluded(a, T, Pp, j, j, ovf, st) || leg_occluded(a, Pp, Q, j, W.ta, ovf, st, W.tb) ||
-        leg_occluded(a, Q, R, W.ta, W.tb, ovf, st))
-      return;
-  } else {
-    if (leg_occluded(a, T, Q, W.ta, W.tb, ovf, st) || leg_occluded(a, Q, Pp, j, W.ta, ovf, st, W.tb) ||
-        leg_occluded(a, Pp, R, j, j, ovf, st))
-      return;
-  }
+  const d3w P[4] = {T, first ? Pp : Q, first ? Q : Pp, R};
+  const int e0 = first ? j : W.ta, e1 = first ? j : W.tb, e2 = first ? W.ta : j, e3 = first ? W.tb : j;
+  const int ex[4][2] = {{-1, -1}, {e0, e1}, {e2, e3}, {-1, -1}};
+  if (legs_occluded(a, P, ex, 4, ovf, st)) return;
   unsigned fl = 0;
   const double n = W.n, phip = g.phip, phi = g.phi;
   d3w e = D3(W.e[0], W.e[1], W.e[2]);
@@ -1372,8 +1421,7 @@ __device__ __forceinline__ void diffract_refl_pair(const PathArgs& a, unsigned l
     tri64(a, W.tb, x0, x1, x2, mb);
   }
   zd r0s, r0h, rns, rnh;
-  fresnel_d(ma, a.freq, fabs(sin(phip)), r0s, r0h);
-  fresnel_d(mb, a.freq, fabs(sin(n * M_PI - phi)), rns, rnh);
+  fresnel_faces(ma, fabs(sin(phip)), mb, fabs(sin(n * M_PI - phi)), a.freq, r0s, r0h, rns, rnh);
   const UtdParts up = utd_parts(n, phi, phip, beta0, L, k, fl);
   zd Ds = utd_coeff(up, r0s, rns);
   zd Dh = utd_coeff(up, r0h, rnh);
@@ -1418,6 +1466,7 @@ __device__ __forceinline__ void diffract_refl_pair(const PathArgs& a, unsigned l
     proj = zvdot(E2, prx);
   }
   zd amp = proj * A * (lam / (4.0 * M_PI));
+  if (diff_lane() != 0) return;  // one lane of the group writes the record
   unsigned uu = atomicAdd(&a.ctr->n_unique, 1u);
   if (uu >= a.ucap) {
     atomicOr(&a.ctr->err, ERR_UNIQUE_OVERFLOW);
@@ -1765,36 +1814,231 @@ __device__ __forceinline__ bool plane_reachable(const RPlane& Pl, float3 S, floa
   return leg_window(Pl, S, A, B, m, lo, hi);
 }
 
+// ---- what an end point can see ----
+// In built-up scenes most reflector planes and wedges are hidden from a given
+// end point (and from one another) behind one wall, and every real leg must
+// be free: so the planes and wedges that are certainly hidden from an end
+// point as a whole take no part as its first reflection or as the wedge it
+// sees directly, and two wedges hidden from each other are no chain's
+// neighbours. A target is hidden when one convex wall quad -- two static coplanar
+// triangles that share an edge -- is crossed strictly inside, by the margins
+// of leg_surely_blocked, by the legs to every corner of the target: the
+// crossings of the legs to the points between the corners lie between
+// theirs. The quads tried are those the leg to the target's middle crosses.
+
+__device__ __forceinline__ float3 end_point(const PathArgs& a, int ntx, int x) {
+  const float4 v = x < ntx ? a.txs[x] : a.rx[x - ntx];
+  return f3(v.x, v.y, v.z);
+}
+
+// Does quad q (q[0].w != 0) cut off point X from E with margin?
+__device__ __forceinline__ bool quad_between(const float4* __restrict__ q, float3 E, float3 X, float eps_occ) {
+  const float4 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3];
+  if (q0.w == 0.0f) return false;
+  const float3 c[4] = {f3(q0.x, q0.y, q0.z), f3(q1.x, q1.y, q1.z), f3(q2.x, q2.y, q2.z), f3(q3.x, q3.y, q3.z)};
+  const float3 dv = f3(X.x - E.x, X.y - E.y, X.z - E.z);
+  const float dl = sqrtf(fdot3(dv, dv));
+  const float3 nv = cross3(f3(c[1].x - c[0].x, c[1].y - c[0].y, c[1].z - c[0].z),
+                           f3(c[2].x - c[0].x, c[2].y - c[0].y, c[2].z - c[0].z));
+  const float nn = sqrtf(fdot3(nv, nv)), dn = fdot3(dv, nv);
+  if (!(dl > 0.0f && fabsf(dn) > 1e-3f * dl * nn)) return false;
+  const float u = fdot3(f3(c[0].x - E.x, c[0].y - E.y, c[0].z - E.z), nv) / dn;
+  const float slack = 2e-3f + 1e-6f * (fabsf(E.x) + fabsf(E.y) + fabsf(E.z) + dl);
+  const float mu = 0.01f * (1.0f + dl * nn / fabsf(dn)) + slack, nu = mu / dl;
+  if (!(u > eps_occ + nu && u < 1.0f - eps_occ - nu)) return false;
+  const float3 H = f3(E.x + dv.x * u, E.y + dv.y * u, E.z + dv.z * u);
+  for (int k = 0; k < 4; ++k) {
+    const float3 a = c[k], b = c[(k + 1) & 3];
+    const float3 e = f3(b.x - a.x, b.y - a.y, b.z - a.z);
+    const float el = sqrtf(fdot3(e, e));
+    if (el > 0.0f && !(fdot3(cross3(e, f3(H.x - a.x, H.y - a.y, H.z - a.z)), nv) > mu * el * nn)) return false;
+  }
+  return true;
+}
+
+// What is to be hidden: from E0 the box lo..hi (kind 0) or the segment lo-hi
+// (1), or from the segment E0-E1 the segment lo-hi (2: the crossings of the
+// legs between two segments on either side of a plane are convex
+// combinations of those of the four legs between their ends).
+struct HiddenCase {
+  int kind;
+  float3 E0, E1, lo, hi;
+};
+// Is it certainly hidden behind one quad?
+__device__ __noinline__ bool surely_hidden(const PathArgs& a, const HiddenCase& h, TStack& st) {
+  const float3 lo = h.lo, hi = h.hi;
+  const float3 mid = f3(0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z));
+  const float3 E = h.kind < 2 ? h.E0 : f3(0.5f * (h.E0.x + h.E1.x), 0.5f * (h.E0.y + h.E1.y), 0.5f * (h.E0.z + h.E1.z));
+  const RayPre rp = ray_pre(E, f3(mid.x - E.x, mid.y - E.y, mid.z - E.z));
+  st.reset();
+  int cur = a.bvh.root0;  // static triangles only
+  for (int visits = 0; visits <= a.bvh.max_visits; ++visits) {
+    if (cur == kEmpty) {
+      if (st.empty()) break;
+      cur = st.pop();
+      continue;
+    }
+    if (cur >= 0) {
+      const float4* n = a.bvh.nodes + 4 * (size_t)DCEM_IDX(cur, a.bvh.nnodes);
+      float4 n0 = __ldg(n), n1 = __ldg(n + 1), n2 = __ldg(n + 2), n3 = __ldg(n + 3);
+      float tn0, tn1;
+      const bool h0 = slab(rp, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, 1.0f, tn0);
+      const bool h1 = slab(rp, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, 1.0f, tn1);
+      const int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
+      if (h0 && h1) {
+        if (!st.push(c1)) return false;
+        cur = c0;
+      } else {
+        cur = h0 ? c0 : h1 ? c1 : kEmpty;
+      }
+      continue;
+    }
+    const int id = __float_as_int(__ldg(&a.bvh.tris[3 * (size_t)DCEM_IDX(~cur, a.bvh.ntris)]).w);
+    cur = kEmpty;
+    const float4* q = a.quads + 4 * (size_t)DCEM_IDX(id, a.bvh.ntris);
+    bool all = quad_between(q, E, mid, a.eps_occ);
+    for (int k = 0; all && k < (h.kind == 0 ? 8 : 2 * h.kind); ++k) {
+      const float3 X = h.kind ? ((k & 1) ? hi : lo) : f3((k & 1) ? hi.x : lo.x, (k & 2) ? hi.y : lo.y, (k & 4) ? hi.z : lo.z);
+      all = quad_between(q, h.kind == 2 ? ((k & 2) ? h.E1 : h.E0) : E, X, a.eps_occ);
+    }
+    if (all) return true;
+  }
+  return false;
+}
+
+// Per end point the planes, then the wedges (in the order wperm) it may see,
+// one warp per word. A wedge the end point is inside of is not seen. Both
+// orders are spatial, so that a warp's legs run close together.
+__global__ void __launch_bounds__(64) k_diff_visible(PathArgs a, int ntx) {
+  extern __shared__ int sstk[];
+  TStack st;
+  bind_stack(st, sstk, kStackTrace);
+  const int npw = (a.nrp + 31) / 32, row = npw + a.nwc, lane = threadIdx.x & 31;
+  const long nitem = (long)(ntx + a.nrx) * row, nwarp = (long)gridDim.x * (blockDim.x >> 5);
+  for (long it = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < nitem; it += nwarp) {
+    const int x = (int)(it / row), c = (int)(it - (long)x * row);
+    const float3 E = end_point(a, ntx, x);
+    bool see = false;
+    if (c < npw) {
+      const int p = c * 32 + lane;
+      if (p < a.nrp) {
+        const float* b = a.rplanes[p].box;
+        see = !surely_hidden(a, HiddenCase{0, E, E, f3(b[0], b[1], b[2]), f3(b[3], b[4], b[5])}, st);
+      }
+    } else {
+      const int i = (c - npw) * kWedgeCluster + lane;
+      if (i < a.nw) {
+        const WedgeF W = a.wf[a.wperm[i]];
+        float3 A, B;
+        edge_ends(W, A, B);
+        see = !surely_inside(W, E) && !surely_hidden(a, HiddenCase{1, E, E, A, B}, st);
+      }
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, see);
+    if (lane == 0) a.vis[it] = m;
+  }
+}
+// The wedges some transmitter (words 0 .. nwc - 1) or some receiver sees, and
+// lists of the groups that hold any (per side a count, then the groups).
+__global__ void __launch_bounds__(256) k_diff_visible_any(PathArgs a, int ntx) {
+  __shared__ unsigned cnt;
+  const int npw = (a.nrp + 31) / 32, row = npw + a.nwc, side = blockIdx.x;
+  const int ng = (a.nw + kWedgeGroup - 1) / kWedgeGroup;
+  int* list = a.vis_grp + (size_t)side * (ng + 1);
+  if (threadIdx.x == 0) cnt = 0u;
+  __syncthreads();
+  for (int c0 = 0; c0 < a.nwc; c0 += 32) {  // lanes: words, warps: end points
+    __shared__ unsigned part[32];
+    const int c = c0 + (threadIdx.x & 31);
+    if (threadIdx.x < 32) part[threadIdx.x] = 0u;
+    __syncthreads();
+    if (c < a.nwc) {
+      unsigned m = 0;
+      const int x1 = side ? ntx + a.nrx : ntx;
+      for (int x = (side ? ntx : 0) + (threadIdx.x >> 5); x < x1; x += 8) m |= a.vis[(long)x * row + npw + c];
+      atomicOr(&part[threadIdx.x & 31], m);
+    }
+    __syncthreads();
+    if (threadIdx.x < 32 && c < a.nwc) {
+      const unsigned m = part[threadIdx.x];
+      a.vis_any[side * a.nwc + c] = m;
+      for (int k = 0; k < 4; ++k)
+        if ((m >> (8 * k)) & 0xffu) list[1 + atomicAdd(&cnt, 1u)] = 4 * c + k;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) list[0] = (int)cnt;
+}
+__device__ __forceinline__ bool sees_plane(const PathArgs& a, int x, int p) {
+  const int npw = (a.nrp + 31) / 32;
+  return (a.vis[(long)x * (npw + a.nwc) + p / 32] >> (p & 31)) & 1u;
+}
+// (i: the wedge's place in the order wperm)
+__device__ __forceinline__ bool sees_wedge(const PathArgs& a, int x, int i) {
+  const int npw = (a.nrp + 31) / 32;
+  return (a.vis[(long)x * (npw + a.nwc) + npw + i / kWedgeCluster] >> (i % kWedgeCluster)) & 1u;
+}
+
+// (as sees_wedge, for wedge w; true when the rows are not built)
+__device__ __forceinline__ bool end_sees(const PathArgs& a, int x, int w) { return !a.vis || sees_wedge(a, x, a.wplace[w]); }
+__device__ __forceinline__ bool wedges_hidden(const PathArgs& a, const WedgeF& A, const WedgeF& B, TStack& st) {
+  HiddenCase h;
+  h.kind = 2;
+  edge_ends(A, h.E0, h.E1);
+  edge_ends(B, h.lo, h.hi);
+  return surely_hidden(a, h, st);
+}
+
 // The relation of consecutive wedges in a chain, once per frame (moving
 // wedges change it): distinct, no shared vertex, not on one line, neither
 // edge in a face plane of the other, each edge partly in the other's
-// exterior; one bit per ordered pair (w1, w2) in a.drel.
+// exterior; one bit per ordered pair (w1, w2) in a.drel. It is symmetric: a
+// warp takes 32 pairs w1 < w2 of one w1 and sets both bits. With chains of
+// three wedges the pairs hidden from each other are dropped here (every
+// triple holds two; 8 x 8 city: 335k triples become a tenth); with chains of
+// two only those k_diff_pairs lists are tested, there.
 __global__ void __launch_bounds__(256) k_diff_rel(PathArgs a) {
-  const long nw = a.nw, total = nw * nw;
-  for (long idx = (long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (long)gridDim.x * blockDim.x) {
-    const int w1 = (int)(idx / nw), w2 = (int)(idx - (long)w1 * nw);
-    bool rel = w1 != w2;
+  extern __shared__ int sstk[];
+  TStack st;
+  bind_stack(st, sstk, kStackTrace);
+  const long nw = a.nw, nch = (nw + 31) / 32, nitem = nw * nch;
+  const int lane = threadIdx.x & 31;
+  const long nwarp = (long)gridDim.x * (blockDim.x >> 5);
+  for (long it = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < nitem; it += nwarp) {
+    const int w1 = (int)(it / nch), w2 = (int)(it - (long)w1 * nch) * 32 + lane;
+    bool rel = w1 < w2 && w2 < nw;
+    if (!__any_sync(0xffffffffu, rel)) continue;
     if (rel) {  // the FP32 exterior tests first: they reject most pairs
       const WedgeF fa = a.wf[w1], fb = a.wf[w2];
-      float3 pa, qa;
+      float3 pa, qa, pb, qb;
       edge_ends(fa, pa, qa);
-      const float m = fmaxf(pre_margin_m(pa), pre_margin_m(qa));
+      edge_ends(fb, pb, qb);
+      const float m = fmaxf(fmaxf(pre_margin_m(pa), pre_margin_m(qa)), fmaxf(pre_margin_m(pb), pre_margin_m(qb)));
       rel = edge_sees(fa, fb, m) && edge_sees(fb, fa, m);
+      if (rel && a.diff_order >= 3) rel = !wedges_hidden(a, fa, fb, st);
     }
     if (rel) {
       const Wedge &A = a.wedges[w1], &B = a.wedges[w2];
       rel = !share_vertex(A, B) && !collinear_edges(A, B) && !in_face_plane(A, B) && !in_face_plane(B, A);
     }
-    if (rel) atomicOr(&a.drel[idx >> 5], 1u << (idx & 31));
+    if (rel) {
+      const long x = (long)w1 * nw + w2, y = (long)w2 * nw + w1;
+      atomicOr(&a.drel[x >> 5], 1u << (x & 31));
+      atomicOr(&a.drel[y >> 5], 1u << (y & 31));
+    }
   }
 }
 
 // Ordered pairs (w1, w2) per source (transmitter or transmitter image) that
 // can start a path of order >= 2: in the relation (k_diff_rel), the
 // transmitter outside w1, some point of edge 2 beyond the incident shadow
-// boundary of the transmitter at w1, and a Keller point on w1 possible
-// between the transmitter and edge 2 (keller_on_edge).
+// boundary of the transmitter at w1, a Keller point on w1 possible between
+// the transmitter and edge 2 (keller_on_edge), and neither w1 hidden from the
+// (real) transmitter nor w2 from w1.
 __global__ void __launch_bounds__(256) k_diff_pairs(PathArgs a, int nsrc) {
+  extern __shared__ int sstk[];
+  TStack st;
+  bind_stack(st, sstk, kStackTrace);
   const long nw = a.nw, total = (long)nsrc * nw * nw;
   const int lane = threadIdx.x & 31;
   const long stride = (long)gridDim.x * blockDim.x;
@@ -1807,7 +2051,7 @@ __global__ void __launch_bounds__(256) k_diff_pairs(PathArgs a, int nsrc) {
       long r = idx - (long)t * nw * nw;
       w1 = (int)(r / nw);
       w2 = (int)(r - (long)w1 * nw);
-      if ((a.drel[r >> 5] >> (r & 31)) & 1u) {
+      if (((a.drel[r >> 5] >> (r & 31)) & 1u) && (t >= a.dntx || end_sees(a, t, w1))) {
         const WedgeF fa = a.wf[w1], fb = a.wf[w2];
         float3 T = chain_source32(a, t), P, Q;
         edge_ends(fb, P, Q);
@@ -1818,6 +2062,7 @@ __global__ void __launch_bounds__(256) k_diff_pairs(PathArgs a, int nsrc) {
           float mg = 0.1f + 1e-4f * (fabsf(T.x) + fabsf(T.y) + fabsf(T.z) + fa.len);
           keep = plane_reachable(a.rplanes[(t - a.dntx) % a.nrpr], T, A1, B1, mg);
         }
+        if (keep && a.diff_order < 3) keep = !wedges_hidden(a, fa, fb, st);
       }
     }
     unsigned mk = __ballot_sync(0xffffffffu, keep);
@@ -1828,6 +2073,7 @@ __global__ void __launch_bounds__(256) k_diff_pairs(PathArgs a, int nsrc) {
     if (keep) {
       if (at < a.dseq2_cap) a.dseq2[at] = make_int4(t, w1, w2, -1);
       else atomicOr(&a.ctr->err, ERR_DIFF_OVERFLOW);
+      if (a.dobs1) atomicOr(&a.dsecond[w2 >> 5], 1u << (w2 & 31));
     }
   }
 }
@@ -1949,7 +2195,7 @@ __global__ void __launch_bounds__(256) k_diff_mid_pairs(PathArgs a) {
     const int w1 = (int)(r % a.nw), t = (int)(r / a.nw);
     const WedgeF fa = a.wf[w1];
     const float3 T = chain_source32(a, t);
-    if (surely_inside(fa, T)) continue;  // warp-uniform
+    if (surely_inside(fa, T) || !end_sees(a, t, w1)) continue;  // warp-uniform
     const RPlane& Pl = a.rplanes[p];
     const float3 n = f3(Pl.nf[0], Pl.nf[1], Pl.nf[2]);
     float3 A0, A1;
@@ -2024,9 +2270,15 @@ __global__ void __launch_bounds__(256) k_diff_triples(PathArgs a) {
 }
 
 // FP32 Keller points of a chain (the pre-test's estimate): Newton's method
-// as in keller_chain, in FP32, from the edges' midpoints. Returns true when
-// the cosine mismatch fell below 2e-6 at every edge, or a full Newton step
-// would move no point by more than step_tol (metres).
+// as in keller_chain, in FP32, from the edges' midpoints, with the iterates
+// kept within kKellerBox metres of the edges (coordinates at that bound with
+// the slope pointing out stay there; the rest take the reduced step).
+// Returns 1 when the cosine mismatch fell below 2e-6 at every edge, or a full
+// Newton step would move no point by more than step_tol (metres); -1 when
+// the minimum certainly lies off an edge: the length is convex, so at any
+// points y on the edges it is at least L(t) + g.(y - t), and that exceeds
+// L(t) for all of them by more than the slope's rounding; else 0.
+constexpr float kKellerBox = 1.0f;
 __device__ __forceinline__ float chain_len32(const WedgeF* W, int m, float3 T, float3 R, const float* t) {
   float3 prev = T;
   float L = 0.0f;
@@ -2039,7 +2291,7 @@ __device__ __forceinline__ float chain_len32(const WedgeF* W, int m, float3 T, f
   float3 d = f3(R.x - prev.x, R.y - prev.y, R.z - prev.z);
   return L + sqrtf(fdot3(d, d));
 }
-__device__ bool keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, float step_tol) {
+__device__ int keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, float step_tol) {
   for (int i = 0; i < m; ++i) t[i] = 0.5f * W[i].len;
   float Lc = chain_len32(W, m, T, R, t);
   for (int it = 0; it < 30; ++it) {
@@ -2047,11 +2299,14 @@ __device__ bool keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, f
     X[0] = T;
     for (int i = 0; i < m; ++i) X[i + 1] = edge_point(W[i], t[i]);
     X[m + 1] = R;
-    float g[3] = {0.0f, 0.0f, 0.0f}, H[3][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
+    float serr[4], g[3] = {0.0f, 0.0f, 0.0f}, H[3][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
     for (int j = 0; j <= m; ++j) {
       float3 d = f3(X[j + 1].x - X[j].x, X[j + 1].y - X[j].y, X[j + 1].z - X[j].z);
       float l = sqrtf(fdot3(d, d));
-      if (!(l > 0.0f)) return false;
+      if (!(l > 0.0f)) return 0;
+      // rounding of this leg's direction (as in keller_on_edge)
+      serr[j] = 2e-5f + 2e-6f * (fabsf(X[j].x) + fabsf(X[j].y) + fabsf(X[j].z) + fabsf(X[j + 1].x) +
+                                 fabsf(X[j + 1].y) + fabsf(X[j + 1].z)) / l;
       float3 u = f3(d.x / l, d.y / l, d.z / l);
       int ia = j - 1, ib = j;
       float ca = ia >= 0 ? fdot3(W[ia].e, u) : 0.0f, cb = ib < m ? fdot3(W[ib].e, u) : 0.0f;
@@ -2069,9 +2324,23 @@ __device__ bool keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, f
         H[ib][ia] += h;
       }
     }
+    float cut = 0.0f;
+    for (int i = 0; i < m; ++i) {
+      const float err = serr[i] + serr[i + 1], far = fmaxf(fabsf(t[i]), fabsf(W[i].len - t[i]));
+      cut += fminf(-g[i] * t[i], g[i] * (W[i].len - t[i])) - err * far;
+    }
+    if (cut > 0.0f) return -1;
     float gmax = 0.0f;
-    for (int i = 0; i < m; ++i) gmax = fmaxf(gmax, fabsf(g[i]));
-    if (gmax < 2e-6f) return true;
+    bool bound = false;
+    for (int i = 0; i < m; ++i) {
+      if ((t[i] <= -kKellerBox && g[i] > 0.0f) || (t[i] >= W[i].len + kKellerBox && g[i] < 0.0f)) {
+        bound = true;  // held at the bound
+        g[i] = 0.0f;
+        for (int j = 0; j < m; ++j) H[i][j] = H[j][i] = i == j ? 1.0f : 0.0f;
+      }
+      gmax = fmaxf(gmax, fabsf(g[i]));
+    }
+    if (gmax < 2e-6f) return bound ? 0 : 1;
     float A[3][4], dx[3];
     for (int i = 0; i < m; ++i) {
       for (int j = 0; j < m; ++j) A[i][j] = H[i][j];
@@ -2081,7 +2350,7 @@ __device__ bool keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, f
       int piv = c;
       for (int r = c + 1; r < m; ++r)
         if (fabsf(A[r][c]) > fabsf(A[piv][c])) piv = r;
-      if (!(fabsf(A[piv][c]) > 1e-30f)) return false;
+      if (!(fabsf(A[piv][c]) > 1e-30f)) return 0;
       if (piv != c)
         for (int j = 0; j <= m; ++j) {
           float x = A[c][j];
@@ -2103,7 +2372,7 @@ __device__ bool keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, f
     float step = 1.0f, tn[3] = {t[0], t[1], t[2]};
     bool moved = false;
     for (int q = 0; q < 30; ++q) {
-      for (int i = 0; i < m; ++i) tn[i] = t[i] + step * dx[i];
+      for (int i = 0; i < m; ++i) tn[i] = fminf(fmaxf(t[i] + step * dx[i], -kKellerBox), W[i].len + kKellerBox);
       float Ln = chain_len32(W, m, T, R, tn);
       if (Ln <= Lc * (1.0f + 1e-6f)) {
         Lc = fminf(Lc, Ln);
@@ -2112,13 +2381,13 @@ __device__ bool keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, f
       }
       step *= 0.5f;
     }
-    if (!moved) return gmax < 1e-4f;
+    if (!moved) return gmax < 1e-4f && !bound ? 1 : 0;
     for (int i = 0; i < m; ++i) t[i] = tn[i];
     // the full Newton step (the quadratic model's distance to the
     // stationary point) below step_tol: close enough for the margins
-    if (dfull < step_tol) return true;
+    if (dfull < step_tol && !bound) return 1;
   }
-  return false;
+  return 0;
 }
 
 // Position margin of the FP32 Keller estimate: 5 cm plus 1e-5 of the
@@ -2200,8 +2469,10 @@ __device__ __noinline__ bool leg_surely_blocked(const Bvh& bvh, float3 o, float3
 // reject anything.
 __device__ __noinline__ bool chain_possible(const WedgeF* W, int m, float3 T, float3 R, float* t, bool* solved) {
   float mt = chain_margin(T, R);
-  *solved = keller32(W, m, T, R, t, 0.1f * mt);
-  if (!*solved) return true;
+  const int kr = keller32(W, m, T, R, t, 0.1f * mt);
+  *solved = kr > 0;
+  if (kr < 0) return false;
+  if (kr == 0) return true;
   float3 X[5];
   X[0] = T;
   for (int i = 0; i < m; ++i) {
@@ -2246,6 +2517,7 @@ __device__ __noinline__ bool chain_possible(const WedgeF* W, int m, float3 T, fl
 // the last edge must be able to cross its plane inside the box.
 __device__ __forceinline__ bool multi_stage1(const PathArgs& a, int4 sq, bool three, int rho) {
   const bool mid = !three && sq.w <= -2, obs_img = rho >= a.nrx;
+  if (!obs_img && !end_sees(a, a.dntx + rho, three ? sq.w : sq.z)) return false;
   WedgeF fl = a.wf[three ? sq.w : sq.z];
   const WedgeF fp = a.wf[three ? sq.z : sq.y];
   float3 R = chain_observer32(a, rho), P, Q;
@@ -2264,6 +2536,33 @@ __device__ __forceinline__ bool multi_stage1(const PathArgs& a, int4 sq, bool th
     keep = plane_reachable(a.rplanes[(rho - a.nrx) % a.nrpr], R, A1, B1, mg);
   }
   return keep;
+}
+
+// Stage 1 of a triple depends on its last two wedges and the receiver only,
+// and the triples share their last pairs (8 x 8 city: 112k triples, a few
+// thousand pairs): one bit per (related pair whose first wedge is the second
+// of some pair, receiver), in rows of dobs1_row words. One warp per related
+// pair, its lanes over the receivers.
+__global__ void __launch_bounds__(256) k_diff_stage1(PathArgs a) {
+  const long nw = a.nw, nch = (nw + 31) / 32, nitem = nw * nch;
+  const int lane = threadIdx.x & 31;
+  const long nwarp = (long)gridDim.x * (blockDim.x >> 5);
+  for (long it = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < nitem; it += nwarp) {
+    const int wp = (int)(it / nch), w0 = (int)(it - (long)wp * nch) * 32;
+    if (!((a.dsecond[wp >> 5] >> (wp & 31)) & 1u)) continue;
+    const long bit = (long)wp * nw + w0 + lane;
+    const bool rel = w0 + lane < nw && ((a.drel[bit >> 5] >> (bit & 31)) & 1u);
+    for (unsigned rm = __ballot_sync(0xffffffffu, rel); rm; rm &= rm - 1u) {
+      const int wl = w0 + __ffs(rm) - 1;
+      unsigned* row = a.dobs1 + ((size_t)wp * nw + wl) * a.dobs1_row;
+      for (int c = 0; c < a.dobs1_row; ++c) {
+        const int r = 32 * c + lane;
+        const unsigned m =
+            __ballot_sync(0xffffffffu, r < a.nrx && multi_stage1(a, make_int4(0, 0, wp, wl), true, r));
+        if (lane == 0) row[c] = m;
+      }
+    }
+  }
 }
 
 // Stage 2 for a pair with a reflection between its wedges: the chain over w1
@@ -2418,7 +2717,13 @@ __global__ void __launch_bounds__(256) k_diff_multi_pre(PathArgs a) {
     const bool more = item < nitem;
     if (more) {
       const long rho = r0 + lane;
-      const bool pass = rho < r1 && multi_stage1(a, sq, e >= n2, (int)rho);
+      bool pass = rho < r1;
+      if (pass) {
+        if (a.dobs1 && e >= n2 && rho < a.nrx)
+          pass = (a.dobs1[((size_t)sq.z * a.nw + sq.w) * a.dobs1_row + (rho >> 5)] >> (rho & 31)) & 1u;
+        else
+          pass = multi_stage1(a, sq, e >= n2, (int)rho);
+      }
       const unsigned mk = __ballot_sync(0xffffffffu, pass);
       if (pass) wq[wid][qn + __popc(mk & ((1u << lane) - 1u))] = e * nobs + rho;
       qn += __popc(mk);
@@ -2462,9 +2767,32 @@ __device__ __forceinline__ double chain_len(const Wedge* const* E, int m, d3w T,
   return L + sqrt(dotw(d, d));
 }
 
+// Where Newton's method starts (the length is convex, so the start decides
+// the number of steps, not the result): one wedge's closed form, a chain's
+// FP32 Keller points where that estimate converges, else the midpoints. An
+// FP64 step costs some two thousand cycles of dependent operations; from the
+// midpoints a chain takes 5 to 50, from these starts two or three.
+__device__ __forceinline__ void keller_start(const Wedge* const* E, int m, d3w T, d3w R, double* t) {
+  if (m == 1) {
+    const d3w e = D3(E[0]->e[0], E[0]->e[1], E[0]->e[2]), p0 = D3(E[0]->p0[0], E[0]->p0[1], E[0]->p0[2]);
+    const d3w dt = T - p0, dr = R - p0;
+    const double zt = dotw(dt, e), zr = dotw(dr, e);
+    const d3w pt = dt - e * zt, pr = dr - e * zr;
+    const double rt = sqrt(dotw(pt, pt)), rr = sqrt(dotw(pr, pr));
+    t[0] = rt + rr > 0.0 ? zt + (zr - zt) * rt / (rt + rr) : 0.5 * E[0]->len;
+    return;
+  }
+  WedgeF W[3];
+  float tf[3];
+  for (int i = 0; i < m; ++i) W[i] = wedge_f(*E[i]);
+  const bool ok =
+      keller32(W, m, f3((float)T.x, (float)T.y, (float)T.z), f3((float)R.x, (float)R.y, (float)R.z), tf, 1e-3f) > 0;
+  for (int i = 0; i < m; ++i) t[i] = ok ? (double)tf[i] : 0.5 * E[i]->len;
+}
+
 // Keller points: the stationary point (the minimum: the length is convex in
 // t) of the unfolded length over the edge parameters, by Newton's method
-// from the edges' midpoints (at most 50 steps), a step that does not
+// from keller_start (at most 50 steps), a step that does not
 // shorten the chain halved (at most 40 times) until the cosine mismatch is
 // below 1e-8 or the Newton decrement below 1e-15 of the length, full steps
 // after that; converged when every edge's mismatch is below 1e-12. A leg shorter than kLegMin stops it: the
@@ -2472,7 +2800,7 @@ __device__ __forceinline__ double chain_len(const Wedge* const* E, int m, d3w T,
 // where Keller's law has no solution.
 constexpr double kLegMin = 1e-6;
 __device__ bool keller_chain(const Wedge* const* E, int m, d3w T, d3w R, double* t) {
-  for (int i = 0; i < m; ++i) t[i] = 0.5 * E[i]->len;
+  keller_start(E, m, T, R, t);
   double Lc = chain_len(E, m, T, R, t);
   for (int it = 0; it < 50; ++it) {
     d3w X[5];
@@ -2504,9 +2832,17 @@ __device__ bool keller_chain(const Wedge* const* E, int m, d3w T, d3w R, double*
         H[ib][ia] += h;
       }
     }
-    double gmax = 0.0;
-    for (int i = 0; i < m; ++i) gmax = fmax(gmax, fabs(g[i]));
+    double gmax = 0.0, cut = 0.0;
+    for (int i = 0; i < m; ++i) {
+      gmax = fmax(gmax, fabs(g[i]));
+      cut += fmin(-g[i] * t[i], g[i] * (E[i]->len - t[i]));
+    }
     if (gmax < 1e-12) return true;
+    // convex: at any y the length is at least L(t) + g.(y - t), so when that
+    // exceeds L(t) for every y on the edges (by more than rounding), the
+    // minimum lies off an edge and the chain is rejected (kinks off the edges
+    // otherwise take the 50 steps of 40 halvings: 4.1M cycles for one chain)
+    if (cut > 1e-9 * Lc) return false;
     // H dx = -g by elimination with partial pivoting
     double A[3][4], dx[3];
     for (int i = 0; i < m; ++i) {
@@ -2690,12 +3026,7 @@ __device__ __noinline__ void diffract_mid(const PathArgs& a, int4 sq, int r, dou
   // the real legs: two excluded triangles at each point
   const d3w Y[5] = {T, Q1, Pp, Q2, R};
   const int ex[5][2] = {{-1, -1}, {A.ta, A.tb}, {j, j}, {B.ta, B.tb}, {-1, -1}};
-  for (int q = 0; q < 4; ++q) {
-    const d3w dv = Y[q + 1] - Y[q];
-    RayPre rp = ray_pre(f3((float)Y[q].x, (float)Y[q].y, (float)Y[q].z), f3((float)dv.x, (float)dv.y, (float)dv.z));
-    if (any_hit(a.bvh, rp, a.eps_occ, 1.0f - a.eps_occ, ex[q][0], ex[q][1], ovf, st, ex[q + 1][0], ex[q + 1][1]))
-      return;
-  }
+  if (legs_occluded(a, Y, ex, 5, ovf, st)) return;
   unsigned fl = 0;
   const d3w u = D3(a.pol.x, a.pol.y, a.pol.z);
   d3w ip = (Q1 - T) * (1.0 / ell[0]);
@@ -2734,8 +3065,7 @@ __device__ __noinline__ void diffract_mid(const PathArgs& a, int4 sq, int r, dou
     const float4 mb =
         a.mats[__float_as_int(a.tris[3 * (size_t)DCEM_IDX(a.slot_of_id[DCEM_IDX(W.tb, a.bvh.ntris)], a.bvh.ntris) + 1].w)];
     zd r0s, r0h, rns, rnh;
-    fresnel_d(ma, a.freq, fabs(sin(phip[i])), r0s, r0h);
-    fresnel_d(mb, a.freq, fabs(sin(nn * M_PI - phi[i])), rns, rnh);
+    fresnel_faces(ma, fabs(sin(phip[i])), mb, fabs(sin(nn * M_PI - phi[i])), a.freq, r0s, r0h, rns, rnh);
     const UtdParts up = utd_parts(nn, phi[i], phip[i], beta0, L, k, fl);
     const zd Ds = utd_coeff(up, r0s, rns), Dh = utd_coeff(up, r0h, rnh);
     sincos(-k * s, &sn, &cs);
@@ -2750,6 +3080,7 @@ __device__ __noinline__ void diffract_mid(const PathArgs& a, int4 sq, int r, dou
   }
   const d3w prx = polw(u, ip * -1.0, fl);
   const zd amp = zvdot(Ev, prx) * (lam / (4.0 * M_PI));
+  if (diff_lane() != 0) return;  // one lane of the group writes the record
   unsigned uu = atomicAdd(&a.ctr->n_unique, 1u);
   if (uu >= a.ucap) {
     atomicOr(&a.ctr->err, ERR_UNIQUE_OVERFLOW);
@@ -2847,12 +3178,7 @@ __device__ __noinline__ void diffract_multi(const PathArgs& a, unsigned long lon
   for (int i = 0; i < m; ++i) { Y[ny] = X[i + 1]; ex[ny][0] = E[i]->ta; ex[ny][1] = E[i]->tb; ++ny; }
   if (last) { Y[ny] = Pp; ex[ny][0] = ex[ny][1] = j; ++ny; }
   Y[ny] = R; ex[ny][0] = ex[ny][1] = -1; ++ny;
-  for (int q = 0; q + 1 < ny; ++q) {
-    d3w dv = Y[q + 1] - Y[q];
-    RayPre rp = ray_pre(f3((float)Y[q].x, (float)Y[q].y, (float)Y[q].z), f3((float)dv.x, (float)dv.y, (float)dv.z));
-    if (any_hit(a.bvh, rp, a.eps_occ, 1.0f - a.eps_occ, ex[q][0], ex[q][1], ovf, st, ex[q + 1][0], ex[q + 1][1]))
-      return;
-  }
+  if (legs_occluded(a, Y, ex, ny, ovf, st)) return;
   unsigned fl = 0;
   const d3w u = D3(a.pol.x, a.pol.y, a.pol.z);
   d3w ip = (X[1] - X[0]) * (1.0 / ell[0]);  // the real direction into Q_1
@@ -2893,8 +3219,7 @@ __device__ __noinline__ void diffract_multi(const PathArgs& a, unsigned long lon
     const float4 mb =
         a.mats[__float_as_int(a.tris[3 * (size_t)DCEM_IDX(a.slot_of_id[DCEM_IDX(W.tb, a.bvh.ntris)], a.bvh.ntris) + 1].w)];
     zd r0s, r0h, rns, rnh;
-    fresnel_d(ma, a.freq, fabs(sin(phip[i])), r0s, r0h);
-    fresnel_d(mb, a.freq, fabs(sin(nn * M_PI - phi[i])), rns, rnh);
+    fresnel_faces(ma, fabs(sin(phip[i])), mb, fabs(sin(nn * M_PI - phi[i])), a.freq, r0s, r0h, rns, rnh);
     const UtdParts up = utd_parts(nn, phi[i], phip[i], beta0, L, k, fl);
     zd Ds = utd_coeff(up, r0s, rns), Dh = utd_coeff(up, r0h, rnh);
     sincos(-k * s, &sn, &cs);
@@ -2917,6 +3242,7 @@ __device__ __noinline__ void diffract_multi(const PathArgs& a, unsigned long lon
   zd amp = zvdot(Ev, prx) * (lam / (4.0 * M_PI));
   double Ltot = 0.0;
   for (int q = 0; q <= m; ++q) Ltot += ell[q];
+  if (diff_lane() != 0) return;  // one lane of the group writes the record
   unsigned uu = atomicAdd(&a.ctr->n_unique, 1u);
   if (uu >= a.ucap) {
     atomicOr(&a.ctr->err, ERR_UNIQUE_OVERFLOW);
@@ -3139,7 +3465,7 @@ __device__ __forceinline__ ReflCand refl_decode(const PathArgs& a, int nlinks, u
 // the two at the wedge costs a few percent of testing every (kind, link,
 // plane pair) block on its own (8 x 8 city blocks, 64 receivers, 321 planes:
 // 19.8M blocks, 24.5 ms; this form 1.2 ms in all):
-//   k_refl_visible the planes and wedges each end point may see at all
+//   k_diff_visible the planes and wedges each end point may see at all
 //   k_refl_single  every (end point, plane): the wedges that the image sees
 //                  through the plane's box. Such a side with no reflection
 //                  on the other end gives the one-reflection candidates;
@@ -3225,163 +3551,8 @@ __device__ __forceinline__ int octet_wedge(const PathArgs& a, int g, unsigned& g
 __device__ __forceinline__ float3 plane_image(const RPlane& P, float3 X) {
   return mirror32(X, f3(P.nf[0], P.nf[1], P.nf[2]), P.cf);
 }
-__device__ __forceinline__ float3 end_point(const PathArgs& a, int ntx, int x) {
-  const float4 v = x < ntx ? a.txs[x] : a.rx[x - ntx];
-  return f3(v.x, v.y, v.z);
-}
 __device__ __forceinline__ float image_margin(float3 X, float3 Y) {
   return 0.1f + 1e-4f * (fabsf(X.x) + fabsf(X.y) + fabsf(X.z) + fabsf(Y.x) + fabsf(Y.y) + fabsf(Y.z));
-}
-
-// ---- what an end point can see ----
-// In built-up scenes most reflector planes and wedges are hidden from a given
-// end point behind one wall, and every real leg from an end point must be
-// free: so the planes and wedges that are certainly hidden from it as a
-// whole take no part as its first reflection or as the wedge it sees
-// directly. (8 x 8 city blocks: the side lists shrink four to eight times a
-// side.) A target is hidden when one convex wall quad -- two static coplanar
-// triangles that share an edge -- is crossed strictly inside, by the margins
-// of leg_surely_blocked, by the legs to every corner of the target: the
-// crossings of the legs to the points between the corners lie between
-// theirs. The quads tried are those the leg to the target's middle crosses.
-
-// Does quad q (q[0].w != 0) cut off point X from E with margin?
-__device__ __forceinline__ bool quad_between(const float4* __restrict__ q, float3 E, float3 X, float eps_occ) {
-  const float4 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3];
-  if (q0.w == 0.0f) return false;
-  const float3 c[4] = {f3(q0.x, q0.y, q0.z), f3(q1.x, q1.y, q1.z), f3(q2.x, q2.y, q2.z), f3(q3.x, q3.y, q3.z)};
-  const float3 dv = f3(X.x - E.x, X.y - E.y, X.z - E.z);
-  const float dl = sqrtf(fdot3(dv, dv));
-  const float3 nv = cross3(f3(c[1].x - c[0].x, c[1].y - c[0].y, c[1].z - c[0].z),
-                           f3(c[2].x - c[0].x, c[2].y - c[0].y, c[2].z - c[0].z));
-  const float nn = sqrtf(fdot3(nv, nv)), dn = fdot3(dv, nv);
-  if (!(dl > 0.0f && fabsf(dn) > 1e-3f * dl * nn)) return false;
-  const float u = fdot3(f3(c[0].x - E.x, c[0].y - E.y, c[0].z - E.z), nv) / dn;
-  const float slack = 2e-3f + 1e-6f * (fabsf(E.x) + fabsf(E.y) + fabsf(E.z) + dl);
-  const float mu = 0.01f * (1.0f + dl * nn / fabsf(dn)) + slack, nu = mu / dl;
-  if (!(u > eps_occ + nu && u < 1.0f - eps_occ - nu)) return false;
-  const float3 H = f3(E.x + dv.x * u, E.y + dv.y * u, E.z + dv.z * u);
-  for (int k = 0; k < 4; ++k) {
-    const float3 a = c[k], b = c[(k + 1) & 3];
-    const float3 e = f3(b.x - a.x, b.y - a.y, b.z - a.z);
-    const float el = sqrtf(fdot3(e, e));
-    if (el > 0.0f && !(fdot3(cross3(e, f3(H.x - a.x, H.y - a.y, H.z - a.z)), nv) > mu * el * nn)) return false;
-  }
-  return true;
-}
-
-// Are all points of the box lo..hi, or (seg) of the segment lo-hi, certainly
-// hidden from E behind one quad?
-__device__ __noinline__ bool surely_hidden(const PathArgs& a, float3 E, float3 lo, float3 hi, bool seg, TStack& st) {
-  const float3 mid = f3(0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z));
-  const RayPre rp = ray_pre(E, f3(mid.x - E.x, mid.y - E.y, mid.z - E.z));
-  st.reset();
-  int cur = a.bvh.root0;  // static triangles only
-  for (int visits = 0; visits <= a.bvh.max_visits; ++visits) {
-    if (cur == kEmpty) {
-      if (st.empty()) break;
-      cur = st.pop();
-      continue;
-    }
-    if (cur >= 0) {
-      const float4* n = a.bvh.nodes + 4 * (size_t)DCEM_IDX(cur, a.bvh.nnodes);
-      float4 n0 = __ldg(n), n1 = __ldg(n + 1), n2 = __ldg(n + 2), n3 = __ldg(n + 3);
-      float tn0, tn1;
-      const bool h0 = slab(rp, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, 1.0f, tn0);
-      const bool h1 = slab(rp, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, 1.0f, tn1);
-      const int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
-      if (h0 && h1) {
-        if (!st.push(c1)) return false;
-        cur = c0;
-      } else {
-        cur = h0 ? c0 : h1 ? c1 : kEmpty;
-      }
-      continue;
-    }
-    const int id = __float_as_int(__ldg(&a.bvh.tris[3 * (size_t)DCEM_IDX(~cur, a.bvh.ntris)]).w);
-    cur = kEmpty;
-    const float4* q = a.quads + 4 * (size_t)DCEM_IDX(id, a.bvh.ntris);
-    bool all = quad_between(q, E, mid, a.eps_occ);
-    for (int k = 0; all && k < (seg ? 2 : 8); ++k) {
-      const float3 X = seg ? (k ? hi : lo) : f3((k & 1) ? hi.x : lo.x, (k & 2) ? hi.y : lo.y, (k & 4) ? hi.z : lo.z);
-      all = quad_between(q, E, X, a.eps_occ);
-    }
-    if (all) return true;
-  }
-  return false;
-}
-
-// Per end point the planes, then the wedges (in the order wperm) it may see,
-// one warp per word. A wedge the end point is inside of is not seen. Both
-// orders are spatial, so that a warp's legs run close together.
-__global__ void __launch_bounds__(64) k_refl_visible(PathArgs a, int ntx) {
-  extern __shared__ int sstk[];
-  TStack st;
-  bind_stack(st, sstk, kStackTrace);
-  const int npw = (a.nrp + 31) / 32, row = npw + a.nwc, lane = threadIdx.x & 31;
-  const long nitem = (long)(ntx + a.nrx) * row, nwarp = (long)gridDim.x * (blockDim.x >> 5);
-  for (long it = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < nitem; it += nwarp) {
-    const int x = (int)(it / row), c = (int)(it - (long)x * row);
-    const float3 E = end_point(a, ntx, x);
-    bool see = false;
-    if (c < npw) {
-      const int p = c * 32 + lane;
-      if (p < a.nrp) {
-        const float* b = a.rplanes[p].box;
-        see = !surely_hidden(a, E, f3(b[0], b[1], b[2]), f3(b[3], b[4], b[5]), false, st);
-      }
-    } else {
-      const int i = (c - npw) * kWedgeCluster + lane;
-      if (i < a.nw) {
-        const WedgeF W = a.wf[a.wperm[i]];
-        float3 A, B;
-        edge_ends(W, A, B);
-        see = !surely_inside(W, E) && !surely_hidden(a, E, A, B, true, st);
-      }
-    }
-    const unsigned m = __ballot_sync(0xffffffffu, see);
-    if (lane == 0) a.vis[it] = m;
-  }
-}
-// The wedges some transmitter (words 0 .. nwc - 1) or some receiver sees, and
-// lists of the groups that hold any (per side a count, then the groups).
-__global__ void __launch_bounds__(256) k_refl_visible_any(PathArgs a, int ntx) {
-  __shared__ unsigned cnt;
-  const int npw = (a.nrp + 31) / 32, row = npw + a.nwc, side = blockIdx.x;
-  const int ng = (a.nw + kWedgeGroup - 1) / kWedgeGroup;
-  int* list = a.vis_grp + (size_t)side * (ng + 1);
-  if (threadIdx.x == 0) cnt = 0u;
-  __syncthreads();
-  for (int c0 = 0; c0 < a.nwc; c0 += 32) {  // lanes: words, warps: end points
-    __shared__ unsigned part[32];
-    const int c = c0 + (threadIdx.x & 31);
-    if (threadIdx.x < 32) part[threadIdx.x] = 0u;
-    __syncthreads();
-    if (c < a.nwc) {
-      unsigned m = 0;
-      const int x1 = side ? ntx + a.nrx : ntx;
-      for (int x = (side ? ntx : 0) + (threadIdx.x >> 5); x < x1; x += 8) m |= a.vis[(long)x * row + npw + c];
-      atomicOr(&part[threadIdx.x & 31], m);
-    }
-    __syncthreads();
-    if (threadIdx.x < 32 && c < a.nwc) {
-      const unsigned m = part[threadIdx.x];
-      a.vis_any[side * a.nwc + c] = m;
-      for (int k = 0; k < 4; ++k)
-        if ((m >> (8 * k)) & 0xffu) list[1 + atomicAdd(&cnt, 1u)] = 4 * c + k;
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) list[0] = (int)cnt;
-}
-__device__ __forceinline__ bool sees_plane(const PathArgs& a, int x, int p) {
-  const int npw = (a.nrp + 31) / 32;
-  return (a.vis[(long)x * (npw + a.nwc) + p / 32] >> (p & 31)) & 1u;
-}
-// (i: the wedge's place in the order wperm)
-__device__ __forceinline__ bool sees_wedge(const PathArgs& a, int x, int i) {
-  const int npw = (a.nrp + 31) / 32;
-  return (a.vis[(long)x * (npw + a.nwc) + npw + i / kWedgeCluster] >> (i % kWedgeCluster)) & 1u;
 }
 
 // Two FIFO queues per warp in shared memory, so that each stage runs on full
@@ -3889,12 +4060,7 @@ __device__ __noinline__ void diffract_refl2(const PathArgs& a, unsigned long lon
   P[ny] = X[1]; ex[ny][0] = W.ta; ex[ny][1] = W.tb; ++ny;
   for (int i = 0; i < na; ++i) { P[ny] = Y[nb + i]; ex[ny][0] = ex[ny][1] = pj[nb + i]; ++ny; }
   P[ny] = R; ex[ny][0] = ex[ny][1] = -1; ++ny;
-  for (int q = 0; q + 1 < ny; ++q) {
-    const d3w dv = P[q + 1] - P[q];
-    RayPre rp = ray_pre(f3((float)P[q].x, (float)P[q].y, (float)P[q].z), f3((float)dv.x, (float)dv.y, (float)dv.z));
-    if (any_hit(a.bvh, rp, a.eps_occ, 1.0f - a.eps_occ, ex[q][0], ex[q][1], ovf, st, ex[q + 1][0], ex[q + 1][1]))
-      return;
-  }
+  if (legs_occluded(a, P, ex, ny, ovf, st)) return;
   unsigned fl = 0;
   const d3w u = D3(a.pol.x, a.pol.y, a.pol.z);
   const d3w ip = (X[1] - X[0]) * (1.0 / ell[0]);  // the real direction into Q
@@ -3924,8 +4090,7 @@ __device__ __noinline__ void diffract_refl2(const PathArgs& a, unsigned long lon
     const float4 mb =
         a.mats[__float_as_int(a.tris[3 * (size_t)DCEM_IDX(a.slot_of_id[DCEM_IDX(W.tb, a.bvh.ntris)], a.bvh.ntris) + 1].w)];
     zd r0s, r0h, rns, rnh;
-    fresnel_d(ma, a.freq, fabs(sin(phip[0])), r0s, r0h);
-    fresnel_d(mb, a.freq, fabs(sin(nn * M_PI - phi[0])), rns, rnh);
+    fresnel_faces(ma, fabs(sin(phip[0])), mb, fabs(sin(nn * M_PI - phi[0])), a.freq, r0s, r0h, rns, rnh);
     const UtdParts up = utd_parts(nn, phi[0], phip[0], beta0, L, k, fl);
     const zd Ds = utd_coeff(up, r0s, rns), Dh = utd_coeff(up, r0h, rnh);
     sincos(-k * s, &sn, &cs);
@@ -3942,6 +4107,7 @@ __device__ __noinline__ void diffract_refl2(const PathArgs& a, unsigned long lon
   }
   const d3w prx = polw(u, din * -1.0, fl);
   const zd amp = zvdot(Ev, prx) * (lam / (4.0 * M_PI));
+  if (diff_lane() != 0) return;  // one lane of the group writes the record
   unsigned uu = atomicAdd(&a.ctr->n_unique, 1u);
   if (uu >= a.ucap) {
     atomicOr(&a.ctr->err, ERR_UNIQUE_OVERFLOW);
@@ -4008,8 +4174,9 @@ __global__ void __launch_bounds__(256) k_diffract_pre(PathArgs a, int nlinks) {
 // same whatever the number of active lanes, but with the few survivors left
 // after the occlusion test the pipe is mostly idle (12% busy on the city) and
 // the time is the longest lane's chain of dependent operations plus the
-// other lanes' divergent branches: so survivor i goes to block i mod grid,
-// slot i / grid, and the slots fill the warps one lane at a time.
+// other lanes' divergent branches: so a survivor takes a group of four lanes
+// (see utd_parts), survivor i goes to block i mod grid, slot i / grid, and the
+// slots fill the warps one group at a time.
 constexpr int kDiffThreads = 256;
 __global__ void __launch_bounds__(kDiffThreads) k_diffract(PathArgs a) {
   extern __shared__ int sstk[];
@@ -4018,8 +4185,9 @@ __global__ void __launch_bounds__(kDiffThreads) k_diffract(PathArgs a) {
   const unsigned n = min(a.ctr->n_dexact, a.dsurv_cap);
   const double k = 2.0 * M_PI * a.freq / 299792458.0, lam = 299792458.0 / a.freq;
   unsigned ovf = 0;
-  const unsigned slot = (threadIdx.x & 31) * (kDiffThreads / 32) + (threadIdx.x >> 5);
-  for (unsigned i = blockIdx.x + gridDim.x * slot; i < n; i += gridDim.x * blockDim.x) {
+  constexpr unsigned kWarps = kDiffThreads / 32, kGroups = kDiffThreads / kDiffLanes;
+  const unsigned slot = (threadIdx.x & 31) / kDiffLanes * kWarps + (threadIdx.x >> 5);
+  for (unsigned i = blockIdx.x + gridDim.x * slot; i < n; i += gridDim.x * kGroups) {
     const unsigned long long c = a.dexact[i];
     const unsigned kind = (unsigned)(c >> kKindShift);
     if (kind == 2u && ((c >> 61) & 1ull)) diffract_refl2(a, c & kRefl2Mask, k, lam, ovf, st);
@@ -4178,6 +4346,11 @@ cudaError_t launch_diffract(const PathArgs& args, int nlinks, int sms, cudaStrea
   if (a.rplanes && a.nrp > 0)
     k_wedge_boxes<<<(a.nw + 255) / 256, 256, 0, st>>>(a.wf, a.wperm, a.nw, a.wgbox);
   if (nlinks > 0) {
+    if (a.vis) {  // what the end points see: with reflector planes or chains
+      const long nvis = (long)(nlinks / a.nrx + a.nrx) * ((a.nrp + 31) / 32 + a.nwc);
+      k_diff_visible<<<(int)std::min<long>((nvis + 1) / 2, 16L * sms), 64, 64 * kStackTrace * sizeof(int), st>>>(
+          a, nlinks / a.nrx);
+    }
     long total = (long)nlinks * a.nw;
     long g = std::min<long>((total + 255) / 256, 8L * sms);
     k_diffract_pre<<<(int)std::max<long>(g, 1), 256, 0, st>>>(a, nlinks);
@@ -4189,9 +4362,7 @@ cudaError_t launch_diffract(const PathArgs& args, int nlinks, int sms, cudaStrea
         cudaMemsetAsync(a.wobs_cnt, 0, sizeof(unsigned) * (size_t)a.nw, st);
         cudaMemsetAsync(a.rmask, 0, sizeof(unsigned) * (size_t)(ntx + a.nrx) * a.nrp * a.nwc, st);
       }
-      const long nvis = (long)(ntx + a.nrx) * ((a.nrp + 31) / 32 + a.nwc);
-      k_refl_visible<<<(int)std::min<long>((nvis + 1) / 2, 16L * sms), 64, 64 * kStackTrace * sizeof(int), st>>>(a, ntx);
-      k_refl_visible_any<<<2, 256, 0, st>>>(a, ntx);
+      k_diff_visible_any<<<2, 256, 0, st>>>(a, ntx);
       k_refl_single<<<warps(((long)ntx * a.rsub + a.nrx) * a.nrp), 256, 0, st>>>(a, ntx, nlinks);
       if (a.drefl2) {
         k_refl_room<<<(a.nw + 255) / 256, 256, 0, st>>>(a);
@@ -4208,13 +4379,19 @@ cudaError_t launch_diffract(const PathArgs& args, int nlinks, int sms, cudaStrea
       int nsrc = b.dntx * (1 + b.nrpr);
       long tp = (long)nsrc * a.nw * a.nw;
       cudaMemsetAsync(a.drel, 0, sizeof(unsigned) * (((size_t)a.nw * a.nw + 31) / 32), st);
-      k_diff_rel<<<(int)std::max<long>(std::min<long>(((long)a.nw * a.nw + 255) / 256, 8L * sms), 1), 256, 0, st>>>(b);
-      k_diff_pairs<<<(int)std::max<long>(std::min<long>((tp + 255) / 256, 8L * sms), 1), 256, 0, st>>>(b, nsrc);
+      if (a.dobs1) cudaMemsetAsync(a.dsecond, 0, sizeof(unsigned) * (size_t)((a.nw + 31) / 32), st);
+      const size_t ssm = 256 * kStackTrace * sizeof(int);
+      const long rw = (long)a.nw * ((a.nw + 31) / 32);
+      k_diff_rel<<<(int)std::max<long>(std::min<long>((rw + 7) / 8, 8L * sms), 1), 256, ssm, st>>>(b);
+      k_diff_pairs<<<(int)std::max<long>(std::min<long>((tp + 255) / 256, 8L * sms), 1), 256, ssm, st>>>(b, nsrc);
       if (a.dmid && a.rplanes && a.nrp > 0) {
         long nblk = (long)b.dntx * a.nw * a.nrp;
         k_diff_mid_pairs<<<(int)std::max<long>(std::min<long>((nblk + 7) / 8, 8L * sms), 1), 256, 0, st>>>(b);
       }
-      if (a.diff_order >= 3) k_diff_triples<<<8 * sms, 256, 0, st>>>(b);
+      if (a.diff_order >= 3) {
+        k_diff_triples<<<8 * sms, 256, 0, st>>>(b);
+        if (a.dobs1) k_diff_stage1<<<8 * sms, 256, 0, st>>>(b);
+      }
       k_diff_multi_pre<<<8 * sms, 256, 256 * kStackTrace * sizeof(int), st>>>(b);
     }
     k_diff_unblocked<<<8 * sms, 64, 64 * kStackTrace * sizeof(int), st>>>(b, nlinks);

@@ -57,6 +57,7 @@ struct PathArgs {
   // kWedgeCluster, and the boxes of the groups of kWedgeGroup (6 floats
   // each, every frame)
   const int* wperm;
+  const int* wplace;              // ... and each wedge's place in it
   float* wgbox;
   int nwc;
   unsigned long long* dsurv;      // candidates past the FP32 pre-tests
@@ -97,6 +98,12 @@ struct PathArgs {
   int4* dseq3;
   unsigned dseq3_cap;
   unsigned* drel;
+  // order 3: the receivers past stage 1 at each related pair (null: the rows
+  // would take too much memory, stage 1 is then run per triple), and the
+  // wedges that are second in some pair (bits)
+  unsigned* dobs1;
+  int dobs1_row;
+  unsigned* dsecond;
   // validation reuse (coherent frames; Sec. III "Propagation path caching"):
   // the previous frame's records of its distinct keys, found through a hash
   // table of their link keys, are copied when nothing they depend on moved
