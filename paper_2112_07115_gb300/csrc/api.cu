@@ -198,7 +198,7 @@ struct FramePlan {
   unsigned* sticky_n_next;  // sticky mode: this frame's kept-path count (persistent)
   cudaEvent_t ev[10];
   cudaStream_t side;     // second branch of the frame (compact copy, end-of-frame state)
-  cudaEvent_t br[4];     // its fork and join events
+  cudaEvent_t br[5];     // its fork and join events
 };
 
 struct FrameGraph {
@@ -385,7 +385,7 @@ struct dcem_scene {
   unsigned last_ncand = 0;
   cudaEvent_t ev[10] = {};
   cudaStream_t side = nullptr;   // the frame's second branch (see enqueue_frame)
-  cudaEvent_t br[4] = {};
+  cudaEvent_t br[5] = {};
   int launches = 0;  // kernels launched since the last completed frame
   int last_use_q = 0;  // closest-hit kernel of the last frame (TraceArgs::use_q)
   // closest-hit configuration (dcem_scene_set_trace_config / dcem_scene_autotune)
@@ -1836,7 +1836,7 @@ static void make_plan(dcem_scene* s, int nrx, const dcem_params* p, bool coheren
   P.bucket_cnt = s->bucket_cnt;
   for (int i = 0; i < 10; ++i) P.ev[i] = s->ev[i];
   P.side = s->side;
-  for (int i = 0; i < 4; ++i) P.br[i] = s->br[i];
+  for (int i = 0; i < 5; ++i) P.br[i] = s->br[i];
 }
 
 // Event record on a stream, or an event-record node when the stream is being
@@ -1856,6 +1856,10 @@ static TraceArgs frame_trace_args(const FramePlan& P) {
   return a;
 }
 
+// Does the frame preparation run beside the closest hit: in full frames
+// (coherent ones mark before it) whose stages are not timed.
+static bool prep_beside(const FramePlan& P, bool tm) { return !P.coherent && !tm; }
+
 // The frame's device work before the closest hit, in stream order (timing
 // events only with `timed`).
 static int enqueue_pre(const FramePlan& P, int sms, cudaStream_t st, bool cap, bool timed) {
@@ -1867,10 +1871,17 @@ static int enqueue_pre(const FramePlan& P, int sms, cudaStream_t st, bool cap, b
   CK(cudaMemcpyAsync(P.txs, P.txs_h, sizeof(float4) * P.nsets, cudaMemcpyHostToDevice, st));
   if (P.nlinks > P.nrx) CK(cudaMemsetAsync(P.bucket_cnt, 0, sizeof(unsigned) * P.nlinks, st));
   // second branch: the compact node copy, concurrent with the frame
-  // preparation and the marking pass (joined before the closest hit)
-  if (P.use_q) {
+  // preparation and the marking pass (joined before the closest hit). A full
+  // frame's preparation (the receivers' tree) is first needed by the capture
+  // pass, so it runs on that branch too, beside the closest hit (two CTAs:
+  // 14 us on the highway, 190 us with 4096 receivers), unless the stages are
+  // timed one by one.
+  const bool beside = prep_beside(P, tm);
+  if (P.use_q || beside) {
     CK(cudaEventRecord(P.br[0], st));
     CK(cudaStreamWaitEvent(P.side, P.br[0], 0));
+  }
+  if (P.use_q) {
     launch_quantize4(P.nodes, P.q4_bound, P.q4_count, P.q4_kid, P.q4_src, P.root_box, P.has0, P.has1, P.qnodes,
                      P.qframe, P.side);
     CK(cudaGetLastError());
@@ -1878,7 +1889,8 @@ static int enqueue_pre(const FramePlan& P, int sms, cudaStream_t st, bool cap, b
   }
   if (P.q.vc_next_key)  // the key table this frame builds for the next one
     CK(cudaMemsetAsync(P.q.vc_next_key, 0, sizeof(unsigned long long) * P.q.vc_cap, st));
-  CK(launch_frame_prep(P.fp, st));
+  CK(launch_frame_prep(P.fp, beside ? P.side : st));
+  if (beside) CK(cudaEventRecord(P.br[4], P.side));
   if (tm) CK(rec(P.ev[1], st, cap));
   if (P.coherent) {
     CK(launch_mark(P.a, P.c, sms, st));
@@ -1909,6 +1921,7 @@ static int enqueue_trace(const FramePlan& P, int sms, cudaStream_t st, bool cap,
 static int enqueue_post(const FramePlan& P, int sms, cudaStream_t st, bool cap, bool timed) {
   bool tm = P.tm && timed;
   TraceArgs a = frame_trace_args(P);
+  if (prep_beside(P, tm)) CK(cudaStreamWaitEvent(st, P.br[4], 0));
   if (P.R > 0) CK(launch_capture(a, sms, st));
   if (tm) CK(rec(P.ev[4], st, cap));
   CK(launch_dedupe(P.q, sms * 4, st));
@@ -2002,7 +2015,7 @@ static int plan_frame(dcem_scene* s, int nrx, const dcem_params* p, bool coheren
   // kernels of this frame: prep, [mark, carry], trace, capture, dedupe x2, validate x3, reduce, end
   s->launches += 2 + (coherent ? 2 : 0) + (s->R > 0 ? 2 + P.a.max_trans : 0) + 5 + (nrx > 0 ? 1 : 0) +
                  (P.q.vc_next_key ? 1 : 0) +
-                 (P.use_q ? 1 : 0) + (P.q.link_off ? 1 : 0) + (P.q.sticky_prev ? 1 : 0) +
+                 (P.use_q ? 1 : 0) + (P.q.link_off ? (P.nlinks > 65536 ? 2 : 1) : 0) + (P.q.sticky_prev ? 1 : 0) +
                  diffraction_launches(P);
   s->graph_replayed = 0;
   FrameGraph& G = s->fgraph[s->cur];
@@ -2540,7 +2553,7 @@ int dcem_batch_trace(dcem_batch* b, const float* const* tx, const int32_t* ntx, 
       P.a.use_q = 0;
       s->last_use_q = 3;  // every scene's rays in one launch
       s->launches += 2 + (coh[i] ? 2 : 0) + (s->R > 0 ? 1 : 0) + 5 + (nrx[i] > 0 ? 1 : 0) +
-                     (P.q.vc_next_key ? 1 : 0) + (P.use_q ? 1 : 0) + (P.q.link_off ? 1 : 0) +
+                     (P.q.vc_next_key ? 1 : 0) + (P.use_q ? 1 : 0) + (P.q.link_off ? (P.nlinks > 65536 ? 2 : 1) : 0) +
                      (P.q.sticky_prev ? 1 : 0) + diffraction_launches(P) + (i == 0 ? 1 : 0);
       s->graph_replayed = 0;
       b->h_tab[i] = frame_trace_args(P);

@@ -291,9 +291,15 @@ __device__ __forceinline__ d3 pol_of(d3 u, d3 d, unsigned& flags) {
 //                complex amplitude (FP64); valid paths go to their link's
 //                bucket
 // ---------------------------------------------------------------------------
-// Distinct keys are few (thousands): thread t of block b takes keys
-// b + gridDim * t, so that every SM gets a share.
+// Distinct keys are few (a thousand) in most frames and tens of thousands
+// with many transmitters. Few: thread t of block b takes keys b + gridDim * t,
+// so that every SM gets a share.
 __device__ __forceinline__ unsigned spread_index(unsigned i) { return blockIdx.x + gridDim.x * i; }
+// The FP64 kernels are launched with four times the blocks that the few-keys
+// case wants (there, more warps with fewer lanes each only add FP64 warp
+// instructions); all of them work when there are many keys.
+constexpr unsigned kManyKeys = 16384;
+__device__ __forceinline__ unsigned key_blocks(unsigned nu) { return nu > kManyKeys ? gridDim.x : gridDim.x / 4; }
 
 // Validation reuse (Sec. III "Propagation path caching": the cached paths
 // are re-checked each frame; here a check is skipped when its result cannot
@@ -341,8 +347,10 @@ __global__ void __launch_bounds__(64) k_val_geom(PathArgs a) {
   bind_stack(st, sstk, kStackSmall);
   unsigned nu = min(a.ctr->n_unique, a.ucap);
   const bool reuse = a.reuse && a.ctr->n_moved_boxes <= a.mv_cap;
+  const unsigned nb = key_blocks(nu);
+  if (blockIdx.x >= nb) return;
   for (unsigned t = threadIdx.x;; t += blockDim.x) {
-    unsigned u = spread_index(t);
+    unsigned u = blockIdx.x + nb * t;
     if (u >= nu) break;
     int ci = a.uniq[u];
     PathRec rec;
@@ -557,11 +565,162 @@ struct FieldEnds {
   unsigned fl0, fl1;
 };
 
+// The coefficients of bounce j (1..k) of path X: incoming X[j-1] -> X[j],
+// outgoing X[j] -> X[j+1].
+__device__ __forceinline__ void bounce_coef(const PathArgs& a, const d3* X, int id, int j, double wfac, BounceCoef& c) {
+  const float4* tp = a.tris + 3 * (size_t)DCEM_IDX(a.slot_of_id[DCEM_IDX(id & ~kTransBit, a.bvh.ntris)], a.bvh.ntris);
+  float4 p0 = tp[0], p1 = tp[1], p2 = tp[2];
+  const float4 mt = a.mats[__float_as_int(p1.w)];
+  if (id & kTransBit) {  // penetration loss L dB: field times 10^(-L/20)
+    c.trans = 1;
+    c.te_re = pow(10.0, -(double)mt.w / 20.0);
+    return;
+  }
+  c.trans = 0;
+  d3 din = dir_of(X[j - 1], X[j]), dout = dir_of(X[j], X[j + 1]);
+  d3 q0 = mk3(p0.x, p0.y, p0.z);
+  d3 nh = du(dx(mk3(p1.x, p1.y, p1.z) - q0, mk3(p2.x, p2.y, p2.z) - q0));
+  double ct = fabs(dd(din, nh));
+  d3 sv = dx(din, nh);
+  double sn = dn(sv);
+  if (sn < 1e-12) {  // normal incidence: any unit vector perpendicular to n
+    d3 ax = fabs(nh.x) < 0.9 ? mk3(1, 0, 0) : mk3(0, 1, 0);
+    sv = du(dx(nh, ax));
+  } else {
+    sv = sv * (1.0 / sn);
+  }
+  d3 pin = dx(sv, din), pout = dx(sv, dout);
+  zd gte, gtm;
+  if (mt.z != 0.0f) {
+    gte = Z(-1.0);
+    gtm = Z(1.0);
+  } else {
+    zd ec = Z((double)mt.x, (double)mt.y * wfac);
+    zd root = zsqrt(ec - Z(1.0 - ct * ct));
+    gte = zdiv(Z(ct) - root, Z(ct) + root);
+    gtm = zdiv(ec * ct - root, ec * ct + root);
+  }
+  c.sv[0] = sv.x; c.sv[1] = sv.y; c.sv[2] = sv.z;
+  c.pin[0] = pin.x; c.pin[1] = pin.y; c.pin[2] = pin.z;
+  c.pout[0] = pout.x; c.pout[1] = pout.y; c.pout[2] = pout.z;
+  c.te_re = gte.re; c.te_im = gte.im;
+  c.tm_re = gtm.re; c.tm_im = gtm.im;
+}
+__device__ __forceinline__ void bounce_field(const BounceCoef& c, z3& E) {
+  if (c.trans) {
+    E.x = E.x * c.te_re;
+    E.y = E.y * c.te_re;
+    E.z = E.z * c.te_re;
+    return;
+  }
+  const d3 sv = mk3(c.sv[0], c.sv[1], c.sv[2]), pin = mk3(c.pin[0], c.pin[1], c.pin[2]),
+           pout = mk3(c.pout[0], c.pout[1], c.pout[2]);
+  zd ts = Z(c.te_re, c.te_im) * zdot(E, sv), tpp = Z(c.tm_re, c.tm_im) * zdot(E, pin);
+  E.x = ts * sv.x + tpp * pout.x;
+  E.y = ts * sv.y + tpp * pout.y;
+  E.z = ts * sv.z + tpp * pout.z;
+}
+// Phase k L reduced modulo 2 pi: subtract the nearest multiple of 2 pi, the
+// product n * 2 pi taken exactly by an FMA against a two-part 2 pi.
+__device__ __forceinline__ void path_phase(double freq, double L, double* sn, double* cs) {
+  double kl = 2.0 * M_PI * freq / 299792458.0 * L;
+  double nq = rint(kl * (0.5 / M_PI));
+  double ph = fma(-nq, 6.283185307179586, kl);
+  ph = fma(-nq, 2.4492935982947064e-16, ph);
+  sincos(ph, sn, cs);
+}
+// The amplitude from the field at the receiver, the record completed and its
+// place in the link's bucket.
+__device__ __forceinline__ void field_done(const PathArgs& a, PathRec& rec, const d3* X, unsigned u, const z3& E, d3 prx,
+                                           double sn, double cs, unsigned fl) {
+  const int k = rec.depth;
+  zd proj = zdot(E, prx);
+  double lam = 299792458.0 / a.freq;
+  double g = lam / (4.0 * M_PI) / rec.len;
+  double re = proj.re * cs + proj.im * sn, im = proj.im * cs - proj.re * sn;
+  rec.valid = 1;
+  rec.flags |= fl;
+  rec.amp_re = re * g;
+  rec.amp_im = im * g;
+  for (int j = 0; j < k; ++j) {
+    rec.pts[j][0] = (float)X[j + 1].x;
+    rec.pts[j][1] = (float)X[j + 1].y;
+    rec.pts[j][2] = (float)X[j + 1].z;
+  }
+  int rxi = rec.rx;
+  unsigned pos = atomicAdd(&a.bucket_cnt[rxi], 1u);
+  if (pos < (unsigned)a.bucket_cap) a.bucket[(size_t)rxi * a.bucket_cap + pos] = (int)u;
+  else atomicOr(&a.ctr->err, ERR_BUCKET_OVERFLOW);
+  atomicAdd(&a.ctr->n_valid, 1u);
+  if (a.sticky_next) {  // kept for the next frame
+    if (rec.flags & DCEM_PATH_STICKY) atomicAdd(&a.ctr->n_sticky_valid, 1u);
+    unsigned q = atomicAdd(&a.ctr->n_sticky_next, 1u);
+    if (q < a.sticky_cap) {
+      StickyKey sk;
+      sk.link = rxi;
+      sk.depth = k;
+      for (int j = 0; j < kMaxRefl; ++j) sk.tri[j] = rec.tri[j];
+      a.sticky_next[q] = sk;
+    }
+  }
+}
+
+// With many keys the FP64 pipe's throughput binds, not one key's latency: a
+// lane takes a whole key (the same operations in the same order), and the
+// valid keys (a third of an urban frame's) wait in a per-warp queue so that
+// the warp's FP64 instructions run on full lanes.
+__device__ __noinline__ void field_many(const PathArgs& a, unsigned nu, unsigned* queue) {
+  const int lane = threadIdx.x & 31;
+  const d3 upol = mk3(a.pol.x, a.pol.y, a.pol.z);
+  const double wfac = -1.0 / (2.0 * M_PI * a.freq * 8.8541878128e-12);
+  const unsigned nwarp = gridDim.x * (blockDim.x >> 5);
+  int n = 0;  // waiting (warp-uniform)
+  auto take = [&](int m) {
+    if (lane < m) {
+      const unsigned u = queue[n - m + lane];
+      PathRec& rec = a.prec[u];
+      const int k = rec.depth;
+      const d3* X = reinterpret_cast<const d3*>(a.vpts) + (size_t)u * (kMaxRefl + 2);
+      unsigned fl = 0;
+      const d3 e0 = pol_of(upol, dir_of(X[0], X[1]), fl);
+      z3 E = {Z(e0.x), Z(e0.y), Z(e0.z)};
+      for (int j = 1; j <= k; ++j) {
+        BounceCoef c;
+        bounce_coef(a, X, rec.tri[j - 1], j, wfac, c);
+        bounce_field(c, E);
+      }
+      const d3 prx = pol_of(upol, dir_of(X[k + 1], X[k]), fl);
+      double sn, cs;
+      path_phase(a.freq, rec.len, &sn, &cs);
+      field_done(a, rec, X, u, E, prx, sn, cs, fl);
+    }
+    n -= m;
+    __syncwarp();
+  };
+  for (unsigned u0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; u0 < nu; u0 += 32 * nwarp) {
+    const unsigned u = u0 + lane;
+    const bool valid = u < nu && a.vstate[u] == 1;
+    const unsigned m = __ballot_sync(0xffffffffu, valid);
+    if (valid) queue[n + __popc(m & ((1u << lane) - 1u))] = u;
+    n += __popc(m);
+    __syncwarp();
+    if (n >= 32) take(32);
+  }
+  if (n > 0) take(n);
+}
+
 __global__ void __launch_bounds__(kFieldThreads) k_val_field(PathArgs a) {
   constexpr int kGroups = kFieldThreads / kFieldLanes;
   __shared__ BounceCoef scoef[kGroups][kMaxRefl];
   __shared__ FieldEnds sends[kGroups];
+  __shared__ unsigned squeue[kFieldThreads / 32][64];
   const unsigned nu = min(a.ctr->n_unique, a.ucap);
+  if (nu > kManyKeys) {
+    field_many(a, nu, squeue[threadIdx.x >> 5]);
+    return;
+  }
+  const unsigned nb = key_blocks(nu);
+  if (blockIdx.x >= nb) return;
   const int grp = threadIdx.x / kFieldLanes, gl = threadIdx.x % kFieldLanes;
   const unsigned gmask = ((1u << kFieldLanes) - 1u) << ((threadIdx.x & 31) & ~(kFieldLanes - 1));
   const d3 upol = mk3(a.pol.x, a.pol.y, a.pol.z);
@@ -569,56 +728,13 @@ __global__ void __launch_bounds__(kFieldThreads) k_val_field(PathArgs a) {
   BounceCoef* C = scoef[grp];
   FieldEnds& ends = sends[grp];
   for (unsigned it = 0;; ++it) {
-    unsigned u = blockIdx.x + gridDim.x * (grp + kGroups * it);
+    unsigned u = blockIdx.x + nb * (grp + kGroups * it);
     if (u >= nu) break;
     if (a.vstate[u] != 1) continue;
     PathRec& rec = a.prec[u];
     const int k = rec.depth;
     const d3* X = reinterpret_cast<const d3*>(a.vpts) + (size_t)u * (kMaxRefl + 2);
-    const double L = rec.len;
-    // bounce j (1..k): incoming X[j-1] -> X[j], outgoing X[j] -> X[j+1]
-    for (int j = 1 + gl; j <= k; j += kFieldLanes) {
-      BounceCoef& c = C[j - 1];
-      const int id = rec.tri[j - 1];
-      const float4* tp = a.tris + 3 * (size_t)DCEM_IDX(a.slot_of_id[DCEM_IDX(id & ~kTransBit, a.bvh.ntris)],
-                                                        a.bvh.ntris);
-      float4 p0 = tp[0], p1 = tp[1], p2 = tp[2];
-      const float4 mt = a.mats[__float_as_int(p1.w)];
-      if (id & kTransBit) {  // penetration loss L dB: field times 10^(-L/20)
-        c.trans = 1;
-        c.te_re = pow(10.0, -(double)mt.w / 20.0);
-        continue;
-      }
-      c.trans = 0;
-      d3 din = dir_of(X[j - 1], X[j]), dout = dir_of(X[j], X[j + 1]);
-      d3 q0 = mk3(p0.x, p0.y, p0.z);
-      d3 nh = du(dx(mk3(p1.x, p1.y, p1.z) - q0, mk3(p2.x, p2.y, p2.z) - q0));
-      double ct = fabs(dd(din, nh));
-      d3 sv = dx(din, nh);
-      double sn = dn(sv);
-      if (sn < 1e-12) {  // normal incidence: any unit vector perpendicular to n
-        d3 ax = fabs(nh.x) < 0.9 ? mk3(1, 0, 0) : mk3(0, 1, 0);
-        sv = du(dx(nh, ax));
-      } else {
-        sv = sv * (1.0 / sn);
-      }
-      d3 pin = dx(sv, din), pout = dx(sv, dout);
-      zd gte, gtm;
-      if (mt.z != 0.0f) {
-        gte = Z(-1.0);
-        gtm = Z(1.0);
-      } else {
-        zd ec = Z((double)mt.x, (double)mt.y * wfac);
-        zd root = zsqrt(ec - Z(1.0 - ct * ct));
-        gte = zdiv(Z(ct) - root, Z(ct) + root);
-        gtm = zdiv(ec * ct - root, ec * ct + root);
-      }
-      c.sv[0] = sv.x; c.sv[1] = sv.y; c.sv[2] = sv.z;
-      c.pin[0] = pin.x; c.pin[1] = pin.y; c.pin[2] = pin.z;
-      c.pout[0] = pout.x; c.pout[1] = pout.y; c.pout[2] = pout.z;
-      c.te_re = gte.re; c.te_im = gte.im;
-      c.tm_re = gtm.re; c.tm_im = gtm.im;
-    }
+    for (int j = 1 + gl; j <= k; j += kFieldLanes) bounce_coef(a, X, rec.tri[j - 1], j, wfac, C[j - 1]);
     // the ends, on lanes that hold no bounce of a path of up to 5 bounces
     if (gl == kFieldLanes - 1) {
       unsigned f = 0;
@@ -631,63 +747,13 @@ __global__ void __launch_bounds__(kFieldThreads) k_val_field(PathArgs a) {
       ends.prx[0] = prx.x; ends.prx[1] = prx.y; ends.prx[2] = prx.z;
       ends.fl1 = f;
     } else if (gl == kFieldLanes - 3) {
-      // phase k L reduced modulo 2 pi: subtract the nearest multiple of 2 pi,
-      // the product n * 2 pi taken exactly by an FMA against a two-part 2 pi
-      double kl = 2.0 * M_PI * a.freq / 299792458.0 * L;
-      double nq = rint(kl * (0.5 / M_PI));
-      double ph = fma(-nq, 6.283185307179586, kl);
-      ph = fma(-nq, 2.4492935982947064e-16, ph);
-      sincos(ph, &ends.sn, &ends.cs);
+      path_phase(a.freq, rec.len, &ends.sn, &ends.cs);
     }
     __syncwarp(gmask);
     if (gl == 0) {
       z3 E = {Z(ends.e0[0]), Z(ends.e0[1]), Z(ends.e0[2])};
-      for (int j = 0; j < k; ++j) {
-        const BounceCoef& c = C[j];
-        if (c.trans) {
-          E.x = E.x * c.te_re;
-          E.y = E.y * c.te_re;
-          E.z = E.z * c.te_re;
-          continue;
-        }
-        const d3 sv = mk3(c.sv[0], c.sv[1], c.sv[2]), pin = mk3(c.pin[0], c.pin[1], c.pin[2]),
-                 pout = mk3(c.pout[0], c.pout[1], c.pout[2]);
-        zd ts = Z(c.te_re, c.te_im) * zdot(E, sv), tpp = Z(c.tm_re, c.tm_im) * zdot(E, pin);
-        E.x = ts * sv.x + tpp * pout.x;
-        E.y = ts * sv.y + tpp * pout.y;
-        E.z = ts * sv.z + tpp * pout.z;
-      }
-      const unsigned fl = ends.fl0 | ends.fl1;
-      const double sn = ends.sn, cs = ends.cs;
-      zd proj = zdot(E, mk3(ends.prx[0], ends.prx[1], ends.prx[2]));
-      double lam = 299792458.0 / a.freq;
-      double g = lam / (4.0 * M_PI) / L;
-      double re = proj.re * cs + proj.im * sn, im = proj.im * cs - proj.re * sn;
-      rec.valid = 1;
-      rec.flags |= fl;
-      rec.amp_re = re * g;
-      rec.amp_im = im * g;
-      for (int j = 0; j < k; ++j) {
-        rec.pts[j][0] = (float)X[j + 1].x;
-        rec.pts[j][1] = (float)X[j + 1].y;
-        rec.pts[j][2] = (float)X[j + 1].z;
-      }
-      int rxi = rec.rx;
-      unsigned pos = atomicAdd(&a.bucket_cnt[rxi], 1u);
-      if (pos < (unsigned)a.bucket_cap) a.bucket[(size_t)rxi * a.bucket_cap + pos] = (int)u;
-      else atomicOr(&a.ctr->err, ERR_BUCKET_OVERFLOW);
-      atomicAdd(&a.ctr->n_valid, 1u);
-      if (a.sticky_next) {  // kept for the next frame
-        if (rec.flags & DCEM_PATH_STICKY) atomicAdd(&a.ctr->n_sticky_valid, 1u);
-        unsigned q = atomicAdd(&a.ctr->n_sticky_next, 1u);
-        if (q < a.sticky_cap) {
-          StickyKey sk;
-          sk.link = rxi;
-          sk.depth = k;
-          for (int j = 0; j < kMaxRefl; ++j) sk.tri[j] = rec.tri[j];
-          a.sticky_next[q] = sk;
-        }
-      }
+      for (int j = 0; j < k; ++j) bounce_field(C[j], E);
+      field_done(a, rec, X, u, E, mk3(ends.prx[0], ends.prx[1], ends.prx[2]), ends.sn, ends.cs, ends.fl0 | ends.fl1);
     }
     __syncwarp(gmask);  // the group's shared records are free again
   }
@@ -4206,128 +4272,231 @@ __global__ void __launch_bounds__(kDiffThreads) k_diffract(PathArgs a) {
 // ---------------------------------------------------------------------------
 constexpr int kReduceThreads = 256;
 
-// Exclusive scan of the links' valid-path counts (one CTA: each thread sums
-// a contiguous run of links, the run totals are scanned in shared memory,
-// then each thread writes its run's offsets).
-__global__ void __launch_bounds__(1024) k_link_scan(const unsigned* __restrict__ cnt, int n, unsigned cap,
-                                                    unsigned* __restrict__ off) {
-  __shared__ unsigned part[1024];
-  int tid = threadIdx.x;
-  int per = (n + 1023) / 1024;
-  int lo = min(n, tid * per), hi = min(n, lo + per);
-  unsigned sum = 0;
-  for (int i = lo; i < hi; ++i) sum += min(cnt[i], cap);
-  part[tid] = sum;
+// Output offsets of many links (above kScanLinks): the valid paths of each
+// group of kReduceGroup links, then (more than kReduceGroup groups) an
+// exclusive scan of the groups. (One CTA scanning every link took 110 us for
+// 65,536 links, each thread walking its own run of counts.)
+constexpr int kReduceGroup = 256;
+__global__ void __launch_bounds__(kReduceGroup) k_link_sums(const unsigned* __restrict__ cnt, int n, unsigned cap,
+                                                            unsigned* __restrict__ sums) {
+  const int i = blockIdx.x * kReduceGroup + threadIdx.x;
+  unsigned v = i < n ? min(cnt[i], cap) : 0u;
+  v = __reduce_add_sync(0xffffffffu, v);
+  __shared__ unsigned part[kReduceGroup / 32];
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
   __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {
-    unsigned v = tid >= o ? part[tid - o] : 0u;
-    __syncthreads();
-    part[tid] += v;
-    __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < kReduceGroup / 32; ++k) v += part[k];
+    sums[blockIdx.x] = v;
   }
-  unsigned base = tid ? part[tid - 1] : 0u;
-  for (int i = lo; i < hi; ++i) {
-    off[i] = base;
-    base += min(cnt[i], cap);
+}
+__global__ void __launch_bounds__(1024) k_link_scan(unsigned* __restrict__ sums, int n) {
+  __shared__ unsigned part[32];
+  __shared__ unsigned carry;
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid == 0) carry = 0u;
+  for (int i0 = 0; i0 < n; i0 += 1024) {
+    const unsigned v = i0 + tid < n ? sums[i0 + tid] : 0u;
+    unsigned x = v;
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) part[tid >> 5] = x;
+    __syncthreads();
+    if (tid < 32) {
+      unsigned p = part[tid];
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, p, o);
+        if (lane >= o) p += y;
+      }
+      part[tid] = p;
+    }
+    __syncthreads();
+    const unsigned before = carry + (tid >= 32 ? part[(tid >> 5) - 1] : 0u) + x - v;
+    if (i0 + tid < n) sums[i0 + tid] = before;
+    __syncthreads();
+    if (tid == 0) carry += part[31];
+    __syncthreads();
   }
 }
 
-__global__ void __launch_bounds__(kReduceThreads) k_reduce(PathArgs a) {
+// The record of a distinct key as it goes to the caller.
+__device__ __forceinline__ void write_path(const PathArgs& a, const PathRec& p, unsigned o) {
+  if (o >= a.pout_cap) return;
+  dcem_path q;
+  q.rx = p.rx % a.nrx;
+  q.tx = p.rx / a.nrx;
+  q.reserved = 0;
+  q.depth = p.depth;
+  for (int j = 0; j < kMaxRefl; ++j) {
+    q.tri[j] = p.tri[j];
+    q.pts[j][0] = p.pts[j][0];
+    q.pts[j][1] = p.pts[j][1];
+    q.pts[j][2] = p.pts[j][2];
+  }
+  q.flags = p.flags;
+  q.ray = p.ray >= 0 ? a.ray_perm[p.ray] : -1;
+  q.key = p.key;
+  q.len_m = p.len;
+  q.delay_s = p.len / 299792458.0;
+  q.amp_re = p.amp_re;
+  q.amp_im = p.amp_im;
+  a.pout[o] = q;
+}
+// A link's sums as field and powers: thread k of the first half of 2 n
+// threads takes link r0 + k's field and coherent power, of the second half
+// its incoherent power (a logarithm is some 60 dependent FP64 operations, so
+// the block's links take theirs side by side).
+__device__ __forceinline__ void write_links(const PathArgs& a, int r0, int n, const double (*sum)[3]) {
+  const int tid = threadIdx.x;
+  if (tid >= 2 * n) return;
+  const int k = tid < n ? tid : tid - n, r = r0 + k;
+  const double fr = sum[k][0], fi = sum[k][1], w = tid < n ? fr * fr + fi * fi : sum[k][2];
+  if (tid < n && a.out_field) {
+    a.out_field[2 * (size_t)r] = fr;
+    a.out_field[2 * (size_t)r + 1] = fi;
+  }
+  double* out = tid < n ? a.out_pc : a.out_pi;
+  if (out) out[r] = 10.0 * log10(a.tx_power * w) + 30.0;
+}
+
+// One warp per link with up to 32 paths (nearly all: the keys are sorted and
+// the sums formed in registers), then the block together for each link with
+// more. The sums' order is one for both: position i of the sorted paths goes
+// to partial sum i mod 256, in order, then a fixed binary tree over the 256
+// partial sums -- whose upper levels add zeros when there are few paths, so
+// the warp takes the last five only. One CTA per link took 548 us for 65,536
+// links with 21,700 paths. A block takes `per` links: eight, or one while
+// there are few links, which may then hold dozens of paths each (the office:
+// 48 links with 14 paths on average, 12 us one a block, 41 us eight).
+constexpr int kReduceWarps = kReduceThreads / 32;
+__global__ void __launch_bounds__(kReduceThreads) k_reduce(PathArgs a, int nlinks, int per) {
   extern __shared__ unsigned long long skey[];   // bucket_cap keys, then bucket_cap ints
   int* sidx = reinterpret_cast<int*>(skey + a.bucket_cap);
-  __shared__ double red[4][kReduceThreads];
-  __shared__ unsigned soff;
-  int r = blockIdx.x, tid = threadIdx.x;
-  int cnt = (int)min(a.bucket_cnt[r], (unsigned)a.bucket_cap);
-  // output offset: valid paths of all lower links (scanned beforehand when
-  // there are many links)
-  if (tid == 0) soff = a.link_off ? a.link_off[r] : 0u;
-  __syncthreads();
-  if (!a.link_off) {
-    unsigned part = 0;
-    for (int q = tid; q < r; q += kReduceThreads) part += min(a.bucket_cnt[q], (unsigned)a.bucket_cap);
-    for (int off = 16; off > 0; off >>= 1) part += __shfl_down_sync(0xffffffffu, part, off);
-    if ((tid & 31) == 0) atomicAdd(&soff, part);
+  __shared__ double red[3][kReduceThreads], sums[kReduceWarps][3];
+  __shared__ unsigned scnt[kReduceWarps], part[kReduceWarps];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int r0 = blockIdx.x * per, rw = wid < per ? r0 + wid : nlinks;
+  const unsigned cap = (unsigned)a.bucket_cap;
+  // paths of the links before this block's: the groups' offsets or sums, and
+  // the links of the own group (of all links when there are no groups)
+  const int g = r0 / kReduceGroup, ng = (nlinks + kReduceGroup - 1) / kReduceGroup;
+  unsigned before = 0;
+  if (a.link_off) {
+    if (ng > kReduceGroup) before = tid == 0 ? a.link_off[g] : 0u;
+    else before = tid < g ? a.link_off[tid] : 0u;
   }
-  int np2 = 1;
-  while (np2 < cnt) np2 <<= 1;
-  for (int i = tid; i < np2; i += kReduceThreads) {
-    if (i < cnt) {
-      int u = DCEM_IDX(a.bucket[(size_t)r * a.bucket_cap + i], a.ucap);
-      skey[i] = a.prec[u].key;
-      sidx[i] = u;
-    } else {
-      skey[i] = ~0ull;
-      sidx[i] = -1;
+  for (int q = (a.link_off ? g * kReduceGroup : 0) + tid; q < r0; q += kReduceThreads) before += min(a.bucket_cnt[q], cap);
+  before = __reduce_add_sync(0xffffffffu, before);
+  const int cnt = rw < nlinks ? (int)min(a.bucket_cnt[rw], cap) : 0;
+  if (lane == 0) {
+    part[wid] = before;
+    scnt[wid] = (unsigned)cnt;
+  }
+  // the warp's keys, sorted across its lanes (an odd-even merge network over
+  // the next power of two)
+  unsigned long long key = ~0ull;
+  int idx = -1;
+  if (cnt <= 32 && lane < cnt) {
+    idx = DCEM_IDX(a.bucket[(size_t)rw * a.bucket_cap + lane], a.ucap);
+    key = a.prec[idx].key;
+  }
+  if (cnt <= 32) {
+    for (int k = 2; k < 2 * cnt; k <<= 1)
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        const unsigned long long ok = __shfl_xor_sync(0xffffffffu, key, j);
+        const int oi = __shfl_xor_sync(0xffffffffu, idx, j);
+        const bool low = (lane & j) == 0, up = (lane & k) == 0;
+        if (low == up ? ok < key : ok > key) {
+          key = ok;
+          idx = oi;
+        }
+      }
+  }
+  __syncthreads();
+  unsigned off = 0;
+  for (int k = 0; k < kReduceWarps; ++k) off += part[k];
+  const unsigned base = off;
+  for (int k = 0; k < wid; ++k) off += scnt[k];
+  if (cnt <= 32 && rw < nlinks) {
+    double sre = 0.0, sim = 0.0, sinc = 0.0;
+    if (lane < cnt) {
+      const PathRec& p = a.prec[idx];
+      sre += p.amp_re;
+      sim += p.amp_im;
+      sinc += p.amp_re * p.amp_re + p.amp_im * p.amp_im;
+      write_path(a, p, off + (unsigned)lane);
+    }
+    for (int s = 16; s > 0; s >>= 1) {
+      sre += __shfl_down_sync(0xffffffffu, sre, s);
+      sim += __shfl_down_sync(0xffffffffu, sim, s);
+      sinc += __shfl_down_sync(0xffffffffu, sinc, s);
+    }
+    if (lane == 0) {
+      sums[wid][0] = sre;
+      sums[wid][1] = sim;
+      sums[wid][2] = sinc;
     }
   }
-  __syncthreads();
-  for (int k = 2; k <= np2; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
+  off = base;
+  for (int k = 0; k < per; ++k) {  // links with more paths, the block together
+    const int n = (int)scnt[k];
+    if (n > 32) {
+      const int r = r0 + k;
+      int np2 = 1;
+      while (np2 < n) np2 <<= 1;
+      __syncthreads();
       for (int i = tid; i < np2; i += kReduceThreads) {
-        int ixj = i ^ j;
-        if (ixj > i) {
-          unsigned long long x = skey[i], y = skey[ixj];
-          bool up = (i & k) == 0;
-          if ((x > y) == up) {
-            skey[i] = y; skey[ixj] = x;
-            int t = sidx[i]; sidx[i] = sidx[ixj]; sidx[ixj] = t;
-          }
+        if (i < n) {
+          int u = DCEM_IDX(a.bucket[(size_t)r * a.bucket_cap + i], a.ucap);
+          skey[i] = a.prec[u].key;
+          sidx[i] = u;
+        } else {
+          skey[i] = ~0ull;
+          sidx[i] = -1;
         }
       }
       __syncthreads();
-    }
-  }
-  // fixed-order sums: thread t takes sorted positions t, t+256, ... in order,
-  // then a fixed binary tree over the 256 partial sums
-  double sre = 0.0, sim = 0.0, sinc = 0.0;
-  unsigned off = soff;
-  for (int i = tid; i < cnt; i += kReduceThreads) {
-    const PathRec& p = a.prec[sidx[i]];
-    sre += p.amp_re;
-    sim += p.amp_im;
-    sinc += p.amp_re * p.amp_re + p.amp_im * p.amp_im;
-    unsigned o = off + (unsigned)i;
-    if (o < a.pout_cap) {
-      dcem_path q;
-      q.rx = p.rx % a.nrx;
-      q.tx = p.rx / a.nrx;
-      q.reserved = 0;
-      q.depth = p.depth;
-      for (int j = 0; j < kMaxRefl; ++j) {
-        q.tri[j] = p.tri[j];
-        q.pts[j][0] = p.pts[j][0];
-        q.pts[j][1] = p.pts[j][1];
-        q.pts[j][2] = p.pts[j][2];
+      for (int kk = 2; kk <= np2; kk <<= 1) {
+        for (int j = kk >> 1; j > 0; j >>= 1) {
+          for (int i = tid; i < np2; i += kReduceThreads) {
+            int ixj = i ^ j;
+            if (ixj > i) {
+              unsigned long long x = skey[i], y = skey[ixj];
+              bool up = (i & kk) == 0;
+              if ((x > y) == up) {
+                skey[i] = y; skey[ixj] = x;
+                int t = sidx[i]; sidx[i] = sidx[ixj]; sidx[ixj] = t;
+              }
+            }
+          }
+          __syncthreads();
+        }
       }
-      q.flags = p.flags;
-      q.ray = p.ray >= 0 ? a.ray_perm[p.ray] : -1;
-      q.key = p.key;
-      q.len_m = p.len;
-      q.delay_s = p.len / 299792458.0;
-      q.amp_re = p.amp_re;
-      q.amp_im = p.amp_im;
-      a.pout[o] = q;
+      double sre = 0.0, sim = 0.0, sinc = 0.0;
+      for (int i = tid; i < n; i += kReduceThreads) {
+        const PathRec& p = a.prec[sidx[i]];
+        sre += p.amp_re;
+        sim += p.amp_im;
+        sinc += p.amp_re * p.amp_re + p.amp_im * p.amp_im;
+        write_path(a, p, off + (unsigned)i);
+      }
+      red[0][tid] = sre;
+      red[1][tid] = sim;
+      red[2][tid] = sinc;
+      __syncthreads();
+      for (int s = kReduceThreads / 2; s > 0; s >>= 1) {
+        if (tid < s)
+          for (int q = 0; q < 3; ++q) red[q][tid] += red[q][tid + s];
+        __syncthreads();
+      }
+      if (tid < 3) sums[k][tid] = red[tid][0];
     }
+    off += scnt[k];
   }
-  red[0][tid] = sre;
-  red[1][tid] = sim;
-  red[2][tid] = sinc;
   __syncthreads();
-  for (int s = kReduceThreads / 2; s > 0; s >>= 1) {
-    if (tid < s)
-      for (int q = 0; q < 3; ++q) red[q][tid] += red[q][tid + s];
-    __syncthreads();
-  }
-  if (tid == 0) {
-    double fr = red[0][0], fi = red[1][0], pinc = red[2][0];
-    if (a.out_field) {
-      a.out_field[2 * (size_t)r] = fr;
-      a.out_field[2 * (size_t)r + 1] = fi;
-    }
-    if (a.out_pc) a.out_pc[r] = 10.0 * log10(a.tx_power * (fr * fr + fi * fi)) + 30.0;
-    if (a.out_pi) a.out_pi[r] = 10.0 * log10(a.tx_power * pinc) + 30.0;
-  }
+  write_links(a, r0, min(per, nlinks - r0), sums);
 }
 
 // ---------------------------------------------------------------------------
@@ -4407,10 +4576,12 @@ cudaError_t launch_sticky_probe(const PathArgs& a, int grid, cudaStream_t st) {
 
 cudaError_t launch_validate(const PathArgs& a, int grid, cudaStream_t st) {
   const size_t gsm = 64 * kStackSmall * sizeof(int);
-  if (a.prec_df) k_val_geom<df><<<grid, 64, gsm, st>>>(a);
-  else k_val_geom<double><<<grid, 64, gsm, st>>>(a);
-  k_val_occ<<<grid, 64, 64 * kStackTrace * sizeof(int), st>>>(a);
-  k_val_field<<<grid, kFieldThreads, 0, st>>>(a);
+  if (a.prec_df) k_val_geom<df><<<4 * grid, 64, gsm, st>>>(a);
+  else k_val_geom<double><<<4 * grid, 64, gsm, st>>>(a);
+  // (key, sub-segment) items: one or two lanes of every warp while they are
+  // few, so that a warp waits for few different traversals
+  k_val_occ<<<4 * grid, 64, 64 * kStackTrace * sizeof(int), st>>>(a);
+  k_val_field<<<4 * grid, kFieldThreads, 0, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -4440,14 +4611,19 @@ cudaError_t launch_vcache_build(const PathArgs& a, int grid, cudaStream_t st) {
 
 cudaError_t launch_reduce(const PathArgs& a, int nlinks, cudaStream_t st) {
   if (nlinks <= 0) return cudaSuccess;
-  if (a.link_off) k_link_scan<<<1, 1024, 0, st>>>(a.bucket_cnt, nlinks, (unsigned)a.bucket_cap, a.link_off);
+  if (a.link_off) {
+    const int ng = (nlinks + kReduceGroup - 1) / kReduceGroup;
+    k_link_sums<<<ng, kReduceGroup, 0, st>>>(a.bucket_cnt, nlinks, (unsigned)a.bucket_cap, a.link_off);
+    if (ng > kReduceGroup) k_link_scan<<<1, 1024, 0, st>>>(a.link_off, ng);
+  }
   size_t smem = (size_t)a.bucket_cap * (sizeof(unsigned long long) + sizeof(int));
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_reduce, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
     attr = true;
   }
-  k_reduce<<<nlinks, kReduceThreads, smem, st>>>(a);
+  const int per = nlinks <= 1024 ? 1 : kReduceWarps;
+  k_reduce<<<(nlinks + per - 1) / per, kReduceThreads, smem, st>>>(a, nlinks, per);
   return cudaGetLastError();
 }
 

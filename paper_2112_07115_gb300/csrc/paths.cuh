@@ -27,7 +27,7 @@ struct PathArgs {
   int* bucket;                    // links x bucket_cap distinct-key indices of valid paths
   unsigned* bucket_cnt;           // links (link = transmitter * nrx + receiver)
   int bucket_cap;                 // power of two
-  unsigned* link_off;             // links: output offset of each link's paths (many links), or null
+  unsigned* link_off;             // groups of links: their paths, or their output offsets (many links); or null
   dcem_path* pout;                // ordered output (link, key): caller's device buffer or staging
   unsigned pout_cap;
   double* out_field;              // links x 2 (re, im), or null
@@ -138,8 +138,9 @@ cudaError_t launch_validate(const PathArgs& a, int grid, cudaStream_t st);
 cudaError_t launch_vcache_build(const PathArgs& a, int grid, cudaStream_t st);
 // First-order edge diffraction paths of every (link, wedge) (after validation).
 cudaError_t launch_diffract(const PathArgs& a, int nlinks, int sms, cudaStream_t st);
-// Per-link sums and ordered output; links above kScanLinks take their output
-// offsets from a scan (a.link_off) instead of summing the lower links' counts.
+// Per-link sums and ordered output; more links than kScanLinks take their
+// output offsets from sums over groups (a.link_off) instead of summing the
+// lower links' counts.
 constexpr int kScanLinks = 4096;
 cudaError_t launch_reduce(const PathArgs& a, int nlinks, cudaStream_t st);
 
