@@ -568,12 +568,13 @@ int dcem_path_gradients(dcem_scene* s, const float* tx, const float* rx, int32_t
  * reverse-mode (adjoint) kernel, evaluated at the parameters theta, and the
  * gradient of a loss of the received powers: the field of Sec. III step 6
  * (Eq. 1 with the spreading of Eq. 3) over the fixed paths, differentiated by
- * one backward sweep per path. The kernel keeps only the path's vertices from
- * its forward sweep (FP64 image sources and back-trace) and recomputes each
- * bounce's directions, polarisation basis, Fresnel coefficients and incident
- * field from them during the backward sweep; an object's translation reaches
- * the vertices through the tangent of the image geometry. The cost per path
- * does not grow with the number of parameters.
+ * one backward sweep per path. From the path's vertices (FP64 image sources
+ * and back-trace) each bounce's directions, polarisation basis and Fresnel
+ * coefficients are formed once; the field is carried forward and its adjoint
+ * back through them; an object's translation reaches the vertices through the
+ * tangent of the image geometry. The cost per path does not grow with the
+ * number of parameters, and a call that asks for values only (field,
+ * pcoh_dbm) stops after the forward sweep.
  *   theta       n_params values, or NULL for the scene's current values:
  *               eps_r, sigma of every material, then the x, y translation of
  *               every rigid object (absolute: an object's triangles are

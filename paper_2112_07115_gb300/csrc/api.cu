@@ -2620,8 +2620,8 @@ int dcem_scene_gradient_size(const dcem_scene* s, int32_t* n_params) {
 }  // extern "C"
 
 // Field derivatives over a fixed path topology: forward mode (one thread per
-// (path, parameter)) at the scene's parameters, or the adjoint kernel (one
-// thread per path) at theta (null: the scene's parameters).
+// (path, parameter)) at the scene's parameters, or the adjoint kernel (eight
+// lanes per path) at theta (null: the scene's parameters).
 static int path_derivs(dcem_scene* s, const float* tx, const float* rx, int32_t nrx, int32_t rx_ptr_kind,
                        const dcem_path* paths, int32_t n_paths, const dcem_params* p, const double* theta,
                        const double* pcoh_bar, int32_t ptr_kind, double* field, double* pcoh_dbm, double* dfield,
@@ -2664,8 +2664,8 @@ static int path_derivs(dcem_scene* s, const float* tx, const float* rx, int32_t 
   if (rx_ptr_kind == DCEM_PTR_HOST) {
     std::vector<float4> h((size_t)nrx);
     for (int i = 0; i < nrx; ++i) h[i] = make_float4(rx[3 * i], rx[3 * i + 1], rx[3 * i + 2], 0.0f);
+    // (pageable: the call returns once h has been read)
     CK(cudaMemcpyAsync(s->g_rx, h.data(), sizeof(float4) * nrx, cudaMemcpyHostToDevice, st));
-    CK(cudaStreamSynchronize(st));  // h goes out of scope
   } else {
     CK(launch_pack_rx(rx, nrx, s->g_rx, st));
   }
@@ -2739,10 +2739,13 @@ static int path_derivs(dcem_scene* s, const float* tx, const float* rx, int32_t 
   g.err = s->g_err;
   g.field = dev && field ? field : G;
   g.pcoh = dev && pcoh_dbm ? pcoh_dbm : G + o_pc;
-  g.dfield = dev && dfield ? dfield : G + o_df;
+  // without derivatives wanted the kernels stop at the value; the rows of
+  // dfield are written when wanted, or as scratch when they outgrow shared memory
+  g.need_d = !adjoint || dfield || dpcoh_dbm || theta_bar;
+  g.dfield = dfield ? (dev ? dfield : G + o_df) : np > kGradShared ? G + o_df : nullptr;
   g.dpcoh = dev && dpcoh_dbm ? dpcoh_dbm : G + o_dp;
   g.theta_bar = theta_bar ? (dev ? theta_bar : G + o_tb) : nullptr;
-  CK(adjoint ? launch_adjoint(g, st) : launch_gradients(g, st));
+  CK(adjoint ? launch_adjoint(g, s->sms, st) : launch_gradients(g, st));
   s->launches += (n_paths > 0 ? 1 : 0) + 1 + (rx_ptr_kind == DCEM_PTR_DEVICE ? 1 : 0) + (g.theta_bar ? 1 : 0);
   unsigned err = 0;
   CK(cudaMemcpyAsync(&err, s->g_err, sizeof(unsigned), cudaMemcpyDeviceToHost, st));

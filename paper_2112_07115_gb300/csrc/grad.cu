@@ -16,6 +16,8 @@
 // receiver, so results are the same in every run.
 #include "grad.cuh"
 
+#include <algorithm>
+
 namespace dcem {
 namespace {
 
@@ -256,73 +258,89 @@ __global__ void k_grad_items(GradArgs g) {
   }
 }
 
-// One warp per receiver: its paths are contiguous (grouped by rx).
-__global__ void k_grad_reduce(GradArgs g, int nparam) {
-  int r = (int)((blockIdx.x * (long)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (r >= g.nrx) return;
-  int lo = 0, hi = 0;
-  if (lane == 0) {
-    int a = 0, b = g.n_paths;  // first path with rx >= r
+// One block per receiver: its paths are contiguous (grouped by rx). The items
+// of a path belong to distinct parameters, so the block's threads add a
+// path's items side by side, path after path (every sum in path order), to
+// accumulators in shared memory while the parameters fit there. (One lane
+// adding all items in global memory took 108 us for 256 receivers.)
+constexpr int kGradThreads = 128;
+__global__ void __launch_bounds__(kGradThreads) k_grad_reduce(GradArgs g, int nparam) {
+  extern __shared__ double sacc[];
+  __shared__ int range[2];
+  __shared__ double se[2];
+  const int r = blockIdx.x, tid = threadIdx.x;
+  if (tid < 2) {  // the first path with rx >= r, and with rx > r
+    int a = 0, b = g.n_paths;
     while (a < b) {
-      int m = (a + b) >> 1;
-      if (g.paths[m].rx < r) a = m + 1; else b = m;
+      const int m = (a + b) >> 1;
+      if (g.paths[m].rx < r + tid) a = m + 1; else b = m;
     }
-    lo = a;
-    b = g.n_paths;  // first path with rx > r
-    while (a < b) {
-      int m = (a + b) >> 1;
-      if (g.paths[m].rx <= r) a = m + 1; else b = m;
-    }
-    hi = a;
+    range[tid] = a;
   }
-  lo = __shfl_sync(0xffffffffu, lo, 0);
-  hi = __shfl_sync(0xffffffffu, hi, 0);
-  double* df = g.dfield + 2 * (size_t)r * nparam;
-  for (int t = lane; t < 2 * nparam; t += 32) df[t] = 0.0;
-  __syncwarp();
+  double* out = g.dfield ? g.dfield + 2 * (size_t)r * nparam : nullptr;
+  double* df = nparam <= kGradShared ? sacc : out;
+  if (g.need_d)
+    for (int t = tid; t < 2 * nparam; t += kGradThreads) df[t] = 0.0;
+  __syncthreads();
+  const int lo = range[0], hi = range[1];
   double er = 0.0, ei = 0.0;
-  if (lane == 0) {
-    for (long it = (long)lo * g.W; it < (long)hi * g.W; ++it) {
-      int pm = g.param[it];
-      double2 v = g.items[it];
+  for (int p = lo; p < hi; ++p) {
+    for (int q = tid; q < (g.need_d ? g.W : 1); q += kGradThreads) {
+      const long it = (long)p * g.W + q;
+      const int pm = g.param[it];
       if (pm == -2) {
+        const double2 v = g.items[it];
         er += v.x;
         ei += v.y;
       } else if (pm >= 0) {
+        const double2 v = g.items[it];
         df[2 * pm] += v.x;
         df[2 * pm + 1] += v.y;
       }
     }
+    __syncthreads();
+  }
+  if (tid == 0) {
     if (g.field) {
       g.field[2 * (size_t)r] = er;
       g.field[2 * (size_t)r + 1] = ei;
     }
+    const double p = er * er + ei * ei;
+    if (g.pcoh) g.pcoh[r] = p > 0.0 ? 10.0 * log10(g.tx_power * p) + 30.0 : -INFINITY;
+    se[0] = er;
+    se[1] = ei;
   }
-  __syncwarp();
-  er = __shfl_sync(0xffffffffu, er, 0);
-  ei = __shfl_sync(0xffffffffu, ei, 0);
-  if (g.pcoh && lane == 0) {
-    double p = er * er + ei * ei;
-    g.pcoh[r] = p > 0.0 ? 10.0 * log10(g.tx_power * p) + 30.0 : -INFINITY;
-  }
+  if (!g.need_d) return;
+  __syncthreads();
+  er = se[0];
+  ei = se[1];
+  if (out && df != out)
+    for (int t = tid; t < 2 * nparam; t += kGradThreads) out[t] = df[t];
   if (g.dpcoh) {
     // P = P_t |E|^2: dP = 2 P_t Re(conj(E) dE), d(dBm) = 10 / ln 10 * dP / P
-    double p = er * er + ei * ei;
-    for (int t = lane; t < nparam; t += 32) {
-      double dp = 2.0 * (er * df[2 * t] + ei * df[2 * t + 1]);
-      g.dpcoh[(size_t)r * nparam + t] = p > 0.0 ? 4.342944819032518 * dp / p : 0.0;
+    const double p = er * er + ei * ei;
+    for (int t = tid; t < nparam; t += kGradThreads) {
+      const double dr = df[2 * t], di = df[2 * t + 1];
+      const double dp = 2.0 * (er * dr + ei * di);
+      g.dpcoh[(size_t)r * nparam + t] = p > 0.0 && (dr != 0.0 || di != 0.0) ? 4.342944819032518 * dp / p : 0.0;
     }
   }
 }
 
 // ---------------------------------------------------------------------------
-// reverse mode: one thread per path
+// reverse mode: eight lanes per path
 // ---------------------------------------------------------------------------
 // The forward sweep evaluates the path's geometry in FP64 (image sources,
-// back-trace) and keeps only its vertices X_0 .. X_{k+1} (the checkpoint);
-// the field state of a bounce (directions, polarisation basis, Fresnel
-// coefficients, the field before it) is recomputed from the vertices when the
-// backward sweep needs it. The backward sweep carries d a / d v for every
+// back-trace: one lane, the only long chain) and keeps its vertices
+// X_0 .. X_{k+1}. A bounce's field quantities (directions, polarisation
+// basis, Fresnel coefficients) depend on the vertices only, so each lane
+// forms those of its own bounce; carrying the field forward and its adjoint
+// back through them is short; then each lane differentiates its own bounce,
+// and the parameters' tangents are shared out likewise. Everything of a path
+// waits in shared memory. FP64 runs at a small fraction of the FP32 rate and
+// a path is a chain of dependent operations: one thread per path that
+// recomputed every earlier bounce for each one took 385 us a call (300 paths,
+// up to 4 bounces). The backward sweep carries d a / d v for every
 // intermediate v (complex: the field is holomorphic in its complex
 // intermediates) from a back to the vertices and to each bounce's complex
 // permittivity. A material's eps_r and sigma take d a / d eps_c directly; an
@@ -336,7 +354,7 @@ __device__ __forceinline__ R3 r3(double x, double y, double z) { return R3{x, y,
 __device__ __forceinline__ R3 operator+(R3 a, R3 b) { return r3(a.x + b.x, a.y + b.y, a.z + b.z); }
 __device__ __forceinline__ R3 operator-(R3 a, R3 b) { return r3(a.x - b.x, a.y - b.y, a.z - b.z); }
 __device__ __forceinline__ R3 operator*(R3 a, double s) { return r3(a.x * s, a.y * s, a.z * s); }
-__device__ __forceinline__ double rdot(R3 a, R3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
+__device__ __forceinline__ double rdot(R3 a, R3 b) { return fma(a.z, b.z, fma(a.y, b.y, a.x * b.x)); }
 __device__ __forceinline__ R3 rcross(R3 a, R3 b) {
   return r3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
 }
@@ -349,7 +367,9 @@ struct Zc {
 __device__ __forceinline__ Zc zc(double r, double i = 0.0) { return Zc{r, i}; }
 __device__ __forceinline__ Zc operator+(Zc a, Zc b) { return zc(a.re + b.re, a.im + b.im); }
 __device__ __forceinline__ Zc operator-(Zc a, Zc b) { return zc(a.re - b.re, a.im - b.im); }
-__device__ __forceinline__ Zc operator*(Zc a, Zc b) { return zc(a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re); }
+__device__ __forceinline__ Zc operator*(Zc a, Zc b) {
+  return zc(fma(a.re, b.re, -(a.im * b.im)), fma(a.re, b.im, a.im * b.re));
+}
 __device__ __forceinline__ Zc operator*(Zc a, double s) { return zc(a.re * s, a.im * s); }
 __device__ __forceinline__ Zc operator/(Zc a, Zc b) {
   double d = b.re * b.re + b.im * b.im;
@@ -373,7 +393,9 @@ __device__ __forceinline__ Z3 operator+(const Z3& a, const Z3& b) { return Z3{a.
 __device__ __forceinline__ Z3 operator-(const Z3& a, const Z3& b) { return Z3{a.x - b.x, a.y - b.y, a.z - b.z}; }
 __device__ __forceinline__ Z3 operator*(const Z3& a, Zc s) { return Z3{a.x * s, a.y * s, a.z * s}; }
 __device__ __forceinline__ Z3 operator*(const Z3& a, double s) { return Z3{a.x * s, a.y * s, a.z * s}; }
-__device__ __forceinline__ Zc zdot(const Z3& a, R3 v) { return a.x * v.x + a.y * v.y + a.z * v.z; }
+__device__ __forceinline__ Zc zdot(const Z3& a, R3 v) {
+  return zc(fma(a.z.re, v.z, fma(a.y.re, v.y, a.x.re * v.x)), fma(a.z.im, v.z, fma(a.y.im, v.y, a.x.im * v.x)));
+}
 __device__ __forceinline__ Z3 zcross(R3 a, const Z3& b) {  // real x complex
   return Z3{b.z * a.y - b.y * a.z, b.x * a.z - b.z * a.x, b.y * a.x - b.x * a.y};
 }
@@ -449,119 +471,174 @@ __device__ __forceinline__ Z3 bounce_apply(const Bounce& b, const Z3& E) {
   return z3of(b.sv, b.te * zdot(E, b.sv)) + z3of(b.pout, b.tm * zdot(E, b.pin));
 }
 
-__global__ void k_grad_adjoint(GradArgs g) {
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < g.n_paths; p += gridDim.x * blockDim.x) {
-    const dcem_path& P = g.paths[p];
-    const long base = (long)p * g.W;
-    for (int q = 0; q < g.W; ++q) g.param[base + q] = -1;
-    const int k = P.depth;
+constexpr int kAdjLanes = 8, kAdjGroups = 32 / kAdjLanes;
+// A path's state in shared memory (index j: bounce j + 1, i: leg or vertex).
+struct AdjPath {
+  R3 V0[kMaxRefl], Nn[kMaxRefl], img[kMaxRefl + 1], X[kMaxRefl + 2], dv[kMaxRefl + 1];
+  double ell[kMaxRefl + 1], er[kMaxRefl], sg[kMaxRefl], nn[kMaxRefl], den[kMaxRefl], sp[kMaxRefl];
+  int mat[kMaxRefl], obj[kMaxRefl], pec[kMaxRefl];
+  Bounce b[kMaxRefl];
+  Z3 Em[kMaxRefl], Eb[kMaxRefl];       // the field before a bounce, the adjoint of the field after it
+  Z3 din[kMaxRefl], dout[kMaxRefl];    // adjoints of a bounce's incoming and outgoing directions
+  Z3 t[kMaxRefl + 1];                  // adjoint of a leg's vector
+  Zc ebar[kMaxRefl];                   // adjoint of a bounce's permittivity
+  Pol pol0, polr;
+  Z3 E0b, Er;                          // adjoint of the field at the Tx, the field at the Rx
+  Z3 p0, pr;                           // the polarisations' part of the end legs' adjoints
+  Zc ph, Pbar, Lbar;
+  double L;
+  int bad;
+};
+
+// One path per group of kAdjLanes lanes, `ppw` groups of each warp at work.
+__global__ void __launch_bounds__(32) k_grad_adjoint(GradArgs g, int ppw) {
+  __shared__ AdjPath sh[kAdjGroups];
+  const int gl = threadIdx.x % kAdjLanes, grp = threadIdx.x / kAdjLanes;
+  AdjPath& s = sh[grp];
+  const int p = blockIdx.x * ppw + grp;
+  bool act = grp < ppw && p < g.n_paths;
+  const dcem_path& P = g.paths[act ? p : 0];
+  const long base = (long)p * g.W;
+  const int k = act ? P.depth : 0;
+  if (act) {
+    for (int q = gl; q < g.W; q += kAdjLanes) g.param[base + q] = -1;
     bool good = k >= 0 && k <= g.max_refl && P.rx >= 0 && P.rx < g.nrx;
     for (int j = 0; good && j < k; ++j) good = P.tri[j] >= 0 && P.tri[j] < g.ntri;
     if (!good) {
-      atomicOr(g.err, 2u);
-      continue;
+      if (gl == 0) atomicOr(g.err, 2u);
+      act = false;
+    } else if (gl == 0) {
+      if (p > 0 && g.paths[p - 1].rx > P.rx) atomicOr(g.err, 1u);
+      s.bad = 0;
     }
-    if (p > 0 && g.paths[p - 1].rx > P.rx) atomicOr(g.err, 1u);
-    // ---- forward sweep: geometry in FP64 at theta
-    const double wfac = -1.0 / (2.0 * kPi * g.freq * kEps0);
-    R3 V0[kMaxRefl], Nn[kMaxRefl], img[kMaxRefl + 1], X[kMaxRefl + 2];
-    double er[kMaxRefl], sg[kMaxRefl];
-    int mat[kMaxRefl], obj[kMaxRefl];
-    bool pec[kMaxRefl];
-    const R3 tx = r3(g.tx[0], g.tx[1], g.tx[2]);
-    const float4 rv = g.rx[P.rx];
-    bool ok = true;
-    img[0] = tx;
-    for (int j = 0; j < k && ok; ++j) {
+  }
+  __syncwarp();
+  // ---- forward sweep: the triangles at theta
+  const double wfac = -1.0 / (2.0 * kPi * g.freq * kEps0);
+  const R3 tx = r3(g.tx[0], g.tx[1], g.tx[2]), u = r3(g.pol[0], g.pol[1], g.pol[2]);
+  if (act)
+    for (int j = gl; j < k; j += kAdjLanes) {
       const int id = P.tri[j];
       const float4* t = g.tris + 3 * (size_t)g.slot_of_id[id];
-      obj[j] = g.tri_obj[id];
+      const int ob = g.tri_obj[id], m = g.tri_mat[id];
       R3 off = r3(0.0, 0.0, 0.0);
-      if (g.theta && obj[j] >= 0) {
-        const double* th = g.theta + 2 * g.nmat + 2 * obj[j];
-        const float* xf = g.xf + 12 * (size_t)obj[j];
+      if (g.theta && ob >= 0) {
+        const double* th = g.theta + 2 * g.nmat + 2 * ob;
+        const float* xf = g.xf + 12 * (size_t)ob;
         off = r3(th[0] - (double)xf[3], th[1] - (double)xf[7], 0.0);
       }
       R3 v0 = r3(t[0].x, t[0].y, t[0].z) + off, v1 = r3(t[1].x, t[1].y, t[1].z) + off,
          v2 = r3(t[2].x, t[2].y, t[2].z) + off;
       R3 n = rcross(v1 - v0, v2 - v0);
-      double nn = rdot(n, n);
-      if (!(nn > 0.0)) ok = false;
-      img[j + 1] = img[j] - n * (2.0 * rdot(img[j] - v0, n) / nn);
-      V0[j] = v0;
-      Nn[j] = n;
-      mat[j] = g.tri_mat[id];
-      const float4 mt = g.mats[mat[j]];
-      pec[j] = mt.z != 0.0f;
-      er[j] = g.theta ? g.theta[2 * mat[j]] : (double)mt.x;
-      sg[j] = g.theta ? g.theta[2 * mat[j] + 1] : (double)mt.y;
+      s.nn[j] = rdot(n, n);
+      s.V0[j] = v0;
+      s.Nn[j] = n;
+      const float4 mt = g.mats[m];
+      s.mat[j] = m;
+      s.obj[j] = ob;
+      s.pec[j] = mt.z != 0.0f;
+      s.er[j] = g.theta ? g.theta[2 * m] : (double)mt.x;
+      s.sg[j] = g.theta ? g.theta[2 * m + 1] : (double)mt.y;
+      if (!(s.nn[j] > 0.0)) s.bad = 1;
     }
-    X[0] = tx;
-    X[k + 1] = r3(rv.x, rv.y, rv.z);
-    for (int j = k; j >= 1 && ok; --j) {
-      R3 dir = img[j] - X[j + 1];
-      double den = rdot(dir, Nn[j - 1]);
+  __syncwarp();
+  if (act && gl == 0 && !s.bad) {  // image sources, back-trace
+    R3 I = tx;
+    s.img[0] = I;
+    for (int j = 0; j < k; ++j) {
+      I = I - s.Nn[j] * (2.0 * rdot(I - s.V0[j], s.Nn[j]) / s.nn[j]);
+      s.img[j + 1] = I;
+    }
+    const float4 rv = g.rx[P.rx];
+    R3 Y = r3(rv.x, rv.y, rv.z);
+    s.X[0] = tx;
+    s.X[k + 1] = Y;
+    for (int j = k; j >= 1; --j) {
+      const R3 dir = s.img[j] - Y;
+      const double den = rdot(dir, s.Nn[j - 1]);
       if (den == 0.0) {
-        ok = false;
+        s.bad = 1;
         break;
       }
-      double s = rdot(V0[j - 1] - X[j + 1], Nn[j - 1]) / den;
-      X[j] = X[j + 1] + dir * s;
+      const double q = rdot(s.V0[j - 1] - Y, s.Nn[j - 1]) / den;
+      s.den[j - 1] = den;
+      s.sp[j - 1] = q;
+      Y = Y + dir * q;
+      s.X[j] = Y;
     }
-    R3 dv[kMaxRefl + 1];
-    double ell[kMaxRefl + 1], L = 0.0;
-    for (int i = 0; i <= k && ok; ++i) {
-      R3 e = X[i + 1] - X[i];
-      ell[i] = rnorm(e);
-      if (!(ell[i] > 0.0)) ok = false;
-      else dv[i] = e * (1.0 / ell[i]);
-      L += ell[i];
+  }
+  __syncwarp();
+  if (act && !s.bad)
+    for (int i = gl; i <= k; i += kAdjLanes) {
+      const R3 e = s.X[i + 1] - s.X[i];
+      const double l = rnorm(e);
+      s.ell[i] = l;
+      s.dv[i] = e * (1.0 / l);
+      if (!(l > 0.0)) s.bad = 1;
     }
-    if (!ok) {
-      atomicOr(g.err, 4u);
-      continue;
+  __syncwarp();
+  if (act && s.bad) {
+    if (gl == 0) atomicOr(g.err, 4u);
+    act = false;
+  }
+  // ---- the bounces, the end polarisations, the phase
+  if (act) {
+    for (int j = gl; j < k; j += kAdjLanes)
+      s.b[j] = bounce_of(s.dv[j], s.dv[j + 1], s.Nn[j], s.er[j], s.sg[j], s.pec[j] != 0, wfac);
+    if (gl == kAdjLanes - 1) s.pol0 = pol_fwd(u, s.dv[0]);
+    if (gl == kAdjLanes - 2) s.polr = pol_fwd(u, s.dv[k] * -1.0);
+    if (gl == kAdjLanes - 3) {
+      double L = 0.0, sp, cp;
+      for (int i = 0; i <= k; ++i) L += s.ell[i];
+      sincos(2.0 * kPi * g.freq / kC0 * L, &sp, &cp);
+      s.ph = zc(cp, -sp);  // e^{-j k L}
+      s.L = L;
     }
-    // ---- the field (the bounces are recomputed from the vertices below)
-    const R3 u = r3(g.pol[0], g.pol[1], g.pol[2]);
-    const Pol pol0 = pol_fwd(u, dv[0]);
-    const Z3 E0 = Z3{zc(pol0.n.x), zc(pol0.n.y), zc(pol0.n.z)};
-    Z3 E = E0;
-    for (int j = 1; j <= k; ++j)
-      E = bounce_apply(bounce_of(dv[j - 1], dv[j], Nn[j - 1], er[j - 1], sg[j - 1], pec[j - 1], wfac), E);
-    const R3 mdk = dv[k] * -1.0;
-    const Pol polr = pol_fwd(u, mdk);
-    const double lam = kC0 / g.freq, kw = 2.0 * kPi * g.freq / kC0, K = lam / (4.0 * kPi);
-    double sp, cp;
-    sincos(kw * L, &sp, &cp);
-    const Zc ph = zc(cp, -sp);  // e^{-j k L}
-    const Zc Pp = zdot(E, polr.n);
-    const Zc a = Pp * ph * (K / L);
-    // ---- backward sweep from a-bar = 1
-    Z3 Xb[kMaxRefl + 2], db[kMaxRefl + 1];
-    const Z3 z0 = Z3{zc(0.0), zc(0.0), zc(0.0)};
-    for (int i = 0; i <= k + 1; ++i) Xb[i] = z0;
-    for (int i = 0; i <= k; ++i) db[i] = z0;
-    Zc ebar[kMaxRefl];
-    const Zc Pbar = ph * (K / L);
-    const Zc Lbar = a * zc(-1.0 / L, -kw);
-    Z3 Eb = z3of(polr.n, Pbar);
-    db[k] = db[k] - pol_bwd(polr, mdk, E * Pbar);  // the Rx polarisation is taken along -d_k
-    for (int j = k; j >= 1; --j) {
-      // the field before bounce j, recomputed from the vertices
-      Z3 Em = E0;
-      for (int q = 1; q < j; ++q)
-        Em = bounce_apply(bounce_of(dv[q - 1], dv[q], Nn[q - 1], er[q - 1], sg[q - 1], pec[q - 1], wfac), Em);
-      const Bounce b = bounce_of(dv[j - 1], dv[j], Nn[j - 1], er[j - 1], sg[j - 1], pec[j - 1], wfac);
+  }
+  __syncwarp();
+  // ---- the field forward, its adjoint back (from a-bar = 1)
+  if (act && gl == 0) {
+    const R3 e = s.pol0.n;
+    Z3 E = Z3{zc(e.x), zc(e.y), zc(e.z)};
+    for (int j = 0; j < k; ++j) {
+      s.Em[j] = E;
+      E = bounce_apply(s.b[j], E);
+    }
+    const double lam = kC0 / g.freq, K = lam / (4.0 * kPi);
+    const Zc a = zdot(E, s.polr.n) * s.ph * (K / s.L);
+    g.items[base] = make_double2(a.re, a.im);
+    g.param[base] = -2;
+    if (g.need_d) {
+      s.Er = E;
+      s.Pbar = s.ph * (K / s.L);
+      s.Lbar = a * zc(-1.0 / s.L, -(2.0 * kPi * g.freq / kC0));
+      Z3 Eb = z3of(s.polr.n, s.Pbar);
+      for (int j = k - 1; j >= 0; --j) {
+        const Bounce& b = s.b[j];
+        s.Eb[j] = Eb;
+        Eb = z3of(b.sv, zdot(Eb, b.sv) * b.te) + z3of(b.pin, zdot(Eb, b.pout) * b.tm);
+      }
+      s.E0b = Eb;
+    }
+  }
+  if (!g.need_d) return;
+  __syncwarp();
+  // ---- each bounce differentiated at its own directions
+  if (act) {
+    for (int j = gl; j < k; j += kAdjLanes) {
+      const Bounce b = s.b[j];
+      const Z3 Em = s.Em[j], Eb = s.Eb[j];
+      const R3 di = s.dv[j], dq = s.dv[j + 1];
       const Zc es = zdot(Em, b.sv), ep = zdot(Em, b.pin);
       const Zc A = b.te * es, B = b.tm * ep;
       const Zc Ab = zdot(Eb, b.sv), Bb = zdot(Eb, b.pout);
       Z3 svb = Eb * A + Em * (Ab * b.te);
       const Z3 poutb = Eb * B;
       const Z3 pinb = Em * (Bb * b.tm);
-      const Zc teb = Ab * es, tmb = Bb * ep;
-      Eb = z3of(b.sv, Ab * b.te) + z3of(b.pin, Bb * b.tm);
-      ebar[j - 1] = zc(0.0);
+      Z3 din = zcross(pinb, b.sv);
+      Zc eb = zc(0.0);
       if (!b.pec) {
+        const Zc teb = Ab * es, tmb = Bb * ep;
         const Zc r = b.root, cc = zc(b.c), c2 = zc(b.c * b.c);
         const Zc Dte = cc + r, Dtm = b.ec * b.c + r;
         const Zc w = r - c2 / r;                      // r - c^2 / r
@@ -570,81 +647,97 @@ __global__ void k_grad_adjoint(GradArgs g) {
         const Zc dtm_dc = b.ec * w * 2.0 / (Dtm * Dtm);
         const Zc dtm_de = cc * (r * 2.0 - b.ec / r) / (Dtm * Dtm);
         const Zc cb = teb * dte_dc + tmb * dtm_dc;
-        ebar[j - 1] = teb * dte_de + tmb * dtm_de;
-        db[j - 1] = db[j - 1] + z3of(b.nh, cb * b.sgn);
+        eb = teb * dte_de + tmb * dtm_de;
+        din = din + z3of(b.nh, cb * b.sgn);
       }
-      svb = svb + zcross(dv[j - 1], pinb) + zcross(dv[j], poutb);
-      db[j - 1] = db[j - 1] + zcross(pinb, b.sv);
-      db[j] = db[j] + zcross(poutb, b.sv);
+      svb = svb + zcross(di, pinb) + zcross(dq, poutb);
       if (!b.fixed_s) {
-        Z3 vb = (svb - z3of(b.sv, zdot(svb, b.sv))) * (1.0 / b.vn);
-        db[j - 1] = db[j - 1] + zcross(b.nh, vb);
+        const Z3 vb = (svb - z3of(b.sv, zdot(svb, b.sv))) * (1.0 / b.vn);
+        din = din + zcross(b.nh, vb);
       }
+      s.ebar[j] = eb;
+      s.din[j] = din;
+      s.dout[j] = zcross(poutb, b.sv);
     }
-    db[0] = db[0] + pol_bwd(pol0, dv[0], Eb);
-    // directions and lengths -> vertices
-    for (int i = 0; i <= k; ++i) {
-      Z3 t = (db[i] - z3of(dv[i], zdot(db[i], dv[i]))) * (1.0 / ell[i]);
-      t = t + z3of(dv[i], Lbar);
-      Xb[i + 1] = Xb[i + 1] + t;
-      Xb[i] = Xb[i] - t;
+    if (gl == kAdjLanes - 1) s.p0 = pol_bwd(s.pol0, s.dv[0], s.E0b);
+    // the Rx polarisation is taken along -d_k
+    if (gl == kAdjLanes - 2) s.pr = pol_bwd(s.polr, s.dv[k] * -1.0, s.Er * s.Pbar);
+  }
+  __syncwarp();
+  // directions and lengths -> the legs' vectors
+  if (act)
+    for (int i = gl; i <= k; i += kAdjLanes) {
+      Z3 db = i < k ? s.din[i] : s.pr * -1.0;
+      if (i > 0) db = db + s.dout[i - 1];
+      if (i == 0) db = db + s.p0;
+      s.t[i] = (db - z3of(s.dv[i], zdot(db, s.dv[i]))) * (1.0 / s.ell[i]) + z3of(s.dv[i], s.Lbar);
     }
-    // ---- outputs: the value, then each parameter at its first bounce
-    g.items[base] = make_double2(a.re, a.im);
-    g.param[base] = -2;
-    for (int j = 0; j < k; ++j) {
-      if (!pec[j]) {
-        bool first = true;
-        for (int q = 0; q < j; ++q) first = first && mat[q] != mat[j];
-        if (first) {
-          Zc de = zc(0.0);
-          for (int q = j; q < k; ++q)
-            if (mat[q] == mat[j]) de = de + ebar[q];
-          g.items[base + 1 + 4 * j] = make_double2(de.re, de.im);                 // d / d eps_r
-          g.param[base + 1 + 4 * j] = 2 * mat[j];
-          g.items[base + 2 + 4 * j] = make_double2(-de.im * wfac, de.re * wfac);  // d / d sigma
-          g.param[base + 2 + 4 * j] = 2 * mat[j] + 1;
-        }
-      }
-      if (obj[j] >= 0) {
-        bool first = true;
-        for (int q = 0; q < j; ++q) first = first && obj[q] != obj[j];
-        if (!first) continue;
-        for (int ax = 0; ax < 2; ++ax) {
-          // tangent of the image geometry when every plane of object obj[j] moves along axis ax
-          R3 ti[kMaxRefl + 1], tX[kMaxRefl + 2];
-          ti[0] = r3(0, 0, 0);
-          for (int q = 0; q < k; ++q) {
-            R3 dv0 = obj[q] == obj[j] ? r3(ax == 0 ? 1.0 : 0.0, ax == 1 ? 1.0 : 0.0, 0.0) : r3(0, 0, 0);
-            ti[q + 1] = ti[q] - Nn[q] * (2.0 * rdot(ti[q] - dv0, Nn[q]) / rdot(Nn[q], Nn[q]));
-          }
-          tX[k + 1] = r3(0, 0, 0);
-          for (int q = k; q >= 1; --q) {
-            R3 dv0 = obj[q - 1] == obj[j] ? r3(ax == 0 ? 1.0 : 0.0, ax == 1 ? 1.0 : 0.0, 0.0) : r3(0, 0, 0);
-            R3 dir = img[q] - X[q + 1], tdir = ti[q] - tX[q + 1];
-            double den = rdot(dir, Nn[q - 1]), tden = rdot(tdir, Nn[q - 1]);
-            double s = rdot(V0[q - 1] - X[q + 1], Nn[q - 1]) / den;
-            double ts = (rdot(dv0 - tX[q + 1], Nn[q - 1]) - s * tden) / den;
-            tX[q] = tX[q + 1] + dir * ts + tdir * s;
-          }
-          Zc da = zc(0.0);
-          for (int i = 1; i <= k; ++i) da = da + zdot(Xb[i], tX[i]);
-          g.items[base + 3 + ax + 4 * j] = make_double2(da.re, da.im);
-          g.param[base + 3 + ax + 4 * j] = 2 * g.nmat + 2 * obj[j] + ax;
-        }
-      }
+  __syncwarp();
+  if (!act) return;
+  // ---- outputs: each parameter at its first bounce
+  for (int j = gl; j < k; j += kAdjLanes) {
+    bool first = !s.pec[j];
+    for (int q = 0; q < j; ++q) first = first && s.mat[q] != s.mat[j];
+    if (!first) continue;
+    Zc de = zc(0.0);
+    for (int q = j; q < k; ++q)
+      if (s.mat[q] == s.mat[j]) de = de + s.ebar[q];
+    g.items[base + 1 + 4 * j] = make_double2(de.re, de.im);                 // d / d eps_r
+    g.param[base + 1 + 4 * j] = 2 * s.mat[j];
+    g.items[base + 2 + 4 * j] = make_double2(-de.im * wfac, de.re * wfac);  // d / d sigma
+    g.param[base + 2 + 4 * j] = 2 * s.mat[j] + 1;
+  }
+  for (int ja = gl; ja < 2 * k; ja += kAdjLanes) {
+    const int j = ja >> 1, ax = ja & 1;
+    bool first = s.obj[j] >= 0;
+    for (int q = 0; q < j; ++q) first = first && s.obj[q] != s.obj[j];
+    if (!first) continue;
+    // tangent of the image geometry when every plane of object obj[j] moves
+    // along axis ax: of the images, then of the vertices from the last back
+    // (the images' tangents are kept, the vertices' contracted at once)
+    R3 ti[kMaxRefl + 1];
+    ti[0] = r3(0, 0, 0);
+    const R3 e = r3(ax == 0 ? 1.0 : 0.0, ax == 1 ? 1.0 : 0.0, 0.0);
+    for (int q = 0; q < k; ++q) {
+      const R3 d0 = s.obj[q] == s.obj[j] ? e : r3(0, 0, 0);
+      ti[q + 1] = ti[q] - s.Nn[q] * (2.0 * rdot(ti[q] - d0, s.Nn[q]) / s.nn[q]);
     }
+    Zc da = zc(0.0);
+    R3 tX = r3(0, 0, 0);
+    for (int q = k; q >= 1; --q) {
+      const R3 d0 = s.obj[q - 1] == s.obj[j] ? e : r3(0, 0, 0);
+      const R3 dir = s.img[q] - s.X[q + 1], tdir = ti[q] - tX;
+      const double sq = s.sp[q - 1];
+      const double ts = (rdot(d0 - tX, s.Nn[q - 1]) - sq * rdot(tdir, s.Nn[q - 1])) / s.den[q - 1];
+      tX = tX + dir * ts + tdir * sq;
+      da = da + zdot(s.t[q - 1] - s.t[q], tX);  // vertex q ends leg q - 1 and starts leg q
+    }
+    g.items[base + 3 + ax + 4 * j] = make_double2(da.re, da.im);
+    g.param[base + 3 + ax + 4 * j] = 2 * g.nmat + 2 * s.obj[j] + ax;
   }
 }
 
 // Vector-Jacobian product of the received powers: one thread per parameter,
-// receivers summed in order.
+// receivers summed in order, sixteen receivers' values loaded at a time (the
+// sum itself is short; one load per addition took 69 us for 256 receivers).
 __global__ void k_theta_bar(GradArgs g, int nparam) {
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nparam; t += gridDim.x * blockDim.x) {
-    double acc = 0.0;
-    for (int r = 0; r < g.nrx; ++r) acc += g.pcoh_bar[r] * g.dpcoh[(size_t)r * nparam + t];
-    g.theta_bar[t] = acc;
+  constexpr int kBatch = 16;
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= nparam) return;
+  double acc = 0.0;
+  for (int r0 = 0; r0 < g.nrx; r0 += kBatch) {
+    double v[kBatch], w[kBatch];
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i) {
+      const int r = min(r0 + i, g.nrx - 1);
+      v[i] = g.dpcoh[(size_t)r * nparam + t];
+      w[i] = g.pcoh_bar[r];
+    }
+#pragma unroll
+    for (int i = 0; i < kBatch; ++i)
+      if (r0 + i < g.nrx) acc += w[i] * v[i];
   }
+  g.theta_bar[t] = acc;
 }
 
 __global__ void k_pack_rx(const float* __restrict__ rx3, int n, float4* out) {
@@ -659,11 +752,22 @@ cudaError_t launch_pack_rx(const float* rx3, int n, float4* out, cudaStream_t st
   return cudaGetLastError();
 }
 
-cudaError_t launch_adjoint(const GradArgs& a, cudaStream_t st) {
-  if (a.n_paths > 0) k_grad_adjoint<<<(a.n_paths + 63) / 64, 64, 0, st>>>(a);
+static void launch_grad_reduce(const GradArgs& a, int nparam, cudaStream_t st) {
+  if (a.nrx <= 0) return;
+  const size_t smem = a.need_d && nparam <= kGradShared ? 2 * sizeof(double) * (size_t)nparam : 0;
+  k_grad_reduce<<<a.nrx, kGradThreads, smem, st>>>(a, nparam);
+}
+
+cudaError_t launch_adjoint(const GradArgs& a, int sms, cudaStream_t st) {
+  if (a.n_paths > 0) {
+    // one path per warp while there are few, so that a path's FP64 chain has
+    // a scheduler to itself; four when they are many
+    const int ppw = std::max(1, std::min(kAdjGroups, a.n_paths / (8 * sms)));
+    k_grad_adjoint<<<(a.n_paths + ppw - 1) / ppw, 32, 0, st>>>(a, ppw);
+  }
   int nparam = grad_nparam(a.nmat, a.nobj);
-  if (a.nrx > 0) k_grad_reduce<<<(a.nrx + 3) / 4, 128, 0, st>>>(a, nparam);
-  if (a.theta_bar && nparam > 0) k_theta_bar<<<(nparam + 127) / 128, 128, 0, st>>>(a, nparam);
+  launch_grad_reduce(a, nparam, st);
+  if (a.theta_bar && nparam > 0) k_theta_bar<<<(nparam + 31) / 32, 32, 0, st>>>(a, nparam);
   return cudaGetLastError();
 }
 
@@ -673,10 +777,7 @@ cudaError_t launch_gradients(const GradArgs& a, cudaStream_t st) {
     long b = (total + 127) / 128;
     k_grad_items<<<(int)(b < 65535 ? b : 65535), 128, 0, st>>>(a);
   }
-  if (a.nrx > 0) {
-    int nparam = grad_nparam(a.nmat, a.nobj);
-    k_grad_reduce<<<(a.nrx + 3) / 4, 128, 0, st>>>(a, nparam);
-  }
+  launch_grad_reduce(a, grad_nparam(a.nmat, a.nobj), st);
   return cudaGetLastError();
 }
 
