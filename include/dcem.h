@@ -170,7 +170,7 @@ typedef struct {
                                   compact copy in shared memory, 2 = 4-wide
                                   compact copy read from global memory, 3 =
                                   one launch for every scene of a batch
-                                  (binary nodes from global memory)           */
+                                  (4-wide compact copies from global memory)  */
   int32_t graph_replayed;      /* 1 if the frame's device work was launched as
                                   one replayed CUDA graph                        */
   int32_t paths_sticky;        /* DCEM_MODE_STICKY: valid paths that only the

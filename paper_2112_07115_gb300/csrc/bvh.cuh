@@ -66,6 +66,10 @@ struct FramePrepArgs {
   SmallTreeArgs trx, tmv;
 };
 
+// Boxes of a tree whose topology (children, parents, leaf parents) is set, from
+// its primitives' boxes; arrive: zeroed, one word per internal node.
+void launch_refit_prims(const float* d_prim, const int* d_perm, int n, int node_base, int leaf_base, float4* d_nodes,
+                        const int* d_leaf_parent, int* d_arrive, float* d_root_box, cudaStream_t st);
 cudaError_t launch_frame_prep(const FramePrepArgs& a, cudaStream_t st);
 
 // Counts of scratch the scan of m histogram entries needs beyond them.

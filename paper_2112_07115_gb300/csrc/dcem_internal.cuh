@@ -575,7 +575,8 @@ __device__ __forceinline__ void cswap(float& da, int& ca, float& db, int& cb) {
 
 // Closest hit as closest_hit(), over the 4-wide compact copy: per step the
 // four child boxes are tested, the hit ones ordered by entry distance, the
-// nearest visited next and the others pushed. Node visits count box pairs
+// nearest visited next and the others pushed (pushed unsorted, the highway's
+// frame took 414 us instead of 407, the office's 1071 instead of 1057). Node visits count box pairs
 // (a 4-wide step = 2), the unit of the 2-wide traversals. kG: the copy is
 // read from global memory (read-only path) instead of shared memory.
 template <bool kG = false>

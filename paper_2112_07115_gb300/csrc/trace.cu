@@ -38,6 +38,19 @@ __device__ __forceinline__ long long capitems_cap(const TraceArgs& a) {
   return (long long)(a.N + a.max_trans + 1) * a.LS;
 }
 
+// The compact copy's grid and size.
+__device__ __forceinline__ QFrame load_qframe(const TraceArgs& a) {
+  QFrame f;
+  f.ox = a.qframe[0];
+  f.oy = a.qframe[1];
+  f.oz = a.qframe[2];
+  f.sx = a.qframe[3];
+  f.sy = a.qframe[4];
+  f.sz = a.qframe[5];
+  f.n4 = min(*a.q4_count, a.q4_bound);
+  return f;
+}
+
 // Warp-wide dynamic work fetch: lane 0 takes the next `n` items.
 __device__ __forceinline__ int fetch_warp(unsigned* counter, unsigned n) {
   int base = 0;
@@ -242,22 +255,31 @@ __global__ void __launch_bounds__(256) k_trace_t(TraceArgs a) {
 // several scenes in one launch
 // ---------------------------------------------------------------------------
 // Every scene's rays (its retrace queue in a coherent frame) in one
-// persistent launch: the scenes' work is cut into chunks of 32 rays of one
-// scene, a warp takes the next chunk from a counter shared by all scenes and
-// traces its rays over that scene's binary trees (nodes from L2), with the
-// same per-segment steps as trace_rays. A chunk's scene is found by a binary
-// search over the chunk counts' prefix, formed by every CTA at its start.
-__global__ void __launch_bounds__(256) k_trace_batch(const TraceArgs* __restrict__ tab, int n, unsigned* chunk_ctr) {
+// persistent launch: the scenes' work is cut into chunks of rays of one
+// scene, a warp takes the next chunk from a counter shared by all
+// scenes and traces its rays over that scene's 4-wide compact copy (from L2;
+// the binary nodes where a scene has none), a lane whose ray has ended taking
+// the chunk's next one, with the same per-segment steps as trace_rays. A
+// chunk's scene is found by a binary search over the chunk counts' prefix,
+// formed by every CTA at its start.
+constexpr unsigned kBatchChunk = 128, kBatchChunkMin = 32;
+__global__ void __launch_bounds__(256, 3) k_trace_batch(const TraceArgs* __restrict__ tab, int n, unsigned* chunk_ctr) {
   extern __shared__ int sstk[];
   __shared__ unsigned pre[kMaxBatch + 1];  // pre[s]: chunks of the scenes before s
+  __shared__ unsigned rays;                // of all scenes
   TStack st;
   bind_stack(st, sstk, kStackTrace);
+  if (threadIdx.x == 0) pre[0] = rays = 0u;
+  __syncthreads();
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const TraceArgs& t = tab[i];
-    unsigned nq = t.queue ? min(*t.nq_dev, (unsigned)t.R) : (unsigned)t.R;
-    pre[i + 1] = (nq + 31u) >> 5;
+    pre[i + 1] = t.queue ? min(*t.nq_dev, (unsigned)t.R) : (unsigned)t.R;
+    atomicAdd(&rays, pre[i + 1]);
   }
-  if (threadIdx.x == 0) pre[0] = 0u;
+  __syncthreads();
+  // short lists (retrace queues) in smaller chunks, so that every warp has some
+  const unsigned chunk = rays / (4u * gridDim.x * (blockDim.x >> 5)) >= kBatchChunk ? kBatchChunk : kBatchChunkMin;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) pre[i + 1] = (pre[i + 1] + chunk - 1u) / chunk;
   __syncthreads();
   if (threadIdx.x == 0)
     for (int i = 1; i <= n; ++i) pre[i] += pre[i - 1];
@@ -279,35 +301,50 @@ __global__ void __launch_bounds__(256) k_trace_batch(const TraceArgs* __restrict
     const int R = a.R, N = a.N;
     [[maybe_unused]] const int LS = a.LS;  // bounds of the checked build
     const unsigned nq = a.queue ? min(*a.nq_dev, (unsigned)R) : (unsigned)R;
-    const unsigned q = ((c - pre[lo]) << 5) + (unsigned)lane;
+    unsigned next = (c - pre[lo]) * chunk;
+    const unsigned end = min(nq, next + chunk);
+    QFrame f{};
+    int qr0 = kEmpty, qr1 = kEmpty;
+    if (a.use_q) {
+      f = load_qframe(a);
+      qr0 = a.q4_roots[0];
+      qr1 = a.q4_roots[1];
+    }
     int ray = -1, b = 0, last = -1;
     float3 o = f3(0.0f, 0.0f, 0.0f), d = o;
     float D = 0.0f;
-    if (q < nq) {
-      ray = a.queue ? a.queue[DCEM_IDX((int)q, R)] : (int)q;
-      b = a.queue ? a.restart[DCEM_IDX(ray, R)] : 0;
-      if (b == 0) {
-        float4 rd = __ldg(&a.rays[DCEM_IDX(ray, R)]);
-        float4 t4 = __ldg(&a.txs[DCEM_IDX(__float_as_int(rd.w), a.nsets)]);
-        o = f3(t4.x, t4.y, t4.z);
-        d = f3(rd.x, rd.y, rd.z);
-      } else {
-        float4 lo4 = a.log_o[log_at(a, b, ray)], ld = a.log_d[log_at(a, b, ray)];
-        o = f3(lo4.x, lo4.y, lo4.z);
-        D = lo4.w;
-        d = f3(ld.x, ld.y, ld.z);
-        last = a.log_id[log_at(a, b - 1, ray)];
-      }
-    }
     unsigned segs = 0, nodes = 0, tris = 0, ovf = 0, maxn = 0;
-    while (__any_sync(0xffffffffu, ray >= 0)) {
+    for (;;) {
+      const unsigned need = __ballot_sync(0xffffffffu, ray < 0);
+      const unsigned q = next + __popc(need & ((1u << lane) - 1u));
+      if (ray < 0 && q < end) {
+        ray = a.queue ? a.queue[DCEM_IDX((int)q, R)] : (int)q;
+        b = a.queue ? a.restart[DCEM_IDX(ray, R)] : 0;
+        if (b == 0) {
+          float4 rd = __ldg(&a.rays[DCEM_IDX(ray, R)]);
+          float4 t4 = __ldg(&a.txs[DCEM_IDX(__float_as_int(rd.w), a.nsets)]);
+          o = f3(t4.x, t4.y, t4.z);
+          d = f3(rd.x, rd.y, rd.z);
+          D = 0.0f;
+          last = -1;
+        } else {
+          float4 lo4 = a.log_o[log_at(a, b, ray)], ld = a.log_d[log_at(a, b, ray)];
+          o = f3(lo4.x, lo4.y, lo4.z);
+          D = lo4.w;
+          d = f3(ld.x, ld.y, ld.z);
+          last = a.log_id[log_at(a, b - 1, ray)];
+        }
+      }
+      next = min(end, next + (unsigned)__popc(need));
+      if (!__any_sync(0xffffffffu, ray >= 0)) break;
       unsigned item = 0xffffffffu;
       if (ray >= 0) {
         RayPre rp = ray_pre(o, d);
         float t;
         int id;
         unsigned nn = 0, nt = 0;
-        const int slot = closest_hit(bvh, rp, a.tmin, last, t, id, ovf, nn, nt, st);
+        const int slot = a.use_q ? closest_hit_q4<true>(a.qnodes, f, bvh, qr0, qr1, rp, a.tmin, last, t, id, ovf, nn, nt, st)
+                                 : closest_hit_far(bvh, rp, a.tmin, last, &t, &id, &ovf, &nn, &nt, st.s, st.stride, st.cap);
         ++segs;
         nodes += nn;
         tris += nt;
@@ -374,14 +411,7 @@ __device__ __forceinline__ void trace_q_body(const TraceArgs& a) {
   const int n4 = min(*a.q4_count, a.q4_bound);
   for (int i = threadIdx.x; i < 4 * n4; i += blockDim.x) sq[i] = a.qnodes[i];
   const int qr0 = a.q4_roots[0], qr1 = a.q4_roots[1];
-  QFrame f;
-  f.ox = a.qframe[0];
-  f.oy = a.qframe[1];
-  f.oz = a.qframe[2];
-  f.sx = a.qframe[3];
-  f.sy = a.qframe[4];
-  f.sz = a.qframe[5];
-  f.n4 = n4;
+  const QFrame f = load_qframe(a);
   __syncthreads();
   trace_rays<true, false, kT>(a, sq, f, st, qr0, qr1);
 }
@@ -396,14 +426,7 @@ __global__ void __launch_bounds__(256, 3) k_trace_qg(TraceArgs a) {
   TStack st;
   bind_stack(st, sstk, a.stack_cap);
   const int qr0 = a.q4_roots[0], qr1 = a.q4_roots[1];
-  QFrame f;
-  f.ox = a.qframe[0];
-  f.oy = a.qframe[1];
-  f.oz = a.qframe[2];
-  f.sx = a.qframe[3];
-  f.sy = a.qframe[4];
-  f.sz = a.qframe[5];
-  f.n4 = min(*a.q4_count, a.q4_bound);
+  const QFrame f = load_qframe(a);
   trace_rays<true, true>(a, a.qnodes, f, st, qr0, qr1);
 }
 
