@@ -724,54 +724,77 @@ struct SmallBvh {
   int cap;                           // leaves the tree's arrays hold (nodes: cap - 1)
 };
 
-// Slab test returning the clipped parameter interval [tn, tf] within [0, tcap].
-__device__ __forceinline__ bool slab_io(const RayPre& r, float lox, float hix, float loy, float hiy,
-                                        float loz, float hiz, float tcap, float& tn, float& tf) {
-  float t0x = __fmul_rn(__fsub_rn(lox, r.o.x), r.inv.x), t1x = __fmul_rn(__fsub_rn(hix, r.o.x), r.inv.x);
-  float t0y = __fmul_rn(__fsub_rn(loy, r.o.y), r.inv.y), t1y = __fmul_rn(__fsub_rn(hiy, r.o.y), r.inv.y);
-  float t0z = __fmul_rn(__fsub_rn(loz, r.o.z), r.inv.z), t1z = __fmul_rn(__fsub_rn(hiz, r.o.z), r.inv.z);
-  tn = fmax3(fminf(t0x, t1x), fminf(t0y, t1y), fmaxf(fminf(t0z, t1z), 0.0f));
-  tf = fmin3(fmaxf(t0x, t1x), fmaxf(t0y, t1y), fminf(fmaxf(t0z, t1z), tcap));
+// The capture cone of a segment against a box of receivers. A receiver
+// captured at parameter s lies within rho(s) = alpha (D + s) of o + s d, so
+// along each axis o + s d - rho(s) <= R <= o + s d + rho(s), and with R in the
+// box these are linear inequalities in s: s (d + alpha) >= lo - o - alpha D
+// and s (d - alpha) <= hi - o + alpha D. With d >= 0 the first is a lower
+// bound of s and the second an upper one while d > alpha, else (the cone
+// spreads faster than it moves along the axis) a lower one too: a box beside
+// the segment is reached only where the cone has grown to it. With d < 0 the
+// sides change places. The box can hold a captured receiver only if the three axes'
+// intervals meet within [0, tend]. One pass of a multiply-add per plane, and
+// tighter than the segment against the box grown by the radius at its end and
+// again at the exit, which it replaces (urban grid's capture pass 976 -> 806 us,
+// highway 56 -> 53). Margins (0.1% of the radius, 1 cm and 4e-7 of the
+// coordinates) exceed the FP32 rounding.
+struct ConeRay {
+  float nx, ny, nz, mx, my, mz;  // near planes: s >= plane * n + m
+  float fx, fy, fz, gx, gy, gz;  // far planes: s <= plane * f + g,
+  float hx, hy, hz, kx, ky, kz;  // or s >= plane * h + k (the other pair bounds nothing)
+  bool px, py, pz;               // d >= 0: near plane lo
+};
+__device__ __forceinline__ void cone_axis(float o, float d, float a, float c, float& n, float& m, float& f, float& g,
+                                          float& h, float& k, bool& p) {
+  p = d >= 0.0f;
+  const float s = p ? 1.0f : -1.0f;
+  // near: (lo - c - o) / (d + a), or (hi + c - o) / (d - a)
+  n = __fdividef(1.0f, __fmaf_rn(s, a, d));
+  m = __fmul_rn(__fmaf_rn(-s, c, -o), n);
+  // far: (hi + c - o) / (d - a), or (lo - c - o) / (d + a)
+  const float e = __fmaf_rn(-s, a, d), i = __fdividef(1.0f, e), j = __fmul_rn(__fmaf_rn(s, c, -o), i);
+  const bool upper = s * e > 1e-6f, lower = s * e < -1e-6f;
+  f = upper ? i : 0.0f;
+  g = upper ? j : 3.4e38f;
+  h = lower ? i : 0.0f;
+  k = lower ? j : -3.4e38f;
+}
+__device__ __forceinline__ ConeRay cone_ray(float3 o, float3 d, float D, float tend, float alpha) {
+  const float a = alpha * 1.001f, c = __fmaf_rn(a, D, 0.01f + 4e-7f * (fabsf(o.x) + fabsf(o.y) + fabsf(o.z) + tend));
+  ConeRay r;
+  cone_axis(o.x, d.x, a, c, r.nx, r.mx, r.fx, r.gx, r.hx, r.kx, r.px);
+  cone_axis(o.y, d.y, a, c, r.ny, r.my, r.fy, r.gy, r.hy, r.ky, r.py);
+  cone_axis(o.z, d.z, a, c, r.nz, r.mz, r.fz, r.gz, r.hz, r.kz, r.pz);
+  return r;
+}
+// The parameters [tn, tf] at which the cone can hold a point of the box.
+__device__ __forceinline__ bool cone_box(const ConeRay& r, float tend, float lox, float hix, float loy, float hiy,
+                                         float loz, float hiz, float& tf) {
+  const float x0 = r.px ? lox : hix, x1 = r.px ? hix : lox, y0 = r.py ? loy : hiy, y1 = r.py ? hiy : loy,
+              z0 = r.pz ? loz : hiz, z1 = r.pz ? hiz : loz;
+  const float near3 = fmax3(__fmaf_rn(x0, r.nx, r.mx), __fmaf_rn(y0, r.ny, r.my), __fmaf_rn(z0, r.nz, r.mz));
+  const float grown = fmax3(__fmaf_rn(x1, r.hx, r.kx), __fmaf_rn(y1, r.hy, r.ky), __fmaf_rn(z1, r.hz, r.kz));
+  const float tn = fmax3(near3, grown, 0.0f);
+  tf = fmin3(__fmaf_rn(x1, r.fx, r.gx), __fmaf_rn(y1, r.fy, r.gy), fminf(__fmaf_rn(z1, r.fz, r.gz), tend));
   return slab_accept(tn, tf);
 }
 
-// Conservative filter for the capture cone of a segment against a box of
-// receivers: false only if no point of the box can pass `captured`. A point
-// captured at parameter s lies within rho(s) = alpha (D + s) of the segment,
-// so the segment meets the box grown by rho(tend); within that clipped
-// interval [tn, tf] the radius is at most rho(tf), so the segment also meets
-// the box grown by rho(tf). Margins (0.1% and 1 cm) exceed FP32 rounding.
-__device__ __forceinline__ bool cone_box(const RayPre& r, float D, float tend, float alpha, float lox,
-                                         float hix, float loy, float hiy, float loz, float hiz) {
-  float a = alpha * 1.001f;
-  float g = a * (D + tend) + 0.01f;
-  float tn, tf;
-  if (!slab_io(r, lox - g, hix + g, loy - g, hiy + g, loz - g, hiz + g, tend, tn, tf)) return false;
-  g = a * (D + fminf(tf * 1.00001f, tend)) + 0.01f;
-  return slab_io(r, lox - g, hix + g, loy - g, hiy + g, loz - g, hiz + g, tend, tn, tf);
-}
-
-// Every receiver whose reception sphere captures the segment (r.o, d, D,
+// Every receiver whose reception sphere captures the segment (o, d, D,
 // tend) is passed to emit(rx index). Returns false on a malformed tree or a
 // stack overflow.
 template <class Emit>
-__device__ __forceinline__ bool capture_tree(const SmallBvh& t, const float4* __restrict__ rx,
-                                             const RayPre& r, float3 d, float D, float tend, float alpha,
-                                             TStack& st, Emit&& emit) {
+__device__ __forceinline__ bool capture_tree(const SmallBvh& t, const float4* __restrict__ rx, float3 o, float3 d,
+                                             float D, float tend, float alpha, TStack& st, Emit&& emit) {
   int root = *t.root;
   if (root == kEmpty) return true;
-  // Every receiver lies in the root box, so a capture at s puts the segment
-  // within rho(s) <= rho(te) of that box: clip the culling length te to the
-  // exit of the box grown by the largest radius, twice (the second time
-  // with the radius at the first exit). The exact test keeps tend.
-  float te = tend;
+  const ConeRay r = cone_ray(o, d, D, tend, alpha);
+  // every receiver lies in the root box: the culling length ends at its exit
+  // (the exact test keeps tend)
+  float te;
   {
     const float* rb = t.root_box;
-    for (int it = 0; it < 2; ++it) {
-      float g = alpha * 1.001f * (D + te) + 0.01f, tn, tf;
-      if (!slab_io(r, rb[0] - g, rb[3] + g, rb[1] - g, rb[4] + g, rb[2] - g, rb[5] + g, te, tn, tf)) return true;
-      te = fminf(te, tf * 1.00001f + 1e-6f);
-    }
+    if (!cone_box(r, tend, rb[0], rb[3], rb[1], rb[4], rb[2], rb[5], te)) return true;
+    te = fminf(tend, te * 1.00001f + 1e-6f);
   }
   st.reset();
   int cur = root;
@@ -779,15 +802,23 @@ __device__ __forceinline__ bool capture_tree(const SmallBvh& t, const float4* __
     if (cur < 0) {
       int ri = t.perm[DCEM_IDX(~cur, t.cap)];
       float4 v = rx[DCEM_IDX(ri, t.cap)];
-      if (captured(r.o, d, D, tend, alpha, f3(v.x, v.y, v.z))) emit(ri);
+      if (captured(o, d, D, tend, alpha, f3(v.x, v.y, v.z))) emit(ri);
     } else {
       const float4* n = t.nodes + 4 * (size_t)DCEM_IDX(cur, t.cap - 1);
       float4 n0 = n[0], n1 = n[1], n2 = n[2], n3 = n[3];
       int c0 = __float_as_int(n3.x), c1 = __float_as_int(n3.y);
-      bool m0 = cone_box(r, D, te, alpha, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y);
-      bool m1 = cone_box(r, D, te, alpha, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w);
-      if (m1 && !st.push(c1)) return false;
-      if (m0 && !st.push(c0)) return false;
+      float tf;
+      bool m0 = cone_box(r, te, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, tf);
+      bool m1 = cone_box(r, te, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, tf);
+      if (m0 && m1) {
+        if (!st.push(c1)) return false;
+        cur = c0;
+        continue;
+      }
+      if (m0 || m1) {
+        cur = m0 ? c0 : c1;
+        continue;
+      }
     }
     if (st.empty()) return true;
     cur = st.pop();

@@ -476,13 +476,7 @@ __global__ void __launch_bounds__(256) k_capture(TraceArgs a) {
                                        : 0;
       float alpha = __ldg(&a.txs[DCEM_IDX(set, a.nsets)].w);
       int link0 = set * a.nrx;
-      RayPre rp;
-      rp.o = o;
-      float dx = fabsf(d.x) < 1e-30f ? copysignf(1e-30f, d.x) : d.x;
-      float dy = fabsf(d.y) < 1e-30f ? copysignf(1e-30f, d.y) : d.y;
-      float dz = fabsf(d.z) < 1e-30f ? copysignf(1e-30f, d.z) : d.z;
-      rp.inv = f3(__fdiv_rn(1.0f, dx), __fdiv_rn(1.0f, dy), __fdiv_rn(1.0f, dz));
-      if (!capture_tree(rxt, rx, rp, d, D, tend, alpha, st, [&](int r) {
+      if (!capture_tree(rxt, rx, o, d, D, tend, alpha, st, [&](int r) {
             if (!reused || a.rx_moved[r]) emit_cand(a, ray, b, link0 + r);
           }))
         ovf = 1u;
