@@ -2108,7 +2108,7 @@ static int enqueue_post(const FramePlan& P, int sms, cudaStream_t st, bool cap, 
   CK(launch_dedupe(P.q, sms * 4, st));
   if (P.q.sticky_prev) CK(launch_sticky_probe(P.q, sms * 4, st));
   if (tm) CK(rec(P.ev[5], st, cap));
-  CK(launch_validate(P.q, sms * 4, st));
+  CK(launch_validate(P.q, P.nlinks, sms * 4, st));
   if (P.q.vc_next_key) CK(launch_vcache_build(P.q, sms * 4, st));
   if (P.q.wedges) CK(launch_diffract(P.q, P.nlinks, sms, st));
   if (tm) CK(rec(P.ev[6], st, cap));
@@ -2193,8 +2193,8 @@ static int plan_frame(dcem_scene* s, int nrx, const dcem_params* p, bool coheren
   FramePlan& P = s->plan;
   make_plan(s, nrx, p, coherent, out, P);
   s->last_use_q = P.use_q;
-  // kernels of this frame: prep, [mark, carry], trace, capture, dedupe x2, validate x3, reduce, end
-  s->launches += 2 + (coherent ? 2 : 0) + (s->R > 0 ? 2 + P.a.max_trans : 0) + 5 + (nrx > 0 ? 1 : 0) +
+  // kernels of this frame: prep, [mark, carry], trace, capture, dedupe x2, validate (x3 with many links), reduce, end
+  s->launches += 2 + (coherent ? 2 : 0) + (s->R > 0 ? 2 + P.a.max_trans : 0) + (P.nlinks <= kFewLinks ? 3 : 5) + (nrx > 0 ? 1 : 0) +
                  (P.q.vc_next_key ? 1 : 0) +
                  (P.use_q ? 1 : 0) + (P.q.link_off ? (P.nlinks > 65536 ? 2 : 1) : 0) + (P.q.sticky_prev ? 1 : 0) +
                  diffraction_launches(P);
@@ -2734,7 +2734,7 @@ int dcem_batch_trace(dcem_batch* b, const float* const* tx, const int32_t* ntx, 
       // binary nodes of a scene without one, or configured so)
       P.use_q = P.a.use_q = P.use_q ? 2 : 0;
       s->last_use_q = 3;  // every scene's rays in one launch
-      s->launches += 2 + (coh[i] ? 2 : 0) + (s->R > 0 ? 1 : 0) + 5 + (nrx[i] > 0 ? 1 : 0) +
+      s->launches += 2 + (coh[i] ? 2 : 0) + (s->R > 0 ? 1 : 0) + (P.nlinks <= kFewLinks ? 3 : 5) + (nrx[i] > 0 ? 1 : 0) +
                      (P.q.vc_next_key ? 1 : 0) + (P.use_q ? 1 : 0) + (P.q.link_off ? (P.nlinks > 65536 ? 2 : 1) : 0) +
                      (P.q.sticky_prev ? 1 : 0) + diffraction_launches(P) + (i == 0 ? 1 : 0);
       s->graph_replayed = 0;

@@ -283,7 +283,8 @@ __device__ __forceinline__ d3 pol_of(d3 u, d3 d, unsigned& flags) {
 }
 
 // ---------------------------------------------------------------------------
-// validation + field in three kernels:
+// validation + field, with many links in three kernels (k_validate: with few,
+// in one):
 //   k_val_geom   one thread per distinct key: image sources, back-trace,
 //                reflection points inside their triangles (FP64)
 //   k_val_occ    one thread per (key, sub-segment): FP32 any-hit occlusion
@@ -338,8 +339,45 @@ __device__ __forceinline__ bool vc_reusable(const PathArgs& a, int pu, int rxi, 
   return true;
 }
 
-// T = double (FP64) or df (double-float) for every step of the geometry;
-// path points and length are stored in FP64 either way.
+// The steps of the geometry, T = double (FP64) or df (double-float); path
+// points and length are stored in FP64 either way. Both validation kernels
+// below run these same operations, so a key's result does not depend on which
+// of them took it.
+// An interaction's triangle and its (unnormalised) normal: false when it has
+// none, or is a transmission (ids with kTransBit) through an opaque material.
+template <class T>
+__device__ __forceinline__ bool val_triangle(const PathArgs& a, int id, v3<T>& v0, v3<T>& v1, v3<T>& v2, v3<T>& n) {
+  const float4* tp = a.tris + 3 * (size_t)DCEM_IDX(a.slot_of_id[DCEM_IDX(id & ~kTransBit, a.bvh.ntris)], a.bvh.ntris);
+  const float4 p0 = tp[0], p1 = tp[1], p2 = tp[2];
+  v0 = vof<T>(p0.x, p0.y, p0.z);
+  v1 = vof<T>(p1.x, p1.y, p1.z);
+  v2 = vof<T>(p2.x, p2.y, p2.z);
+  n = vcross(v1 - v0, v2 - v0);
+  const bool opaque = (id & kTransBit) && !(a.mats[__float_as_int(p1.w)].w >= 0.0f);
+  return !opaque && pos(vdot(n, n));
+}
+// step 3: the image of I in the plane of (v0, n), nn = n.n
+template <class T>
+__device__ __forceinline__ v3<T> val_image(v3<T> I, v3<T> v0, v3<T> n, T nn) {
+  return I - scale(n, sc_of<T>(2.0f) * vdot(I - v0, n) / nn);
+}
+// step 4: where the leg from X toward Y crosses the plane, the parameter
+// within (lo, 1); false when it does not
+template <class T>
+__device__ __forceinline__ bool val_cross(v3<T> X, v3<T> Y, v3<T> v0, v3<T> n, T lo, T& s, v3<T>& P) {
+  const v3<T> dir = Y - X;
+  const T den = vdot(dir, n);
+  if (zero(den)) return false;
+  s = vdot(v0 - X, n) / den;
+  P = X + scale(dir, s);
+  return pos(s - lo) && neg(s - sc_of<T>(1.0f));
+}
+template <class T>
+__device__ __forceinline__ bool val_inside(v3<T> v0, v3<T> v1, v3<T> v2, v3<T> n, v3<T> x) {
+  return !(neg(vdot(vcross(v1 - v0, x - v0), n)) || neg(vdot(vcross(v2 - v1, x - v1), n)) ||
+           neg(vdot(vcross(v0 - v2, x - v2), n)));
+}
+
 template <class T>
 __global__ void __launch_bounds__(64) k_val_geom(PathArgs a) {
   extern __shared__ int sstk[];
@@ -425,46 +463,29 @@ __global__ void __launch_bounds__(64) k_val_geom(PathArgs a) {
     float4 rxv = a.rx[rxi % a.nrx], txv = a.txs[rxi / a.nrx];
     v3<T> X[kMaxRefl + 2], V0[kMaxRefl], V1[kMaxRefl], V2[kMaxRefl], Nn[kMaxRefl];
     v3<T> tx = vof<T>(txv.x, txv.y, txv.z), rx = vof<T>(rxv.x, rxv.y, rxv.z);
-    const T two = sc_of<T>(2.0f), one = sc_of<T>(1.0f);
     bool ok = true;
-    // interactions: reflections, and transmissions (kTransBit) straight
-    // through a transmitting triangle; rj lists the reflections
+    // interactions: reflections (rj lists them), and transmissions straight
+    // through a transmitting triangle
     int rj[kMaxRefl], m = 0;
-    bool isT[kMaxRefl];
     for (int j = 0; j < k && ok; ++j) {
-      isT[j] = (ids[j] & kTransBit) != 0;
-      const float4* tp = a.tris + 3 * (size_t)DCEM_IDX(a.slot_of_id[DCEM_IDX(ids[j] & ~kTransBit, a.bvh.ntris)],
-                                                        a.bvh.ntris);
-      float4 p0 = tp[0], p1 = tp[1], p2 = tp[2];
-      if (isT[j] && !(a.mats[__float_as_int(p1.w)].w >= 0.0f)) ok = false;
-      V0[j] = vof<T>(p0.x, p0.y, p0.z);
-      V1[j] = vof<T>(p1.x, p1.y, p1.z);
-      V2[j] = vof<T>(p2.x, p2.y, p2.z);
-      v3<T> n = vcross(V1[j] - V0[j], V2[j] - V0[j]);
-      if (!pos(vdot(n, n))) ok = false;
-      Nn[j] = n;
-      if (!isT[j]) rj[m++] = j;
+      ok = val_triangle(a, ids[j], V0[j], V1[j], V2[j], Nn[j]);
+      if (!(ids[j] & kTransBit)) rj[m++] = j;
     }
-    // step 3: image sources I_1..I_m in the planes of the reflecting triangles
+    // image sources I_1..I_m in the planes of the reflecting triangles
     v3<T> img[kMaxRefl + 1];
     img[0] = tx;
     for (int q = 0; q < m && ok; ++q) {
       int j = rj[q];
-      T nn = vdot(Nn[j], Nn[j]);
-      img[q + 1] = img[q] - scale(Nn[j], two * vdot(img[q] - V0[j], Nn[j]) / nn);
+      img[q + 1] = val_image(img[q], V0[j], Nn[j], vdot(Nn[j], Nn[j]));
     }
-    // step 4: back-trace from the receiver; XR = reflection points
+    // back-trace from the receiver; XR = reflection points
     v3<T> XR[kMaxRefl + 2];
     XR[0] = tx;
     XR[m + 1] = rx;
     for (int q = m; q >= 1 && ok; --q) {
       int j = rj[q - 1];
-      v3<T> dir = img[q] - XR[q + 1];
-      T den = vdot(dir, Nn[j]);
-      if (zero(den)) { ok = false; break; }
-      T sp = vdot(V0[j] - XR[q + 1], Nn[j]) / den;
-      if (!(pos(sp) && neg(sp - one))) { ok = false; break; }
-      XR[q] = XR[q + 1] + scale(dir, sp);
+      T sp;
+      ok = val_cross(XR[q + 1], img[q], V0[j], Nn[j], sc_of<T>(0.0f), sp, XR[q]);
     }
     // the interaction points in order: a transmission crosses its plane on
     // the straight piece between the surrounding reflection points, after
@@ -475,22 +496,16 @@ __global__ void __launch_bounds__(64) k_val_geom(PathArgs a) {
       int q = 0;
       T s_prev = sc_of<T>(0.0f);
       for (int j = 0; j < k && ok; ++j) {
-        if (!isT[j]) {
+        if (!(ids[j] & kTransBit)) {
           X[j + 1] = XR[++q];
           s_prev = sc_of<T>(0.0f);
         } else {
-          v3<T> A = XR[q], dir = XR[q + 1] - XR[q];
-          T den = vdot(dir, Nn[j]);
-          if (zero(den)) { ok = false; break; }
-          T sp = vdot(V0[j] - A, Nn[j]) / den;
-          if (!(pos(sp - s_prev) && neg(sp - one))) { ok = false; break; }
-          X[j + 1] = A + scale(dir, sp);
+          T sp;
+          ok = val_cross(XR[q], XR[q + 1], V0[j], Nn[j], s_prev, sp, X[j + 1]);
+          if (!ok) break;
           s_prev = sp;
         }
-        v3<T> v0 = V0[j], v1 = V1[j], v2 = V2[j], n = Nn[j], x = X[j + 1];
-        if (neg(vdot(vcross(v1 - v0, x - v0), n)) || neg(vdot(vcross(v2 - v1, x - v1), n)) ||
-            neg(vdot(vcross(v0 - v2, x - v2), n)))
-          ok = false;
+        ok = val_inside(V0[j], V1[j], V2[j], Nn[j], X[j + 1]);
       }
     }
     T L = sc_of<T>(0.0f);
@@ -756,6 +771,247 @@ __global__ void __launch_bounds__(kFieldThreads) k_val_field(PathArgs a) {
       field_done(a, rec, X, u, E, mk3(ends.prx[0], ends.prx[1], ends.prx[2]), ends.sn, ends.cs, ends.fl0 | ends.fl1);
     }
     __syncwarp(gmask);  // the group's shared records are free again
+  }
+}
+
+// ---------------------------------------------------------------------------
+// few links: the three steps in one kernel, a group of lanes per key
+// ---------------------------------------------------------------------------
+// With few links a frame has a few hundred keys, and validation is the time
+// of one key's chain of dependent FP64 operations and loads, three times over
+// (the highway: geometry 33, occlusion 21, field 27 us). Here a group of
+// kFieldLanes lanes takes a key through all three: each lane its own
+// interaction's triangle, normal and inside test, its own leg's length and
+// occlusion, its own bounce's coefficients; only the images, the back-trace
+// and the field's last step run in one lane. The key's state waits in shared
+// memory.
+template <class T>
+struct ValKey {
+  v3<T> v0[kMaxRefl], v1[kMaxRefl], v2[kMaxRefl], n[kMaxRefl], img[kMaxRefl + 1], X[kMaxRefl + 2];
+  T nn[kMaxRefl], leg[kMaxRefl + 1];
+  d3 P[kMaxRefl + 2];
+  BounceCoef coef[kMaxRefl];
+  FieldEnds ends;
+  int ids[kMaxRefl];
+};
+
+template <class T>
+__global__ void __launch_bounds__(kFieldThreads) k_validate(PathArgs a) {
+  constexpr int kGroups = kFieldThreads / kFieldLanes;
+  extern __shared__ int sstk[];
+  __shared__ ValKey<T> skeys[kGroups];
+  TStack st;
+  bind_stack(st, sstk, kStackTrace);
+  const int grp = threadIdx.x / kFieldLanes, gl = threadIdx.x % kFieldLanes;
+  const unsigned gmask = ((1u << kFieldLanes) - 1u) << ((threadIdx.x & 31) & ~(kFieldLanes - 1));
+  ValKey<T>& S = skeys[grp];
+  const unsigned nu = min(a.ctr->n_unique, a.ucap);
+  const bool reuse = a.reuse && a.ctr->n_moved_boxes <= a.mv_cap;
+  const d3 upol = mk3(a.pol.x, a.pol.y, a.pol.z);
+  const double wfac = -1.0 / (2.0 * M_PI * a.freq * 8.8541878128e-12);
+  unsigned ovf = 0;
+  for (unsigned it = 0;; ++it) {
+    const unsigned u = blockIdx.x + gridDim.x * (grp + kGroups * it);
+    if (u >= nu) break;
+    __syncwarp(gmask);  // the group's record is free again
+    // ---- the key
+    const int ci = a.uniq[u];
+    int k, rxi, ray;
+    unsigned fl0 = 0u;
+    unsigned long long lkey = 0ull, key;  // the link key (0: a sticky record) and the record's
+    if (ci >= 0) {
+      const Cand c = a.cand[DCEM_IDX(ci, a.cand_cap)];
+      const int slot = DCEM_IDX(a.cand_slot[DCEM_IDX(ci, a.cand_cap)], a.hcap);
+      key = lkey = a.hkey[slot];
+      k = cand_seg(c);
+      rxi = cand_rx(c);
+      ray = c.ray;
+      for (int j = gl; j < kMaxRefl; j += kFieldLanes) S.ids[j] = j < k ? log_id_at(a, j, ray) : -1;
+      __syncwarp(gmask);
+      if (gl == 0) {  // the slot is no longer needed: the table stays empty for the next frame
+        a.hkey[slot] = 0ull;
+        a.hrep[slot] = ~0ull;
+      }
+      // the record's key leaves the transmitter out: (receiver, depth,
+      // sequence), as a single-transmitter frame has it
+      if (rxi >= a.nrx) key = seq_key(rxi % a.nrx, k, [&](int j) { return S.ids[j]; });
+      if (ray >= a.R0) ray = a.inst_root[DCEM_IDX(ray - a.R0, a.R - a.R0)];  // reported as its primary ray
+    } else {  // sticky mode: a kept path that no capture of this frame has
+      const StickyKey& sk = a.sticky_prev[~ci];
+      k = sk.depth;
+      rxi = sk.link;
+      ray = -1;
+      for (int j = gl; j < kMaxRefl; j += kFieldLanes) S.ids[j] = j < k ? sk.tri[j] : -1;
+      __syncwarp(gmask);
+      key = seq_key(rxi % a.nrx, k, [&](int j) { return S.ids[j]; });
+      fl0 = DCEM_PATH_STICKY;
+    }
+    if (a.ckey && gl == 0) a.ckey[u] = lkey;
+    PathRec& rec = a.prec[u];
+    d3* xs = reinterpret_cast<d3*>(a.vpts) + (size_t)u * (kMaxRefl + 2);
+    // ---- the previous frame's record, when nothing it depends on moved (vc_reusable, shared out)
+    if (reuse && lkey) {
+      const int pu = vc_find(a, lkey);
+      if (pu >= 0) {
+        const int ps = a.prev_vstate[pu];
+        const d3* src = reinterpret_cast<const d3*>(a.prev_vpts) + (size_t)pu * (kMaxRefl + 2);
+        bool same = !a.rx_moved[rxi % a.nrx];
+        for (int j = gl; j < k && same; j += kFieldLanes) {
+          const int o = a.tri_obj[S.ids[j] & ~(kTransBit | kDiffBit)];
+          same = !(o >= 0 && a.obj_moved[o]);
+        }
+        if (ps != 0)  // (invalid geometry depends on nothing else)
+          for (int j = gl; j <= k && same; j += kFieldLanes) {
+            const d3 p0 = src[j], dv = src[j + 1] - p0;
+            const RayPre rp =
+                ray_pre(f3((float)p0.x, (float)p0.y, (float)p0.z), f3((float)dv.x, (float)dv.y, (float)dv.z));
+            same = !seg_hits_tree(a.mvt, rp, 1.0f, st);
+          }
+        if (__all_sync(gmask, same)) {
+          const bool valid = ps == 1 || ps == 3;
+          if (ps != 0)
+            for (int j = gl; j <= k + 1; j += kFieldLanes) xs[j] = src[j];
+          const int* from = reinterpret_cast<const int*>(&a.prev_prec[pu]);
+          int* to = reinterpret_cast<int*>(&rec);
+          static_assert(sizeof(PathRec) % sizeof(int) == 0, "record copied by words");
+          for (int w = gl; w < (int)(sizeof(PathRec) / sizeof(int)); w += kFieldLanes) to[w] = from[w];
+          __syncwarp(gmask);
+          if (gl == 0) {
+            rec.ray = ray;  // this frame's representative
+            a.vstate[u] = valid ? 3 : ps;  // 3: valid, reused
+            if (valid) {
+              unsigned pos = atomicAdd(&a.bucket_cnt[rxi], 1u);
+              if (pos < (unsigned)a.bucket_cap) a.bucket[(size_t)rxi * a.bucket_cap + pos] = (int)u;
+              else atomicOr(&a.ctr->err, ERR_BUCKET_OVERFLOW);
+              atomicAdd(&a.ctr->n_valid, 1u);
+            }
+            atomicAdd(&a.ctr->n_val_reused, 1u);
+          }
+          continue;
+        }
+      }
+    }
+    // ---- geometry
+    const float4 rxv = a.rx[rxi % a.nrx], txv = a.txs[rxi / a.nrx];
+    bool ok = true;
+    for (int j = gl; j < k; j += kFieldLanes) {
+      v3<T> v0, v1, v2, n;
+      ok = val_triangle(a, S.ids[j], v0, v1, v2, n) && ok;
+      S.v0[j] = v0;
+      S.v1[j] = v1;
+      S.v2[j] = v2;
+      S.n[j] = n;
+      S.nn[j] = vdot(n, n);
+    }
+    ok = __all_sync(gmask, ok);
+    if (ok && gl == 0) {
+      S.X[0] = vof<T>(txv.x, txv.y, txv.z);
+      S.X[k + 1] = vof<T>(rxv.x, rxv.y, rxv.z);
+      // images of the transmitter, by interaction (a transmission keeps the last)
+      v3<T> I = S.X[0];
+      for (int j = 0; j < k; ++j) {
+        if (!(S.ids[j] & kTransBit)) I = val_image(I, S.v0[j], S.n[j], S.nn[j]);
+        S.img[j + 1] = I;
+      }
+      // reflection points, from the receiver back
+      v3<T> Y = S.X[k + 1];
+      T sp;
+      for (int j = k - 1; j >= 0 && ok; --j) {
+        if (S.ids[j] & kTransBit) continue;
+        v3<T> P;
+        ok = val_cross(Y, S.img[j + 1], S.v0[j], S.n[j], sc_of<T>(0.0f), sp, P);
+        S.X[j + 1] = Y = P;
+      }
+      // transmissions cross the straight piece between the surrounding
+      // reflection points, each after the previous one of its piece
+      v3<T> A = S.X[0];
+      T s_prev = sc_of<T>(0.0f);
+      for (int j = 0; j < k && ok; ++j) {
+        if (!(S.ids[j] & kTransBit)) {
+          A = S.X[j + 1];
+          s_prev = sc_of<T>(0.0f);
+          continue;
+        }
+        int e = j + 1;  // the piece's end: the next reflection, or the receiver
+        while (e < k && (S.ids[e] & kTransBit)) ++e;
+        ok = val_cross(A, S.X[e + 1], S.v0[j], S.n[j], s_prev, sp, S.X[j + 1]);
+        s_prev = sp;
+      }
+    }
+    ok = __shfl_sync(gmask, (int)ok, 0, kFieldLanes) != 0;
+    T L = sc_of<T>(0.0f);
+    if (ok) {
+      __syncwarp(gmask);
+      for (int j = gl; j < k; j += kFieldLanes) ok = val_inside(S.v0[j], S.v1[j], S.v2[j], S.n[j], S.X[j + 1]) && ok;
+      for (int j = gl; j <= k; j += kFieldLanes) {
+        const v3<T> e = S.X[j + 1] - S.X[j];
+        S.leg[j] = root(vdot(e, e));
+      }
+      for (int j = gl; j <= k + 1; j += kFieldLanes)
+        S.P[j] = mk3(to_d(S.X[j].x), to_d(S.X[j].y), to_d(S.X[j].z));
+      ok = __all_sync(gmask, ok);
+      __syncwarp(gmask);
+      for (int j = 0; j <= k; ++j) L = L + S.leg[j];
+      ok = ok && pos(L);
+    }
+    int state = ok ? 1 : 0;  // 0: no geometry, 1: valid, 2: occluded
+    if (ok) {
+      for (int j = gl; j <= k + 1; j += kFieldLanes) xs[j] = S.P[j];
+      // ---- occlusion: the legs
+      bool hit = false;
+      for (int j = gl; j <= k; j += kFieldLanes) {
+        const d3 p0 = S.P[j], dv = S.P[j + 1] - p0;
+        const RayPre rp = ray_pre(f3((float)p0.x, (float)p0.y, (float)p0.z), f3((float)dv.x, (float)dv.y, (float)dv.z));
+        const int ex0 = j >= 1 ? S.ids[j - 1] & ~kTransBit : -1, ex1 = j < k ? S.ids[j] & ~kTransBit : -1;
+        hit = any_hit(a.bvh, rp, a.eps_occ, 1.0f - a.eps_occ, ex0, ex1, ovf, st) || hit;
+      }
+      if (__any_sync(gmask, hit)) state = 2;
+    }
+    // ---- the record, and the field of a valid path
+    const double len = ok ? to_d(L) : 0.0;
+    for (int j = gl; j < kMaxRefl; j += kFieldLanes) {
+      rec.tri[j] = S.ids[j];
+      rec.pts[j][0] = rec.pts[j][1] = rec.pts[j][2] = 0.0f;
+    }
+    if (gl == 0) {
+      rec.key = key;
+      rec.rx = rxi;
+      rec.depth = k;
+      rec.ray = ray;
+      rec.flags = fl0;
+      rec.valid = 0;
+      rec.pad = 0;
+      rec.len = len;
+      rec.amp_re = rec.amp_im = 0.0;
+      a.vstate[u] = state;
+    }
+    if (state != 1) continue;
+    for (int j = 1 + gl; j <= k; j += kFieldLanes) bounce_coef(a, S.P, S.ids[j - 1], j, wfac, S.coef[j - 1]);
+    // the ends, on lanes that hold no bounce of a path of up to 5 bounces
+    if (gl == kFieldLanes - 1) {
+      unsigned f = 0;
+      d3 e0 = pol_of(upol, dir_of(S.P[0], S.P[1]), f);
+      S.ends.e0[0] = e0.x; S.ends.e0[1] = e0.y; S.ends.e0[2] = e0.z;
+      S.ends.fl0 = f;
+    } else if (gl == kFieldLanes - 2) {
+      unsigned f = 0;
+      d3 prx = pol_of(upol, dir_of(S.P[k + 1], S.P[k]), f);
+      S.ends.prx[0] = prx.x; S.ends.prx[1] = prx.y; S.ends.prx[2] = prx.z;
+      S.ends.fl1 = f;
+    } else if (gl == kFieldLanes - 3) {
+      path_phase(a.freq, len, &S.ends.sn, &S.ends.cs);
+    }
+    __syncwarp(gmask);
+    if (gl == 0) {
+      z3 E = {Z(S.ends.e0[0]), Z(S.ends.e0[1]), Z(S.ends.e0[2])};
+      for (int j = 0; j < k; ++j) bounce_field(S.coef[j], E);
+      field_done(a, rec, S.P, u, E, mk3(S.ends.prx[0], S.ends.prx[1], S.ends.prx[2]), S.ends.sn, S.ends.cs,
+                 S.ends.fl0 | S.ends.fl1);
+    }
+  }
+  if (ovf) {
+    atomicAdd(&a.ctr->stack_overflow, 1u);
+    atomicOr(&a.ctr->err, ERR_STACK);
   }
 }
 
@@ -4574,13 +4830,19 @@ cudaError_t launch_sticky_probe(const PathArgs& a, int grid, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_validate(const PathArgs& a, int grid, cudaStream_t st) {
+cudaError_t launch_validate(const PathArgs& a, int nlinks, int grid, cudaStream_t st) {
+  const size_t osm = 64 * kStackTrace * sizeof(int);
+  if (nlinks <= kFewLinks) {
+    if (a.prec_df) k_validate<df><<<grid, kFieldThreads, osm, st>>>(a);
+    else k_validate<double><<<grid, kFieldThreads, osm, st>>>(a);
+    return cudaGetLastError();
+  }
   const size_t gsm = 64 * kStackSmall * sizeof(int);
   if (a.prec_df) k_val_geom<df><<<4 * grid, 64, gsm, st>>>(a);
   else k_val_geom<double><<<4 * grid, 64, gsm, st>>>(a);
   // (key, sub-segment) items: one or two lanes of every warp while they are
   // few, so that a warp waits for few different traversals
-  k_val_occ<<<4 * grid, 64, 64 * kStackTrace * sizeof(int), st>>>(a);
+  k_val_occ<<<4 * grid, 64, osm, st>>>(a);
   k_val_field<<<4 * grid, kFieldThreads, 0, st>>>(a);
   return cudaGetLastError();
 }

@@ -132,7 +132,11 @@ cudaError_t launch_dedupe(const PathArgs& a, int grid, cudaStream_t st);
 // Sticky mode: the previous frame's valid paths whose key no capture of this
 // frame has join the distinct keys (validated like them).
 cudaError_t launch_sticky_probe(const PathArgs& a, int grid, cudaStream_t st);
-cudaError_t launch_validate(const PathArgs& a, int grid, cudaStream_t st);
+// Frames of at most kFewLinks links validate in one kernel, a group of lanes
+// per key (a few hundred keys: latency); more links in three (tens of thousands
+// of keys: throughput).
+constexpr int kFewLinks = 1024;
+cudaError_t launch_validate(const PathArgs& a, int nlinks, int grid, cudaStream_t st);
 // The table of this frame's distinct keys for the next frame's validation
 // reuse (after validation, before diffraction adds its records).
 cudaError_t launch_vcache_build(const PathArgs& a, int grid, cudaStream_t st);
