@@ -154,7 +154,9 @@ __device__ __forceinline__ d3 dx(d3 a, d3 b) {
   return mk3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
 }
 __device__ __forceinline__ double dn(d3 a) { return sqrt(dd(a, a)); }
-__device__ __forceinline__ d3 du(d3 a) { return a * (1.0 / dn(a)); }
+// (a reciprocal square root is one chain of dependent operations, a square
+// root and a division are two; both are within an ulp or two)
+__device__ __forceinline__ d3 du(d3 a) { return a * rsqrt(dd(a, a)); }
 
 // Double-float numbers (hi + lo, two FP32 values, about 44 significant
 // bits): the validation geometry in this precision runs on the FP32 pipe.
@@ -222,6 +224,7 @@ struct v3 {
 template <class T> __device__ __forceinline__ v3<T> operator+(v3<T> a, v3<T> b) { return {a.x + b.x, a.y + b.y, a.z + b.z}; }
 template <class T> __device__ __forceinline__ v3<T> operator-(v3<T> a, v3<T> b) { return {a.x - b.x, a.y - b.y, a.z - b.z}; }
 template <class T> __device__ __forceinline__ v3<T> scale(v3<T> a, T s) { return {a.x * s, a.y * s, a.z * s}; }
+// (not fused: path lengths stay equal to those of a plain FP64 evaluation)
 template <class T> __device__ __forceinline__ T vdot(v3<T> a, v3<T> b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 template <class T> __device__ __forceinline__ v3<T> vcross(v3<T> a, v3<T> b) {
   return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
@@ -243,16 +246,18 @@ __device__ __forceinline__ zd operator*(zd a, zd b) {
 }
 __device__ __forceinline__ zd operator*(zd a, double s) { return Z(a.re * s, a.im * s); }
 __device__ __forceinline__ zd zdiv(zd a, zd b) {
-  double d = b.re * b.re + b.im * b.im;
-  return Z((a.re * b.re + a.im * b.im) / d, (a.im * b.re - a.re * b.im) / d);
+  const double r = 1.0 / fma(b.re, b.re, b.im * b.im);
+  return Z(fma(a.re, b.re, a.im * b.im) * r, fma(a.im, b.re, -(a.re * b.im)) * r);
 }
 __device__ __forceinline__ zd zexp(zd a) {
   double m = exp(a.re), sn, cs;
   sincos(a.im, &sn, &cs);
   return Z(m * cs, m * sn);
 }
-__device__ __forceinline__ zd zsqrt(zd a) {  // principal branch
-  double r = hypot(a.re, a.im);
+// principal branch (the squares cannot overflow: a permittivity from FP32
+// material constants)
+__device__ __forceinline__ zd zsqrt(zd a) {
+  double r = sqrt(fma(a.re, a.re, a.im * a.im));
   double x = sqrt(0.5 * (r + fabs(a.re)));
   if (x == 0.0) return Z(0.0, 0.0);
   double y = a.im / (2.0 * x);
@@ -272,14 +277,14 @@ __device__ __forceinline__ d3 dir_of(d3 a, d3 b) { return du(b - a); }  // unit 
 // (a fixed axis instead when u is along d; the path is then flagged).
 __device__ __forceinline__ d3 pol_of(d3 u, d3 d, unsigned& flags) {
   d3 p = u - d * dd(u, d);
-  double n = dn(p);
-  if (n < 1e-9) {
+  double n2 = dd(p, p);
+  if (n2 < 1e-18) {
     flags |= DCEM_PATH_POL_DEGENERATE;
     d3 ax = fabs(d.x) < 0.9 ? mk3(1, 0, 0) : mk3(0, 1, 0);
     p = ax - d * dd(ax, d);
-    n = dn(p);
+    n2 = dd(p, p);
   }
-  return p * (1.0 / n);
+  return p * rsqrt(n2);
 }
 
 // ---------------------------------------------------------------------------
@@ -356,7 +361,9 @@ __device__ __forceinline__ bool val_triangle(const PathArgs& a, int id, v3<T>& v
   const bool opaque = (id & kTransBit) && !(a.mats[__float_as_int(p1.w)].w >= 0.0f);
   return !opaque && pos(vdot(n, n));
 }
-// step 3: the image of I in the plane of (v0, n), nn = n.n
+// step 3: the image of I in the plane of (v0, n), nn = n.n (2 / nn formed
+// beside the normals would take the division off the chain of images, but its
+// rounding reaches the path length: three times the phase error)
 template <class T>
 __device__ __forceinline__ v3<T> val_image(v3<T> I, v3<T> v0, v3<T> n, T nn) {
   return I - scale(n, sc_of<T>(2.0f) * vdot(I - v0, n) / nn);
@@ -597,12 +604,12 @@ __device__ __forceinline__ void bounce_coef(const PathArgs& a, const d3* X, int 
   d3 nh = du(dx(mk3(p1.x, p1.y, p1.z) - q0, mk3(p2.x, p2.y, p2.z) - q0));
   double ct = fabs(dd(din, nh));
   d3 sv = dx(din, nh);
-  double sn = dn(sv);
-  if (sn < 1e-12) {  // normal incidence: any unit vector perpendicular to n
+  double sn2 = dd(sv, sv);
+  if (sn2 < 1e-24) {  // normal incidence: any unit vector perpendicular to n
     d3 ax = fabs(nh.x) < 0.9 ? mk3(1, 0, 0) : mk3(0, 1, 0);
     sv = du(dx(nh, ax));
   } else {
-    sv = sv * (1.0 / sn);
+    sv = sv * rsqrt(sn2);
   }
   d3 pin = dx(sv, din), pout = dx(sv, dout);
   zd gte, gtm;
@@ -1176,7 +1183,7 @@ __device__ __forceinline__ double dotw(d3w a, d3w b) { return fma(a.z, b.z, fma(
 __device__ __forceinline__ d3w crossw(d3w a, d3w b) {
   return D3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
 }
-__device__ __forceinline__ d3w unitw(d3w a) { return a * (1.0 / sqrt(dotw(a, a))); }
+__device__ __forceinline__ d3w unitw(d3w a) { return a * rsqrt(dotw(a, a)); }
 __device__ __forceinline__ d3w polw(d3w u, d3w d, unsigned& fl) {
   d3w p = u - d * dotw(u, d);
   double n = sqrt(dotw(p, p));
