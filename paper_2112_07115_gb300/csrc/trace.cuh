@@ -35,7 +35,7 @@ struct TraceArgs {
   int use_q;               // closest-hit kernel: 0 binary nodes (k_trace), 1 the 4-wide compact
                            // copy from shared memory (k_trace_q), 2 from global memory (k_trace_qg)
   int stack_cap;           // shared-memory stack entries per thread
-  int block;               // threads per CTA of kernels 0 and 2 (kernel 1: kTraceQThreads)
+  int block;               // threads per CTA of kernels 0 and 2 (kernel 1: up to kTraceQThreads)
   float4* log_o;           // (N+1) x R: origin, unfolded length D
   float4* log_d;           // (N+1) x R: direction, hit t (+inf escaped)
   int* log_id;             // (N+1) x R: hit triangle id or -1
