@@ -33,8 +33,6 @@ enum : unsigned { NA_ERR_RX_RANGE = 1u, NA_ERR_PER_RX = 2u };
 struct NaScratch {
   unsigned count[kNaMaxRx];    // paths per receiver
   unsigned offset[kNaMaxRx];   // exclusive prefix sum of count
-  unsigned err;                // error bits of the current call
-  unsigned pad[63];
   int order[kNaMaxPaths];      // path indices grouped by receiver
 };
 
@@ -47,17 +45,17 @@ static __device__ __align__(256) NaScratch g_na_scratch;
 // the receivers of its eighth of the records in shared memory (a record's
 // rank among them stays in a register), each then scans its eighth of the
 // receivers over the eight counts, and places its records: 9 us for 16,384
-// records and 1024 receivers. As four kernels
-// with counters in device memory (clear, count, scan, place) it was 13 us
-// and three launches more; one CTA alone (25 us) reads the records' receiver
-// numbers, 128 bytes apart or more, at one SM's rate.
+// records and 1024 receivers. As four kernels with counters in device memory
+// (clear, count, scan, place) it was 13 us and three launches more; one CTA
+// alone (25 us) reads the records' receiver numbers, 192 bytes apart, at one
+// SM's rate.
 constexpr int kNaCluster = 8, kNaGroupThreads = 1024;
 constexpr int kNaPerThread = kNaMaxPaths / (kNaCluster * kNaGroupThreads);
 constexpr int kNaSlice = kNaMaxRx / kNaCluster;
 static_assert(kNaSlice <= kNaGroupThreads, "one receiver of the slice per thread");
 
 __global__ void __cluster_dims__(kNaCluster, 1, 1) __launch_bounds__(kNaGroupThreads)
-    k_na_group(NaScratch* s, const dcem_path* __restrict__ p, int n, int nrx) {
+    k_na_group(NaScratch* s, unsigned* err, const dcem_path* __restrict__ p, int n, int nrx) {
   __shared__ unsigned cnt[kNaMaxRx];          // paths per receiver, then their first places
   __shared__ unsigned total[kNaCluster], errs[kNaCluster], part[32];
   cg::cluster_group cl = cg::this_cluster();
@@ -126,7 +124,7 @@ __global__ void __cluster_dims__(kNaCluster, 1, 1) __launch_bounds__(kNaGroupThr
   if (me == 0 && tid == 0) {
     unsigned e = 0;
     for (int c = 0; c < kNaCluster; ++c) e |= errs[c];
-    s->err = e;
+    *err = e;
   }
 }
 
@@ -261,6 +259,7 @@ __global__ void __launch_bounds__(kNaThreads) k_na_reduce(const NaScratch* s, co
 // Per-device address of g_na_scratch, looked up once per device.
 std::mutex g_na_mutex;
 NaScratch* g_na_addr[kNaMaxDevices] = {};
+unsigned* g_na_err[kNaMaxDevices] = {};   // error bits of the current call, in mapped host memory
 bool g_na_attr[kNaMaxDevices] = {};
 
 int na_status(cudaError_t e) {
@@ -283,6 +282,7 @@ extern "C" int dcem_reduce_paths_noalloc(const dcem_path* paths, int32_t n_paths
   if (e != cudaSuccess) return na_status(e);
   if (dev < 0 || dev >= kNaMaxDevices) return DCEM_ERR_CUDA;
   NaScratch* s = nullptr;
+  unsigned *err = nullptr, *err_d = nullptr;
   {
     std::lock_guard<std::mutex> lock(g_na_mutex);
     if (!g_na_addr[dev]) {
@@ -291,6 +291,12 @@ extern "C" int dcem_reduce_paths_noalloc(const dcem_path* paths, int32_t n_paths
       e = cudaGetSymbolAddress(&ptr, g_na_scratch);
       if (e != cudaSuccess) return na_status(e);
       g_na_addr[dev] = static_cast<NaScratch*>(ptr);
+    }
+    if (!g_na_err[dev]) {
+      void* ptr = nullptr;
+      e = cudaHostAlloc(&ptr, 64, cudaHostAllocMapped);
+      if (e != cudaSuccess) return na_status(e);
+      g_na_err[dev] = static_cast<unsigned*>(ptr);
     }
     if (!g_na_attr[dev]) {
       size_t smem = (size_t)kNaMaxPerRx * (sizeof(unsigned long long) + sizeof(int));
@@ -304,10 +310,15 @@ extern "C" int dcem_reduce_paths_noalloc(const dcem_path* paths, int32_t n_paths
       g_na_attr[dev] = true;
     }
     s = g_na_addr[dev];
+    err = g_na_err[dev];
+    void* ptr = nullptr;
+    e = cudaHostGetDevicePointer(&ptr, err, 0);
+    if (e != cudaSuccess) return na_status(e);
+    err_d = static_cast<unsigned*>(ptr);
   }
   if (nrx == 0) return DCEM_OK;  // the set-up call
   cudaStream_t st = (cudaStream_t)stream;
-  k_na_group<<<kNaCluster, kNaGroupThreads, 0, st>>>(s, paths, n_paths, nrx);
+  k_na_group<<<kNaCluster, kNaGroupThreads, 0, st>>>(s, err_d, paths, n_paths, nrx);
   // receivers per CTA: enough CTAs for every SM (four fit by shared memory),
   // no more than a warp each
   const int per = std::min(kNaWarps, (nrx + 511) / 512);
@@ -316,11 +327,11 @@ extern "C" int dcem_reduce_paths_noalloc(const dcem_path* paths, int32_t n_paths
                                                               p_inc_dbm);
   e = cudaGetLastError();
   if (e != cudaSuccess) return na_status(e);
-  unsigned err = 0;
-  e = cudaMemcpyAsync(&err, &s->err, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  // the error bits come with the end of the kernels, without a copy of their own
+  e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return na_status(e);
-  if (err & NA_ERR_RX_RANGE) return DCEM_ERR_ARG;
-  if (err & NA_ERR_PER_RX) return DCEM_ERR_CAPACITY;
+  const unsigned bits = *static_cast<volatile unsigned*>(err);
+  if (bits & NA_ERR_RX_RANGE) return DCEM_ERR_ARG;
+  if (bits & NA_ERR_PER_RX) return DCEM_ERR_CAPACITY;
   return DCEM_OK;
 }

@@ -4605,7 +4605,7 @@ __device__ __forceinline__ void write_path(const PathArgs& a, const PathRec& p, 
   q.delay_s = p.len / 299792458.0;
   q.amp_re = p.amp_re;
   q.amp_im = p.amp_im;
-  a.pout[o] = q;
+  (o < a.hrec_cap ? a.hrec : a.pout)[o] = q;
 }
 // A link's sums as field and powers: thread k of the first half of 2 n
 // threads takes link r0 + k's field and coherent power, of the second half

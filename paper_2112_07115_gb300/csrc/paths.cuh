@@ -30,6 +30,8 @@ struct PathArgs {
   unsigned* link_off;             // groups of links: their paths, or their output offsets (many links); or null
   dcem_path* pout;                // ordered output (link, key): caller's device buffer or staging
   unsigned pout_cap;
+  dcem_path* hrec;                // first hrec_cap records: mapped host memory in place of pout
+  unsigned hrec_cap;
   double* out_field;              // links x 2 (re, im), or null
   double* out_pc;                 // links P_coh dBm, or null
   double* out_pi;                 // links P_inc dBm, or null
