@@ -58,6 +58,13 @@ __device__ __forceinline__ int fetch_warp(unsigned* counter, unsigned n) {
   return __shfl_sync(0xffffffffu, base, 0);
 }
 
+// The ray slot at place q of the order in which rays are taken: chunks of 32
+// slots (so that a warp still takes rays close in direction), those first
+// whose rays stay longest in the scene.
+__device__ __forceinline__ int ray_at(const TraceArgs& a, int q) {
+  return __ldg(&a.ray_order[DCEM_IDX(q >> 5, (a.R + 31) >> 5)]) * 32 + (q & 31);
+}
+
 // Persistent traversal with a per-lane ray fetch: every lane traces one
 // segment of its own ray per step, and a lane whose ray has ended takes the
 // next ray of the queue at once (one atomic per warp for all such lanes), so
@@ -123,7 +130,7 @@ __device__ __forceinline__ void trace_rays(const TraceArgs& a, const uint4* qn, 
             ntr = (inf >> 4) & 15;
             set = inf >> 8;
           } else {
-            ray = a.queue ? a.queue[DCEM_IDX(q, R)] : q;
+            ray = a.queue ? a.queue[DCEM_IDX(q, R)] : ray_at(a, q);
             b = a.queue ? a.restart[DCEM_IDX(ray, R)] : 0;
             nr = b;
             ntr = 0;
@@ -318,7 +325,7 @@ __global__ void __launch_bounds__(256, 3) k_trace_batch(const TraceArgs* __restr
       const unsigned need = __ballot_sync(0xffffffffu, ray < 0);
       const unsigned q = next + __popc(need & ((1u << lane) - 1u));
       if (ray < 0 && q < end) {
-        ray = a.queue ? a.queue[DCEM_IDX((int)q, R)] : (int)q;
+        ray = a.queue ? a.queue[DCEM_IDX((int)q, R)] : ray_at(a, (int)q);
         b = a.queue ? a.restart[DCEM_IDX(ray, R)] : 0;
         if (b == 0) {
           float4 rd = __ldg(&a.rays[DCEM_IDX(ray, R)]);
@@ -528,8 +535,7 @@ __global__ void __launch_bounds__(256) k_mark(TraceArgs a, CoherentArgs c) {
   constexpr int kPre = 5;  // segments held in registers (later ones are loaded when tested)
   const long nwarps = (long)((gridDim.x * blockDim.x) >> 5);
   for (long b0 = (long)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; b0 < R; b0 += 32 * nwarps) {
-    const int base = (int)b0;
-    const int ray = base + lane;
+    const int ray = ray_at(a, (int)b0) + lane;  // the retrace queue keeps the order, too
     const bool in = ray < R;
     float4 plo[kPre], pld[kPre];
 #pragma unroll

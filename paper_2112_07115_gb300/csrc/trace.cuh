@@ -10,6 +10,7 @@ struct TraceArgs {
   const float4* rays;      // R unit directions (xyz), .w = the ray's set (int bits)
   const float4* txs;       // per ray set: transmitter position (xyz) and the
                            // effective capture spacing alpha_t / sqrt(3) (w)
+  const int* ray_order;    // order in which chunks of 32 ray slots are taken (ray_at)
   int nsets;
   int R, N;                // rays, reflections
   int LS;                  // segment-log stride: R, plus the child slots with transmission
