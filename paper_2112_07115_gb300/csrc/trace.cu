@@ -452,46 +452,110 @@ __device__ __forceinline__ char* stage_receivers(const TraceArgs& a, char* p, co
   return stage_tree(a.rxt, max(a.nrx - 1, 0), a.nrx, reinterpret_cast<char*>(srx + a.nrx), rxt);
 }
 
+// A segment of the capture list as its thread holds it.
+struct CapSeg {
+  unsigned it;             // list entry, or kNoSeg
+  float4 lo, ld;
+  int set;                 // the ray's set (a transmission child: its parent's)
+};
+constexpr unsigned kNoSeg = 0xffffffffu;
+
+__device__ __forceinline__ unsigned cap_entry(const TraceArgs& a, unsigned base, unsigned total) {
+  const unsigned q = base + (threadIdx.x & 31);
+  return q < total ? a.capitems[DCEM_IDX(q, capitems_cap(a))] : kNoSeg;
+}
+__device__ __forceinline__ CapSeg cap_load(const TraceArgs& a, unsigned it) {
+  CapSeg s;
+  s.it = it;
+  s.lo = s.ld = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  s.set = 0;
+  if (it != kNoSeg) {
+    const int ray = (int)((it & 0x7fffffffu) >> 4), b = (int)(it & 15u);
+    s.lo = a.log_o[log_at(a, b, ray)];
+    s.ld = a.log_d[log_at(a, b, ray)];
+    if (ray >= a.R) s.set = a.inst[DCEM_IDX(ray - a.R, a.child_cap)] >> 8;
+    else if (a.nsets > 1) s.set = __float_as_int(__ldg(reinterpret_cast<const float*>(a.rays) + 4 * (size_t)ray + 3));
+  }
+  return s;
+}
+
+// The kernel is bound by memory round trips (the list, the log records it
+// points to, the work counter), so a warp has three batches of 32 segments
+// under way: while one is tested, the next one's records, the entries of the
+// one after it and the place of the one after that are being fetched, and
+// captures are collected per warp in shared memory and go to the candidate
+// list 32 or more at a time (one at a time, every capture held its warp up
+// for a round trip to the list's counter).
+constexpr int kCapWarps = 256 / 32;
+constexpr unsigned kCapOut = 96;
+
 template <bool kS>
 __global__ void __launch_bounds__(256) k_capture(TraceArgs a) {
   extern __shared__ __align__(16) int sstk[];
+  __shared__ Cand out[kCapWarps][kCapOut];
+  __shared__ unsigned n_out[kCapWarps];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (lane == 0) n_out[wid] = 0u;
+  __syncwarp();
   TStack st;
   bind_stack(st, sstk, kStackSmall);
   SmallBvh rxt = a.rxt;
   const float4* rx = a.rx;
+  const unsigned total = min(a.ctr->n_capitems, (unsigned)a.LS * (unsigned)(a.N + a.max_trans + 1));
+  // the first three batches by place, so that a short list takes all warps
+  const unsigned round = gridDim.x * blockDim.x;
+  unsigned here = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u, next = here + round, then = next + round;
+  CapSeg cur = cap_load(a, cap_entry(a, here, total));
+  unsigned entry = cap_entry(a, next, total);
   if (kS) {
     stage_receivers(a, reinterpret_cast<char*>(sstk + blockDim.x * kStackSmall), rx, rxt);
     __syncthreads();
   }
-  const int R = a.R, LS = a.LS;
-  const unsigned total = min(a.ctr->n_capitems, (unsigned)LS * (unsigned)(a.N + a.max_trans + 1));
+  auto flush = [&](unsigned n) {
+    n = min(n, kCapOut);
+    unsigned at = 0;
+    if (lane == 0) at = atomicAdd(&a.ctr->n_cand, n);
+    at = __shfl_sync(0xffffffffu, at, 0);
+    for (unsigned k = lane; k < n; k += 32) {
+      if (at + k < a.cand_cap) a.cand[at + k] = out[wid][k];
+      else atomicOr(&a.ctr->err, ERR_CAND_OVERFLOW);
+    }
+    __syncwarp();
+    if (lane == 0) n_out[wid] = 0u;
+    __syncwarp();
+  };
   unsigned ovf = 0;
-  for (;;) {
-    int base = fetch_warp(&a.ctr->work_capture, 32u);
-    if ((unsigned)base >= total) break;
-    unsigned q = (unsigned)base + (threadIdx.x & 31);
-    if (q < total) {
-      unsigned it = a.capitems[q];
-      bool reused = (it & 0x80000000u) != 0u;
-      int ray = (int)((it & 0x7fffffffu) >> 4), b = (int)(it & 15u);
-      float4 lo = a.log_o[log_at(a, b, ray)], ld = a.log_d[log_at(a, b, ray)];
-      float3 o = f3(lo.x, lo.y, lo.z), d = f3(ld.x, ld.y, ld.z);
-      float D = lo.w, t = ld.w;
-      float tend = isinf(t) ? a.escape : t;
-      // the ray's set: its capture spacing, and the link of its captures
-      // (a transmission child: its parent's)
-      int set = ray >= R ? (a.inst[DCEM_IDX(ray - R, a.child_cap)] >> 8)
-                         : a.nsets > 1 ? __float_as_int(__ldg(reinterpret_cast<const float*>(a.rays) + 4 * (size_t)ray + 3))
-                                       : 0;
-      float alpha = __ldg(&a.txs[DCEM_IDX(set, a.nsets)].w);
-      int link0 = set * a.nrx;
-      if (!capture_tree(rxt, rx, o, d, D, tend, alpha, st, [&](int r) {
-            if (!reused || a.rx_moved[r]) emit_cand(a, ray, b, link0 + r);
-          }))
+  while (here < total) {
+    unsigned more = 0;
+    if (lane == 0) more = 3 * round + atomicAdd(&a.ctr->work_capture, 32u);
+    const unsigned entry2 = cap_entry(a, then, total);
+    const CapSeg s = cur;
+    cur = cap_load(a, entry);
+    if (s.it != kNoSeg) {
+      const bool reused = (s.it & 0x80000000u) != 0u;
+      const int ray = (int)((s.it & 0x7fffffffu) >> 4), b = (int)(s.it & 15u);
+      const float tend = isinf(s.ld.w) ? a.escape : s.ld.w;
+      // the set's capture spacing, and the link of its captures
+      const float alpha = __ldg(&a.txs[DCEM_IDX(s.set, a.nsets)].w);
+      const int link0 = s.set * a.nrx;
+      if (!capture_tree(rxt, rx, f3(s.lo.x, s.lo.y, s.lo.z), f3(s.ld.x, s.ld.y, s.ld.z), s.lo.w, tend, alpha, st,
+                        [&](int r) {
+                          if (reused && !a.rx_moved[r]) return;
+                          const unsigned k = atomicAdd(&n_out[wid], 1u);
+                          if (k < kCapOut) out[wid][k] = Cand{ray, ((link0 + r) << 4) | b};
+                          else emit_cand(a, ray, b, link0 + r);
+                        }))
         ovf = 1u;
     }
     __syncwarp();
+    const unsigned held = n_out[wid];
+    if (held >= 32u) flush(held);
+    here = next;
+    next = then;
+    then = __shfl_sync(0xffffffffu, more, 0);
+    entry = entry2;
   }
+  if (n_out[wid]) flush(n_out[wid]);
   if (ovf) {
     atomicAdd(&a.ctr->stack_overflow, 1u);
     atomicOr(&a.ctr->err, ERR_STACK);
