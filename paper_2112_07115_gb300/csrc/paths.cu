@@ -4293,12 +4293,18 @@ __global__ void __launch_bounds__(64) k_diff_unblocked(PathArgs a, int nlinks) {
   // few candidates: a few lanes of every warp, so that all SMs share the
   // traversals' latency; many: full warps of consecutive candidates (which
   // come from one warp above, so their legs run close together)
+  // Up to 16 candidates an SM all go on: the exact stage takes them side by
+  // side and its time is one candidate's either way, while the longest of the
+  // legs here takes 50 us (1113 candidates on a highway, of which 472 would
+  // stay: 1016 us for two frames with the test, 935 without; 1643 in an 8 x 8
+  // city, of which 227 would stay: 638 and 640).
+  const bool all = n <= 2u * gridDim.x;
   const unsigned nwarp = gridDim.x * (blockDim.x >> 5), per = min(32u, max(1u, (n + nwarp - 1) / nwarp));
   for (unsigned i0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per; i0 < n; i0 += nwarp * per) {
     const unsigned i = i0 + lane;
     const bool mine = lane < (int)per && i < n;
     const unsigned long long code = mine ? a.dsurv[i] : 0ull;
-    const bool keep = mine && !diff_blocked(a, nlinks, code, st);
+    const bool keep = mine && (all || !diff_blocked(a, nlinks, code, st));
     const unsigned mk = __ballot_sync(0xffffffffu, keep);
     if (!mk) continue;
     unsigned at = 0;
