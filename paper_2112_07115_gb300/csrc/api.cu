@@ -693,7 +693,7 @@ static bool uses_vis(const dcem_scene* s) {
 // and the host copies them on once the frame has ended. With four
 // copies into pageable memory and a second synchronisation instead, a frame of
 // 8 links took 135 rather than 125 us, a coherent one 114 rather than 98; the
-// rest of a large frame's results still goes that way. 256 KB per scene, from
+// rest of a large frame's results still goes that way. 0.3 MB per scene, from
 // its first frame with host results on.
 constexpr unsigned kHostRecs = 1024;
 constexpr int kHostLinks = 2048;

@@ -884,49 +884,6 @@ __device__ __forceinline__ unsigned qenc_hi(float v, float o, float s) {
   return d < 0.0f ? 0u : (unsigned)d;
 }
 
-// Compact copy of both trees (layout and grid in dcem_internal.cuh): the
-// grid pads the union of the root boxes by 1 m + 1e-3 of its largest extent
-// on every side, so every box lies well inside it, with 65000 steps across
-// each padded axis.
-__global__ void k_quantize(const float4* __restrict__ nodes, int nn, const float* __restrict__ root_box,
-                           int has0, int has1, uint4* qn, float* qframe) {
-  float lo[3] = {3.4e38f, 3.4e38f, 3.4e38f}, hi[3] = {-3.4e38f, -3.4e38f, -3.4e38f};
-  for (int t = 0; t < 2; ++t) {
-    if (!(t == 0 ? has0 : has1)) continue;
-    for (int k = 0; k < 3; ++k) {
-      float a = root_box[6 * t + k], b = root_box[6 * t + 3 + k];
-      if (isfinite(a)) lo[k] = fminf(lo[k], a);
-      if (isfinite(b)) hi[k] = fmaxf(hi[k], b);
-    }
-  }
-  float ext = 0.0f;
-  for (int k = 0; k < 3; ++k) {
-    if (!(hi[k] >= lo[k])) { lo[k] = 0.0f; hi[k] = 0.0f; }
-    ext = fmaxf(ext, hi[k] - lo[k]);
-  }
-  float pad = 1.0f + 1e-3f * ext;
-  float o[3], sc[3];
-  for (int k = 0; k < 3; ++k) {
-    o[k] = lo[k] - pad;
-    sc[k] = fmaxf((hi[k] - lo[k] + 2.0f * pad) / 65000.0f, 1e-6f);
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0)
-    for (int k = 0; k < 3; ++k) { qframe[k] = o[k]; qframe[3 + k] = sc[k]; }
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += gridDim.x * blockDim.x) {
-    float4 n0 = nodes[4 * (size_t)i], n1 = nodes[4 * (size_t)i + 1], n2 = nodes[4 * (size_t)i + 2],
-           n3 = nodes[4 * (size_t)i + 3];
-    // child 0: lo (n0.x, n0.z, n2.x), hi (n0.y, n0.w, n2.y); child 1 likewise
-    unsigned w[6] = {qenc_lo(n0.x, o[0], sc[0]) | (qenc_hi(n0.y, o[0], sc[0]) << 16),
-                     qenc_lo(n0.z, o[1], sc[1]) | (qenc_hi(n0.w, o[1], sc[1]) << 16),
-                     qenc_lo(n2.x, o[2], sc[2]) | (qenc_hi(n2.y, o[2], sc[2]) << 16),
-                     qenc_lo(n1.x, o[0], sc[0]) | (qenc_hi(n1.y, o[0], sc[0]) << 16),
-                     qenc_lo(n1.z, o[1], sc[1]) | (qenc_hi(n1.w, o[1], sc[1]) << 16),
-                     qenc_lo(n2.z, o[2], sc[2]) | (qenc_hi(n2.w, o[2], sc[2]) << 16)};
-    qn[2 * (size_t)i] = make_uint4(w[0], w[1], w[2], w[3]);
-    qn[2 * (size_t)i + 1] = make_uint4(w[4], w[5], __float_as_uint(n3.x), __float_as_uint(n3.y));
-  }
-}
-
 // ---------------------------------------------------------------------------
 // 4-wide compact copy of both trees (layout in dcem_internal.cuh)
 // ---------------------------------------------------------------------------
@@ -1013,8 +970,11 @@ __device__ __forceinline__ unsigned qword(float lo, float hi, float o, float s) 
   return qenc_lo(lo, o, s) | (qenc_hi(hi, o, s) << 16);
 }
 
-// Per frame: the 4-wide compact nodes from the current binary child boxes,
-// on the grid of k_quantize (written to qframe by the first thread).
+// Per frame: the 4-wide compact nodes from the current binary child boxes.
+// The grid (dcem_internal.cuh; written to qframe by the first thread) pads
+// the union of the root boxes by 1 m + 1e-3 of its largest extent on every
+// side, so every box lies well inside it, with 65000 steps across each
+// padded axis.
 __global__ void k_quantize4(const float4* __restrict__ nodes, const int* __restrict__ n4p,
                             const int4* __restrict__ kid4, const int4* __restrict__ src4,
                             const float* __restrict__ root_box, int has0, int has1, uint4* q4, float* qframe) {
@@ -1180,14 +1140,6 @@ void launch_place_tris(const float* d_v9, const int* d_sel, const int* d_perm, c
   if (n > 0)
     k_place_tris<<<nblk(n, 256), 256, 0, st>>>(d_v9, d_sel, d_perm, d_tri_mat, d_tri_obj, n, leaf_base,
                                                d_tris, d_objv, d_slot_of_id);
-}
-
-void launch_quantize(const float4* d_nodes, int nn, const float* d_root_box, int has0, int has1, uint4* d_qn,
-                     float* d_qframe, cudaStream_t st) {
-  int g = (nn + 255) / 256;
-  if (g < 1) g = 1;
-  if (g > 1024) g = 1024;
-  k_quantize<<<g, 256, 0, st>>>(d_nodes, nn, d_root_box, has0, has1, d_qn, d_qframe);
 }
 
 

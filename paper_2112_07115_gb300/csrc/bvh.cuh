@@ -126,11 +126,6 @@ cudaError_t launch_dyn_update(const DynUpdateArgs& a, cudaStream_t st);
 // Shared memory the one-CTA update needs (must stay within 227 KB).
 size_t dyn_update_smem(int nd, int nobj);
 
-// Compact copy of the nn nodes of both trees (2 uint4 per node) and its
-// frame (origin.xyz, step.xyz), from the current node boxes and root boxes.
-void launch_quantize(const float4* d_nodes, int nn, const float* d_root_box, int has0, int has1, uint4* d_qn,
-                     float* d_qframe, cudaStream_t st);
-
 // 4-wide compact copy: map the binary trees (nn internal nodes, 2 root codes)
 // to 4-wide nodes once per topology (one CTA, nn <= 8192), then encode the
 // child boxes every frame. n4 and the 4-wide roots stay on the device.
@@ -144,7 +139,9 @@ cudaError_t launch_bvh4_map(const float4* d_nodes, int nn, const int* d_roots, i
                             int* d_n4, int* d_roots4, int* d_scratch, cudaStream_t st);
 void launch_quantize4(const float4* d_nodes, int n4_bound, const int* d_n4, const int4* d_kid4, const int4* d_src4,
                       const float* d_root_box, int has0, int has1, uint4* d_q4, float* d_qframe, cudaStream_t st);
-// At most (2 + 2 nn) / 3 internal nodes of two trees lie at even depth.
+// 4-wide nodes of two trees at most: one with a 4-wide child absorbs three
+// binary nodes and has at most four such children, the others absorb one or
+// more, so nn >= 3 i + l and l <= 3 i + 1 per tree.
 inline int bvh4_bound(int nn) { return (2 + 2 * nn) / 3; }
 
 // Per frame: world vertices of the moving triangles, per-object boxes and the

@@ -418,10 +418,9 @@ __device__ __forceinline__ int closest_hit(const Bvh& bvh, const RayPre& r, floa
 // ---------------------------------------------------------------------------
 // compact nodes for shared memory: child boxes as 16-bit codes on a per-frame
 // grid (origin O, step S_k on axis k) that contains both trees, rounded
-// outward by three steps, so a code box always contains the exact box. 32
-// bytes per node: words 0-2 = child 0 axes x, y, z, words 3-5 = child 1
-// axes, words 6-7 = child ids; each axis word holds the lo code in its low
-// half and the hi code in its high half.
+// outward by three steps, so a code box always contains the exact box. Each
+// box has one word per axis with the lo code in its low half and the hi code
+// in its high half.
 //
 // The slab test runs in grid units: with F = 2^23 + code (the float whose
 // bits are 0x4B00'code', built by one byte permute) the plane parameter is
@@ -499,68 +498,8 @@ static __device__ __noinline__ int closest_hit_far(const Bvh bvh, const RayPre r
   return slot;
 }
 
-// Closest hit as closest_hit(), with the nodes read from the compact copy
-// (shared memory). Same triangle test and tie rule, so the same result.
-__device__ __forceinline__ int closest_hit_q(const uint4* qn, const QFrame& f, const Bvh& bvh, const RayPre& r,
-                                             float tmin, int excl, float& t_best, int& id_best, unsigned& overflow,
-                                             unsigned& n_nodes, unsigned& n_tris, TStack& st) {
-  QRay q;
-  if (!qray_make(f, r, q))
-    return closest_hit_far(bvh, r, tmin, excl, &t_best, &id_best, &overflow, &n_nodes, &n_tris, st.s, st.stride,
-                           st.cap);
-  st.reset();
-  t_best = __int_as_float(0x7f800000);
-  id_best = 0x7fffffff;
-  int slot_best = -1;
-  if (bvh.root1 != kEmpty) st.push(bvh.root1);
-  int cur = bvh.root0;
-  if (cur == kEmpty) cur = st.empty() ? kEmpty : st.pop();
-  for (int visits = 0; cur != kEmpty; ++visits) {
-    if (visits > bvh.max_visits) {
-      overflow = 1u;
-      break;
-    }
-    if (cur >= 0) {
-      ++n_nodes;
-      const int ci = DCEM_IDX(cur, bvh.nnodes);
-      uint4 a = qn[2 * ci], b = qn[2 * ci + 1];
-      float tn0, tn1;
-      bool h0 = qslab(q, a.x, a.y, a.z, t_best, tn0);
-      bool h1 = qslab(q, a.w, b.x, b.y, t_best, tn1);
-      int c0 = (int)b.z, c1 = (int)b.w;
-      if (h0 && h1) {
-        int nearc = tn0 <= tn1 ? c0 : c1, farc = tn0 <= tn1 ? c1 : c0;
-        if (!st.push(farc)) overflow = 1u;
-        cur = nearc;
-      } else if (h0) {
-        cur = c0;
-      } else if (h1) {
-        cur = c1;
-      } else {
-        cur = st.empty() ? kEmpty : st.pop();
-      }
-    } else {
-      int slot = ~cur;
-      ++n_tris;
-      float3 v0, v1, v2;
-      int id;
-      load_tri(bvh.tris, DCEM_IDX(slot, bvh.ntris), v0, v1, v2, id);
-      float t;
-      if (id != excl && tri_hit(r, v0, v1, v2, t) && t > tmin) {
-        if (t < t_best || (t == t_best && id < id_best)) {
-          t_best = t;
-          id_best = id;
-          slot_best = slot;
-        }
-      }
-      cur = st.empty() ? kEmpty : st.pop();
-    }
-  }
-  return slot_best;
-}
-
 // 4-wide compact nodes (shared memory), 64 bytes each: words 0-11 = the axis
-// words of children 0-3 (x, y, z per child, as in the 2-wide copy), words
+// words of children 0-3 (x, y, z per child), words
 // 12-15 = the child codes (4-wide node index, leaf ~slot, or kEmpty with an
 // inverted box that no ray meets).
 //

@@ -47,7 +47,7 @@ static __device__ __align__(256) NaScratch g_na_scratch;
 // receivers over the eight counts, and places its records: 9 us for 16,384
 // records and 1024 receivers. As four kernels with counters in device memory
 // (clear, count, scan, place) it was 13 us and three launches more; one CTA
-// alone (25 us) reads the records' receiver numbers, 192 bytes apart, at one
+// alone (25 us) reads the records' receiver numbers, 224 bytes apart, at one
 // SM's rate.
 constexpr int kNaCluster = 8, kNaGroupThreads = 1024;
 constexpr int kNaPerThread = kNaMaxPaths / (kNaCluster * kNaGroupThreads);

@@ -13,7 +13,7 @@
 //           triangle of the sequence;
 //   step 4  path validation: the back-trace from the receiver through the
 //           images must cross each plane inside its triangle, and every
-//           sub-segment must be unoccluded (FP32 any-hit over the LBVH);
+//           sub-segment must be unoccluded (FP32 any-hit over the trees);
 //   step 6  per valid path: total length, delay, and the complex amplitude
 //           of the ray field (Eq. 1) with the free-space spreading of Eq. 3
 //           (exponent 2) and one Fresnel TE/TM reflection per bounce, with

@@ -2,7 +2,7 @@
 //
 // Sec. III "Backward ray tracing", steps 1-2: every ray of the sampled sphere
 // is traced from the transmitter through up to N specular reflections; each
-// segment's closest hit comes from a stack traversal of the two LBVH trees
+// segment's closest hit comes from a stack traversal of the two trees
 // (static scene, moving objects) with a watertight FP32 triangle test, and
 // each segment is tested against every receiver's reception sphere. Every
 // segment is logged (origin, direction, unfolded length, hit) so that the
@@ -49,13 +49,6 @@ __device__ __forceinline__ QFrame load_qframe(const TraceArgs& a) {
   f.sz = a.qframe[5];
   f.n4 = min(*a.q4_count, a.q4_bound);
   return f;
-}
-
-// Warp-wide dynamic work fetch: lane 0 takes the next `n` items.
-__device__ __forceinline__ int fetch_warp(unsigned* counter, unsigned n) {
-  int base = 0;
-  if ((threadIdx.x & 31) == 0) base = (int)atomicAdd(counter, n);
-  return __shfl_sync(0xffffffffu, base, 0);
 }
 
 // The ray slot at place q of the order in which rays are taken: chunks of 32
