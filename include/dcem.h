@@ -338,8 +338,9 @@ int dcem_scene_set_diffraction(dcem_scene* s, int32_t on, int32_t* n_wedges);
  * Fresnel reflection at P. Record: depth 2, tri = {P's triangle id,
  * wedge | DCEM_TRI_DIFFRACT} or {wedge | DCEM_TRI_DIFFRACT, triangle id},
  * pts = the two points in path order, ray = -1. on = 0 turns it off.
- * *n_planes (may be NULL): the reflector-plane count. Cost: one pre-test
- * thread per (link, wedge, plane, order) per frame. With diffraction chains
+ * *n_planes (may be NULL): the reflector-plane count. Cost: one warp per
+ * (transmitter or receiver, plane it sees) per frame, its lanes over the
+ * wedges, then the exact test per candidate. With diffraction chains
  * on (dcem_scene_set_diffraction_order, max_order m >= 2) the reflection also
  * comes before or after every chain of 2..m wedges: the chain from the
  * transmitter's image or toward the receiver's image in the plane (Keller
@@ -360,7 +361,9 @@ int dcem_scene_set_diffraction(dcem_scene* s, int32_t on, int32_t* n_wedges);
  * at each reflection in the real directions and the UTD coefficient over the
  * unfolded distances. Record: depth 3, tri = the two triangle ids and
  * wedge | DCEM_TRI_DIFFRACT in path order, pts = the three points. Cost: one
- * warp per (kind, link, plane pair) per frame, its lanes over the wedges.
+ * thread per (transmitter or receiver, plane, plane) per frame, a warp over
+ * the wedges for those within reach; with one reflection on each side, the
+ * transmitters' (plane, wedge) sides against the receivers'.
  * on = 3 adds, to on = 2 and with diffraction chains on (max_order >= 2), a
  * reflection between the two wedges of an order-2 chain: Tx -> Q1 -> P ->
  * Q2 -> Rx, by image theory the chain over the first wedge and the second

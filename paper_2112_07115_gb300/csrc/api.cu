@@ -160,11 +160,17 @@ __global__ void k_ray_keys(const float4* __restrict__ d, int n, unsigned* keys, 
 // million-ray highway's SMs had work for 258,000 of the kernel's 386,000
 // cycles on average (a frame 358 us, in this order 346). The last chunk may
 // be short and stays last.
-__global__ void k_chunk_keys(const float4* __restrict__ rays, int n, const float* __restrict__ box, unsigned* keys,
-                             unsigned* idx) {
+__global__ void k_chunk_keys(const float4* __restrict__ rays, int n, const float* __restrict__ box, int has0,
+                             int has1, unsigned* keys, unsigned* idx) {
   float e[3], diag = 0.0f;
-  for (int k = 0; k < 3; ++k) {  // static and moving triangles; an empty box is inverted
-    e[k] = fmaxf(fmaxf(box[3 + k], box[9 + k]) - fminf(box[k], box[6 + k]), 1e-6f);
+  for (int k = 0; k < 3; ++k) {  // static and moving triangles
+    float lo = 3.4e38f, hi = -3.4e38f;
+    for (int t = 0; t < 2; ++t) {
+      if (!(t == 0 ? has0 : has1)) continue;
+      lo = fminf(lo, box[6 * t + k]);
+      hi = fmaxf(hi, box[6 * t + 3 + k]);
+    }
+    e[k] = fmaxf(hi - lo, 1e-6f);
     diag += e[k] * e[k];
   }
   diag = sqrtf(diag);
@@ -1563,7 +1569,8 @@ int dcem_scene_set_ray_sets(dcem_scene* s, const float* dirs, const int32_t* n_r
       if (!e) {
         k_gather_rays<<<g, 256, 0, s->st>>>(src, v0, n, s->rays, s->ray_perm);
         const int nc = (n + 31) / 32;
-        k_chunk_keys<<<std::min((nc + 255) / 256, 1024), 256, 0, s->st>>>(s->rays, n, s->root_box, k0, v0);
+        const int gc = std::min((nc + 255) / 256, 1024);
+        k_chunk_keys<<<gc, 256, 0, s->st>>>(s->rays, n, s->root_box, s->ns > 0, s->nd > 0, k0, v0);
         e = sort_pairs_u32(k0, v0, k1, v1, hist, nc, 8, s->st);
         if (!e) e = cudaMemcpyAsync(s->ray_order, v0, sizeof(unsigned) * nc, cudaMemcpyDeviceToDevice, s->st);
       }
