@@ -2237,8 +2237,15 @@ __device__ __noinline__ bool surely_hidden(const PathArgs& a, const HiddenCase& 
 
 // Per end point the planes, then the wedges (in the order wperm) it may see,
 // one warp per word. A wedge the end point is inside of is not seen. Both
-// orders are spatial, so that a warp's legs run close together.
-__global__ void __launch_bounds__(64) k_diff_visible(PathArgs a, int ntx) {
+// orders are spatial, so that a warp's legs run close together. Without
+// `test` everything else counts as seen: scenes with few planes (a road and
+// its barriers) are open, and a highway's 480,000 legs of up to 2 km cost 240
+// us a frame and hid nothing.
+constexpr int kOpenPlanes = 16;
+// Neither do they pay for one reflection without chains, whose candidates are
+// cheap to form: 8 x 8 city blocks with 10, 30 and 60 receivers 542, 587 and
+// 648 us a frame with the tests, 365, 453 and 531 without.
+__global__ void __launch_bounds__(64) k_diff_visible(PathArgs a, int ntx, bool test) {
   extern __shared__ int sstk[];
   TStack st;
   bind_stack(st, sstk, kStackTrace);
@@ -2252,7 +2259,7 @@ __global__ void __launch_bounds__(64) k_diff_visible(PathArgs a, int ntx) {
       const int p = c * 32 + lane;
       if (p < a.nrp) {
         const float* b = a.rplanes[p].box;
-        see = !surely_hidden(a, HiddenCase{0, E, E, f3(b[0], b[1], b[2]), f3(b[3], b[4], b[5])}, st);
+        see = !test || !surely_hidden(a, HiddenCase{0, E, E, f3(b[0], b[1], b[2]), f3(b[3], b[4], b[5])}, st);
       }
     } else {
       const int i = (c - npw) * kWedgeCluster + lane;
@@ -2260,7 +2267,7 @@ __global__ void __launch_bounds__(64) k_diff_visible(PathArgs a, int ntx) {
         const WedgeF W = a.wf[a.wperm[i]];
         float3 A, B;
         edge_ends(W, A, B);
-        see = !surely_inside(W, E) && !surely_hidden(a, HiddenCase{1, E, E, A, B}, st);
+        see = !surely_inside(W, E) && !(test && surely_hidden(a, HiddenCase{1, E, E, A, B}, st));
       }
     }
     const unsigned m = __ballot_sync(0xffffffffu, see);
@@ -3793,7 +3800,7 @@ __device__ __forceinline__ ReflCand refl_decode(const PathArgs& a, int nlinks, u
 // against a wedge, and the receiver's. Forming each side once and joining
 // the two at the wedge costs a few percent of testing every (kind, link,
 // plane pair) block on its own (8 x 8 city blocks, 64 receivers, 321 planes:
-// 19.8M blocks, 24.5 ms; this form 1.2 ms in all):
+// 19.8M blocks, 24.5 ms; this form 1.9 ms in all):
 //   k_diff_visible the planes and wedges each end point may see at all
 //   k_refl_single  every (end point, plane): the wedges that the image sees
 //                  through the plane's box. Such a side with no reflection
@@ -4026,22 +4033,25 @@ __device__ __forceinline__ void refl_flush(const PathArgs& a, int ntx, int nlink
   if (r.ct > r.ch) refl_candidates_take(a, nlinks, cq, r.ch, r.ct - r.ch);
 }
 
-// One warp per (end point, plane): lanes test the wedge groups' boxes first
-// (most are out of the image's window), then the wedges, four groups at once.
-__global__ void __launch_bounds__(256) k_refl_single(PathArgs a, int ntx, int nlinks) {
+// One warp per (end point, plane) and part of the wedge groups (`parts` of
+// them while there are few end points and planes: in an open scene every
+// group is in the image's window): lanes test the groups' boxes first, then
+// the wedges, four groups at once.
+__global__ void __launch_bounds__(256) k_refl_single(PathArgs a, int ntx, int nlinks, int parts) {
   __shared__ ReflQueues Q;
-  const long nitem = ((long)ntx * a.rsub + a.nrx) * a.nrp;
+  const long nitem = ((long)ntx * a.rsub + a.nrx) * a.nrp * parts;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const long nwarp = (long)gridDim.x * kReflWarps;
   const int ng = (a.nw + kWedgeGroup - 1) / kWedgeGroup;
   ReflRing r;
-  for (long it = (long)blockIdx.x * kReflWarps + wid; it < nitem; it += nwarp) {
+  for (long u = (long)blockIdx.x * kReflWarps + wid; u < nitem; u += nwarp) {
+    const long it = u / parts;
     const int p = (int)(it % a.nrp), v = (int)(it / a.nrp), x = item_end(a, ntx, v);
     if (!sees_plane(a, x, p)) continue;
     const RPlane& Pl = a.rplanes[p];
     const float3 E = end_point(a, ntx, x), X = plane_image(Pl, E);
     const float m = image_margin(E, X);
-    for (int g0 = 0; g0 < ng; g0 += 32) {
+    for (int g0 = 32 * (int)(u % parts); g0 < ng; g0 += 32 * parts) {
       const bool near = g0 + lane < ng && image_sees_group(a, Pl, g0 + lane, X, m, nullptr, X);
       for (unsigned gm = __ballot_sync(0xffffffffu, near); gm;) {
         const int i = octet_wedge(a, g0 + lane, gm);
@@ -4073,17 +4083,18 @@ __global__ void k_refl_room(PathArgs a) {
 }
 
 // The receivers' one-reflection sides into their wedges' lists, from the
-// mask words: one warp per (receiver, plane).
-__global__ void __launch_bounds__(256) k_refl_lists(PathArgs a, int ntx) {
-  const long nitem = (long)a.nrx * a.nrp;
+// mask words: one warp per (receiver, plane) and part of the words.
+__global__ void __launch_bounds__(256) k_refl_lists(PathArgs a, int ntx, int parts) {
+  const long nitem = (long)a.nrx * a.nrp * parts;
   const int lane = threadIdx.x & 31;
   const long nwarp = (long)gridDim.x * (blockDim.x >> 5);
-  for (long it = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < nitem; it += nwarp) {
-    const int p = (int)(it % a.nrp), rx = (int)(it / a.nrp);
+  for (long u = (long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); u < nitem; u += nwarp) {
+    const long it = u / parts;
+    const int p = (int)(it % a.nrp), rx = (int)(it / a.nrp), part = (int)(u % parts);
     const float3 X = plane_image(a.rplanes[p], end_point(a, ntx, ntx + rx));
     const unsigned* row = a.rmask + ((long)(ntx + rx) * a.nrp + p) * a.nwc;
     for (int c0 = 0; c0 < a.nwc; c0 += 32) {
-      const unsigned word = c0 + lane < a.nwc ? row[c0 + lane] : 0u;
+      const unsigned word = c0 + lane < a.nwc && (c0 + lane) % parts == part ? row[c0 + lane] : 0u;
       for (unsigned cm = __ballot_sync(0xffffffffu, word != 0); cm; cm &= cm - 1u) {
         const int src = __ffs(cm) - 1;
         const unsigned wd = __shfl_sync(0xffffffffu, word, src);
@@ -4141,16 +4152,18 @@ __global__ void __launch_bounds__(256) k_refl_join(PathArgs a, int ntx, int nlin
 // Both reflections on one side of the wedge: lanes take (end point, first
 // plane from it, second plane) and keep those whose second plane's box the
 // image can reach through the first's; for each of them the warp tests the
-// groups' boxes against the double image, then the groups' wedges.
-__global__ void __launch_bounds__(256) k_refl_double(PathArgs a, int ntx, int nlinks) {
+// groups' boxes against the double image, then the groups' wedges. `per`
+// items a warp: 32, or fewer so that all warps have one (a highway's 8 planes
+// and 201 end points make 14,400 items, nearly all of them within reach).
+__global__ void __launch_bounds__(256, 3) k_refl_double(PathArgs a, int ntx, int nlinks, int per) {
   __shared__ ReflQueues Q;
   const long nitem = ((long)ntx * a.rsub + a.nrx) * a.nrp * a.nrp;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const long stride = (long)gridDim.x * blockDim.x;
+  const long stride = (long)gridDim.x * kReflWarps * per;
   const int ng = (a.nw + kWedgeGroup - 1) / kWedgeGroup;
   ReflRing r;
-  for (long base = (long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < nitem; base += stride) {
-    const long it = base + lane;
+  for (long base = ((long)blockIdx.x * kReflWarps + wid) * per; base < nitem; base += stride) {
+    const long it = lane < per ? base + lane : nitem;
     int v = 0, pa = 0, pb = 0;
     float m = 0.0f;
     bool pass = false;
@@ -4193,6 +4206,57 @@ __global__ void __launch_bounds__(256) k_refl_double(PathArgs a, int ntx, int nl
     }
   }
   refl_flush(a, ntx, nlinks, Q.side[wid], Q.cand[wid], r);
+}
+
+// The same candidates link by link, for open scenes with few transmitters:
+// nearly every wedge is within reach of every double image there, so forming
+// the sides first saves nothing, and the Keller point's place on the edge (a
+// tenth of a side's work) drops most pairs. One warp per (side, link, plane,
+// plane). A highway (8 planes, 2400 wedges, 200 links): 1.55 ms a frame by
+// k_refl_double, 0.57 ms by this.
+__global__ void __launch_bounds__(256, 3) k_refl_direct(PathArgs a, int ntx, int nlinks) {
+  __shared__ unsigned long long cq[kReflWarps][kReflRing];
+  const long nitem = 2L * nlinks * a.nrp * a.nrp;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const long nwarp = (long)gridDim.x * kReflWarps;
+  const int ng = (a.nw + kWedgeGroup - 1) / kWedgeGroup;
+  ReflRing r;
+  for (long it = (long)blockIdx.x * kReflWarps + wid; it < nitem; it += nwarp) {
+    const int pb = (int)(it % a.nrp);
+    long q = it / a.nrp;
+    const int pa = (int)(q % a.nrp);
+    q /= a.nrp;
+    const int link = (int)(q % nlinks), t = link / a.nrx, rx = ntx + link % a.nrx;
+    const bool tx = q < nlinks;
+    const int x = tx ? t : rx, y = tx ? rx : t;
+    if (pa == pb || !sees_plane(a, x, pa)) continue;
+    const RPlane &Pa = a.rplanes[pa], &Pb = a.rplanes[pb];
+    const float3 E = end_point(a, ntx, x), Y = end_point(a, ntx, y), X1 = plane_image(Pa, E), X = plane_image(Pb, X1);
+    const float m = image_margin(E, X);
+    float lo[3] = {Pb.box[0], Pb.box[1], Pb.box[2]}, hi[3] = {Pb.box[3], Pb.box[4], Pb.box[5]};
+    if (!box_window(Pa, X1, m, lo, hi)) continue;
+    for (int g0 = 0; g0 < ng; g0 += 32) {
+      const int g = g0 + lane;
+      const bool near = g < ng && image_sees_group(a, Pb, g, X, m, &Pa, X1);
+      for (unsigned gm = __ballot_sync(0xffffffffu, near); gm;) {
+        const int i = octet_wedge(a, g, gm);
+        bool ok = i >= 0 && sees_wedge(a, y, i);
+        unsigned long long code = 0;
+        if (ok) {
+          const int w = a.wperm[i];
+          const WedgeF& W = a.wf[w];
+          WedgeSide me, o;
+          float3 p;
+          side_zr(W, X, me, p);
+          side_zr(W, Y, o, p);
+          ok = side_keller(W.len, me, o);
+          code = refl2_code(a, nlinks, tx ? 0 : 2, link, tx ? pa : pb, tx ? pb : pa, w);
+        }
+        refl_push(a, nlinks, cq[wid], r, ok, code);
+      }
+    }
+  }
+  if (r.ct > r.ch) refl_candidates_take(a, nlinks, cq[wid], r.ch, r.ct - r.ch);
 }
 
 // ---- occlusion before the exact stage ----
@@ -4284,7 +4348,7 @@ __device__ __forceinline__ bool diff_blocked(const PathArgs& a, int nlinks, unsi
   return false;
 }
 
-__global__ void __launch_bounds__(64) k_diff_unblocked(PathArgs a, int nlinks) {
+__global__ void __launch_bounds__(64) k_diff_unblocked(PathArgs a, int nlinks, bool open) {
   extern __shared__ int sstk[];
   TStack st;
   bind_stack(st, sstk, kStackTrace);
@@ -4293,18 +4357,25 @@ __global__ void __launch_bounds__(64) k_diff_unblocked(PathArgs a, int nlinks) {
   // few candidates: a few lanes of every warp, so that all SMs share the
   // traversals' latency; many: full warps of consecutive candidates (which
   // come from one warp above, so their legs run close together)
-  // Up to 16 candidates an SM all go on: the exact stage takes them side by
+  // Up to 64 candidates an SM all go on: the exact stage takes them side by
   // side and its time is one candidate's either way, while the longest of the
   // legs here takes 50 us (1113 candidates on a highway, of which 472 would
   // stay: 1016 us for two frames with the test, 935 without; 1643 in an 8 x 8
   // city, of which 227 would stay: 638 and 640).
-  const bool all = n <= 2u * gridDim.x;
+  // So do all of an open scene's, nearly none of which is blocked. They keep
+  // their order, in which survivors of one kind stand together: the exact
+  // stage's warps then run one kind's code.
+  if (n <= 8u * gridDim.x || open) {
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) a.dexact[i] = a.dsurv[i];
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr->n_dexact = n;
+    return;
+  }
   const unsigned nwarp = gridDim.x * (blockDim.x >> 5), per = min(32u, max(1u, (n + nwarp - 1) / nwarp));
   for (unsigned i0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per; i0 < n; i0 += nwarp * per) {
     const unsigned i = i0 + lane;
     const bool mine = lane < (int)per && i < n;
     const unsigned long long code = mine ? a.dsurv[i] : 0ull;
-    const bool keep = mine && (all || !diff_blocked(a, nlinks, code, st));
+    const bool keep = mine && !diff_blocked(a, nlinks, code, st);
     const unsigned mk = __ballot_sync(0xffffffffu, keep);
     if (!mk) continue;
     unsigned at = 0;
@@ -4785,9 +4856,10 @@ cudaError_t launch_diffract(const PathArgs& args, int nlinks, int sms, cudaStrea
     k_wedge_boxes<<<(a.nw + 255) / 256, 256, 0, st>>>(a.wf, a.wperm, a.nw, a.wgbox);
   if (nlinks > 0) {
     if (a.vis) {  // what the end points see: with reflector planes or chains
+      const bool test = a.nrp == 0 || (a.nrp > kOpenPlanes && (a.drefl2 || a.diff_order >= 2));
       const long nvis = (long)(nlinks / a.nrx + a.nrx) * ((a.nrp + 31) / 32 + a.nwc);
       k_diff_visible<<<(int)std::min<long>((nvis + 1) / 2, 16L * sms), 64, 64 * kStackTrace * sizeof(int), st>>>(
-          a, nlinks / a.nrx);
+          a, nlinks / a.nrx, test);
     }
     long total = (long)nlinks * a.nw;
     long g = std::min<long>((total + 255) / 256, 8L * sms);
@@ -4801,13 +4873,23 @@ cudaError_t launch_diffract(const PathArgs& args, int nlinks, int sms, cudaStrea
         cudaMemsetAsync(a.rmask, 0, sizeof(unsigned) * (size_t)(ntx + a.nrx) * a.nrp * a.nwc, st);
       }
       k_diff_visible_any<<<2, 256, 0, st>>>(a, ntx);
-      k_refl_single<<<warps(((long)ntx * a.rsub + a.nrx) * a.nrp), 256, 0, st>>>(a, ntx, nlinks);
+      // parts of an item while there are fewer items than warps
+      const long room = 64L * sms;
+      auto parts = [&](long n) { return (int)std::max<long>(1, std::min<long>(8, room / std::max<long>(n, 1))); };
+      const long single = ((long)ntx * a.rsub + a.nrx) * a.nrp, lists = (long)a.nrx * a.nrp;
+      k_refl_single<<<warps(single * parts(single)), 256, 0, st>>>(a, ntx, nlinks, parts(single));
       if (a.drefl2) {
         k_refl_room<<<(a.nw + 255) / 256, 256, 0, st>>>(a);
-        k_refl_lists<<<warps((long)a.nrx * a.nrp), 256, 0, st>>>(a, ntx);
+        k_refl_lists<<<warps(lists * parts(lists)), 256, 0, st>>>(a, ntx, parts(lists));
         k_refl_join<<<warps((long)ntx * a.nrp * a.nwc * kJoinParts), 256, 0, st>>>(a, ntx, nlinks);
-        a.rsub = std::max(1, a.rsub / 4);
-        k_refl_double<<<warps((((long)ntx * a.rsub + a.nrx) * a.nrp * a.nrp + 31) / 32), 256, 0, st>>>(a, ntx, nlinks);
+        auto items = [&] { return ((long)ntx * a.rsub + a.nrx) * a.nrp * a.nrp; };
+        if (a.nrp <= kOpenPlanes && nlinks <= 2 * (ntx + a.nrx)) {
+          k_refl_direct<<<warps(2L * nlinks * a.nrp * a.nrp), 256, 0, st>>>(a, ntx, nlinks);
+        } else {
+          if (items() > 32 * room) a.rsub = std::max(1, a.rsub / 4);
+          const int per = (int)std::max<long>(1, std::min<long>(32, items() / room));
+          k_refl_double<<<warps((items() + per - 1) / per), 256, 0, st>>>(a, ntx, nlinks, per);
+        }
       }
     }
     PathArgs b = a;  // chains: transmitters, and the reflector planes applied to them
@@ -4832,7 +4914,8 @@ cudaError_t launch_diffract(const PathArgs& args, int nlinks, int sms, cudaStrea
       }
       k_diff_multi_pre<<<8 * sms, 256, 256 * kStackTrace * sizeof(int), st>>>(b);
     }
-    k_diff_unblocked<<<8 * sms, 64, 64 * kStackTrace * sizeof(int), st>>>(b, nlinks);
+    k_diff_unblocked<<<8 * sms, 64, 64 * kStackTrace * sizeof(int), st>>>(
+        b, nlinks, a.rplanes && a.nrp > 0 && a.nrp <= kOpenPlanes);
     k_diffract<<<sms, kDiffThreads, kDiffThreads * kStackTrace * sizeof(int), st>>>(b);
   }
   return cudaGetLastError();
