@@ -3628,8 +3628,8 @@ __device__ __noinline__ void diffract_multi(const PathArgs& a, unsigned long lon
 // -> Rx). By image theory the diffraction runs from the transmitter's image
 // in the planes before the wedge (taken in path order) toward the receiver's
 // image in the planes after it (the last one first); the reflection points
-// follow by unfolding back from Q. A block (kind, link, p1, p2) goes to one
-// warp, which queues the block's candidate wedges (k_diffract_refl2_pre).
+// follow by unfolding back from Q. The candidates are formed per side of the
+// wedge (k_refl_single to k_refl_double) or link by link (k_refl_direct).
 // Survivors carry 10 in bits 63-62 and 1 in bit 61 over (block * nw + wedge).
 constexpr unsigned long long kRefl2Tag = kReflTag | (1ull << 61);
 constexpr unsigned long long kRefl2Mask = (1ull << 61) - 1ull;
@@ -4387,7 +4387,7 @@ __global__ void __launch_bounds__(64) k_diff_unblocked(PathArgs a, int nlinks, b
 
 __device__ __forceinline__ d3w mirror_d(d3w x, d3w n, double c) { return x - n * (2.0 * (dotw(n, x) - c)); }
 
-// One survivor of k_diffract_refl2_pre: the images, the Keller point and the
+// One survivor with two reflections: the images, the Keller point and the
 // wedge rules (chain_geometry with one wedge) and the reflection points on
 // the group planes; the member triangles holding those points; everything
 // again on the members' own planes (the oracle's mirrors are the static
