@@ -1118,17 +1118,19 @@ __device__ zd utd_term(double n, double beta, double s, double kL, unsigned& fl)
 // with face reflection factors r0, rn. The prefactor and the four terms do
 // not depend on r0 and rn, so the soft and hard coefficients share them
 // (utd_parts once, utd_coeff per polarisation).
-// The exact stage takes a survivor with a group of kDiffLanes lanes that run
-// the same code on the same values and split what is independent: the four
-// terms here, the two faces' Fresnel factors, the legs' occlusion.
+// The exact stage takes a survivor with a group of kDiffLanes lanes (or, with
+// many survivors, one) that run the same code on the same values and split
+// what is independent: the four terms here, the two faces' Fresnel factors,
+// the legs' occlusion. The values are the same either way.
 constexpr int kDiffLanes = 4;
-__device__ __forceinline__ int diff_lane() { return threadIdx.x & (kDiffLanes - 1); }
+__shared__ int diff_lanes;  // lanes per survivor, set by k_diffract
+__device__ __forceinline__ int diff_lane() { return threadIdx.x & (diff_lanes - 1); }
 __device__ __forceinline__ unsigned diff_mask() {
-  return ((1u << kDiffLanes) - 1u) << ((threadIdx.x & 31) & ~(kDiffLanes - 1));
+  return ((1u << diff_lanes) - 1u) << ((threadIdx.x & 31) & ~(diff_lanes - 1));
 }
 __device__ __forceinline__ zd diff_from(zd v, int lane) {  // the value of a lane of the group
   const unsigned m = diff_mask();
-  return Z(__shfl_sync(m, v.re, lane, kDiffLanes), __shfl_sync(m, v.im, lane, kDiffLanes));
+  return Z(__shfl_sync(m, v.re, lane, diff_lanes), __shfl_sync(m, v.im, lane, diff_lanes));
 }
 struct UtdParts {
   zd pre, t[4];
@@ -1138,9 +1140,14 @@ __device__ UtdParts utd_parts(double n, double phi, double phip, double beta0, d
   UtdParts u;
   u.pre = Z(-h, h) * (1.0 / (2.0 * n * sqrt(2.0 * M_PI * k) * sin(beta0)));  // -e^{-j pi/4} / (...)
   // terms: (phi - phi', +), (phi - phi', -), (phi + phi', -), (phi + phi', +)
-  const int q = diff_lane();
-  const zd t = utd_term(n, q < 2 ? phi - phip : phi + phip, q == 0 || q == 3 ? 1.0 : -1.0, k * L, fl);
-  for (int j = 0; j < 4; ++j) u.t[j] = diff_from(t, j);
+#pragma unroll 1
+  for (int j0 = 0; j0 < 4; j0 += diff_lanes) {
+    const int q = j0 + diff_lane();
+    const zd t = utd_term(n, q < 2 ? phi - phip : phi + phip, q == 0 || q == 3 ? 1.0 : -1.0, k * L, fl);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (j >= j0 && j < j0 + diff_lanes) u.t[j] = diff_from(t, j - j0);
+  }
   return u;
 }
 __device__ zd utd_coeff(const UtdParts& u, zd r0, zd rn) {
@@ -1163,13 +1170,20 @@ __device__ void fresnel_d(float4 mt, double freq, double ct, zd& te, zd& tm) {
 // ... of a wedge's two faces at once (te, tm of face 0, then of face n).
 __device__ __forceinline__ void fresnel_faces(float4 ma, double cta, float4 mb, double ctb, double freq, zd& r0s,
                                               zd& r0h, zd& rns, zd& rnh) {
-  const bool second = diff_lane() & 1;
-  zd te, tm;
-  fresnel_d(second ? mb : ma, freq, second ? ctb : cta, te, tm);
-  r0s = diff_from(te, 0);
-  r0h = diff_from(tm, 0);
-  rns = diff_from(te, 1);
-  rnh = diff_from(tm, 1);
+#pragma unroll 1
+  for (int j = 0; j < 2; j += diff_lanes) {
+    const bool second = (j + diff_lane()) & 1;
+    zd te, tm;
+    fresnel_d(second ? mb : ma, freq, second ? ctb : cta, te, tm);
+    if (j == 0) {
+      r0s = diff_from(te, 0);
+      r0h = diff_from(tm, 0);
+    }
+    if (j == 1 || diff_lanes > 1) {
+      rns = diff_from(te, 1 - j);
+      rnh = diff_from(tm, 1 - j);
+    }
+  }
 }
 
 struct d3w {
@@ -1326,7 +1340,7 @@ __device__ __noinline__ int leg_crossings(const PathArgs& a, d3w p, d3w q, int e
 __device__ __noinline__ bool legs_occluded(const PathArgs& a, const d3w* P, const int (*ex)[2], int n, unsigned& ovf,
                                            TStack& st) {
   bool hit = false;
-  for (int q = diff_lane(); q + 1 < n && !hit; q += kDiffLanes) {
+  for (int q = diff_lane(); q + 1 < n && !hit; q += diff_lanes) {
     const d3w dv = P[q + 1] - P[q];
     const RayPre rp = ray_pre(f3((float)P[q].x, (float)P[q].y, (float)P[q].z),
                               f3((float)dv.x, (float)dv.y, (float)dv.z));
@@ -2614,7 +2628,7 @@ __global__ void __launch_bounds__(256) k_diff_triples(PathArgs a) {
 // the minimum certainly lies off an edge: the length is convex, so at any
 // points y on the edges it is at least L(t) + g.(y - t), and that exceeds
 // L(t) for all of them by more than the slope's rounding; else 0.
-constexpr float kKellerBox = 1.0f;
+constexpr float kKellerBox = 4.0f;  // 1 m kept 40% more chains for the exact stage, 16 m cost more steps than it saved
 __device__ __forceinline__ float chain_len32(const WedgeF* W, int m, float3 T, float3 R, const float* t) {
   float3 prev = T;
   float L = 0.0f;
@@ -4250,7 +4264,7 @@ __global__ void __launch_bounds__(256, 3) k_refl_direct(PathArgs a, int ntx, int
           side_zr(W, X, me, p);
           side_zr(W, Y, o, p);
           ok = side_keller(W.len, me, o);
-          code = refl2_code(a, nlinks, tx ? 0 : 2, link, tx ? pa : pb, tx ? pb : pa, w);
+          if (ok) code = refl2_code(a, nlinks, tx ? 0 : 2, link, tx ? pa : pb, tx ? pb : pa, w);
         }
         refl_push(a, nlinks, cq[wid], r, ok, code);
       }
@@ -4582,7 +4596,9 @@ __global__ void __launch_bounds__(256) k_diffract_pre(PathArgs a, int nlinks) {
 // the time is the longest lane's chain of dependent operations plus the
 // other lanes' divergent branches: so a survivor takes a group of four lanes
 // (see utd_parts), survivor i goes to block i mod grid, slot i / grid, and the
-// slots fill the warps one group at a time.
+// slots fill the warps one group at a time. More than two rounds of groups on
+// every SM (a highway with two reflections: 266 survivors an SM) keep the
+// instruction pipes busy; there a survivor takes one lane.
 constexpr int kDiffThreads = 256;
 __global__ void __launch_bounds__(kDiffThreads) k_diffract(PathArgs a) {
   extern __shared__ int sstk[];
@@ -4591,9 +4607,12 @@ __global__ void __launch_bounds__(kDiffThreads) k_diffract(PathArgs a) {
   const unsigned n = min(a.ctr->n_dexact, a.dsurv_cap);
   const double k = 2.0 * M_PI * a.freq / 299792458.0, lam = 299792458.0 / a.freq;
   unsigned ovf = 0;
-  constexpr unsigned kWarps = kDiffThreads / 32, kGroups = kDiffThreads / kDiffLanes;
-  const unsigned slot = (threadIdx.x & 31) / kDiffLanes * kWarps + (threadIdx.x >> 5);
-  for (unsigned i = blockIdx.x + gridDim.x * slot; i < n; i += gridDim.x * kGroups) {
+  constexpr unsigned kWarps = kDiffThreads / 32;
+  const unsigned lanes = n > 2 * kDiffThreads / kDiffLanes * gridDim.x ? 1 : kDiffLanes;
+  if (threadIdx.x == 0) diff_lanes = (int)lanes;
+  __syncthreads();
+  const unsigned slot = (threadIdx.x & 31) / lanes * kWarps + (threadIdx.x >> 5);
+  for (unsigned i = blockIdx.x + gridDim.x * slot; i < n; i += gridDim.x * (kDiffThreads / lanes)) {
     const unsigned long long c = a.dexact[i];
     const unsigned kind = (unsigned)(c >> kKindShift);
     if (kind == 2u && ((c >> 61) & 1ull)) diffract_refl2(a, c & kRefl2Mask, k, lam, ovf, st);
