@@ -2331,6 +2331,14 @@ __device__ __forceinline__ bool sees_wedge(const PathArgs& a, int x, int i) {
 
 // (as sees_wedge, for wedge w; true when the rows are not built)
 __device__ __forceinline__ bool end_sees(const PathArgs& a, int x, int w) { return !a.vis || sees_wedge(a, x, a.wplace[w]); }
+// Are wedges hidden from each other left out of the relation? For chains of
+// three, and where the transmitters' images in many planes would each test
+// the same pairs again (8 x 8 city, order 2 with one reflection, 321 planes:
+// a frame took 5.0 ms, so and with planes hidden from an end left out
+// 3.2); not in open scenes.
+__device__ __forceinline__ bool hidden_in_relation(const PathArgs& a) {
+  return a.diff_order >= 3 || a.nrpr > kOpenPlanes;
+}
 __device__ __forceinline__ bool wedges_hidden(const PathArgs& a, const WedgeF& A, const WedgeF& B, TStack& st) {
   HiddenCase h;
   h.kind = 2;
@@ -2365,7 +2373,7 @@ __global__ void __launch_bounds__(256) k_diff_rel(PathArgs a) {
       edge_ends(fb, pb, qb);
       const float m = fmaxf(fmaxf(pre_margin_m(pa), pre_margin_m(qa)), fmaxf(pre_margin_m(pb), pre_margin_m(qb)));
       rel = edge_sees(fa, fb, m) && edge_sees(fb, fa, m);
-      if (rel && a.diff_order >= 3) rel = !wedges_hidden(a, fa, fb, st);
+      if (rel && hidden_in_relation(a)) rel = !wedges_hidden(a, fa, fb, st);
     }
     if (rel) {
       const Wedge &A = a.wedges[w1], &B = a.wedges[w2];
@@ -2383,8 +2391,8 @@ __global__ void __launch_bounds__(256) k_diff_rel(PathArgs a) {
 // can start a path of order >= 2: in the relation (k_diff_rel), the
 // transmitter outside w1, some point of edge 2 beyond the incident shadow
 // boundary of the transmitter at w1, a Keller point on w1 possible between
-// the transmitter and edge 2 (keller_on_edge), and neither w1 hidden from the
-// (real) transmitter nor w2 from w1.
+// the transmitter and edge 2 (keller_on_edge), and neither w1 (an image's
+// plane) hidden from the transmitter nor w2 from w1.
 __global__ void __launch_bounds__(256) k_diff_pairs(PathArgs a, int nsrc) {
   extern __shared__ int sstk[];
   TStack st;
@@ -2401,7 +2409,9 @@ __global__ void __launch_bounds__(256) k_diff_pairs(PathArgs a, int nsrc) {
       long r = idx - (long)t * nw * nw;
       w1 = (int)(r / nw);
       w2 = (int)(r - (long)w1 * nw);
-      if (((a.drel[r >> 5] >> (r & 31)) & 1u) && (t >= a.dntx || end_sees(a, t, w1))) {
+      const bool seen = t < a.dntx ? end_sees(a, t, w1)
+                                   : !a.vis || sees_plane(a, (t - a.dntx) / a.nrpr, (t - a.dntx) % a.nrpr);
+      if (seen && ((a.drel[r >> 5] >> (r & 31)) & 1u)) {
         const WedgeF fa = a.wf[w1], fb = a.wf[w2];
         float3 T = chain_source32(a, t), P, Q;
         edge_ends(fb, P, Q);
@@ -2412,7 +2422,7 @@ __global__ void __launch_bounds__(256) k_diff_pairs(PathArgs a, int nsrc) {
           float mg = 0.1f + 1e-4f * (fabsf(T.x) + fabsf(T.y) + fabsf(T.z) + fa.len);
           keep = plane_reachable(a.rplanes[(t - a.dntx) % a.nrpr], T, A1, B1, mg);
         }
-        if (keep && a.diff_order < 3) keep = !wedges_hidden(a, fa, fb, st);
+        if (keep && a.diff_order < 3 && a.nrpr == 0) keep = !wedges_hidden(a, fa, fb, st);
       }
     }
     unsigned mk = __ballot_sync(0xffffffffu, keep);
@@ -2868,6 +2878,7 @@ __device__ __noinline__ bool chain_possible(const WedgeF* W, int m, float3 T, fl
 __device__ __forceinline__ bool multi_stage1(const PathArgs& a, int4 sq, bool three, int rho) {
   const bool mid = !three && sq.w <= -2, obs_img = rho >= a.nrx;
   if (!obs_img && !end_sees(a, a.dntx + rho, three ? sq.w : sq.z)) return false;
+  if (obs_img && a.vis && !sees_plane(a, a.dntx + (rho - a.nrx) / a.nrpr, (rho - a.nrx) % a.nrpr)) return false;
   WedgeF fl = a.wf[three ? sq.w : sq.z];
   const WedgeF fp = a.wf[three ? sq.z : sq.y];
   float3 R = chain_observer32(a, rho), P, Q;
