@@ -750,9 +750,12 @@ cudaError_t launch_trace_batch(const TraceArgs* d_tab, int n, unsigned* chunk_ct
 static size_t rx_stage_bytes(int nrx) { return (size_t)nrx * 16 + stage_bytes(nrx > 1 ? nrx - 1 : 0, nrx); }
 constexpr size_t kStageLimit = 96 * 1024;
 
-static cudaError_t allow_smem(const void* fn, size_t smem) {
-  if (smem <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+// Their dynamic shared memory is allowed up to kStageLimit whatever this call
+// takes: the 48 KB a launch gets otherwise include the kernel's own arrays
+// (6 KB in k_capture), and a constant cannot be lowered by another thread
+// before this one's launch.
+static cudaError_t allow_smem(const void* fn) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStageLimit);
 }
 
 cudaError_t launch_capture(const TraceArgs& a, int sms, cudaStream_t st) {
@@ -761,7 +764,7 @@ cudaError_t launch_capture(const TraceArgs& a, int sms, cudaStream_t st) {
   bool kS = a.nrx <= 1024 && staged <= kStageLimit;
   const void* fn = kS ? (const void*)k_capture<true> : (const void*)k_capture<false>;
   size_t smem = kS ? staged : base;
-  cudaError_t e = allow_smem(fn, smem);
+  cudaError_t e = allow_smem(fn);
   if (e != cudaSuccess) return e;
   int blocks = grid_for((long)a.LS * (a.N + a.max_trans + 1), 256, resident_blocks(fn, sms, smem));
   if (kS) k_capture<true><<<blocks, 256, smem, st>>>(a);
@@ -774,12 +777,12 @@ cudaError_t launch_mark(const TraceArgs& a, const CoherentArgs& c, int sms, cuda
   size_t staged = base + stage_bytes(c.mv_cap > 1 ? c.mv_cap - 1 : 0, 0);
   bool kS = staged <= kStageLimit;
   size_t smem = kS ? staged : base;
-  cudaError_t e = allow_smem(kS ? (const void*)k_mark<true> : (const void*)k_mark<false>, smem);
+  const void* fn = kS ? (const void*)k_mark<true> : (const void*)k_mark<false>;
+  cudaError_t e = allow_smem(fn);
   if (e != cudaSuccess) return e;
   // one wave of resident blocks (each stages the moved-box tree once)
   static size_t key = 0;
   static int resident = 0;
-  const void* fn = kS ? (const void*)k_mark<true> : (const void*)k_mark<false>;
   if (key != smem + kS) {
     resident = resident_blocks(fn, sms, smem);
     key = smem + kS;
