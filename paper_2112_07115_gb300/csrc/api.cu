@@ -1410,6 +1410,9 @@ int dcem_scene_create(const float* tris, int32_t ntri, const int32_t* tri_mat, c
   // static tree (built once)
   launch_tri_boxes(v9, sel_s_d, s->ns, s->prim, st);
   SahTree t;
+  std::vector<int> perm;  // (copied asynchronously, as t.leaf_parent: they live until the stream is synchronised)
+  std::vector<float4> nodes;
+  const int root = 0;
   if (s->ns > 1 && s->ns <= kSahMax) {
     t.prim.resize(s->ns);
     for (int i = 0; i < s->ns; ++i) {
@@ -1426,16 +1429,15 @@ int dcem_scene_create(const float* tris, int32_t ntri, const int32_t* tri_mat, c
     t.parent.assign(s->nint_s, -1);
     t.leaf_parent.assign(s->ns, -1);
     sah_split(t, 0, 0, s->ns, 0, 3);
-    std::vector<int> perm(s->ns);
+    perm.resize(s->ns);
     for (int j = 0; j < s->ns; ++j) perm[j] = t.prim[j].id;
-    std::vector<float4> nodes(4 * (size_t)s->nint_s);
+    nodes.assign(4 * (size_t)s->nint_s, make_float4(0.f, 0.f, 0.f, 0.f));
     for (int i = 0; i < s->nint_s; ++i) {
       float c[3];
       const int v[3] = {t.child[2 * (size_t)i], t.child[2 * (size_t)i + 1], t.parent[i]};
       std::memcpy(c, v, sizeof(c));
       nodes[4 * (size_t)i + 3] = make_float4(c[0], c[1], c[2], 0.0f);
     }
-    const int root = 0;
     CKF(cudaMemcpyAsync(s->nodes, nodes.data(), sizeof(float4) * nodes.size(), cudaMemcpyHostToDevice, st));
     CKF(cudaMemcpyAsync(s->perm, perm.data(), sizeof(int) * s->ns, cudaMemcpyHostToDevice, st));
     CKF(cudaMemcpyAsync(s->leaf_parent, t.leaf_parent.data(), sizeof(int) * s->ns, cudaMemcpyHostToDevice, st));
