@@ -2935,6 +2935,14 @@ static int path_derivs(dcem_scene* s, const float* tx, const float* rx, int32_t 
     return DCEM_OK;
   }
   const int W = 1 + 4 * p->max_refl;
+  // copies from host memory may be made as late as the synchronisation: what
+  // they read outlives it, on every way out
+  std::vector<float4> h;
+  unsigned err = 0;
+  struct Sync {
+    cudaStream_t st;
+    ~Sync() { cudaStreamSynchronize(st); }
+  } sync{st};
   // device copies of the inputs given on the host, scratch, staged outputs
   if ((size_t)nrx > s->g_rx_cap) {
     dfree(s->g_rx);
@@ -2942,9 +2950,8 @@ static int path_derivs(dcem_scene* s, const float* tx, const float* rx, int32_t 
     s->g_rx_cap = (size_t)nrx;
   }
   if (rx_ptr_kind == DCEM_PTR_HOST) {
-    std::vector<float4> h((size_t)nrx);
+    h.resize((size_t)nrx);
     for (int i = 0; i < nrx; ++i) h[i] = make_float4(rx[3 * i], rx[3 * i + 1], rx[3 * i + 2], 0.0f);
-    // (pageable: the call returns once h has been read)
     CK(cudaMemcpyAsync(s->g_rx, h.data(), sizeof(float4) * nrx, cudaMemcpyHostToDevice, st));
   } else {
     CK(launch_pack_rx(rx, nrx, s->g_rx, st));
@@ -3027,7 +3034,6 @@ static int path_derivs(dcem_scene* s, const float* tx, const float* rx, int32_t 
   g.theta_bar = theta_bar ? (dev ? theta_bar : G + o_tb) : nullptr;
   CK(adjoint ? launch_adjoint(g, s->sms, st) : launch_gradients(g, st));
   s->launches += (n_paths > 0 ? 1 : 0) + 1 + (rx_ptr_kind == DCEM_PTR_DEVICE ? 1 : 0) + (g.theta_bar ? 1 : 0);
-  unsigned err = 0;
   CK(cudaMemcpyAsync(&err, s->g_err, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
   if (!dev) {
     cudaMemcpyKind k = cudaMemcpyDeviceToHost;

@@ -51,3 +51,19 @@ for sc in (scenes.city_blocks(n=2), scenes.toy_street()):
     s.close()
 assert L.fake_stale() == 0, L.fake_stale()
 """)
+
+
+def test_sources_of_copies_outlive_them_derivatives(stand_in):
+    _child(stand_in, """
+sc = scenes.toy_street()
+s = dcem.Scene.from_scene(sc)
+before = L.fake_stale()
+prm = dcem.default_params(max_refl=3)
+none = np.zeros(0, dcem.PATH_DTYPE)
+for n in (1, 40):
+    rx = np.ones((n, 3), np.float32)
+    s.gradients(sc.tx, rx, none, prm)
+    s.adjoint(sc.tx, rx, none, prm, theta=s.theta(sc.xf[0]), pcoh_bar=np.ones(n))
+assert L.fake_stale() == before, L.fake_stale() - before
+s.close()
+""")
