@@ -28,6 +28,20 @@ void dfree(T*& p) {
   if (p) cudaFree((void*)p);
   p = nullptr;
 }
+// A buffer of n in place of the one that may be there.
+template <class T>
+cudaError_t renew(T** p, size_t n) {
+  dfree(*p);
+  return dalloc(p, n);
+}
+// ... holding v: null unless its contents are in place.
+template <class T>
+cudaError_t upload(T** p, const std::vector<T>& v) {
+  cudaError_t e = renew(p, v.size());
+  if (e == cudaSuccess) e = cudaMemcpy(*p, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) dfree(*p);
+  return e;
+}
 
 int status_of(cudaError_t e) {
   if (e == cudaSuccess) return DCEM_OK;
@@ -575,16 +589,21 @@ int alloc_build_scratch(dcem_scene* s, int n) {
 // The segment log for W segments per slot over the R primary rays and
 // child_cap transmission children (their restart points, segment counts and
 // instance words too).
+// Here and below, a capacity counts only once all of its buffers are there
+// (else a call after one that ran out of memory would launch on null
+// pointers): it is zero, or the pointer that stands for it null, until then.
 int ensure_log(dcem_scene* s, int W, int child_cap) {
   if (s->logW >= W && s->log_o && s->child_cap == child_cap) return DCEM_OK;
   const int LS = s->R + child_cap;
   dfree(s->log_o); dfree(s->log_d); dfree(s->log_id); dfree(s->capitems);
   size_t n = (size_t)W * (size_t)(LS > 0 ? LS : 1);
+  s->logW = 0;
   CK(dalloc(&s->log_o, n));
   CK(dalloc(&s->log_d, n));
   CK(dalloc(&s->log_id, n));
   CK(dalloc(&s->capitems, n));
   if (child_cap != s->child_cap) {
+    s->child_cap = -1;
     dfree(s->nseg); dfree(s->restart); dfree(s->inst); dfree(s->inst_root);
     CK(dalloc(&s->nseg, LS > 0 ? LS : 1));
     CK(dalloc(&s->restart, LS > 0 ? LS : 1));
@@ -600,6 +619,7 @@ int ensure_log(dcem_scene* s, int W, int child_cap) {
 
 int ensure_paths(dcem_scene* s, unsigned cand_cap, unsigned ucap) {
   if (cand_cap > s->cand_cap) {
+    s->cand_cap = 0;
     dfree(s->cand[0]); dfree(s->cand[1]); dfree(s->cand_slot); dfree(s->hkey); dfree(s->hrep);
     CK(dalloc(&s->cand[0], cand_cap));
     CK(dalloc(&s->cand[1], cand_cap));
@@ -614,6 +634,7 @@ int ensure_paths(dcem_scene* s, unsigned cand_cap, unsigned ucap) {
     s->cache_valid = false;  // previous captures are gone
   }
   if (ucap > s->ucap) {
+    s->ucap = 0;
     dfree(s->uniq); dfree(s->prec); dfree(s->pout); dfree(s->vpts); dfree(s->vstate);
     dfree(s->prec_b); dfree(s->vpts_b); dfree(s->vstate_b); dfree(s->ckey);
     dfree(s->vc_key[0]); dfree(s->vc_key[1]); dfree(s->vc_u[0]); dfree(s->vc_u[1]);
@@ -650,7 +671,6 @@ int ensure_rx(dcem_scene* s, int nrx, int nlinks, int bucket_cap) {
   if (nrx > s->nrx_cap || !s->rx3) {
     int cap = std::max(1, std::max(nrx, s->nrx_cap));
     dfree(s->rx3); dfree(s->rx_cur); dfree(s->rx_traced); dfree(s->rx_moved); dfree(s->moved_list);
-    CK(dalloc(&s->rx3, 3 * (size_t)cap));
     CK(dalloc(&s->rx_cur, cap));
     CK(dalloc(&s->rx_traced, cap));
     CK(dalloc(&s->rx_moved, cap));
@@ -661,6 +681,7 @@ int ensure_rx(dcem_scene* s, int nrx, int nlinks, int bucket_cap) {
     CK(dalloc(&s->rxt_parent, cap));
     CK(dalloc(&s->rxt_perm, cap));
     CK(dalloc(&s->rxt_arrive, cap));
+    CK(dalloc(&s->rx3, 3 * (size_t)cap));
     s->nrx_cap = cap;
     s->cache_valid = false;
   }
@@ -672,10 +693,10 @@ int ensure_rx(dcem_scene* s, int nrx, int nlinks, int bucket_cap) {
       while (bucket_cap > 64 && (size_t)cap * bucket_cap > ((size_t)1 << 26)) bucket_cap >>= 1;
     dfree(s->bucket); dfree(s->bucket_cnt); dfree(s->rxout); dfree(s->link_off);
     s->bucket_cap = first ? bucket_cap : std::max(bucket_cap, s->bucket_cap);
-    CK(dalloc(&s->bucket, (size_t)cap * s->bucket_cap));
     CK(dalloc(&s->bucket_cnt, cap));
     CK(dalloc(&s->rxout, 4 * (size_t)cap));  // staging: field (2 cap), P_coh (cap), P_inc (cap)
     CK(dalloc(&s->link_off, cap));
+    CK(dalloc(&s->bucket, (size_t)cap * s->bucket_cap));
     s->nlink_cap = cap;
     s->cache_valid = false;
   }
@@ -1712,40 +1733,30 @@ int dcem_scene_set_diffraction(dcem_scene* s, int32_t on, int32_t* n_wedges) {
   if (!s || (on != 0 && on != 1)) return DCEM_ERR_ARG;
   if (on && !s->wtopo) {
     std::vector<WedgeTopo> w = find_wedges(s->tris_h, s->tri_obj_h);
-    s->nw = (int)w.size();
-    if (s->nw) {
+    if (!w.empty()) {
+      const int nw = (int)w.size();
       std::vector<int> perm = wedge_order(s->tris_h, s->tri_obj_h, w);
-      s->nwc = (s->nw + kWedgeCluster - 1) / kWedgeCluster;
-      CK(dalloc(&s->wtopo, s->nw));
-      CK(dalloc(&s->wedges, s->nw));
-      CK(dalloc(&s->wedgesf, s->nw));
-      CK(dalloc(&s->wperm, s->nw));
       std::vector<int> place(perm.size());
       for (size_t i = 0; i < perm.size(); ++i) place[perm[i]] = (int)i;
-      CK(dalloc(&s->wplace, s->nw));
-      CK(cudaMemcpy(s->wplace, place.data(), sizeof(int) * place.size(), cudaMemcpyHostToDevice));
-      CK(dalloc(&s->wgbox, 6 * (size_t)((s->nw + kWedgeGroup - 1) / kWedgeGroup)));
-      CK(cudaMemcpy(s->wtopo, w.data(), sizeof(WedgeTopo) * w.size(), cudaMemcpyHostToDevice));
-      CK(cudaMemcpy(s->wperm, perm.data(), sizeof(int) * perm.size(), cudaMemcpyHostToDevice));
+      CK(renew(&s->wedges, nw));
+      CK(renew(&s->wedgesf, nw));
+      CK(renew(&s->wgbox, 6 * (size_t)((nw + kWedgeGroup - 1) / kWedgeGroup)));
+      CK(upload(&s->wplace, place));
+      CK(upload(&s->wperm, perm));
+      CK(upload(&s->wtopo, w));
+      s->nw = nw;
+      s->nwc = (nw + kWedgeCluster - 1) / kWedgeCluster;
     }
   }
   if (on && s->nw && !s->dsurv) {  // grown (and the frame traced again) when a frame needs more
-    CK(dalloc(&s->dsurv, (size_t)1024));
-    CK(dalloc(&s->dexact, (size_t)1024));
+    s->dsurv_cap = 0;
+    CK(renew(&s->dexact, (size_t)1024));
+    CK(renew(&s->dsurv, (size_t)1024));
     s->dsurv_cap = 1024;
   }
   s->diffraction = on != 0;
   if (n_wedges) *n_wedges = s->nw;
   return DCEM_OK;
-}
-
-static cudaError_t upload_quads(dcem_scene* s, const std::vector<float4>& quads) {
-  if (s->quads) return cudaSuccess;
-  cudaError_t e = dalloc(&s->quads, quads.size());
-  if (e == cudaSuccess)
-    e = cudaMemcpy(s->quads, quads.data(), sizeof(float4) * quads.size(), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) dfree(s->quads);
-  return e;
 }
 
 int dcem_scene_set_diffraction_reflections(dcem_scene* s, int32_t on, int32_t* n_planes) {
@@ -1756,15 +1767,12 @@ int dcem_scene_set_diffraction_reflections(dcem_scene* s, int32_t on, int32_t* n
     std::vector<int> members;
     std::vector<float> keys;
     group_planes(s->tris_h, s->tri_obj_h, planes, members, keys);
-    s->nrp = (int)planes.size();
-    if (s->nrp) {
-      CK(dalloc(&s->rplanes, planes.size()));
-      CK(dalloc(&s->rmembers, members.size()));
-      CK(dalloc(&s->rkeys, keys.size()));
-      CK(cudaMemcpy(s->rplanes, planes.data(), sizeof(RPlane) * planes.size(), cudaMemcpyHostToDevice));
-      CK(cudaMemcpy(s->rmembers, members.data(), sizeof(int) * members.size(), cudaMemcpyHostToDevice));
-      CK(cudaMemcpy(s->rkeys, keys.data(), sizeof(float) * keys.size(), cudaMemcpyHostToDevice));
-      CK(upload_quads(s, wall_quads(s->tris_h, s->tri_obj_h, planes, members)));
+    if (!planes.empty()) {
+      if (!s->quads) CK(upload(&s->quads, wall_quads(s->tris_h, s->tri_obj_h, planes, members)));
+      CK(upload(&s->rmembers, members));
+      CK(upload(&s->rkeys, keys));
+      CK(upload(&s->rplanes, planes));
+      s->nrp = (int)planes.size();
     }
   }
   s->diff_refl = on;
@@ -1776,16 +1784,17 @@ int dcem_scene_set_diffraction_order(dcem_scene* s, int32_t max_order) {
   if (!s || max_order < 1 || max_order > 3) return DCEM_ERR_ARG;
   if (max_order > 1 && !s->diffraction) return DCEM_ERR_STATE;
   if (max_order >= 2 && !s->dseq2 && s->nw > 1) {  // lists grown (and the frame traced again) on demand
-    CK(dalloc(&s->dseq2, (size_t)4096));
-    s->dseq2_cap = 4096;
-    CK(dalloc(&s->drel, ((size_t)s->nw * s->nw + 31) / 32));
+    s->dseq2_cap = 0;
+    CK(renew(&s->drel, ((size_t)s->nw * s->nw + 31) / 32));
     if (!s->quads) {
       std::vector<RPlane> planes;
       std::vector<int> members;
       std::vector<float> keys;
       group_planes(s->tris_h, s->tri_obj_h, planes, members, keys);
-      CK(upload_quads(s, wall_quads(s->tris_h, s->tri_obj_h, planes, members)));
+      CK(upload(&s->quads, wall_quads(s->tris_h, s->tri_obj_h, planes, members)));
     }
+    CK(renew(&s->dseq2, (size_t)4096));
+    s->dseq2_cap = 4096;
   }
   if (max_order >= 3 && !s->dseq3 && s->nw > 2) {
     CK(dalloc(&s->dseq3, (size_t)4096));
@@ -2430,20 +2439,21 @@ static int frame_finish(dcem_scene* s, const float* tx, int32_t ntx, const float
         if (n <= cap) return DCEM_OK;
         unsigned long long want = std::max<unsigned long long>(2ull * cap, (unsigned long long)n * 5 / 4 + 1024);
         if (want > 0x7fffffffull) return DCEM_ERR_CAPACITY;
-        dfree(buf);
-        CK(dalloc(&buf, (size_t)want));
+        cap = 0;
+        CK(renew(&buf, (size_t)want));
         cap = (unsigned)want;
         return DCEM_OK;
       };
-      unsigned had = s->dsurv_cap;
-      if ((rc = grow(c[0].n_dsurv, s->dsurv_cap, s->dsurv)) != DCEM_OK) return rc;
-      if (s->dsurv_cap != had) {
-        dfree(s->dexact);
-        CK(dalloc(&s->dexact, (size_t)s->dsurv_cap));
-      }
-      if (s->dobs && (rc = grow(c[0].n_dobs, s->dobs_cap, s->dobs)) != DCEM_OK) return rc;
-      if (s->dseq2 && (rc = grow(c[0].n_dpair, s->dseq2_cap, s->dseq2)) != DCEM_OK) return rc;
-      if (s->dseq3 && (rc = grow(c[0].n_dtrip, s->dseq3_cap, s->dseq3)) != DCEM_OK) return rc;
+      // (the two survivor lists have one capacity)
+      const unsigned had = s->dsurv_cap;
+      unsigned room = had;
+      s->dsurv_cap = 0;
+      if ((rc = grow(c[0].n_dsurv, room, s->dsurv)) != DCEM_OK) return rc;
+      if (room != had) CK(renew(&s->dexact, (size_t)room));
+      s->dsurv_cap = room;
+      if ((rc = grow(c[0].n_dobs, s->dobs_cap, s->dobs)) != DCEM_OK) return rc;
+      if ((rc = grow(c[0].n_dpair, s->dseq2_cap, s->dseq2)) != DCEM_OK) return rc;
+      if ((rc = grow(c[0].n_dtrip, s->dseq3_cap, s->dseq3)) != DCEM_OK) return rc;
     }
     if (err & ERR_BUCKET_OVERFLOW) {
       int nb = s->bucket_cap * 2;
@@ -2945,8 +2955,8 @@ static int path_derivs(dcem_scene* s, const float* tx, const float* rx, int32_t 
   } sync{st};
   // device copies of the inputs given on the host, scratch, staged outputs
   if ((size_t)nrx > s->g_rx_cap) {
-    dfree(s->g_rx);
-    CK(dalloc(&s->g_rx, (size_t)nrx));
+    s->g_rx_cap = 0;
+    CK(renew(&s->g_rx, (size_t)nrx));
     s->g_rx_cap = (size_t)nrx;
   }
   if (rx_ptr_kind == DCEM_PTR_HOST) {
@@ -2959,8 +2969,8 @@ static int path_derivs(dcem_scene* s, const float* tx, const float* rx, int32_t 
   const dcem_path* pd = paths;
   if (ptr_kind == DCEM_PTR_HOST && n_paths > 0) {
     if ((size_t)n_paths > s->g_paths_cap) {
-      dfree(s->g_paths);
-      CK(dalloc(&s->g_paths, (size_t)n_paths));
+      s->g_paths_cap = 0;
+      CK(renew(&s->g_paths, (size_t)n_paths));
       s->g_paths_cap = (size_t)n_paths;
     }
     CK(cudaMemcpyAsync(s->g_paths, paths, sizeof(dcem_path) * n_paths, cudaMemcpyHostToDevice, st));
@@ -2968,10 +2978,9 @@ static int path_derivs(dcem_scene* s, const float* tx, const float* rx, int32_t 
   }
   size_t nitems = (size_t)n_paths * W;
   if (nitems > s->g_items_cap) {
-    dfree(s->g_items);
-    dfree(s->g_param);
-    CK(dalloc(&s->g_items, nitems));
-    CK(dalloc(&s->g_param, nitems));
+    s->g_items_cap = 0;
+    CK(renew(&s->g_items, nitems));
+    CK(renew(&s->g_param, nitems));
     s->g_items_cap = nitems;
   }
   // staging: field 2 nrx, P_coh nrx, dfield 2 nrx np, dpcoh nrx np, theta_bar np,
@@ -2979,8 +2988,8 @@ static int path_derivs(dcem_scene* s, const float* tx, const float* rx, int32_t 
   const size_t o_pc = 2 * (size_t)nrx, o_df = o_pc + nrx, o_dp = o_df + 2 * (size_t)nrx * np,
                o_tb = o_dp + (size_t)nrx * np, o_pb = o_tb + np, o_th = o_pb + nrx, nout = o_th + np;
   if (nout > s->g_out_cap) {
-    dfree(s->g_out);
-    CK(dalloc(&s->g_out, nout));
+    s->g_out_cap = 0;
+    CK(renew(&s->g_out, nout));
     s->g_out_cap = nout;
   }
   double* G = s->g_out;

@@ -1,6 +1,8 @@
 """The host code's memory handling, without a GPU: the library's own objects
 linked to a stand-in for the CUDA runtime (host_runtime.cu) in which kernels
-do nothing. Host buffers outlive the asynchronous copies made from them."""
+do nothing. Host buffers outlive the asynchronous copies made from them, and
+after an allocation that failed, whichever it was, a repeated call finds every
+buffer that its kernels take."""
 import os
 import subprocess
 import sys
@@ -66,4 +68,52 @@ for n in (1, 40):
     s.adjoint(sc.tx, rx, none, prm, theta=s.theta(sc.xf[0]), pcoh_bar=np.ones(n))
 assert L.fake_stale() == before, L.fake_stale() - before
 s.close()
+""")
+
+
+@pytest.mark.parametrize("order,refl", [(1, 2), (3, 1), (3, 3)])
+def test_every_allocation_may_fail(stand_in, order, refl):
+    _child(stand_in, f"""
+order, refl = {order}, {refl}
+sc = scenes.city_blocks(n=2, n_rx=30)
+prm = dcem.default_params(max_refl=3)
+rx = np.asarray(sc.rx[0], np.float32)
+
+def attempt(step):
+    # the call, and once more when an allocation failed
+    try:
+        return step()
+    except dcem.DcemError as e:
+        assert e.status == dcem.ERR_NOMEM, e
+        L.fake_fail_alloc(0)
+        return step()
+
+def steps(s):
+    yield lambda: s.set_rays(scenes.fibonacci_sphere(200))
+    yield lambda: s.set_diffraction(True)
+    yield lambda: s.set_diffraction_reflections(refl)
+    yield lambda: s.set_diffraction_order(order)
+    yield lambda: s.trace(sc.tx, rx[:10], prm)
+    def more():
+        L.fake_overflow(1, 5000, 40000, 9000, 9000)
+        s.trace(sc.tx, np.repeat(rx, 20, 0), prm)
+    yield more
+    yield lambda: s.trace(sc.tx, rx[:10], prm)
+    yield lambda: s.gradients(sc.tx, rx[:9], np.zeros(3, dcem.PATH_DTYPE), prm)
+
+n, seen = 1, 0
+while True:
+    s = dcem.Scene.from_scene(sc)
+    first = L.fake_allocs()
+    for step in steps(s):
+        # the n-th allocation from here on fails, wherever that is
+        L.fake_fail_alloc(max(0, n - (L.fake_allocs() - first)))
+        attempt(step)
+    done = L.fake_allocs() - first
+    s.close()
+    assert L.fake_bad() == 0, (n, L.fake_bad_text())
+    if done < n:
+        break
+    n, seen = n + 1, done
+assert seen > 60, seen
 """)
