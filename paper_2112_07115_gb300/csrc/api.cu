@@ -1108,8 +1108,11 @@ std::vector<float4> wall_quads(const std::vector<float>& tris, const std::vector
 // along the scene meet every one of the long boxes it leaves (the 2 km
 // highway: mean 8.8 -> 8.1 nodes, worst segment 74 -> 142, closest hit 0.18 ->
 // 0.23 ms; the radix tree halves all axes alike). kSahMax bounds the build time
-// on the host (5 ms for 50,000 triangles on eight threads).
-constexpr int kSahMax = 1 << 18, kSahBins = 32, kSahDepth = 45;
+// on the host (5 ms for 50,000 triangles on eight threads); kSahLevels the
+// internal levels, to those that two binary levels a 4-wide one may have
+// (kWideLevels): halving takes over where the triangles left would need the
+// rest. (The scenes here have 6 to 21 levels.)
+constexpr int kSahMax = 1 << 18, kSahBins = 32, kSahLevels = 2 * kWideLevels;
 constexpr float kSahAspect = 8.0f;
 
 struct SahPrim {
@@ -1165,7 +1168,9 @@ inline int sah_bin(const SahPrim& p, int k, float lo, float inv, int bins) {
 void sah_split(SahTree& t, int node, int a, int b, int depth, int fork) {
   const int n = b - a;
   int m = a + n / 2;
-  if (n > 2 && depth < kSahDepth) {
+  int halvings = 0;  // levels of the larger child at most when it is halved on
+  while ((1 << halvings) < n - 1) ++halvings;
+  if (n > 2 && depth + 1 + halvings <= kSahLevels) {
     SahBox c;
     for (int i = a; i < b; ++i)
       for (int k = 0; k < 3; ++k) {

@@ -891,20 +891,27 @@ __device__ __forceinline__ unsigned qenc_hi(float v, float o, float s) {
 // 4-wide nodes, top down: a 4-wide node starts from a binary node's two
 // children and replaces, twice, its internal child with the largest box by
 // that child's two children (taking every second level of the tree, whatever
-// its boxes, visits 4-13% more nodes; urban frame 5.39 -> 5.33 ms, office 1068 ->
-// 1057 us); its remaining internal children become
+// its boxes, visits 4-13% more nodes); its remaining internal children become
 // 4-wide nodes in turn. A 4-wide node takes three binary nodes or holds
 // leaves only, so there are at most (2 nn + 1) / 3. For each child slot it
 // records the child (4-wide index, leaf ~slot, or kEmpty) and where its box
-// lives in the binary records (record << 1 | side). Scratch todo[nn]: the
-// binary node of every 4-wide node so far, in shared memory, or the global
-// array `gscr` when that does not fit.
+// lives in the binary records (record << 1 | side).
+// Growing by area alone could give one 4-wide level per binary level, and a
+// traversal leaves three entries a level waiting: a child whose subtree is too
+// deep to stay (kWideLevels) is replaced before any other. Two levels at a
+// time always fit the bound once a node does, and a node has two children, so
+// the two replacements suffice.
+// Scratch, in shared memory or the global array `gscr` when that does not
+// fit: the binary node of every 4-wide node so far, and each binary node's
+// parent and height (internal levels of its subtree).
 __global__ void __launch_bounds__(1024) k_bvh4_map(const float4* __restrict__ nodes, int nn,
-                                                   const int* __restrict__ roots, int4* kid4, int4* src4,
-                                                   int* n4_out, int* roots4_out, int* gscr) {
+                                                    const int* __restrict__ roots, int4* kid4, int4* src4,
+                                                    int* n4_out, int* roots4_out, int* gscr) {
   extern __shared__ int sm4[];
   int* todo = gscr ? gscr : sm4;
-  __shared__ int total;
+  int* par = todo + nn;
+  int* high = par + nn;
+  __shared__ int total, wide;
   const int tid = threadIdx.x, nt = blockDim.x;
   const int cap = (2 * nn + 2) / 3;
   auto kid = [&](int n, int side) { return reinterpret_cast<const int*>(nodes + 4 * (size_t)n + 3)[side]; };
@@ -913,13 +920,30 @@ __global__ void __launch_bounds__(1024) k_bvh4_map(const float4* __restrict__ no
     const float x = xy.y - xy.x, y = xy.w - xy.z, h = side ? z.w - z.z : z.y - z.x;
     return x * y + y * h + h * x;
   };
+  auto inner = [&](int c) { return c >= 0 && c < nn; };
+  for (int i = tid; i < nn; i += nt) {
+    par[i] = -1;
+    high[i] = 1;
+  }
+  __syncthreads();
+  for (int i = tid; i < nn; i += nt)
+    for (int side = 0; side < 2; ++side)
+      if (inner(kid(i, side))) par[kid(i, side)] = i;
+  __syncthreads();
+  // heights, from the nodes that hold two leaves up, until another branch was higher
+  for (int i = tid; i < nn; i += nt)
+    if (!inner(kid(i, 0)) && !inner(kid(i, 1)))
+      for (int h = 2, p = par[i]; p >= 0 && h < 4096 && atomicMax(&high[p], h) < h; ++h) p = par[p];
+  __syncthreads();
   if (tid == 0) {
     total = 0;
+    wide = kWideLevels;
     for (int r = 0; r < 2; ++r) {
       const int c = roots[r];
-      const bool in = c >= 0 && c < nn;
-      roots4_out[r] = in ? total : c;
-      if (in) todo[total++] = c;
+      roots4_out[r] = inner(c) ? total : c;
+      if (!inner(c)) continue;
+      todo[total++] = c;
+      wide = max(wide, (high[c] + 1) / 2);
     }
   }
   __syncthreads();
@@ -935,12 +959,15 @@ __global__ void __launch_bounds__(1024) k_bvh4_map(const float4* __restrict__ no
       for (int grow = 0; grow < 2; ++grow) {
         int at = -1;
         float best = -1.0f;
+        bool must = false;  // too deep for the next 4-wide level
         for (int j = 0; j < m; ++j) {
-          if (!(k[j] >= 0 && k[j] < nn)) continue;
+          if (!inner(k[j])) continue;
           const float ar = area(sr[j] >> 1, sr[j] & 1);
-          if (at < 0 || ar > best) {
+          const bool deep = level + 1 + (high[k[j]] + 1) / 2 > wide;
+          if (at < 0 || (deep && !must) || (deep == must && ar > best)) {
             at = j;
             best = ar;
+            must = deep;
           }
         }
         if (at < 0) break;
@@ -952,7 +979,7 @@ __global__ void __launch_bounds__(1024) k_bvh4_map(const float4* __restrict__ no
         ++m;
       }
       for (int j = 0; j < m; ++j)
-        if (k[j] >= 0 && k[j] < nn) {
+        if (inner(k[j])) {
           const int w = atomicAdd(&total, 1);
           if (w < cap) todo[w] = k[j];
           k[j] = w < cap ? w : kEmpty;  // (a malformed tree only)
