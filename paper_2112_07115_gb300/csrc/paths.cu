@@ -2630,15 +2630,15 @@ __global__ void __launch_bounds__(256) k_diff_triples(PathArgs a) {
 }
 
 // FP32 Keller points of a chain (the pre-test's estimate): Newton's method
-// as in keller_chain, in FP32, from the edges' midpoints, with the iterates
-// kept within kKellerBox metres of the edges (coordinates at that bound with
-// the slope pointing out stay there; the rest take the reduced step).
-// Returns 1 when the cosine mismatch fell below 2e-6 at every edge, or a full
-// Newton step would move no point by more than step_tol (metres); -1 when
-// the minimum certainly lies off an edge: the length is convex, so at any
-// points y on the edges it is at least L(t) + g.(y - t), and that exceeds
-// L(t) for all of them by more than the slope's rounding; else 0.
-constexpr float kKellerBox = 4.0f;  // 1 m kept 40% more chains for the exact stage, 16 m cost more steps than it saved
+// as in keller_chain, in FP32, from the edges' midpoints. Returns true when
+// the cosine mismatch fell below 2e-6 at every edge, or a full Newton step
+// would move no point by more than step_tol (metres).
+// The iterates may leave the edges: where the length is nearly flat (legs of
+// 200 to 2000 m along a road) only the converged point shows how far off its
+// edge it lies. Held within 4 m of the edges and cut by convexity instead, a
+// highway's chains of two with every reflection left 145,370 candidates for
+// the FP64 stage, not 59,700 (24.0 ms a frame, so 20.0), three wedges on a
+// 1 km road 13,831, not 126, and the 8 x 8 city 432, not 307 (1446, so 1246 us).
 __device__ __forceinline__ float chain_len32(const WedgeF* W, int m, float3 T, float3 R, const float* t) {
   float3 prev = T;
   float L = 0.0f;
@@ -2651,7 +2651,7 @@ __device__ __forceinline__ float chain_len32(const WedgeF* W, int m, float3 T, f
   float3 d = f3(R.x - prev.x, R.y - prev.y, R.z - prev.z);
   return L + sqrtf(fdot3(d, d));
 }
-__device__ int keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, float step_tol) {
+__device__ bool keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, float step_tol) {
   for (int i = 0; i < m; ++i) t[i] = 0.5f * W[i].len;
   float Lc = chain_len32(W, m, T, R, t);
   for (int it = 0; it < 30; ++it) {
@@ -2659,14 +2659,11 @@ __device__ int keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, fl
     X[0] = T;
     for (int i = 0; i < m; ++i) X[i + 1] = edge_point(W[i], t[i]);
     X[m + 1] = R;
-    float serr[4], g[3] = {0.0f, 0.0f, 0.0f}, H[3][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
+    float g[3] = {0.0f, 0.0f, 0.0f}, H[3][3] = {{0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f}};
     for (int j = 0; j <= m; ++j) {
       float3 d = f3(X[j + 1].x - X[j].x, X[j + 1].y - X[j].y, X[j + 1].z - X[j].z);
       float l = sqrtf(fdot3(d, d));
-      if (!(l > 0.0f)) return 0;
-      // rounding of this leg's direction (as in keller_on_edge)
-      serr[j] = 2e-5f + 2e-6f * (fabsf(X[j].x) + fabsf(X[j].y) + fabsf(X[j].z) + fabsf(X[j + 1].x) +
-                                 fabsf(X[j + 1].y) + fabsf(X[j + 1].z)) / l;
+      if (!(l > 0.0f)) return false;
       float3 u = f3(d.x / l, d.y / l, d.z / l);
       int ia = j - 1, ib = j;
       float ca = ia >= 0 ? fdot3(W[ia].e, u) : 0.0f, cb = ib < m ? fdot3(W[ib].e, u) : 0.0f;
@@ -2684,23 +2681,9 @@ __device__ int keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, fl
         H[ib][ia] += h;
       }
     }
-    float cut = 0.0f;
-    for (int i = 0; i < m; ++i) {
-      const float err = serr[i] + serr[i + 1], far = fmaxf(fabsf(t[i]), fabsf(W[i].len - t[i]));
-      cut += fminf(-g[i] * t[i], g[i] * (W[i].len - t[i])) - err * far;
-    }
-    if (cut > 0.0f) return -1;
     float gmax = 0.0f;
-    bool bound = false;
-    for (int i = 0; i < m; ++i) {
-      if ((t[i] <= -kKellerBox && g[i] > 0.0f) || (t[i] >= W[i].len + kKellerBox && g[i] < 0.0f)) {
-        bound = true;  // held at the bound
-        g[i] = 0.0f;
-        for (int j = 0; j < m; ++j) H[i][j] = H[j][i] = i == j ? 1.0f : 0.0f;
-      }
-      gmax = fmaxf(gmax, fabsf(g[i]));
-    }
-    if (gmax < 2e-6f) return bound ? 0 : 1;
+    for (int i = 0; i < m; ++i) gmax = fmaxf(gmax, fabsf(g[i]));
+    if (gmax < 2e-6f) return true;
     float A[3][4], dx[3];
     for (int i = 0; i < m; ++i) {
       for (int j = 0; j < m; ++j) A[i][j] = H[i][j];
@@ -2710,7 +2693,7 @@ __device__ int keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, fl
       int piv = c;
       for (int r = c + 1; r < m; ++r)
         if (fabsf(A[r][c]) > fabsf(A[piv][c])) piv = r;
-      if (!(fabsf(A[piv][c]) > 1e-30f)) return 0;
+      if (!(fabsf(A[piv][c]) > 1e-30f)) return false;
       if (piv != c)
         for (int j = 0; j <= m; ++j) {
           float x = A[c][j];
@@ -2732,7 +2715,7 @@ __device__ int keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, fl
     float step = 1.0f, tn[3] = {t[0], t[1], t[2]};
     bool moved = false;
     for (int q = 0; q < 30; ++q) {
-      for (int i = 0; i < m; ++i) tn[i] = fminf(fmaxf(t[i] + step * dx[i], -kKellerBox), W[i].len + kKellerBox);
+      for (int i = 0; i < m; ++i) tn[i] = t[i] + step * dx[i];
       float Ln = chain_len32(W, m, T, R, tn);
       if (Ln <= Lc * (1.0f + 1e-6f)) {
         Lc = fminf(Lc, Ln);
@@ -2741,13 +2724,13 @@ __device__ int keller32(const WedgeF* W, int m, float3 T, float3 R, float* t, fl
       }
       step *= 0.5f;
     }
-    if (!moved) return gmax < 1e-4f && !bound ? 1 : 0;
+    if (!moved) return gmax < 1e-4f;
     for (int i = 0; i < m; ++i) t[i] = tn[i];
     // the full Newton step (the quadratic model's distance to the
     // stationary point) below step_tol: close enough for the margins
-    if (dfull < step_tol && !bound) return 1;
+    if (dfull < step_tol) return true;
   }
-  return 0;
+  return false;
 }
 
 // Position margin of the FP32 Keller estimate: 5 cm plus 1e-5 of the
@@ -2829,10 +2812,8 @@ __device__ __noinline__ bool leg_surely_blocked(const Bvh& bvh, float3 o, float3
 // reject anything.
 __device__ __noinline__ bool chain_possible(const WedgeF* W, int m, float3 T, float3 R, float* t, bool* solved) {
   float mt = chain_margin(T, R);
-  const int kr = keller32(W, m, T, R, t, 0.1f * mt);
-  *solved = kr > 0;
-  if (kr < 0) return false;
-  if (kr == 0) return true;
+  *solved = keller32(W, m, T, R, t, 0.1f * mt);
+  if (!*solved) return true;
   float3 X[5];
   X[0] = T;
   for (int i = 0; i < m; ++i) {
@@ -3147,7 +3128,7 @@ __device__ __forceinline__ void keller_start(const Wedge* const* E, int m, d3w T
   float tf[3];
   for (int i = 0; i < m; ++i) W[i] = wedge_f(*E[i]);
   const bool ok =
-      keller32(W, m, f3((float)T.x, (float)T.y, (float)T.z), f3((float)R.x, (float)R.y, (float)R.z), tf, 1e-3f) > 0;
+      keller32(W, m, f3((float)T.x, (float)T.y, (float)T.z), f3((float)R.x, (float)R.y, (float)R.z), tf, 1e-3f);
   for (int i = 0; i < m; ++i) t[i] = ok ? (double)tf[i] : 0.5 * E[i]->len;
 }
 
