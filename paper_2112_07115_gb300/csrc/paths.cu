@@ -4590,7 +4590,9 @@ __global__ void __launch_bounds__(256) k_diffract_pre(PathArgs a, int nlinks) {
 // (see utd_parts), survivor i goes to block i mod grid, slot i / grid, and the
 // slots fill the warps one group at a time. More than two rounds of groups on
 // every SM (a highway with two reflections: 266 survivors an SM) keep the
-// instruction pipes busy; there a survivor takes one lane.
+// instruction pipes busy; there a survivor takes one lane, and the slots fill
+// one warp after the other (spread over the warps, every warp instruction of
+// the FP64 pipe had a few lanes: 767 us for that highway, so 548).
 constexpr int kDiffThreads = 256;
 __global__ void __launch_bounds__(kDiffThreads) k_diffract(PathArgs a) {
   extern __shared__ int sstk[];
@@ -4603,7 +4605,7 @@ __global__ void __launch_bounds__(kDiffThreads) k_diffract(PathArgs a) {
   const unsigned lanes = n > 2 * kDiffThreads / kDiffLanes * gridDim.x ? 1 : kDiffLanes;
   if (threadIdx.x == 0) diff_lanes = (int)lanes;
   __syncthreads();
-  const unsigned slot = (threadIdx.x & 31) / lanes * kWarps + (threadIdx.x >> 5);
+  const unsigned slot = lanes == 1 ? threadIdx.x : (threadIdx.x & 31) / lanes * kWarps + (threadIdx.x >> 5);
   for (unsigned i = blockIdx.x + gridDim.x * slot; i < n; i += gridDim.x * (kDiffThreads / lanes)) {
     const unsigned long long c = a.dexact[i];
     const unsigned kind = (unsigned)(c >> kKindShift);

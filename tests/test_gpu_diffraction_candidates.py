@@ -1,4 +1,6 @@
-"""How many diffraction candidates reach the FP64 stage, on the GPU."""
+"""How many diffraction candidates reach the FP64 stage, and the forms that
+stage takes with their number, on the GPU."""
+import numpy as np
 import pytest
 
 from paper_2112_07115_gb300 import dcem, scenes
@@ -38,4 +40,38 @@ def test_chains_off_their_edges_are_dropped_in_fp32(stream, vehicles, length, or
     s = _scene(stream, sc, order, refl)
     f = s.trace(sc.tx, sc.rx[0], P.gpu_params(sc))
     assert 0 < f.stats["diff_candidates"] <= 1.1 * count
+    s.close()
+
+
+def _ids(p):
+    p = p[p["ray"] < 0]
+    return sorted((int(q["depth"]), *q["tri"].tolist(), q["len_m"], q["amp_re"], q["amp_im"]) for q in p)
+
+
+@pytest.mark.parametrize("where,nrx,order,refl", [("city", 64, 1, 2), ("city", 64, 2, 2), ("city", 600, 1, 2),
+                                                  ("road", 200, 1, 2)])
+def test_forms_of_the_exact_stage_agree(stream, where, nrx, order, refl):
+    """A receiver alone has few candidates: none is tested for occlusion and
+    each takes four lanes. The 64 receivers' go through the occlusion test; the
+    600 receivers', and without that test the road's, take one lane each. The
+    paths are the same, bit for bit."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    sc = scenes.city_blocks(n_rx=nrx) if where == "city" else scenes.highway(n_frames=1)
+    s = _scene(stream, sc, order, refl)
+    prm = P.gpu_params(sc, max_refl=3)
+    rx = np.asarray(sc.rx[0])
+    assert rx.shape[0] == nrx
+    whole = s.trace(sc.tx, rx, prm)
+    n = whole.stats["diff_candidates"]
+    one_lane = where == "road" or nrx > 64
+    assert (n > 128 * sms) == one_lane
+    alone = 0
+    for r in range(nrx):
+        one = s.trace(sc.tx, rx[r:r + 1], prm)
+        assert one.stats["diff_candidates"] < 64 * sms
+        alone += one.stats["diff_candidates"]
+        assert _ids(one.paths) == _ids(whole.paths[whole.paths["rx"] == r]), r
+    # the candidates are the receivers' own: untested there are as many together as alone, tested fewer
+    assert alone > 64 * sms and (alone > n if where == "city" else alone == n)
     s.close()
