@@ -304,6 +304,7 @@ struct dcem_scene {
   unsigned* vis = nullptr;     // ... what each end point may see (k_refl_visible), and its words
   size_t vis_cap = 0;
   int nrp = 0;
+  bool open = false;               // ... little is hidden in this scene (measure_open)
   int diff_refl = 0;               // reflections with diffraction (0..3, see the header)
   unsigned* rmask = nullptr;   // two reflections: the pre-test's wedge masks, and their words
   size_t rmask_cap = 0;
@@ -1764,6 +1765,33 @@ int dcem_scene_set_diffraction(dcem_scene* s, int32_t on, int32_t* n_wedges) {
   return DCEM_OK;
 }
 
+// Whether the scene is open (dcem_scene::open), once its planes are there. The
+// survivor list, unused between frames, takes the counts.
+static int measure_open(dcem_scene* s, bool* open) {
+  if (!s->dsurv) return DCEM_OK;
+  PathArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.bvh.nodes = s->nodes;
+  a.bvh.tris = s->tris;
+  a.bvh.root0 = s->root_h[0];
+  a.bvh.root1 = kEmpty;
+  a.bvh.max_visits = 2 * (s->nint_s + s->ns) + 8;
+  a.bvh.nnodes = s->nint_s + s->nint_d;
+  a.bvh.ntris = s->ntri;
+  a.quads = s->quads;
+  a.rplanes = s->rplanes;
+  a.nrp = s->nrp;
+  dcem_params p;
+  dcem_params_default(&p);
+  a.eps_occ = p.eps_occ;
+  unsigned n[2] = {0, 0};
+  CK(launch_hidden_planes(a, reinterpret_cast<unsigned*>(s->dsurv), s->st));
+  CK(cudaMemcpyAsync(n, s->dsurv, sizeof(n), cudaMemcpyDeviceToHost, s->st));
+  CK(cudaStreamSynchronize(s->st));
+  *open = n[0] * kOpenDen <= n[1] * kOpenNum;
+  return DCEM_OK;
+}
+
 int dcem_scene_set_diffraction_reflections(dcem_scene* s, int32_t on, int32_t* n_planes) {
   if (!s || on < 0 || on > 3) return DCEM_ERR_ARG;
   if (on && !s->diffraction) return DCEM_ERR_STATE;
@@ -1778,6 +1806,8 @@ int dcem_scene_set_diffraction_reflections(dcem_scene* s, int32_t on, int32_t* n
       CK(upload(&s->rkeys, keys));
       CK(upload(&s->rplanes, planes));
       s->nrp = (int)planes.size();
+      const int rc = measure_open(s, &s->open);
+      if (rc != DCEM_OK) return rc;
     }
   }
   s->diff_refl = on;
@@ -2077,6 +2107,7 @@ static void make_plan(dcem_scene* s, int nrx, const dcem_params* p, bool coheren
   q.rmembers = dr ? s->rmembers : nullptr;
   q.rkeys = dr ? s->rkeys : nullptr;
   q.nrp = dr ? s->nrp : 0;
+  q.open = dr && s->open ? 1 : 0;
   const bool uv = uses_vis(s);
   q.quads = uv ? s->quads : nullptr;
   q.vis_any = uv ? s->vis : nullptr;

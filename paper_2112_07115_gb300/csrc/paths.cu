@@ -2252,10 +2252,8 @@ __device__ __noinline__ bool surely_hidden(const PathArgs& a, const HiddenCase& 
 // Per end point the planes, then the wedges (in the order wperm) it may see,
 // one warp per word. A wedge the end point is inside of is not seen. Both
 // orders are spatial, so that a warp's legs run close together. Without
-// `test` everything else counts as seen: scenes with few planes (a road and
-// its barriers) are open, and a highway's 480,000 legs of up to 2 km cost 240
-// us a frame and hid nothing.
-constexpr int kOpenPlanes = 16;
+// `test` everything else counts as seen: a road and its barriers are open, and
+// a highway's 480,000 legs of up to 2 km cost 240 us a frame and hid nothing.
 // Neither do they pay for one reflection without chains, whose candidates are
 // cheap to form: 8 x 8 city blocks with 10, 30 and 60 receivers 542, 587 and
 // 648 us a frame with the tests, 365, 453 and 531 without.
@@ -2288,6 +2286,34 @@ __global__ void __launch_bounds__(64) k_diff_visible(PathArgs a, int ntx, bool t
     if (lane == 0) a.vis[it] = m;
   }
 }
+// Pairs of up to kHiddenSample planes: is the one's box hidden from the
+// other's middle? One warp per plane, once per scene (the static triangles do
+// not move).
+constexpr int kHiddenSample = 64;
+__global__ void __launch_bounds__(32) k_hidden_planes(PathArgs a, unsigned* cnt) {
+  extern __shared__ int sstk[];
+  TStack st;
+  bind_stack(st, sstk, kStackTrace);
+  const int n = min(a.nrp, kHiddenSample), lane = threadIdx.x;
+  const int p = (int)((long)blockIdx.x * a.nrp / n);
+  const float* b = a.rplanes[p].box;
+  const float3 E = f3(0.5f * (b[0] + b[3]), 0.5f * (b[1] + b[4]), 0.5f * (b[2] + b[5]));
+  for (int k0 = 0; k0 < n; k0 += 32) {
+    const int k = k0 + lane;
+    const bool in = k < n && k != (int)blockIdx.x;
+    bool hidden = false;
+    if (in) {
+      const float* c = a.rplanes[(int)((long)k * a.nrp / n)].box;
+      hidden = surely_hidden(a, HiddenCase{0, E, E, f3(c[0], c[1], c[2]), f3(c[3], c[4], c[5])}, st);
+    }
+    const unsigned h = __popc(__ballot_sync(0xffffffffu, hidden)), m = __popc(__ballot_sync(0xffffffffu, in));
+    if (lane == 0) {
+      atomicAdd(&cnt[0], h);
+      atomicAdd(&cnt[1], m);
+    }
+  }
+}
+
 // The wedges some transmitter (words 0 .. nwc - 1) or some receiver sees, and
 // lists of the groups that hold any (per side a count, then the groups).
 __global__ void __launch_bounds__(256) k_diff_visible_any(PathArgs a, int ntx) {
@@ -2337,7 +2363,7 @@ __device__ __forceinline__ bool end_sees(const PathArgs& a, int x, int w) { retu
 // a frame took 5.0 ms, so and with planes hidden from an end left out
 // 3.2); not in open scenes.
 __device__ __forceinline__ bool hidden_in_relation(const PathArgs& a) {
-  return a.diff_order >= 3 || a.nrpr > kOpenPlanes;
+  return a.diff_order >= 3 || (a.nrpr > 0 && !a.open);
 }
 __device__ __forceinline__ bool wedges_hidden(const PathArgs& a, const WedgeF& A, const WedgeF& B, TStack& st) {
   HiddenCase h;
@@ -4861,6 +4887,13 @@ cudaError_t launch_dedupe(const PathArgs& a, int grid, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+cudaError_t launch_hidden_planes(const PathArgs& a, unsigned* cnt, cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned), st);
+  if (e != cudaSuccess || a.nrp <= 0) return e;
+  k_hidden_planes<<<std::min(a.nrp, kHiddenSample), 32, 32 * kStackTrace * sizeof(int), st>>>(a, cnt);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_diffract(const PathArgs& args, int nlinks, int sms, cudaStream_t st) {
   PathArgs a = args;
   if (!a.wedges || a.nw <= 0) return cudaSuccess;
@@ -4869,7 +4902,7 @@ cudaError_t launch_diffract(const PathArgs& args, int nlinks, int sms, cudaStrea
     k_wedge_boxes<<<(a.nw + 255) / 256, 256, 0, st>>>(a.wf, a.wperm, a.nw, a.wgbox);
   if (nlinks > 0) {
     if (a.vis) {  // what the end points see: with reflector planes or chains
-      const bool test = a.nrp == 0 || (a.nrp > kOpenPlanes && (a.drefl2 || a.diff_order >= 2));
+      const bool test = a.nrp == 0 || (!a.open && (a.drefl2 || a.diff_order >= 2));
       const long nvis = (long)(nlinks / a.nrx + a.nrx) * ((a.nrp + 31) / 32 + a.nwc);
       k_diff_visible<<<(int)std::min<long>((nvis + 1) / 2, 16L * sms), 64, 64 * kStackTrace * sizeof(int), st>>>(
           a, nlinks / a.nrx, test);
@@ -4896,7 +4929,7 @@ cudaError_t launch_diffract(const PathArgs& args, int nlinks, int sms, cudaStrea
         k_refl_lists<<<warps(lists * parts(lists)), 256, 0, st>>>(a, ntx, parts(lists));
         k_refl_join<<<warps((long)ntx * a.nrp * a.nwc * kJoinParts), 256, 0, st>>>(a, ntx, nlinks);
         auto items = [&] { return ((long)ntx * a.rsub + a.nrx) * a.nrp * a.nrp; };
-        if (a.nrp <= kOpenPlanes && nlinks <= 2 * (ntx + a.nrx)) {
+        if (a.open && nlinks <= 2 * (ntx + a.nrx)) {
           k_refl_direct<<<warps(2L * nlinks * a.nrp * a.nrp), 256, 0, st>>>(a, ntx, nlinks);
         } else {
           if (items() > 32 * room) a.rsub = std::max(1, a.rsub / 4);
@@ -4906,6 +4939,7 @@ cudaError_t launch_diffract(const PathArgs& args, int nlinks, int sms, cudaStrea
       }
     }
     PathArgs b = a;  // chains: transmitters, and the reflector planes applied to them
+    if (a.open) b.vis = nullptr;  // nothing to look up: the rows hold what the pre-tests know
     b.dntx = nlinks / a.nrx;
     b.nrpr = a.rplanes && a.diff_order >= 2 ? a.nrp : 0;
     if (a.diff_order >= 2 && a.nw > 1) {
@@ -4928,7 +4962,7 @@ cudaError_t launch_diffract(const PathArgs& args, int nlinks, int sms, cudaStrea
       k_diff_multi_pre<<<8 * sms, 256, 256 * kStackTrace * sizeof(int), st>>>(b);
     }
     k_diff_unblocked<<<8 * sms, 64, 64 * kStackTrace * sizeof(int), st>>>(
-        b, nlinks, a.rplanes && a.nrp > 0 && a.nrp <= kOpenPlanes);
+        b, nlinks, a.open != 0);
     k_diffract<<<sms, kDiffThreads, kDiffThreads * kStackTrace * sizeof(int), st>>>(b);
   }
   return cudaGetLastError();

@@ -73,6 +73,7 @@ struct PathArgs {
   int nrp;
   const float4* quads;            // per triangle id: the convex wall quad it is part of (corners; .w of
                                   // the first 0: none)
+  int open;                       // 1: an open scene, little of which is hidden (launch_hidden_planes)
   int rsub;                       // runs of receivers per transmitter item (set by launch_diffract)
   unsigned* vis;                  // per end point: bits of the planes, then of the wedges it may see
   unsigned* vis_any;              // the wedges some transmitter, then some receiver may see
@@ -142,6 +143,18 @@ cudaError_t launch_validate(const PathArgs& a, int nlinks, int grid, cudaStream_
 // The table of this frame's distinct keys for the next frame's validation
 // reuse (after validation, before diffraction adds its records).
 cudaError_t launch_vcache_build(const PathArgs& a, int grid, cudaStream_t st);
+// How much of a scene its walls hide: of cnt[1] sampled pairs of reflector
+// planes cnt[0] are hidden from each other (a: the static tree, quads, planes,
+// eps_occ). Open scenes, with at most kOpenNum in kOpenDen of them, go without
+// visibility and occlusion tests, and test both reflections on one side of a
+// wedge link by link. Roads: 0 (barriers in one piece) to 30% (in twenty, each
+// a little further out), 2 x 2 city blocks 30%, 3 x 3 41%, 4 x 4 54%, 8 x 8 75%.
+// us a frame, open / with tests, two reflections and chains of two with one:
+// road in eight pieces 2706 / 5263 and 5142 / 5209, 2 x 2 355 / 426 and 344 /
+// 435, 3 x 3 (60 receivers) 866 / 790 and 554 / 706, 5 x 5 1752 / 1158 and 880
+// / 1026, 8 x 8 14456 / 2376 and 5594 / 3337.
+constexpr unsigned kOpenNum = 3, kOpenDen = 8;
+cudaError_t launch_hidden_planes(const PathArgs& a, unsigned* cnt, cudaStream_t st);
 // First-order edge diffraction paths of every (link, wedge) (after validation).
 cudaError_t launch_diffract(const PathArgs& a, int nlinks, int sms, cudaStream_t st);
 // Per-link sums and ordered output; more links than kScanLinks take their

@@ -34,6 +34,11 @@ extern "C" void fake_check_paths(const char* k, const void* args) {
   };
   auto has = [&](const char* s) { return std::strstr(k, s) != nullptr; };
   const size_t nw = (size_t)a.nw;
+  if (has("k_hidden_planes")) {  // (a set-up kernel: no frame's buffers)
+    need(a.quads, 4 * sizeof(float4) * (size_t)a.bvh.ntris, "wall quads");
+    need(a.rplanes, sizeof(RPlane) * (size_t)a.nrp, "planes");
+    return;
+  }
   need(a.ctr, sizeof(DevCounters), "counters");
   need(a.uniq, sizeof(int) * (size_t)a.ucap, "distinct keys");
   need(a.prec, sizeof(PathRec) * (size_t)a.ucap, "records");

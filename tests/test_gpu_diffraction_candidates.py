@@ -75,3 +75,35 @@ def test_forms_of_the_exact_stage_agree(stream, where, nrx, order, refl):
     # the candidates are the receivers' own: untested there are as many together as alone, tested fewer
     assert alone > 64 * sms and (alone > n if where == "city" else alone == n)
     s.close()
+
+
+def _road(pieces):
+    """The highway with its barriers in `pieces` stretches, each a little further out: more planes, no more walls."""
+    sc = scenes.highway(n_frames=1, n_vehicles=100, n_rays=5_000)
+    t = np.array(sc.tris, np.float32).reshape(-1, 3, 3)
+    wall = (np.asarray(sc.tri_obj) < 0) & (t[:, :, 2].max(1) > 0.1)
+    k = np.minimum((t[:, :, 0].mean(1) / 2000.0 * pieces).astype(int), pieces - 1)
+    t[wall, :, 1] += 0.1 * k[wall, None]
+    sc.tris = t.reshape(np.asarray(sc.tris).shape)
+    return sc
+
+
+@pytest.mark.parametrize("where", ["road", "road in pieces", "city"])
+def test_open_scenes_are_told_by_what_their_walls_hide(stream, where):
+    """Whether the tests of what is hidden are made depends on how much is, not
+    on the number of planes: not along a road, however many pieces its barriers
+    have, but among buildings. (Untested, the receivers have as many candidates
+    together as alone.)"""
+    sc = scenes.city_blocks(n=4, n_rx=100) if where == "city" else _road(8 if "pieces" in where else 1)
+    s = _scene(stream, sc, 1, 2)
+    prm = P.gpu_params(sc, max_refl=3)
+    rx = np.asarray(sc.rx[0])
+    whole = s.trace(sc.tx, rx, prm)
+    alone = 0
+    for r in range(rx.shape[0]):
+        one = s.trace(sc.tx, rx[r:r + 1], prm)
+        alone += one.stats["diff_candidates"]
+        assert _ids(one.paths) == _ids(whole.paths[whole.paths["rx"] == r]), r
+    n = whole.stats["diff_candidates"]
+    assert n < alone if where == "city" else n == alone
+    s.close()
