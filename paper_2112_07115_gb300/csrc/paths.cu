@@ -4614,11 +4614,13 @@ __global__ void __launch_bounds__(256) k_diffract_pre(PathArgs a, int nlinks) {
 // the time is the longest lane's chain of dependent operations plus the
 // other lanes' divergent branches: so a survivor takes a group of four lanes
 // (see utd_parts), survivor i goes to block i mod grid, slot i / grid, and the
-// slots fill the warps one group at a time. More than two rounds of groups on
-// every SM (a highway with two reflections: 266 survivors an SM) keep the
-// instruction pipes busy; there a survivor takes one lane, and the slots fill
-// one warp after the other (spread over the warps, every warp instruction of
-// the FP64 pipe had a few lanes: 767 us for that highway, so 548).
+// slots fill the warps one group at a time. More survivors than an SM holds
+// groups of (64) keep the instruction pipes busy; there a survivor takes one
+// lane, and the slots fill one warp after the other (spread over the warps,
+// every warp instruction of the FP64 pipe had a few lanes: 767 us for a
+// highway with two reflections, 276 survivors an SM, so 548). With 60 an SM
+// (the highway with one) a frame takes 859 us on four lanes, 950 on one; with
+// 105 (60 vehicles, four transmitters, two reflections) 1524 and 1344.
 constexpr int kDiffThreads = 256;
 __global__ void __launch_bounds__(kDiffThreads) k_diffract(PathArgs a) {
   extern __shared__ int sstk[];
@@ -4628,7 +4630,7 @@ __global__ void __launch_bounds__(kDiffThreads) k_diffract(PathArgs a) {
   const double k = 2.0 * M_PI * a.freq / 299792458.0, lam = 299792458.0 / a.freq;
   unsigned ovf = 0;
   constexpr unsigned kWarps = kDiffThreads / 32;
-  const unsigned lanes = n > 2 * kDiffThreads / kDiffLanes * gridDim.x ? 1 : kDiffLanes;
+  const unsigned lanes = n > kDiffThreads / kDiffLanes * gridDim.x ? 1 : kDiffLanes;
   if (threadIdx.x == 0) diff_lanes = (int)lanes;
   __syncthreads();
   const unsigned slot = lanes == 1 ? threadIdx.x : (threadIdx.x & 31) / lanes * kWarps + (threadIdx.x >> 5);
