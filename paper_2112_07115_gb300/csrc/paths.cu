@@ -4380,7 +4380,7 @@ __device__ __forceinline__ bool diff_blocked(const PathArgs& a, int nlinks, unsi
   return false;
 }
 
-__global__ void __launch_bounds__(64) k_diff_unblocked(PathArgs a, int nlinks, bool open) {
+__global__ void __launch_bounds__(64) k_diff_unblocked(PathArgs a, int nlinks, unsigned few) {
   extern __shared__ int sstk[];
   TStack st;
   bind_stack(st, sstk, kStackTrace);
@@ -4389,15 +4389,10 @@ __global__ void __launch_bounds__(64) k_diff_unblocked(PathArgs a, int nlinks, b
   // few candidates: a few lanes of every warp, so that all SMs share the
   // traversals' latency; many: full warps of consecutive candidates (which
   // come from one warp above, so their legs run close together)
-  // Up to 64 candidates an SM all go on: the exact stage takes them side by
-  // side and its time is one candidate's either way, while the longest of the
-  // legs here takes 50 us (1113 candidates on a highway, of which 472 would
-  // stay: 1016 us for two frames with the test, 935 without; 1643 in an 8 x 8
-  // city, of which 227 would stay: 638 and 640).
-  // So do all of an open scene's, nearly none of which is blocked. They keep
-  // their order, in which survivors of one kind stand together: the exact
-  // stage's warps then run one kind's code.
-  if (n <= 8u * gridDim.x || open) {
+  // Up to `few` candidates all go on (diff_few). They keep their order, in
+  // which survivors of one kind stand together: the exact stage's warps then
+  // run one kind's code.
+  if (n <= few) {
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) a.dexact[i] = a.dsurv[i];
     if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr->n_dexact = n;
     return;
@@ -4889,6 +4884,20 @@ cudaError_t launch_dedupe(const PathArgs& a, int grid, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// Candidates that go to the exact stage without the occlusion test. The stage
+// takes a few an SM side by side, its time is one candidate's either way, and
+// the longest of the legs here takes 50 us; a wall in every other leg makes the
+// test pay from 16 candidates an SM on (us a frame with lines at 0, 16 and 64:
+// 4 x 4 city blocks, 12 candidates an SM 661, 691, 683, 20 an SM 784, 785, 810;
+// 5 x 5, two wedges, 25 an SM 1371, 1376, 1486; 3 x 3, 2 an SM 325, 305, 303).
+// Open scenes' legs are hardly ever blocked: none is tested. Without reflector
+// planes there is no telling: 64 (a highway, chains of two, 26 an SM: 2722 with
+// the line at 16, 2632 at 64; 2 km with 16 transmitters, 24 an SM: 481 and 424).
+static unsigned diff_few(const PathArgs& a, int sms) {
+  if (a.open) return 0xffffffffu;
+  return (unsigned)sms * (a.nrp > 0 ? 16u : 64u);
+}
+
 cudaError_t launch_hidden_planes(const PathArgs& a, unsigned* cnt, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned), st);
   if (e != cudaSuccess || a.nrp <= 0) return e;
@@ -4963,8 +4972,7 @@ cudaError_t launch_diffract(const PathArgs& args, int nlinks, int sms, cudaStrea
       }
       k_diff_multi_pre<<<8 * sms, 256, 256 * kStackTrace * sizeof(int), st>>>(b);
     }
-    k_diff_unblocked<<<8 * sms, 64, 64 * kStackTrace * sizeof(int), st>>>(
-        b, nlinks, a.open != 0);
+    k_diff_unblocked<<<8 * sms, 64, 64 * kStackTrace * sizeof(int), st>>>(b, nlinks, diff_few(a, sms));
     k_diffract<<<sms, kDiffThreads, kDiffThreads * kStackTrace * sizeof(int), st>>>(b);
   }
   return cudaGetLastError();
