@@ -354,7 +354,10 @@ __device__ __forceinline__ R3 r3(double x, double y, double z) { return R3{x, y,
 __device__ __forceinline__ R3 operator+(R3 a, R3 b) { return r3(a.x + b.x, a.y + b.y, a.z + b.z); }
 __device__ __forceinline__ R3 operator-(R3 a, R3 b) { return r3(a.x - b.x, a.y - b.y, a.z - b.z); }
 __device__ __forceinline__ R3 operator*(R3 a, double s) { return r3(a.x * s, a.y * s, a.z * s); }
-__device__ __forceinline__ double rdot(R3 a, R3 b) { return fma(a.z, b.z, fma(a.y, b.y, a.x * b.x)); }
+// (not fused: path lengths stay equal to those of a plain FP64 evaluation, and
+// the phase is 600 radians a metre; fused, the gradient case's powers and
+// derivatives were 3.7 and 2.3 times as far from one, in the same time)
+__device__ __forceinline__ double rdot(R3 a, R3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 __device__ __forceinline__ R3 rcross(R3 a, R3 b) {
   return r3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
 }
