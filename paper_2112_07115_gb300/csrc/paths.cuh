@@ -148,7 +148,8 @@ cudaError_t launch_vcache_build(const PathArgs& a, int grid, cudaStream_t st);
 // eps_occ). Open scenes, with at most kOpenNum in kOpenDen of them, go without
 // visibility and occlusion tests, and test both reflections on one side of a
 // wedge link by link. Roads: 0 (barriers in one piece) to 30% (in twenty, each
-// a little further out), 2 x 2 city blocks 30%, 3 x 3 41%, 4 x 4 54%, 8 x 8 75%.
+// a little further out), 2 x 2 city blocks 30 and 33%, 3 x 3 44 and 47%, 4 x 4
+// 55 and 58%, 8 x 8 76 and 78% (two seeds each), an urban grid 97%.
 // us a frame, open / with tests, two reflections and chains of two with one:
 // road in eight pieces 2706 / 5263 and 5142 / 5209, 2 x 2 355 / 426 and 344 /
 // 435, 3 x 3 (60 receivers) 866 / 790 and 554 / 706, 5 x 5 1752 / 1158 and 880
