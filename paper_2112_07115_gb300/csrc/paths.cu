@@ -2348,14 +2348,6 @@ __device__ __forceinline__ bool sees_wedge(const PathArgs& a, int x, int i) {
 
 // (as sees_wedge, for wedge w; true when the rows are not built)
 __device__ __forceinline__ bool end_sees(const PathArgs& a, int x, int w) { return !a.vis || sees_wedge(a, x, a.wplace[w]); }
-// Are wedges hidden from each other left out of the relation? For chains of
-// three, and where the transmitters' images in many planes would each test
-// the same pairs again (8 x 8 city, order 2 with one reflection, 321 planes:
-// a frame took 5.0 ms, so and with planes hidden from an end left out
-// 3.2); not in open scenes.
-__device__ __forceinline__ bool hidden_in_relation(const PathArgs& a) {
-  return a.diff_order >= 3 || (a.nrpr > 0 && !a.open);
-}
 __device__ __forceinline__ bool wedges_hidden(const PathArgs& a, const WedgeF& A, const WedgeF& B, TStack& st) {
   HiddenCase h;
   h.kind = 2;
@@ -2370,8 +2362,9 @@ __device__ __forceinline__ bool wedges_hidden(const PathArgs& a, const WedgeF& A
 // exterior; one bit per ordered pair (w1, w2) in a.drel. It is symmetric: a
 // warp takes 32 pairs w1 < w2 of one w1 and sets both bits. With chains of
 // three wedges the pairs hidden from each other are dropped here (every
-// triple holds two; 8 x 8 city: 335k triples become a tenth), with chains of
-// two where hidden_in_relation says so.
+// triple holds two; 8 x 8 city: 335k triples become a tenth). With chains of
+// two that costs more than it saves: 8 x 8, 5 x 5 and 3 x 3 city blocks with
+// one reflection 2910, 991 and 694 us a frame with it, 2703, 860 and 642 without.
 __global__ void __launch_bounds__(256) k_diff_rel(PathArgs a) {
   extern __shared__ int sstk[];
   TStack st;
@@ -2390,7 +2383,7 @@ __global__ void __launch_bounds__(256) k_diff_rel(PathArgs a) {
       edge_ends(fb, pb, qb);
       const float m = fmaxf(fmaxf(pre_margin_m(pa), pre_margin_m(qa)), fmaxf(pre_margin_m(pb), pre_margin_m(qb)));
       rel = edge_sees(fa, fb, m) && edge_sees(fb, fa, m);
-      if (rel && hidden_in_relation(a)) rel = !wedges_hidden(a, fa, fb, st);
+      if (rel && a.diff_order >= 3) rel = !wedges_hidden(a, fa, fb, st);
     }
     if (rel) {
       const Wedge &A = a.wedges[w1], &B = a.wedges[w2];
@@ -2411,8 +2404,8 @@ __global__ void __launch_bounds__(256) k_diff_rel(PathArgs a) {
 // the transmitter and edge 2 (keller_on_edge), and w1 (an image's plane) not
 // hidden from the transmitter. (No test here of whether w2 is hidden from w1:
 // the traversal took the kernel from 63 to 89 registers and 296 B of stack,
-// for every pair; without it 8 x 8 city blocks take 565 us a frame instead of
-// 682 at order 2, 2942 instead of 3337 with one reflection, and this kernel on
+// for every pair; without it 8 x 8 city blocks took 559 us a frame instead of
+// 682 at order 2, 2890 instead of 3283 with one reflection, and this kernel on
 // a 200-vehicle highway 810 us instead of 1190.)
 __global__ void __launch_bounds__(256) k_diff_pairs(PathArgs a, int nsrc) {
   const long nw = a.nw, total = (long)nsrc * nw * nw;
