@@ -608,7 +608,7 @@ int dcem_path_adjoint(dcem_scene* s, const float* tx, const float* rx, int32_t n
  * owns the whole device memory pool, or a real-time loop that must not call
  * cudaMalloc after start-up (an allocation can synchronise the device and
  * stall the loop). The caller passes the inputs and outputs; the scratch
- * lives in one fixed device array of the library (about 310 KB per device,
+ * lives in one fixed device array of the library (about 295 KB per device,
  * held from the first call on that device until the process exits).
  *   paths      device, n_paths records (e.g. the paths dcem_trace_frame
  *              wrote to a device result); order does not matter

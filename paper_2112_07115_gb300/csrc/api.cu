@@ -169,11 +169,11 @@ __global__ void k_ray_keys(const float4* __restrict__ d, int n, unsigned* keys, 
 // Order in which chunks of 32 sorted rays are taken: first those that stay
 // longest in the scene, by the length of a line along the chunk's middle ray
 // through the box of the scene, in octaves (within one the direction order
-// stays; in half octaves a city of 65,536 links took 4.60 ms, so 4.47). A ray's segments are one chain of dependent loads, so the
-// trace ends when the last long ray does: in direction order, the
-// million-ray highway's SMs had work for 258,000 of the kernel's 386,000
-// cycles on average (a frame 358 us, in this order 346). The last chunk may
-// be short and stays last.
+// stays; in half octaves a city of 65,536 links took 3% longer). A ray's
+// segments are one chain of dependent loads, so the trace ends when the last
+// long ray does: in direction order, the million-ray highway's SMs had work
+// for 258,000 of the kernel's 386,000 cycles on average, and a frame took 3%
+// longer. The last chunk may be short and stays last.
 __global__ void k_chunk_keys(const float4* __restrict__ rays, int n, const float* __restrict__ box, int has0,
                              int has1, unsigned* keys, unsigned* idx) {
   float e[3], diag = 0.0f;
@@ -282,7 +282,7 @@ struct dcem_scene {
   int4* q4_src = nullptr;        // node count and roots (rebuilt with the topology)
   int* q4_count = nullptr;
   int* q4_roots = nullptr;
-  int* q4_scr = nullptr;         // scratch of the 4-wide mapping of large trees
+  int* q4_scr = nullptr;         // scratch of the 4-wide mapping of trees above 17,000 nodes
   int* leaf_parent = nullptr;
   int* tri_obj_d = nullptr;  // triangle id -> rigid object (-1 static)
   std::vector<float> tris_h;   // input vertices (static ones are world space) and objects,
@@ -301,7 +301,7 @@ struct dcem_scene {
   int* rmembers = nullptr;     // ... their triangle ids and sort keys
   float* rkeys = nullptr;
   float4* quads = nullptr;     // ... and per triangle the wall quad it is part of (wall_quads)
-  unsigned* vis = nullptr;     // ... what each end point may see (k_refl_visible), and its words
+  unsigned* vis = nullptr;     // ... what each end point may see (k_diff_visible), and its words
   size_t vis_cap = 0;
   int nrp = 0;
   bool open = false;               // ... little is hidden in this scene (measure_open)
@@ -718,11 +718,10 @@ static bool uses_vis(const dcem_scene* s) {
 }
 // Results for host buffers: the reduction writes the link results (up to
 // kHostLinks links) and the first kHostRecs records into mapped host memory,
-// and the host copies them on once the frame has ended. With four
-// copies into pageable memory and a second synchronisation instead, a frame of
-// 8 links took 135 rather than 125 us, a coherent one 114 rather than 98; the
-// rest of a large frame's results still goes that way. 0.3 MB per scene, from
-// its first frame with host results on.
+// and the host copies them on once the frame has ended. With four copies into
+// pageable memory and a second synchronisation instead, a frame of 8 links took
+// 8% longer, a coherent one 16%; the rest of a large frame's results still goes
+// that way. 0.3 MB per scene, from its first frame with host results on.
 constexpr unsigned kHostRecs = 1024;
 constexpr int kHostLinks = 2048;
 
@@ -1103,12 +1102,12 @@ std::vector<float4> wall_quads(const std::vector<float>& tris, const std::vector
 // frame, so it is worth more than the linear builder gives: top-down binned
 // splits by the surface-area heuristic, in the linear builder's layout (one
 // triangle per leaf, root at node 0). Against the radix tree, 4-wide nodes per
-// segment: urban grid 18.0 -> 14.0 (closest hit 4.07 -> 3.47 ms), city 10.4 ->
-// 7.2, office 8.0 -> 6.9 (0.84 -> 0.72 ms). Not for long narrow scenes: there
-// the heuristic cuts across the narrow sides first, and the rays that graze
-// along the scene meet every one of the long boxes it leaves (the 2 km
-// highway: mean 8.8 -> 8.1 nodes, worst segment 74 -> 142, closest hit 0.18 ->
-// 0.23 ms; the radix tree halves all axes alike). kSahMax bounds the build time
+// segment: urban grid 18.0 -> 14.0 (closest hit 15% shorter), city 10.4 -> 7.2,
+// office 8.0 -> 6.9 (14%). Not for long narrow scenes: there the heuristic cuts
+// across the narrow sides first, and the rays that graze along the scene meet
+// every one of the long boxes it leaves (the 2 km highway: mean 8.8 -> 8.1
+// nodes, worst segment 74 -> 142, closest hit 28% longer; the radix tree halves
+// all axes alike). kSahMax bounds the build time
 // on the host (5 ms for 50,000 triangles on eight threads); kSahLevels the
 // internal levels, to those that two binary levels a 4-wide one may have
 // (kWideLevels): halving takes over where the triangles left would need the

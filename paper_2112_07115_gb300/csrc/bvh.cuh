@@ -127,14 +127,14 @@ cudaError_t launch_dyn_update(const DynUpdateArgs& a, cudaStream_t st);
 size_t dyn_update_smem(int nd, int nobj);
 
 // 4-wide compact copy: map the binary trees (nn internal nodes, 2 root codes)
-// to 4-wide nodes once per topology (one CTA, nn <= 8192), then encode the
-// child boxes every frame. n4 and the 4-wide roots stay on the device.
+// to 4-wide nodes once per topology (one CTA), then encode the child boxes
+// every frame. n4 and the 4-wide roots stay on the device.
 // 4-wide levels a tree may have whatever its boxes: a traversal leaves up to
 // three entries waiting per level, beside the other tree's root and the end
 // mark, and the least room of the closest-hit kernels holds them (8 shared
 // and 49 spilled entries against 2 + 3 x 18; tests/test_gpu_graded_scene.py).
-// A tree of more than twice as many binary levels, which the linear builder
-// only gives to thousands of triangles about one point, has half of those.
+// A tree of more than twice as many binary levels (the linear builder's have
+// up to 63) has half of those.
 constexpr int kWideLevels = 18;
 // Shared memory of the 4-wide mapping of nn binary internal nodes, or 0 when
 // it needs the global scratch (3 nn ints) instead.

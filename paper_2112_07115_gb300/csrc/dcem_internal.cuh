@@ -498,18 +498,17 @@ static __device__ __noinline__ int closest_hit_far(const Bvh bvh, const RayPre r
   return slot;
 }
 
-// 4-wide compact nodes (shared memory), 64 bytes each: words 0-11 = the axis
-// words of children 0-3 (x, y, z per child), words
-// 12-15 = the child codes (4-wide node index, leaf ~slot, or kEmpty with an
-// inverted box that no ray meets).
+// 4-wide compact nodes, 64 bytes each: words 0-11 = the axis words of children
+// 0-3 (x, y, z per child), words 12-15 = the child codes (4-wide node index,
+// leaf ~slot, or kEmpty with an inverted box that no ray meets).
 //
 // The traversal's arithmetic units are its limit (the ALU pipe, which takes
 // every minimum, selection and byte permutation, at 60% and the issue slots
 // at 72% in the office), so a step is written for few instructions: the four
 // entry distances carry their child's number in their last two bits, so that
 // ten integer minima and maxima sort them (25 instructions with the codes
-// swapped along), and the stack ends in a sentinel: 1020 -> 989 us a frame in
-// the office, 4.76 -> 4.64 ms in a city of 65,536 links.
+// swapped along), and the stack ends in a sentinel: 3% of a frame of the
+// office, 2.5% in a city of 65,536 links.
 struct QStack {
   int* s;
   int stride, end, at;        // words; end: of the shared entries
@@ -545,10 +544,10 @@ __device__ __forceinline__ int qkey(const QRay& q, unsigned wx, unsigned wy, uns
 
 // Closest hit as closest_hit(), over the 4-wide compact copy: per step the
 // four child boxes are tested, the hit ones ordered by entry distance, the
-// nearest visited next and the others pushed (pushed unsorted, the highway's
-// frame took 414 us instead of 407, the office's 1071 instead of 1057). Node visits count box pairs
-// (a 4-wide step = 2), the unit of the 2-wide traversals. kG: the copy is
-// read from global memory (read-only path) instead of shared memory.
+// nearest visited next and the others pushed (pushed unsorted, frames of the
+// highway and the office took 1 to 2% longer). Node visits count box pairs (a
+// 4-wide step = 2), the unit of the 2-wide traversals. kG: the copy is read
+// from global memory (read-only path) instead of shared memory.
 template <bool kG = false>
 __device__ __forceinline__ int closest_hit_q4(const uint4* qn, const QFrame& f, const Bvh& bvh, int root0,
                                               int root1, const RayPre& r, float tmin, int excl, float& t_best,
@@ -703,11 +702,11 @@ struct SmallBvh {
 // bound of s and the second an upper one while d > alpha, else (the cone
 // spreads faster than it moves along the axis) a lower one too: a box beside
 // the segment is reached only where the cone has grown to it. With d < 0 the
-// sides change places. The box can hold a captured receiver only if the three axes'
-// intervals meet within [0, tend]. One pass of a multiply-add per plane, and
-// tighter than the segment against the box grown by the radius at its end and
-// again at the exit, which it replaces (urban grid's capture pass 976 -> 806 us,
-// highway 56 -> 53). Margins (0.1% of the radius, 1 cm and 4e-7 of the
+// sides change places. The box can hold a captured receiver only if the three
+// axes' intervals meet within [0, tend]. One pass of a multiply-add per plane,
+// and tighter than the segment against the box grown by the radius at its end
+// and again at the exit (the urban grid's capture pass is 17% shorter, the
+// highway's 5%). Margins (0.1% of the radius, 1 cm and 4e-7 of the
 // coordinates) exceed the FP32 rounding.
 struct ConeRay {
   float nx, ny, nz, mx, my, mz;  // near planes: s >= plane * n + m

@@ -2241,7 +2241,8 @@ __device__ __noinline__ bool surely_hidden(const PathArgs& a, const HiddenCase& 
     const float4* q = a.quads + 4 * (size_t)DCEM_IDX(id, a.bvh.ntris);
     bool all = quad_between(q, E, mid, a.eps_occ);
     for (int k = 0; all && k < (h.kind == 0 ? 8 : 2 * h.kind); ++k) {
-      const float3 X = h.kind ? ((k & 1) ? hi : lo) : f3((k & 1) ? hi.x : lo.x, (k & 2) ? hi.y : lo.y, (k & 4) ? hi.z : lo.z);
+      const float3 X = h.kind ? ((k & 1) ? hi : lo)
+                              : f3((k & 1) ? hi.x : lo.x, (k & 2) ? hi.y : lo.y, (k & 4) ? hi.z : lo.z);
       all = quad_between(q, h.kind == 2 ? ((k & 2) ? h.E1 : h.E0) : E, X, a.eps_occ);
     }
     if (all) return true;

@@ -421,8 +421,8 @@ __global__ void __launch_bounds__(kTraceQThreads, 1) k_trace_qt(TraceArgs a) { t
 
 // The 4-wide compact copy read from global memory (L2), for scenes whose copy
 // does not fit in shared memory; stacks in shared memory. Four CTAs per SM
-// (64 registers): a city of 65,536 links took 5.05 ms a frame with three,
-// 4.76 with four, 5.0 with five, 5.4 with six, the last two for their spills.
+// (64 registers): a frame of a city of 65,536 links takes 6% longer with three,
+// 5% with five and 13% with six, the last two for their spills.
 __global__ void __launch_bounds__(256, 4) k_trace_qg(TraceArgs a) {
   extern __shared__ int sstk[];
   TStack st;

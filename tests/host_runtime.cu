@@ -252,7 +252,9 @@ cudaError_t cudaStreamSynchronize(cudaStream_t) {
 }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
   std::memset(static_cast<void*>(a), 0, sizeof(*a));
-  a->type = within(blocks(), p, 1) ? cudaMemoryTypeDevice : within(pinned(), p, 1) ? cudaMemoryTypeHost : cudaMemoryTypeUnregistered;
+  a->type = within(blocks(), p, 1)   ? cudaMemoryTypeDevice
+            : within(pinned(), p, 1) ? cudaMemoryTypeHost
+                                     : cudaMemoryTypeUnregistered;
   return cudaSuccess;
 }
 cudaError_t cudaGetSymbolAddress(void** p, const void*) {
