@@ -1107,7 +1107,10 @@ std::vector<float4> wall_quads(const std::vector<float>& tris, const std::vector
 // across the narrow sides first, and the rays that graze along the scene meet
 // every one of the long boxes it leaves (the 2 km highway: mean 8.8 -> 8.1
 // nodes, worst segment 74 -> 142, closest hit 28% longer; the radix tree halves
-// all axes alike). kSahMax bounds the build time
+// all axes alike). Roads of 60 to 2000 m (2 to 67 times longer than wide):
+// frames within 1% up to 5 times, 4% longer with these splits at 8, 18% at 67.
+// Rows of buildings, 4 to 48 times longer than wide, would be 6 to 20% shorter
+// with them; above the line they keep the tree that serves roads. kSahMax bounds the build time
 // on the host (5 ms for 50,000 triangles on eight threads); kSahLevels the
 // internal levels, to those that two binary levels a 4-wide one may have
 // (kWideLevels): halving takes over where the triangles left would need the
