@@ -897,13 +897,13 @@ __device__ __forceinline__ unsigned qenc_hi(float v, float o, float s) {
 // records the child (4-wide index, leaf ~slot, or kEmpty) and where its box
 // lives in the binary records (record << 1 | side).
 // Growing by area alone could give one 4-wide level per binary level, and a
-// traversal leaves three entries a level waiting: a child whose subtree is too
-// deep to stay (kWideLevels) is replaced before any other. Two levels at a
-// time always fit the bound once a node does, and a node has two children, so
-// the two replacements suffice.
+// traversal leaves three entries a level waiting: trees that would take more
+// than kWideLevels are mapped again, a child whose subtree is too deep to stay
+// replaced before any other. Two levels at a time always fit the bound once a
+// node does, and a node has two children, so the two replacements suffice.
 // Scratch, in shared memory or the global array `gscr` when that does not
-// fit: the binary node of every 4-wide node so far, and each binary node's
-// parent and height (internal levels of its subtree).
+// fit: the binary node of every 4-wide node so far, and for the second pass
+// each binary node's parent and height (internal levels of its subtree).
 __global__ void __launch_bounds__(1024) k_bvh4_map(const float4* __restrict__ nodes, int nn,
                                                     const int* __restrict__ roots, int4* kid4, int4* src4,
                                                     int* n4_out, int* roots4_out, int* gscr) {
@@ -921,74 +921,82 @@ __global__ void __launch_bounds__(1024) k_bvh4_map(const float4* __restrict__ no
     return x * y + y * h + h * x;
   };
   auto inner = [&](int c) { return c >= 0 && c < nn; };
-  for (int i = tid; i < nn; i += nt) {
-    par[i] = -1;
-    high[i] = 1;
-  }
-  __syncthreads();
-  for (int i = tid; i < nn; i += nt)
-    for (int side = 0; side < 2; ++side)
-      if (inner(kid(i, side))) par[kid(i, side)] = i;
-  __syncthreads();
-  // heights, from the nodes that hold two leaves up, until another branch was higher
-  for (int i = tid; i < nn; i += nt)
-    if (!inner(kid(i, 0)) && !inner(kid(i, 1)))
-      for (int h = 2, p = par[i]; p >= 0 && h < 4096 && atomicMax(&high[p], h) < h; ++h) p = par[p];
-  __syncthreads();
-  if (tid == 0) {
-    total = 0;
-    wide = kWideLevels;
-    for (int r = 0; r < 2; ++r) {
-      const int c = roots[r];
-      roots4_out[r] = inner(c) ? total : c;
-      if (!inner(c)) continue;
-      todo[total++] = c;
-      wide = max(wide, (high[c] + 1) / 2);
-    }
-  }
-  __syncthreads();
   int done = 0;
-  for (int level = 0; level < 4096; ++level) {
-    const int end = min(total, cap);
-    __syncthreads();
-    if (done >= end) break;
-    for (int i = done + tid; i < end; i += nt) {
-      const int n = todo[i];
-      int k[4] = {kid(n, 0), kid(n, 1), kEmpty, kEmpty}, sr[4] = {n << 1, (n << 1) | 1, 0, 0};
-      int m = 2;
-      for (int grow = 0; grow < 2; ++grow) {
-        int at = -1;
-        float best = -1.0f;
-        bool must = false;  // too deep for the next 4-wide level
-        for (int j = 0; j < m; ++j) {
-          if (!inner(k[j])) continue;
-          const float ar = area(sr[j] >> 1, sr[j] & 1);
-          const bool deep = level + 1 + (high[k[j]] + 1) / 2 > wide;
-          if (at < 0 || (deep && !must) || (deep == must && ar > best)) {
-            at = j;
-            best = ar;
-            must = deep;
-          }
-        }
-        if (at < 0) break;
-        const int c = k[at];
-        k[at] = kid(c, 0);
-        sr[at] = c << 1;
-        k[m] = kid(c, 1);
-        sr[m] = (c << 1) | 1;
-        ++m;
+  // by area alone; once more by height when that takes too many levels
+  for (int pass = 0; pass < 2; ++pass) {
+    if (pass) {
+      for (int i = tid; i < nn; i += nt) {
+        par[i] = -1;
+        high[i] = 1;
       }
-      for (int j = 0; j < m; ++j)
-        if (inner(k[j])) {
-          const int w = atomicAdd(&total, 1);
-          if (w < cap) todo[w] = k[j];
-          k[j] = w < cap ? w : kEmpty;  // (a malformed tree only)
-        }
-      kid4[i] = make_int4(k[0], k[1], k[2], k[3]);
-      src4[i] = make_int4(sr[0], sr[1], sr[2], sr[3]);
+      __syncthreads();
+      for (int i = tid; i < nn; i += nt)
+        for (int side = 0; side < 2; ++side)
+          if (inner(kid(i, side))) par[kid(i, side)] = i;
+      __syncthreads();
+      // heights, from the nodes that hold two leaves up, until another branch was higher
+      for (int i = tid; i < nn; i += nt)
+        if (!inner(kid(i, 0)) && !inner(kid(i, 1)))
+          for (int h = 2, p = par[i]; p >= 0 && h < 4096 && atomicMax(&high[p], h) < h; ++h) p = par[p];
+      __syncthreads();
     }
-    done = end;
+    if (tid == 0) {
+      total = 0;
+      wide = kWideLevels;
+      for (int r = 0; r < 2; ++r) {
+        const int c = roots[r];
+        roots4_out[r] = inner(c) ? total : c;
+        if (!inner(c)) continue;
+        todo[total++] = c;
+        if (pass) wide = max(wide, (high[c] + 1) / 2);
+      }
+    }
     __syncthreads();
+    done = 0;
+    for (int level = 0; level < (pass ? 4096 : kWideLevels); ++level) {
+      const int end = min(total, cap);
+      __syncthreads();
+      if (done >= end) break;
+      for (int i = done + tid; i < end; i += nt) {
+        const int n = todo[i];
+        int k[4] = {kid(n, 0), kid(n, 1), kEmpty, kEmpty}, sr[4] = {n << 1, (n << 1) | 1, 0, 0};
+        int m = 2;
+        for (int grow = 0; grow < 2; ++grow) {
+          int at = -1;
+          float best = -1.0f;
+          bool must = false;  // too deep for the next 4-wide level
+          for (int j = 0; j < m; ++j) {
+            if (!inner(k[j])) continue;
+            const float ar = area(sr[j] >> 1, sr[j] & 1);
+            const bool deep = pass && level + 1 + (high[k[j]] + 1) / 2 > wide;
+            if (at < 0 || (deep && !must) || (deep == must && ar > best)) {
+              at = j;
+              best = ar;
+              must = deep;
+            }
+          }
+          if (at < 0) break;
+          const int c = k[at];
+          k[at] = kid(c, 0);
+          sr[at] = c << 1;
+          k[m] = kid(c, 1);
+          sr[m] = (c << 1) | 1;
+          ++m;
+        }
+        for (int j = 0; j < m; ++j)
+          if (inner(k[j])) {
+            const int w = atomicAdd(&total, 1);
+            if (w < cap) todo[w] = k[j];
+            k[j] = w < cap ? w : kEmpty;  // (a malformed tree only)
+          }
+        kid4[i] = make_int4(k[0], k[1], k[2], k[3]);
+        src4[i] = make_int4(sr[0], sr[1], sr[2], sr[3]);
+      }
+      done = end;
+      __syncthreads();
+    }
+    __syncthreads();
+    if (done >= min(total, cap)) break;
   }
   if (tid == 0) *n4_out = min(total, cap);
 }
